@@ -2,8 +2,11 @@
 // generator (integer work, bit-exact).
 #include <math.h>
 
+#include <type_traits>
+
 #include "basis.cuh"
 #include "common.cuh"
+#include "gauss.cuh"
 
 namespace hphi {
 
@@ -144,29 +147,35 @@ __global__ void k_philox_raw(const uint32_t* __restrict__ ctr, const uint32_t* _
 // 0, 0)) gives two 53-bit open-interval uniforms and, by Box-Muller, the pair
 // g0 = sqrt(-2 ln u_a) cos(2 pi u_b), g1 = sqrt(-2 ln u_a) sin(2 pi u_b).  A complex element e
 // is g0 + i g1 of block e; real elements 2p and 2p + 1 are g0 and g1 of block p, so no half
-// of a pair is wasted (GB300 runs the fp64 logarithm and sine / cosine at 1/64 of its fp32
-// rate).  One thread per block.
+// of a pair is wasted.  One thread per block.  fp64 pairs come from the integer transform of
+// gauss.cuh, whose tables each CTA stages in shared memory (random 8- and 16-byte reads).
+__device__ constexpr GaussTables kGaussTables = gauss_detail::make_tables();
+
 template <bool CPLX, bool F64>
-__global__ void k_random(void* __restrict__ v, int64_t n_elem, uint64_t seed) {
+__global__ void __launch_bounds__(kThreads) k_random(void* __restrict__ v, int64_t n_elem, uint64_t seed) {
+  __shared__ std::conditional_t<F64, GaussTables, int> s_tab;
+  if constexpr (F64) {
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(&kGaussTables);
+    for (int k = threadIdx.x; k < (int)(sizeof(GaussTables) / 4); k += kThreads)
+      reinterpret_cast<uint32_t*>(&s_tab)[k] = src[k];
+    __syncthreads();
+  }
+  const bool wide = (reinterpret_cast<uintptr_t>(v) & 15u) == 0;  // both numbers of a pair in one store
   const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
   const int64_t n_blk = CPLX ? n_elem : (n_elem + 1) / 2;
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n_blk; p += (int64_t)gridDim.x * blockDim.x) {
     const uint4 o = philox(make_uint4((uint32_t)p, (uint32_t)((uint64_t)p >> 32), 0u, 0u), key);
     const uint64_t a = ((((uint64_t)o.x) << 32) | o.y) >> 11;
     const uint64_t b = ((((uint64_t)o.z) << 32) | o.w) >> 11;
-    if (F64) {
-      const double ua = ((double)a + 0.5) * (1.0 / 9007199254740992.0);
-      const double ub = ((double)b + 0.5) * (1.0 / 9007199254740992.0);
-      const double rad = sqrt(-2.0 * log(ua));
-      double sn, cs;
-      sincospi(2.0 * ub, &sn, &cs);
-      const double g0 = rad * cs, g1 = rad * sn;
-      if (CPLX) {
-        reinterpret_cast<double2*>(v)[p] = make_double2(g0, g1);
+    if constexpr (F64) {
+      double g0, g1;
+      gauss_pair(a, b, s_tab, g0, g1);
+      double* x = reinterpret_cast<double*>(v) + 2 * p;
+      if (wide && (CPLX || 2 * p + 1 < n_elem)) {
+        *reinterpret_cast<double2*>(x) = make_double2(g0, g1);
       } else {
-        double* x = reinterpret_cast<double*>(v);
-        x[2 * p] = g0;
-        if (2 * p + 1 < n_elem) x[2 * p + 1] = g1;
+        x[0] = g0;
+        if (CPLX || 2 * p + 1 < n_elem) x[1] = g1;
       }
     } else {
       // fp32 storage: the same two uniforms, rounded to fp32 (relative error 2^-24, also in
