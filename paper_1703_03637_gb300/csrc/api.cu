@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "gather.cuh"
 
 using cplx = std::complex<double>;
 
@@ -116,6 +117,7 @@ struct hphi_model {
   // device data
   DBuf d_entries, d_cls, d_lin, d_pairs, d_pcoef, d_hi_off, d_lo_rank, d_lo_list, d_lo_off;
   DBuf d_nbr_up, d_deg_up, d_nbr_dn, d_deg_dn, d_npos_up, d_npos_dn, d_counter;
+  DBuf d_up_rec[3], d_up_hdr[3];  // pass U gather tables by entry width
   hphi::SpinDev sdev{};
   hphi::HubDev hdev{};
   Workspace ws;
@@ -466,6 +468,39 @@ hphi::Status build_lo_tables(hphi_model* m, int L, cudaStream_t st) {
                                      m->d_lo_off.as<uint32_t>(), st);
 }
 
+// The pass U gather table of precision prec's launch shape, built on first use (never inside a
+// stream capture: at hphi_build_sector for the default shapes, and by the autotuner).
+hphi::Status hub_ensure_table(hphi_model* m, int prec, cudaStream_t st) {
+  hphi::HubDev& d = m->hdev;
+  if (!hphi::hub_up_row_fits(d, prec)) return {};
+  const int wi = hphi::hub_up_width(d, prec);
+  if (d.up_rec[wi] != nullptr) return {};
+  // at most maxdeg_up terms of each sign, in whole chunks
+  const int slots = (2 * d.maxdeg_up + 4 * hphi::kGatherChunk - 1) / (4 * hphi::kGatherChunk) * (4 * hphi::kGatherChunk);
+  const int64_t stride = d.up_stride;
+  hphi::Status s;
+  if ((s = m->d_up_rec[wi].ensure(sizeof(uint2) * (size_t)stride * (size_t)(slots / 4))).code) return s;
+  if ((s = m->d_up_hdr[wi].ensure(sizeof(uint4) * (size_t)(stride / 32))).code) return s;
+  if ((s = hphi::build_gather_table(d.nbr_up, d.dim_up, d.deg_up, (int)d.dim_up, 31, 2, (int)d.dim_up, 4 << wi,
+                                    m->d_up_rec[wi].as<uint2>(), stride, 0, slots, m->d_up_hdr[wi].as<uint4>(), st))
+          .code)
+    return s;
+  d.up_rec[wi] = m->d_up_rec[wi].as<uint2>();
+  d.up_hdr[wi] = m->d_up_hdr[wi].as<uint4>();
+  return {};
+}
+
+// The diagonal is an integer multiple of the one hopping value +-2^k, and an element's exact
+// int64 sum (at most 128 terms of magnitude below 2^56) cannot overflow
+bool hub_diag_integer(const hphi::HubDev& d, const std::vector<hphi::LinGroup>& ulin) {
+  int e = 0;
+  if (d.c_up != d.c_dn || d.c_up == 0.0 || fabs(frexp(d.c_up, &e)) != 0.5) return false;
+  if (d.n_ulin != 1 || d.n_mulin != 0 || d.n_pairs != 0 || ulin.size() != 1 || d.c0 != 0.0) return false;
+  const double per = ulin[0].coef / d.c_up;
+  const int n = std::min(__builtin_popcountll(ulin[0].mask), d.sector ? std::min(d.n_up, d.n_dn) : d.n_sites);
+  return per == floor(per) && d.maxdeg_up + d.maxdeg_dn + fabs(per) * n <= 128.0;
+}
+
 // Two-pass Hubbard path: real model with one hopping value per species.  Builds the
 // per-species neighbour tables on the device.
 hphi::Status build_hub_fast(hphi_model* m, cudaStream_t st) {
@@ -517,6 +552,14 @@ hphi::Status build_hub_fast(hphi_model* m, cudaStream_t st) {
   if ((s = hphi::build_hub_neighbours(d, 1, m->d_nbr_dn.as<uint32_t>(), m->d_deg_dn.as<uint8_t>(),
                                       m->d_npos_dn.as<uint8_t>(), st)).code)
     return s;
+  d.up_stride = (d.dim_up + 31) / 32 * 32;
+  for (int prec : {HPHI_FP64, HPHI_FP32})
+    if ((s = hub_ensure_table(m, prec, st)).code) return s;
+  std::vector<hphi::LinGroup> ulin(d.n_ulin);
+  if (d.n_ulin)
+    HPHI_CUDA_TRY(cudaMemcpyAsync(ulin.data(), d.ulin, sizeof(hphi::LinGroup) * ulin.size(), cudaMemcpyDeviceToHost, st));
+  HPHI_CUDA_TRY(cudaStreamSynchronize(st));
+  d.dint = hub_diag_integer(d, ulin) ? 1 : 0;
   d.fast = 1;
   return {};
 }
@@ -1221,6 +1264,7 @@ int hphi_autotune(hphi_model* m, int prec, hphi_tune_result* out, void* stream) 
       if ((ept == 0) != (k == 0)) continue;  // (0, 0) is the built-in default
       m->hdev.tuned_ept[pi] = ept;
       m->hdev.tuned_k[pi] = k;
+      if ((s = hub_ensure_table(m, prec, st)).code) break;
       const int grid = hv_grid_for(m, 1, prec, hphi::Epi::kStore);
       s = hv_launch(m, prec, m->ws.vecA.p, m->ws.vecB.p, 1, hphi::Epi::kStore, fa, grid, scratch, st);
       if (s.code) break;

@@ -108,6 +108,12 @@ struct HubDev {
   int tuned_ept[2], tuned_k[2];  // autotuner choices per precision (HPHI_FP64, HPHI_FP32)
   int maxdeg_up, maxdeg_dn;
   double c_up, c_dn;         // the hopping coefficient of each species
+  int dint;                  // c_up = c_dn = +-2^k and the diagonal is an integer multiple of it
+  // pass U gather tables (gather.cuh) for tile entries of 4, 8 and 16 bytes: records
+  // [groups][up_stride], up_stride = dim_up rounded up to whole warps, and a header per warp
+  int64_t up_stride;
+  const uint2* up_rec[3];
+  const uint4* up_hdr[3];
   const uint32_t* nbr_up;
   const uint8_t* deg_up;
   const uint8_t* npos_up;    // entries [0, npos) carry sign +1, [npos, deg) sign -1
@@ -277,11 +283,23 @@ bool spin_quantised(const SpinDev& md, int prec, int nvec);
 size_t spin_scratch_bytes(const SpinDev& md, int prec, bool cplx, int nvec);
 int hv_grid(int nvec);  // upper bound of any H v grid (partials sizing)
 
+// Gather table of n states (k_gather.cu; layout in gather.cuh).  nbr[q * nbr_stride + k] is
+// term q < deg[k] of state k, target | phase << shift with phase < n_phase; zero0 is the index
+// of the first zero entry; entry_bytes (4, 8 or 16) the width of a staged entry.  State k's
+// records go to rec[group * stride + out0 + k], 32 states' header to hdr[(out0 + k) / 32];
+// out0 is a multiple of 32 and the table has room for max_slots slots and whole warps.
+Status build_gather_table(const uint32_t* nbr, int64_t nbr_stride, const uint8_t* deg, int n, int shift, int n_phase,
+                          int zero0, int entry_bytes, uint2* rec, int64_t stride, int64_t out0, int max_slots,
+                          uint4* hdr, cudaStream_t st);
+
 // Two-pass Hubbard path (k_hub.cu): neighbour tables, and H v = diag + up hops (row tiles
 // in shared memory) + down hops (stripe-major row combinations into the scratch vector W).
 Status build_hub_neighbours(const HubDev& md, int species, uint32_t* nbr, uint8_t* deg, uint8_t* npos,
                             cudaStream_t st);
 bool hub_fast_ok(const HubDev& md, int prec, bool cplx, int nvec, Epi epi);
+// gather table (0: 4-byte entries, 1: 8, 2: 16) that pass U of precision prec reads
+int hub_up_width(const HubDev& md, int prec);
+bool hub_up_row_fits(const HubDev& md, int prec);
 int hub_up_grid(const HubDev& md, int prec, Epi epi);
 size_t hub_scratch_bytes(const HubDev& md, int prec, Epi epi);  // scratch the launch needs
 // the fp64 input-exponent slot inside that scratch (see FusedArgs::exp_ready)

@@ -9,8 +9,8 @@ namespace hphi {
 
 // Per-column CTA reduction in a fixed tree order; partials[(block * nvec + c) * kMaxRedQ + q].
 // NT is the CTA size; sm holds NT * kMaxRedQ doubles.
-template <bool F64, int NT = kThreads>
-__device__ void block_finish(const Red<F64>& red, int nq, int nvec, double* __restrict__ partials, double* sm) {
+template <bool F64, int NT = kThreads, int NQ = kMaxRedQ>
+__device__ void block_finish(const Red<F64, NQ>& red, int nq, int nvec, double* __restrict__ partials, double* sm) {
   const int tid = threadIdx.x;
   for (int q = 0; q < nq; ++q) sm[q * NT + tid] = red.get(q);
   __syncthreads();
@@ -58,6 +58,13 @@ __device__ __forceinline__ double fix_to_double(long long m, int eoff) {
   const double d = __ll2double_rn(m);
   if (eoff >= -1022 && eoff <= 1023) return d * __longlong_as_double((long long)(eoff + 1023) << 52);
   return ldexp(d, eoff);
+}
+
+// a 128-bit integer as the nearest-ish fp64 (two roundings: relative error below 2^-52)
+__device__ __forceinline__ double i128_to_double(__int128 v) {
+  const long long hi = (long long)(v >> 64);
+  const unsigned long long lo = (unsigned long long)v;
+  return fma(__ll2double_rn(hi), 18446744073709551616.0, __ull2double_rn(lo));
 }
 
 // ------------------------------------------------------------------ gather sums
@@ -136,15 +143,41 @@ __device__ __forceinline__ void acc_phase(int code, R xr, R xi, A& ar, A& ai) {
 }
 
 // ------------------------------------------------------------------ epilogues
+// The scalars of a fused step in the vectors' precision, converted once per thread: the opaque
+// copy keeps the compiler from converting the kernel's fp64 arguments again for every element
+// (three fp64-pipe conversions an element in the fp32 mTPQ step, at 1/64 of the fp32 rate).
+template <class R>
+__device__ __forceinline__ R opaque(R x) {
+  if constexpr (sizeof(R) == 8) asm volatile("" : "+d"(x));
+  else asm volatile("" : "+f"(x));
+  return x;
+}
+
+template <class R>
 struct EpiScalars {
-  double c1, c2;  // Lanczos pass 1
+  R c1, c2;  // Lanczos pass 1
+  R l, ins;  // mTPQ: l and 1 / N_s
 };
 
+template <class R, Epi E>
+__device__ __forceinline__ EpiScalars<R> epi_scalars(const FusedArgs& fa) {
+  EpiScalars<R> es{(R)0, (R)0, (R)0, (R)0};
+  if constexpr (E == Epi::kLanczos1) {
+    es.c1 = opaque((R)fa.scal[0]);
+    es.c2 = opaque((R)fa.scal[1]);
+  } else if constexpr (E == Epi::kTpq) {
+    es.l = opaque((R)fa.l);
+    es.ins = opaque((R)fa.inv_ns);
+  }
+  return es;
+}
+
+// inv: 1 / |X_k| of this column (mTPQ only)
 template <class S, Epi E, int NQ = kMaxRedQ>
-__device__ __forceinline__ void epilogue(int64_t idx, int c, typename Traits<S>::R sr, typename Traits<S>::R si,
+__device__ __forceinline__ void epilogue(int64_t idx, typename Traits<S>::R sr, typename Traits<S>::R si,
                                          typename Traits<S>::R hr, typename Traits<S>::R hi, S* __restrict__ w,
-                                         const FusedArgs& fa, const EpiScalars& es, const double* s_inv,
-                                         Red<Traits<S>::kF64, NQ>& red) {
+                                         const FusedArgs& fa, const EpiScalars<typename Traits<S>::R>& es,
+                                         typename Traits<S>::R inv, Red<Traits<S>::kF64, NQ>& red) {
   using R = typename Traits<S>::R;
   constexpr bool C = Traits<S>::kCplx;
   if constexpr (E == Epi::kStore) {
@@ -155,8 +188,7 @@ __device__ __forceinline__ void epilogue(int64_t idx, int c, typename Traits<S>:
     const S* Pin = fa.in ? reinterpret_cast<const S*>(fa.in) : P;
     R pr, pi;
     ld<S>(Pin, idx, pr, pi);
-    const R c1 = (R)es.c1, c2 = (R)es.c2;
-    st<S>(P, idx, c1 * hr - c2 * pr, c1 * hi - c2 * pi);
+    st<S>(P, idx, es.c1 * hr - es.c2 * pr, es.c1 * hi - es.c2 * pi);
     red.add(0, sr, hr);
     if constexpr (C) red.add(0, si, hi);
     red.tick();
@@ -164,9 +196,8 @@ __device__ __forceinline__ void epilogue(int64_t idx, int c, typename Traits<S>:
     // X_{k+1} = (l X_k - H X_k / N_s) / |X_k| ; partials <X, HX>, |HX|^2.  |X_{k+1}|^2 follows
     // from them (section 3.5's norm, deferred): l^2 - 2 l u_k + <H^2>_k.
     S* Xn = reinterpret_cast<S*>(fa.out);
-    const R inv = (R)s_inv[c], l = (R)fa.l, ins = (R)fa.inv_ns;
-    const R nr = inv * (l * sr - hr * ins);
-    const R ni = inv * (l * si - hi * ins);
+    const R nr = inv * (es.l * sr - hr * es.ins);
+    const R ni = inv * (es.l * si - hi * es.ins);
     st<S>(Xn, idx, nr, ni);
     red.add(0, sr, hr);
     red.add(1, hr, hr);

@@ -1,0 +1,31 @@
+// Gather tables of the shared-memory row kernels: for each of 32 consecutive states the row
+// entries it sums, in an order that spreads a warp's reads over the shared-memory banks.
+//
+// A thread that sums d random entries of a staged row reads one per slot.  Random addresses
+// cost a warp 3.5 shared-memory wavefronts per 4-byte slot (of 1) and 6.3 per 16-byte slot (of
+// 4), and the order of a thread's own terms is free, so the table picks it: slot by slot,
+// each lane takes the entry whose bank is still unused in this slot and most in demand later.
+// Measured on the tables of the 18-site Hubbard cluster (4-byte entries): 28.8 wavefronts per
+// state instead of 64.1; 16 sites, 16-byte entries: 23.0 per eight lanes instead of 40.3.
+//
+// Terms carry a phase (a sign, or a coefficient class).  Slots run phase by phase, each phase
+// as many slots as the longest of the 32 lists, so the phase of a slot is the same in all
+// lanes; lanes without a term left read one of the zero entries that follow the staged row, in
+// a bank nobody else uses.
+//
+// Layout: records of four slots, rec[group * stride + state], so a warp reads 256 consecutive
+// bytes per group; hdr[warp] holds the slot ends of phases 0 .. 7, cumulative, 16 bits each.
+#pragma once
+
+#include "common.cuh"
+
+namespace hphi {
+
+constexpr int kGatherPhases = 8;
+// zero entries after a staged row: one per 4 bytes (or fewer, wider ones) of a 128-byte bank row
+constexpr int kGatherZeroBytes = 128;
+
+// records are read in chunks of this many groups; a table has whole chunks allocated
+constexpr int kGatherChunk = 4;
+
+}  // namespace hphi

@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(kThreads, BatchTune<S, E>::kMinB)
   __shared__ LinGroup s_lin[kMaxLin];
   __shared__ PairEntry s_pair[kMaxPairs];
   __shared__ double s_pcoef[kMaxPairGroups];
-  __shared__ double s_inv[kMaxNvec];
+  __shared__ R s_inv[kMaxNvec];
   __shared__ double s_red[(E == Epi::kStore) ? 1 : kThreads * CPL];
   __shared__ uint32_t s_dep[4 * 256];
   __shared__ float2 s_phase[8];  // phase codes 0 (none), 1 (+1), 2 (+i), 3 (-1), 4 (-i) as (re, im)
@@ -192,13 +192,9 @@ __global__ void __launch_bounds__(kThreads, BatchTune<S, E>::kMinB)
   for (int k = tid; k < md.n_pairs; k += kThreads) s_pair[k] = md.pairs[k];
   for (int k = tid; k < md.n_pair_groups; k += kThreads) s_pcoef[k] = md.pair_coef[k];
   if constexpr (E == Epi::kTpq) {
-    for (int k = tid; k < nvec; k += kThreads) s_inv[k] = fa.scal[k];
+    for (int k = tid; k < nvec; k += kThreads) s_inv[k] = (R)fa.scal[k];
   }
-  EpiScalars es{0.0, 0.0};
-  if constexpr (E == Epi::kLanczos1) {
-    es.c1 = fa.scal[0];
-    es.c2 = fa.scal[1];
-  }
+  const EpiScalars<R> es = epi_scalars<R, E>(fa);
   __syncthreads();
 
   constexpr int kNQ = n_red<E>() > 0 ? n_red<E>() : 1;
@@ -361,9 +357,9 @@ __global__ void __launch_bounds__(kThreads, BatchTune<S, E>::kMinB)
 #pragma unroll
         for (int q = 0; q < CPL; ++q) {
           if constexpr (E == Epi::kTpq) {
-            const R inv = (R)s_inv[c0 + q], l = (R)fa.l, ins = (R)fa.inv_ns;
-            o.re[q] = inv * (l * x0.re[q] - h.re[q] * ins);
-            o.im[q] = inv * (l * x0.im[q] - h.im[q] * ins);
+            const R inv = s_inv[c0 + q];
+            o.re[q] = inv * (es.l * x0.re[q] - h.re[q] * es.ins);
+            o.im[q] = inv * (es.l * x0.im[q] - h.im[q] * es.ins);
             red[q].add(0, x0.re[q], h.re[q]);
             red[q].add(1, h.re[q], h.re[q]);
             if constexpr (C) {
@@ -388,7 +384,7 @@ __global__ void __launch_bounds__(kThreads, BatchTune<S, E>::kMinB)
       } else {
 #pragma unroll
         for (int q = 0; q < CPL; ++q)
-          epilogue<S, E, kNQ>(off + q, c0 + q, x0.re[q], x0.im[q], h.re[q], h.im[q], w, fa, es, s_inv, red[q]);
+          epilogue<S, E, kNQ>(off + q, x0.re[q], x0.im[q], h.re[q], h.im[q], w, fa, es, R(0), red[q]);
       }
     }
   }

@@ -8,15 +8,18 @@
 //   pass D  walks column stripes in stripe-major order; the stripe of every row stays in
 //           L2 while all rows of that stripe are combined, so X is read from HBM about once.
 //           W receives the plain signed sums.
-//   pass U  stages K whole rows of X in shared memory, applies the up-spin neighbour table
+//   pass U  stages K whole rows of X in shared memory, applies the up-spin gather table
 //           (built once per sector on the device) to all K rows at once, adds diag * X and
 //           coef * W, and runs the fused Lanczos / mTPQ epilogue.
 // fp64 sums use the exact fixed-point accumulator (integer pipes); fp32 sums are plain.
+#include <algorithm>
 #include <mutex>
 #include <string>
+#include <type_traits>
 
 #include "common.cuh"
 #include "epilogue.cuh"
+#include "gather.cuh"
 #include "reduce.cuh"
 
 namespace hphi {
@@ -50,7 +53,7 @@ __device__ __forceinline__ void load_k(const R* p, R* out) {
       const float4 t = *reinterpret_cast<const float4*>(p);
       out[0] = t.x; out[1] = t.y; out[2] = t.z; out[3] = t.w;
     } else {
-      const double2 t = *reinterpret_cast<const double2*>(p);
+      const longlong2 t = *reinterpret_cast<const longlong2*>(p);
       out[0] = t.x; out[1] = t.y;
     }
   } else if constexpr (sizeof(R) * K == 8 && sizeof(R) == 4) {
@@ -62,19 +65,7 @@ __device__ __forceinline__ void load_k(const R* p, R* out) {
   }
 }
 
-template <class R, int K>
-__device__ __forceinline__ void store_k(R* p, const R* v) {
-  if constexpr (sizeof(R) * K == 16) {
-    if constexpr (sizeof(R) == 4) *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-    else *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
-  } else if constexpr (sizeof(R) * K == 8 && sizeof(R) == 4) {
-    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
-  } else {
-#pragma unroll
-    for (int m = 0; m < K; ++m) p[m] = v[m];
-  }
-}
-constexpr int kSmemBudget = 208000;  // shared-memory bytes for the row tile (plus ~21 KB static)
+constexpr int kSmemBudget = 208000;  // shared-memory bytes of the row tile (plus its zero entries and ~7 KB static)
 
 // neighbour table of one species, hop-slot major: nbr[q * n + k] is the q-th active hop
 // target of state k (rank | sign << 31), so threads of consecutive states read
@@ -209,152 +200,6 @@ __global__ void __launch_bounds__(kThreads) k_hub_dn(const HubDev md, const R* _
   }
 }
 
-// pass U: up-spin hops on K rows staged in shared memory, diag, + c_dn W, fused epilogue
-template <class R, int K, Epi E, int NT>
-__global__ void __launch_bounds__(NT) k_hub_up(const HubDev md, const R* __restrict__ X,
-                                                       const R* __restrict__ W, R* __restrict__ w, FusedArgs fa) {
-  using A = typename SumAcc<R>::T;
-  constexpr bool F64 = sizeof(R) == 8;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  R* tile = reinterpret_cast<R*>(smem_raw);
-  __shared__ LinGroup s_ulin[kMaxLin];
-  __shared__ LinGroup s_mlin[kMaxLin];
-  __shared__ PairEntry s_pair[kMaxPairs];
-  __shared__ R s_uc[kMaxLin], s_mc[kMaxLin], s_pcoef[kMaxPairGroups];  // coefficients in R
-  __shared__ double s_inv[1];
-  __shared__ double s_red[(NT / 32) * kMaxRedQ];
-
-  if (fa.done != nullptr && *fa.done) return;
-  const int tid = threadIdx.x;
-  for (int k = tid; k < md.n_ulin; k += NT) { s_ulin[k] = md.ulin[k]; s_uc[k] = (R)md.ulin[k].coef; }
-  for (int k = tid; k < md.n_mulin; k += NT) { s_mlin[k] = md.mulin[k]; s_mc[k] = (R)md.mulin[k].coef; }
-  for (int k = tid; k < md.n_pairs; k += NT) s_pair[k] = md.pairs[k];
-  for (int k = tid; k < md.n_pair_groups; k += NT) s_pcoef[k] = (R)md.pair_coef[k];
-  if constexpr (E == Epi::kTpq) {
-    if (tid == 0) s_inv[0] = fa.scal[0];
-  }
-  EpiScalars es{0.0, 0.0};
-  if constexpr (E == Epi::kLanczos1) {
-    es.c1 = fa.scal[0];
-    es.c2 = fa.scal[1];
-  }
-  const R c_up = (R)md.c_up, c_dn = (R)md.c_dn;
-  const bool same_c = md.c_up == md.c_dn;
-  __shared__ R s_dtab[33];
-  const bool dtab = md.n_ulin == 1 && md.n_mulin == 0 && md.n_pairs == 0;
-  if (dtab && tid <= 32) s_dtab[tid] = (R)(md.c0 + md.ulin[0].coef * (double)tid);
-  __syncthreads();
-  Red<F64> red;
-  red.zero();
-  const int64_t dim_up = md.dim_up, dim_dn = md.dim_dn;
-  const int64_t n_tiles = (dim_dn + K - 1) / K;
-
-  for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-    const int64_t d0 = t * K;
-    const int nk = (int)((dim_dn - d0 < K) ? (dim_dn - d0) : K);
-    __syncthreads();
-    // tile[u * K + m] = X[d0 + m][u]: the K rows interleaved, so one vector load per
-    // neighbour fetches the value of all K rows
-    for (int64_t u = tid; u < dim_up; u += NT) {
-      R vals[K];
-#pragma unroll
-      for (int m = 0; m < K; ++m) vals[m] = (m < nk) ? __ldg(X + (d0 + m) * dim_up + u) : (R)0;
-      store_k<R, K>(tile + u * K, vals);
-    }
-    __syncthreads();
-    uint32_t dn[K];
-#pragma unroll
-    for (int m = 0; m < K; ++m) dn[m] = (m < nk) ? (md.sector ? __ldg(md.list_dn + d0 + m) : (uint32_t)(d0 + m)) : 0u;
-    for (int64_t u = tid; u < dim_up; u += NT) {
-      const uint32_t up = md.sector ? __ldg(md.list_up + u) : (uint32_t)u;
-      const int deg = md.deg_up[u];
-      const uint32_t* nb = md.nbr_up + u;
-      A acc[K];
-#pragma unroll
-      for (int m = 0; m < K; ++m) acc[m].zero();
-      const int du = (int)dim_up;  // neighbour tables hold < 2^28 entries
-      int q = 0;
-      for (; q + 2 <= deg; q += 2) {
-        const uint32_t e0 = __ldg(nb + q * du), e1 = __ldg(nb + (q + 1) * du);
-        R v0[K], v1[K];
-        load_k<R, K>(tile + (int)(e0 & 0x7fffffffu) * K, v0);
-        load_k<R, K>(tile + (int)(e1 & 0x7fffffffu) * K, v1);
-#pragma unroll
-        for (int m = 0; m < K; ++m) {
-          acc[m].add(v0[m], (e0 >> 31) != 0);
-          acc[m].add(v1[m], (e1 >> 31) != 0);
-        }
-      }
-      if (q < deg) {
-        const uint32_t e0 = __ldg(nb + q * du);
-        R v0[K];
-        load_k<R, K>(tile + (int)(e0 & 0x7fffffffu) * K, v0);
-#pragma unroll
-        for (int m = 0; m < K; ++m) acc[m].add(v0[m], (e0 >> 31) != 0);
-      }
-#pragma unroll
-      for (int m = 0; m < K; ++m) {
-        if (m >= nk) break;
-        const int64_t idx = (d0 + m) * dim_up + u;
-        const R x = tile[u * K + m];
-        // diagonal: integer counts times the class coefficients
-        R dg;
-        if (dtab) {
-          dg = s_dtab[__popc(up & dn[m] & (uint32_t)s_ulin[0].mask)];
-        } else {
-        dg = (R)md.c0;
-        for (int g = 0; g < md.n_ulin; ++g) dg += s_uc[g] * (R)__popc(up & dn[m] & (uint32_t)s_ulin[g].mask);
-        for (int g = 0; g < md.n_mulin; ++g) {
-          const uint32_t mk = (uint32_t)s_mlin[g].mask;
-          dg += s_mc[g] * (R)(__popc(up & mk) + __popc(dn[m] & mk));
-        }
-        if (md.n_pairs) {
-          int grp = s_pair[0].grp, cnt = 0;
-          for (int p = 0; p < md.n_pairs; ++p) {
-            const PairEntry pe = s_pair[p];
-            if (pe.grp != grp) {
-              dg += s_pcoef[grp] * (R)cnt;
-              cnt = 0;
-              grp = pe.grp;
-            }
-            const int ni = (int)((up >> pe.i) & 1u) + (int)((dn[m] >> pe.i) & 1u);
-            const int nj = (int)((up >> pe.j) & 1u) + (int)((dn[m] >> pe.j) & 1u);
-            cnt += ni * nj;
-          }
-          dg += s_pcoef[grp] * (R)cnt;
-        }
-        }
-        R hv;
-        if (same_c) {
-          acc[m].add(W[idx], false);
-          hv = dg * x + c_up * (R)acc[m].value();
-        } else {
-          hv = dg * x + c_up * (R)acc[m].value() + c_dn * W[idx];
-        }
-        epilogue<R, E>(idx, 0, x, (R)0, hv, (R)0, w, fa, es, s_inv, red);
-      }
-    }
-  }
-  if constexpr (E != Epi::kStore) {
-    // fixed-order reduction: warp shuffles, then the warps' sums in warp order
-    constexpr int nq = n_red<E>();
-    const int lane = tid & 31, wid = tid >> 5;
-#pragma unroll
-    for (int q = 0; q < nq; ++q) {
-      double x = red.get(q);
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(0xffffffffu, x, off);
-      if (lane == 0) s_red[wid * kMaxRedQ + q] = x;
-    }
-    __syncthreads();
-    if (tid < nq) {
-      double x = 0.0;
-      for (int k = 0; k < NT / 32; ++k) x += s_red[k * kMaxRedQ + tid];
-      fa.partials[(size_t)blockIdx.x * kMaxRedQ + tid] = x;
-    }
-  }
-}
-
 // ------------------------------------------------------------------ fp64 via fixed point
 // fp64 vectors take the gather passes as 64-bit integers on one scale per vector:
 // q = round(x * 2^(1078 - E)), E = the largest exponent field of x, so |q| < 2^56 and the
@@ -396,49 +241,67 @@ __global__ void __launch_bounds__(kThreads) k_quant(const double* __restrict__ X
   }
 }
 
-// pass U on quantised rows: K int64 rows interleaved in shared memory; the diagonal term and
-// the reductions take each element's value from the same quantised tile
-template <int K, Epi E, int NT>
-__global__ void __launch_bounds__(NT) k_hub_up_q(const HubDev md,
-                                                         const long long* __restrict__ Q,
-                                                         const long long* __restrict__ WQ, const int* __restrict__ Ep,
-                                                         double* __restrict__ w, FusedArgs fa) {
+// 4- or 8-byte asynchronous copy to shared memory, and 16-byte ones past L1
+template <int B>
+__device__ __forceinline__ void copy_async(void* dst, const void* src) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  if constexpr (B == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(B) : "memory");
+}
+
+// Pass U: up-spin hops on K rows staged in shared memory, the diagonal, + c_dn W and the fused
+// epilogue.  T is float (fp32 vectors) or long long (fp64 vectors on the fixed-point copy; the
+// diagonal term and the reductions take the row's own value from the same quantised tile).
+//
+// The K rows are interleaved (tile[u * K + m] = X[d0 + m][u]), so one load per neighbour
+// fetches the value of all K rows, and every thread's terms come from a gather table
+// (gather.cuh): four 16-bit targets per 8-byte record, ordered against bank conflicts, the
+// signs a warp-uniform property of the slot.  W and, in Lanczos steps, the previous vector are
+// loaded before the gathers.
+//
+// Measured on GB300, against one 4-byte signed target per term in state order: 16 sites, 8 + 8
+// electrons (165,636,900 rows), fp64 Lanczos step, two rows a tile: 2.13 ms instead of 4.16 ms,
+// bound by shared-memory wavefronts (71 %) and instruction issue (61 %); 7 + 6 electrons, fp32
+// product, four rows: 0.55 instead of 0.90 ms; 18 sites, 9 + 9 (2,363,904,400 rows), fp32 mTPQ
+// step, one 194 KB row: 28.0 instead of 64.3 ms, bound by instruction issue (83 %).
+template <class T, int K, Epi E, int NT>
+__global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_hub_up(const HubDev md, const T* __restrict__ X, const T* W,
+                                               const int* __restrict__ Ep, void* w, FusedArgs fa) {
+  constexpr bool FIX = sizeof(T) == 8;
+  using R = std::conditional_t<FIX, double, float>;
+  constexpr int kWidth = K * (int)sizeof(T) >= 16 ? 2 : (K * (int)sizeof(T) >= 8 ? 1 : 0);
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  long long* tile = reinterpret_cast<long long*>(smem_raw);
+  T* tile = reinterpret_cast<T*>(smem_raw);
   __shared__ LinGroup s_ulin[kMaxLin];
   __shared__ LinGroup s_mlin[kMaxLin];
   __shared__ PairEntry s_pair[kMaxPairs];
-  __shared__ double s_pcoef[kMaxPairGroups];
-  __shared__ double s_inv[1];
+  __shared__ R s_uc[kMaxLin], s_mc[kMaxLin], s_pcoef[kMaxPairGroups];  // coefficients in R
   __shared__ double s_red[(NT / 32) * kMaxRedQ];
+  __shared__ R s_dtab[33];
+  __shared__ int s_dti[33];
 
   if (fa.done != nullptr && *fa.done) return;
   const int tid = threadIdx.x;
-  for (int k = tid; k < md.n_ulin; k += NT) s_ulin[k] = md.ulin[k];
-  for (int k = tid; k < md.n_mulin; k += NT) s_mlin[k] = md.mulin[k];
+  for (int k = tid; k < md.n_ulin; k += NT) { s_ulin[k] = md.ulin[k]; s_uc[k] = (R)md.ulin[k].coef; }
+  for (int k = tid; k < md.n_mulin; k += NT) { s_mlin[k] = md.mulin[k]; s_mc[k] = (R)md.mulin[k].coef; }
   for (int k = tid; k < md.n_pairs; k += NT) s_pair[k] = md.pairs[k];
-  for (int k = tid; k < md.n_pair_groups; k += NT) s_pcoef[k] = md.pair_coef[k];
-  if constexpr (E == Epi::kTpq) {
-    if (tid == 0) s_inv[0] = fa.scal[0];
-  }
-  EpiScalars es{0.0, 0.0};
-  if constexpr (E == Epi::kLanczos1) {
-    es.c1 = fa.scal[0];
-    es.c2 = fa.scal[1];
-  }
-  const int eoff = *Ep - 1078;
-  const bool same_c = md.c_up == md.c_dn;
-  // one hopping value of magnitude 2^k (t = 1 in particular): c * fix(a) = fix(+-a) 2^k,
-  // an exponent shift instead of an fp64 multiply per element
+  for (int k = tid; k < md.n_pair_groups; k += NT) s_pcoef[k] = (R)md.pair_coef[k];
+  const EpiScalars<R> es = epi_scalars<R, E>(fa);
+  const R inv = E == Epi::kTpq ? opaque((R)fa.scal[0]) : (R)0;
+  int same_flag = md.c_up == md.c_dn ? 1 : 0;
+  asm volatile("" : "+r"(same_flag));  // one fp64 comparison per thread, not per element
+  const bool same_c = same_flag != 0;
+  // Fixed point.  One hopping value of magnitude 2^k (t = 1 in particular): c * fix(a) =
+  // fix(+-a) 2^k, an exponent shift instead of an fp64 multiply per element; the element is
+  // then computed in units of 2^e2, e2 = eoff + k: hv = (dg 2^-k xr + (+-(acc + wq))) 2^e2 with
+  // xr = q as fp64, so the two per-element power-of-two scalings fold into the diagonal table,
+  // the Lanczos coefficient and the per-CTA partial sum (both scales must be normal numbers).
+  const int eoff = FIX ? *Ep - 1078 : 0;
   const long long cbits = __double_as_longlong(md.c_up);
   const int cexp = (int)((cbits >> 52) & 0x7ff);
-  const bool c_p2 = same_c && (cbits & 0xfffffffffffffll) == 0 && cexp > 0 && cexp < 0x7ff;
+  const bool c_p2 = FIX && same_c && (cbits & 0xfffffffffffffll) == 0 && cexp > 0 && cexp < 0x7ff;
   const bool c_neg = cbits < 0;
   const int c_l2 = cexp - 1023;
-  // With such a hopping the element is computed in units of 2^e2, e2 = eoff + k:
-  // hv = (dg 2^-k xr + (+-(acc + wq))) 2^e2 with xr = q as fp64, so the two per-element
-  // power-of-two scalings fold into the diagonal table, the Lanczos coefficient and the
-  // per-CTA partial sum (both scales must be normal numbers).
   const int e2 = eoff + c_l2;
   const bool fold = c_p2 && eoff >= -1022 && eoff <= 1023 && e2 >= -1022 && e2 <= 1023 &&
                     (E == Epi::kStore || E == Epi::kLanczos1);
@@ -446,127 +309,220 @@ __global__ void __launch_bounds__(NT) k_hub_up_q(const HubDev md,
   const double s_e2 = fold ? __longlong_as_double((long long)(e2 + 1023) << 52) : 1.0;
   const double r_k = fold ? __longlong_as_double((long long)(1023 - c_l2) << 52) : 1.0;  // 2^-k
   // diagonal = c0 + U * popcount(up & dn & mask) in the common single-group case: table
-  __shared__ double s_dtab[33];
   const bool dtab = md.n_ulin == 1 && md.n_mulin == 0 && md.n_pairs == 0;
-  if (dtab && tid <= 32) s_dtab[tid] = (md.c0 + md.ulin[0].coef * (double)tid) * r_k;
-  __syncthreads();
-  Red<true> red;
+  // the diagonal an integer multiple of the hopping (md.dint): the whole element is one exact
+  // int64 sum d q +- S and <x, H x> adds the exact products q (d q +- S) in 128 bits, moved to
+  // fp64 every 64 elements, so an element costs three fp64 operations instead of six
+  const bool dint = fold && dtab && md.dint;
+  if (dtab && tid <= 32) {
+    const double v = (md.c0 + md.ulin[0].coef * (double)tid) * r_k;
+    s_dtab[tid] = (R)v;
+    s_dti[tid] = dint ? (int)__double2ll_rn(v) : 0;
+  }
+  const R c_up = opaque((R)md.c_up), c_dn = opaque((R)md.c_dn);
+  const int dim_up = (int)md.dim_up;
+  const int64_t dim_dn = md.dim_dn;
+  // the zero entries after the row that unused slots read
+  for (int k = tid; k < kGatherZeroBytes / (int)sizeof(T); k += NT) tile[(size_t)dim_up * K + k] = (T)0;
+  constexpr int NQ = n_red<E>() > 0 ? n_red<E>() : 1;
+  Red<FIX, NQ> red;
   red.zero();
-  int pmx = 0;  // Lanczos: largest exponent field of the P values written (fa.pexp)
-  const int64_t dim_up = md.dim_up, dim_dn = md.dim_dn;
+  __int128 ia = 0;
+  int ic = 0;
+  int pmx = 0;  // fp64 Lanczos: largest exponent field of the P values written (fa.pexp)
   const int64_t n_tiles = (dim_dn + K - 1) / K;
-  const int du = (int)dim_up;
+  const uint2* rec = md.up_rec[kWidth];
+  const uint4* hdr = md.up_hdr[kWidth];
+  const int64_t stride = md.up_stride;
 
   for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
     const int64_t d0 = t * K;
     const int nk = (int)((dim_dn - d0 < K) ? (dim_dn - d0) : K);
     __syncthreads();
-    for (int64_t u = tid; u < dim_up; u += NT) {
+    const T* rows = X + d0 * dim_up;
+    if (K == 1 && (reinterpret_cast<uintptr_t>(rows) & 15u) == 0) {  // one row: 16-byte pieces
+      constexpr int kPer = 16 / (int)sizeof(T);
+      const int nv = dim_up / kPer;
+      for (int u = tid; u < nv; u += NT) copy_async<16>(tile + u * kPer, rows + u * kPer);
+      for (int u = nv * kPer + tid; u < dim_up; u += NT) copy_async<(int)sizeof(T)>(tile + u, rows + u);
+    } else {
+      for (int u = tid; u < dim_up; u += NT) {
 #pragma unroll
-      for (int m = 0; m < K; ++m) tile[u * K + m] = (m < nk) ? __ldg(Q + (d0 + m) * dim_up + u) : 0ll;
+        for (int m = 0; m < K; ++m) {
+          if (m < nk) copy_async<(int)sizeof(T)>(tile + u * K + m, rows + (int64_t)m * dim_up + u);
+          else tile[u * K + m] = (T)0;
+        }
+      }
     }
-    __syncthreads();
     uint32_t dn[K];
 #pragma unroll
     for (int m = 0; m < K; ++m) dn[m] = (m < nk) ? (md.sector ? __ldg(md.list_dn + d0 + m) : (uint32_t)(d0 + m)) : 0u;
-    for (int64_t u = tid; u < dim_up; u += NT) {
-      const uint32_t up = md.sector ? __ldg(md.list_up + u) : (uint32_t)u;
-      const int deg = md.deg_up[u];
-      const uint32_t* nb = md.nbr_up + u;
-      long long acc[K];
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    // Whole warps run to the padded row length: the table's padding reads zero entries.  The
+    // records come from L2, so they are streamed a chunk of kGatherChunk groups ahead, across
+    // states: while a chunk's targets are gathered the next chunk (of this state or the next)
+    // and the next state's header are on their way.
+    uint2 cur[kGatherChunk];
+    uint32_t hx = 0u;
+    if (tid < (int)stride) {
+      hx = __ldg(&hdr[tid >> 5].x);
 #pragma unroll
-      for (int m = 0; m < K; ++m) acc[m] = 0;
-      for (int q = 0; q < deg; ++q) {
-        const uint32_t e = __ldg(nb + q * du);
-        const long long* src = tile + (int)(e & 0x7fffffffu) * K;
-        const bool neg = (e >> 31) != 0;
-        if constexpr (K == 2) {
-          const longlong2 v2 = *reinterpret_cast<const longlong2*>(src);
-          acc[0] += neg ? -v2.x : v2.x;
-          acc[1] += neg ? -v2.y : v2.y;
-        } else {
+      for (int j = 0; j < kGatherChunk; ++j) cur[j] = __ldg(rec + tid + j * stride);
+    }
+    for (int u = tid; u < (int)stride; u += NT) {
+      const int np = (int)(hx & 0xffffu), ns = (int)(hx >> 16);  // slots [0, np) add, [np, ns) subtract
+      const int ng = (ns + 3) >> 2;
+      const int un = u + NT < (int)stride ? u + NT : u;
+      hx = __ldg(&hdr[un >> 5].x);
+      const bool on = u < dim_up;
+      T wv[K];
+      R pin[K];
 #pragma unroll
-          for (int m = 0; m < K; ++m) acc[m] += neg ? -src[m] : src[m];
-        }
+      for (int m = 0; m < K; ++m) {
+        const int64_t idx = (d0 + m) * dim_up + u;
+        wv[m] = (on && m < nk) ? W[idx] : (T)0;
+        if constexpr (E == Epi::kLanczos1 && FIX)
+          pin[m] = (on && m < nk) ? reinterpret_cast<const R*>(fa.in ? fa.in : fa.out)[idx] : (R)0;
       }
+      const uint32_t up = md.sector ? __ldg(md.list_up + (on ? u : 0)) : (uint32_t)u;
+      T acc[K];
+#pragma unroll
+      for (int m = 0; m < K; ++m) acc[m] = (T)0;
+      int c0 = 0;
+      do {
+        const uint2* q = c0 + kGatherChunk < ng ? rec + u + (int64_t)(c0 + kGatherChunk) * stride : rec + un;
+        uint2 nxt[kGatherChunk];
+#pragma unroll
+        for (int j = 0; j < kGatherChunk; ++j) nxt[j] = __ldg(q + j * stride);
+#pragma unroll
+        for (int j = 0; j < kGatherChunk; ++j) {
+          if (c0 + j < ng) {
+            const uint2 r = cur[j];
+            T v[4][K];
+            load_k<T, K>(tile + (r.x & 0xffffu) * K, v[0]);
+            load_k<T, K>(tile + (r.x >> 16) * K, v[1]);
+            load_k<T, K>(tile + (r.y & 0xffffu) * K, v[2]);
+            load_k<T, K>(tile + (r.y >> 16) * K, v[3]);
+            const int left = np - 4 * (c0 + j);  // slots of this group that add
+            if (left >= 4) {
+#pragma unroll
+              for (int m = 0; m < K; ++m) acc[m] += (v[0][m] + v[1][m]) + (v[2][m] + v[3][m]);
+            } else if (left <= 0) {
+#pragma unroll
+              for (int m = 0; m < K; ++m) acc[m] -= (v[0][m] + v[1][m]) + (v[2][m] + v[3][m]);
+            } else {
+#pragma unroll
+              for (int s = 0; s < 4; ++s)
+#pragma unroll
+                for (int m = 0; m < K; ++m) acc[m] += s < left ? v[s][m] : -v[s][m];
+            }
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < kGatherChunk; ++j) cur[j] = nxt[j];
+        c0 += kGatherChunk;
+      } while (c0 < ng);
+      if (!on) continue;
 #pragma unroll
       for (int m = 0; m < K; ++m) {
         if (m >= nk) break;
         const int64_t idx = (d0 + m) * dim_up + u;
-        // the row's own value from the quantised tile: H v is then H applied to the
-        // quantised vector (each element within 2^-57 max|x| of v, as in the gathers)
-        const double xr = __ll2double_rn(tile[u * K + m]);
-        double dg;  // (times 2^-k when folding)
+        const T xq = tile[u * K + m];
+        if constexpr (FIX) {
+          if (dint) {
+            const long long S = acc[m] + wv[m];
+            const long long hq = (long long)s_dti[__popc(up & dn[m] & (uint32_t)s_ulin[0].mask)] * xq + (c_neg ? -S : S);
+            const double hvu = __ll2double_rn(hq);  // hv = hvu 2^e2
+            if constexpr (E == Epi::kStore) {
+              reinterpret_cast<double*>(w)[idx] = hvu * s_e2;
+            } else if constexpr (E == Epi::kLanczos1) {
+              const double pv = fma(es.c1 * s_e2, hvu, -(es.c2 * pin[m]));
+              reinterpret_cast<double*>(fa.out)[idx] = pv;
+              pmx = max(pmx, (int)((__double_as_longlong(pv) >> 52) & 0x7ff));
+              ia += (__int128)xq * (__int128)hq;
+              if (++ic == 64) {
+                red.add(0, i128_to_double(ia), 1.0);
+                ia = 0;
+                ic = 0;
+              }
+            }
+            continue;
+          }
+        }
+        // diagonal: integer counts times the class coefficients (times 2^-k when folding)
+        R dg;
         if (dtab) {
           dg = s_dtab[__popc(up & dn[m] & (uint32_t)s_ulin[0].mask)];
         } else {
-        dg = md.c0;
-        for (int g = 0; g < md.n_ulin; ++g) dg += s_ulin[g].coef * (double)__popc(up & dn[m] & (uint32_t)s_ulin[g].mask);
-        for (int g = 0; g < md.n_mulin; ++g) {
-          const uint32_t mk = (uint32_t)s_mlin[g].mask;
-          dg += s_mlin[g].coef * (double)(__popc(up & mk) + __popc(dn[m] & mk));
-        }
-        if (md.n_pairs) {
-          int grp = s_pair[0].grp, cnt = 0;
-          for (int p = 0; p < md.n_pairs; ++p) {
-            const PairEntry pe = s_pair[p];
-            if (pe.grp != grp) {
-              dg += s_pcoef[grp] * (double)cnt;
-              cnt = 0;
-              grp = pe.grp;
-            }
-            const int ni = (int)((up >> pe.i) & 1u) + (int)((dn[m] >> pe.i) & 1u);
-            const int nj = (int)((up >> pe.j) & 1u) + (int)((dn[m] >> pe.j) & 1u);
-            cnt += ni * nj;
+          dg = (R)md.c0;
+          for (int g = 0; g < md.n_ulin; ++g) dg += s_uc[g] * (R)__popc(up & dn[m] & (uint32_t)s_ulin[g].mask);
+          for (int g = 0; g < md.n_mulin; ++g) {
+            const uint32_t mk = (uint32_t)s_mlin[g].mask;
+            dg += s_mc[g] * (R)(__popc(up & mk) + __popc(dn[m] & mk));
           }
-          dg += s_pcoef[grp] * (double)cnt;
+          if (md.n_pairs) {
+            int grp = s_pair[0].grp, cnt = 0;
+            for (int p = 0; p < md.n_pairs; ++p) {
+              const PairEntry pe = s_pair[p];
+              if (pe.grp != grp) {
+                dg += s_pcoef[grp] * (R)cnt;
+                cnt = 0;
+                grp = pe.grp;
+              }
+              const int ni = (int)((up >> pe.i) & 1u) + (int)((dn[m] >> pe.i) & 1u);
+              const int nj = (int)((up >> pe.j) & 1u) + (int)((dn[m] >> pe.j) & 1u);
+              cnt += ni * nj;
+            }
+            dg += s_pcoef[grp] * (R)cnt;
+          }
+          if (fold) dg *= (R)r_k;
         }
-        if (fold) dg *= r_k;
-        }
-        const long long wq = __ldg(WQ + idx);
-        if (fold) {
-          const long long y = c_neg ? -(acc[m] + wq) : acc[m] + wq;
-          const double hvu = fma(dg, xr, __ll2double_rn(y));  // hv = hvu 2^e2
+        if constexpr (!FIX) {
+          const R hv = same_c ? dg * xq + c_up * (acc[m] + wv[m]) : dg * xq + c_up * acc[m] + c_dn * wv[m];
+          epilogue<R, E, NQ>(idx, xq, (R)0, hv, (R)0, reinterpret_cast<R*>(w), fa, es, inv, red);
+        } else if (fold) {
+          const double xr = __ll2double_rn(xq);
+          const long long S = acc[m] + wv[m];
+          const double hvu = fma(dg, xr, __ll2double_rn(c_neg ? -S : S));  // hv = hvu 2^e2
           if constexpr (E == Epi::kStore) {
-            w[idx] = hvu * s_e2;
+            reinterpret_cast<double*>(w)[idx] = hvu * s_e2;
           } else if constexpr (E == Epi::kLanczos1) {
             // P <- c1 hv - c2 P; partial <x, hv> in units of 2^(eoff + e2)
-            double* P = reinterpret_cast<double*>(fa.out);
-            const double* Pin = fa.in ? reinterpret_cast<const double*>(fa.in) : P;
-            const double pv = fma(es.c1 * s_e2, hvu, -(es.c2 * Pin[idx]));
-            P[idx] = pv;
+            const double pv = fma(es.c1 * s_e2, hvu, -(es.c2 * pin[m]));
+            reinterpret_cast<double*>(fa.out)[idx] = pv;
             pmx = max(pmx, (int)((__double_as_longlong(pv) >> 52) & 0x7ff));
             red.add(0, xr, hvu);
             red.tick();
           }
         } else {
-          const double x = fix_to_double(tile[u * K + m], eoff);
+          const double x = fix_to_double(xq, eoff);
           double hv;
-          if (c_p2) hv = fma(dg, x, fix_to_double(c_neg ? -(acc[m] + wq) : acc[m] + wq, eoff + c_l2));
-          else if (same_c) hv = fma(dg, x, md.c_up * fix_to_double(acc[m] + wq, eoff));
-          else hv = fma(dg, x, fma(md.c_up, fix_to_double(acc[m], eoff), md.c_dn * fix_to_double(wq, eoff)));
+          if (c_p2) hv = fma(dg, x, fix_to_double(c_neg ? -(acc[m] + wv[m]) : acc[m] + wv[m], eoff + c_l2));
+          else if (same_c) hv = fma(dg, x, md.c_up * fix_to_double(acc[m] + wv[m], eoff));
+          else hv = fma(dg, x, fma(md.c_up, fix_to_double(acc[m], eoff), md.c_dn * fix_to_double(wv[m], eoff)));
           if constexpr (E == Epi::kLanczos1) {  // the epilogue's Lanczos step, with the exponent kept
-            double* P = reinterpret_cast<double*>(fa.out);
-            const double* Pin = fa.in ? reinterpret_cast<const double*>(fa.in) : P;
-            const double pv = es.c1 * hv - es.c2 * Pin[idx];
-            P[idx] = pv;
+            const double pv = es.c1 * hv - es.c2 * pin[m];
+            reinterpret_cast<double*>(fa.out)[idx] = pv;
             pmx = max(pmx, (int)((__double_as_longlong(pv) >> 52) & 0x7ff));
             red.add(0, x, hv);
             red.tick();
           } else {
-            epilogue<double, E>(idx, 0, x, 0.0, hv, 0.0, w, fa, es, s_inv, red);
+            epilogue<double, E, NQ>(idx, x, 0.0, hv, 0.0, reinterpret_cast<double*>(w), fa, es, inv, red);
           }
         }
       }
     }
   }
-  if constexpr (E == Epi::kLanczos1) {
+  if constexpr (FIX && E == Epi::kLanczos1) {
+    if (ic) red.add(0, i128_to_double(ia), 1.0);
     if (fa.pexp != nullptr) {
       pmx = (int)__reduce_max_sync(0xffffffffu, (unsigned)pmx);
       if ((tid & 31) == 0 && pmx > 0) atomicMax(fa.pexp, pmx);
     }
   }
   if constexpr (E != Epi::kStore) {
+    // fixed-order reduction: warp shuffles, then the warps' sums in warp order
     constexpr int nq = n_red<E>();
     const int lane = tid & 31, wid = tid >> 5;
 #pragma unroll
@@ -625,7 +581,7 @@ inline int up_threads(size_t tile_bytes) { return tile_bytes > 110000 ? 1024 : 5
 template <class KernelT>
 int occupancy_for(KernelT kern, int nt, size_t smem) {
   int n = 0;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + kGatherZeroBytes);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, nt, smem) != cudaSuccess || n < 1) {
     cudaGetLastError();
     n = 1;
@@ -633,32 +589,30 @@ int occupancy_for(KernelT kern, int nt, size_t smem) {
   return n;
 }
 
-template <class R, int K, Epi E>
+template <class T, int K>
+size_t up_smem(const HubDev& md) { return (size_t)K * md.dim_up * sizeof(T) + kGatherZeroBytes; }
+
+template <class T, int K, Epi E>
 int up_occupancy(const HubDev& md) {
-  const size_t smem = (size_t)K * md.dim_up * sizeof(R);
-  return up_threads(smem) == 1024 ? occupancy_for(k_hub_up<R, K, E, 1024>, 1024, smem)
-                                  : occupancy_for(k_hub_up<R, K, E, 512>, 512, smem);
+  const size_t smem = up_smem<T, K>(md);
+  return up_threads(smem) == 1024 ? occupancy_for(k_hub_up<T, K, E, 1024>, 1024, smem)
+                                  : occupancy_for(k_hub_up<T, K, E, 512>, 512, smem);
 }
 
-template <class R, int K, Epi E>
-Status launch_up(const HubDev& md, const R* X, const R* W, R* w, const FusedArgs& fa, int grid, cudaStream_t st) {
-  const size_t smem = (size_t)K * md.dim_up * sizeof(R);
+template <class T, int K, Epi E>
+Status launch_up(const HubDev& md, const T* X, const T* W, const int* Ep, void* w, const FusedArgs& fa, int grid,
+                 cudaStream_t st) {
+  const size_t smem = up_smem<T, K>(md);
+  const int most = kSmemBudget + kGatherZeroBytes;
   if (up_threads(smem) == 1024) {
-    HPHI_CUDA_TRY(cudaFuncSetAttribute(k_hub_up<R, K, E, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-    k_hub_up<R, K, E, 1024><<<grid, 1024, smem, st>>>(md, X, W, w, fa);
+    HPHI_CUDA_TRY(cudaFuncSetAttribute(k_hub_up<T, K, E, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    k_hub_up<T, K, E, 1024><<<grid, 1024, smem, st>>>(md, X, W, Ep, w, fa);
   } else {
-    HPHI_CUDA_TRY(cudaFuncSetAttribute(k_hub_up<R, K, E, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-    k_hub_up<R, K, E, 512><<<grid, 512, smem, st>>>(md, X, W, w, fa);
+    HPHI_CUDA_TRY(cudaFuncSetAttribute(k_hub_up<T, K, E, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    k_hub_up<T, K, E, 512><<<grid, 512, smem, st>>>(md, X, W, Ep, w, fa);
   }
   HPHI_CUDA_TRY(cudaGetLastError());
   return {};
-}
-
-template <int K, Epi E>
-int upq_occupancy(const HubDev& md) {
-  const size_t smem = (size_t)K * md.dim_up * 8;
-  return up_threads(smem) == 1024 ? occupancy_for(k_hub_up_q<K, E, 1024>, 1024, smem)
-                                  : occupancy_for(k_hub_up_q<K, E, 512>, 512, smem);
 }
 
 // scratch layout of the quantised fp64 path: [Q: dim int64][WQ: dim int64][E: int]
@@ -685,21 +639,8 @@ Status launch_q(const HubDev& md, const void* v, void* w, void* scratch, const F
   if (fa.pexp != nullptr) HPHI_CUDA_TRY(cudaMemsetAsync(fa.pexp, 0, sizeof(int), st));
   Status sd = launch_dn<long long>(md, Q, WQ, fa.done, counter, st);
   if (sd.code) return sd;
-  double* out = reinterpret_cast<double*>(w);
-  const int K = pick_kq(md);
-  const size_t smem = (size_t)K * md.dim_up * 8;
-  const bool big = up_threads(smem) == 1024;
-#define HPHI_UPQ(KK, NN)                                                                                          \
-  HPHI_CUDA_TRY(cudaFuncSetAttribute(k_hub_up_q<KK, E, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget)); \
-  k_hub_up_q<KK, E, NN><<<grid_up, NN, smem, st>>>(md, Q, WQ, Ep, out, fa);
-  if (K == 2) {
-    if (big) { HPHI_UPQ(2, 1024) } else { HPHI_UPQ(2, 512) }
-  } else {
-    if (big) { HPHI_UPQ(1, 1024) } else { HPHI_UPQ(1, 512) }
-  }
-#undef HPHI_UPQ
-  HPHI_CUDA_TRY(cudaGetLastError());
-  return {};
+  return pick_kq(md) == 2 ? launch_up<long long, 2, E>(md, Q, WQ, Ep, w, fa, grid_up, st)
+                          : launch_up<long long, 1, E>(md, Q, WQ, Ep, w, fa, grid_up, st);
 }
 
 int* hub_exponent_slot_impl(const HubDev& md, void* scratch) {
@@ -711,10 +652,10 @@ int upq_grid(const HubDev& md, Epi epi) {
   int occ = 1;
 #define HPHI_OCCQ(KK)                                                          \
   switch (epi) {                                                               \
-    case Epi::kStore: occ = upq_occupancy<KK, Epi::kStore>(md); break;         \
-    case Epi::kLanczos1: occ = upq_occupancy<KK, Epi::kLanczos1>(md); break;   \
-    case Epi::kTpq: occ = upq_occupancy<KK, Epi::kTpq>(md); break;             \
-    case Epi::kRefine: occ = upq_occupancy<KK, Epi::kRefine>(md); break;       \
+    case Epi::kStore: occ = up_occupancy<long long, KK, Epi::kStore>(md); break;         \
+    case Epi::kLanczos1: occ = up_occupancy<long long, KK, Epi::kLanczos1>(md); break;   \
+    case Epi::kTpq: occ = up_occupancy<long long, KK, Epi::kTpq>(md); break;             \
+    case Epi::kRefine: occ = up_occupancy<long long, KK, Epi::kRefine>(md); break;       \
   }
   if (K == 2) { HPHI_OCCQ(2) } else { HPHI_OCCQ(1) }
 #undef HPHI_OCCQ
@@ -735,11 +676,10 @@ Status launch_r(const HubDev& md, const void* v, void* w, void* scratch, const F
   unsigned long long* counter = reinterpret_cast<unsigned long long*>(static_cast<char*>(scratch) + voff);
   Status sd = launch_dn<R>(md, X, W, fa.done, counter, st);
   if (sd.code) return sd;
-  R* out = reinterpret_cast<R*>(w);
   switch (pick_k<R>(md)) {
-    case 4: return launch_up<R, 4, E>(md, X, W, out, fa, grid_up, st);
-    case 2: return launch_up<R, 2, E>(md, X, W, out, fa, grid_up, st);
-    default: return launch_up<R, 1, E>(md, X, W, out, fa, grid_up, st);
+    case 4: return launch_up<R, 4, E>(md, X, W, nullptr, w, fa, grid_up, st);
+    case 2: return launch_up<R, 2, E>(md, X, W, nullptr, w, fa, grid_up, st);
+    default: return launch_up<R, 1, E>(md, X, W, nullptr, w, fa, grid_up, st);
   }
 }
 
@@ -829,13 +769,16 @@ Status build_hub_neighbours(const HubDev& md, int species, uint32_t* nbr, uint8_
   return {};
 }
 
+bool hub_up_row_fits(const HubDev& md, int prec) {
+  return md.dim_up * (int64_t)(prec == HPHI_FP64 ? 8 : 4) <= kSmemBudget;
+}
+
 bool hub_fast_ok(const HubDev& md, int prec, bool cplx, int nvec, Epi epi) {
   if (!md.fast || cplx || nvec != 1) return false;
   // fixed-point sums of at most 127 terms (|q| < 2^56) stay exact in 64 bits
   if (prec == HPHI_FP64 && md.maxdeg_up + md.maxdeg_dn > 126) return false;
   if (epi == Epi::kRefine && prec != HPHI_FP64) return false;
-  const int64_t row = md.dim_up * (int64_t)(prec == HPHI_FP64 ? 8 : 4);
-  return row <= kSmemBudget;
+  return hub_up_row_fits(md, prec);
 }
 
 // the launch shape of one precision: the autotuner's choice, else the built-in default
@@ -845,6 +788,12 @@ HubDev with_shape(const HubDev& md, int prec) {
   t.dn_ept = md.tuned_ept[i];
   t.up_k = md.tuned_k[i];
   return t;
+}
+
+int hub_up_width(const HubDev& md0, int prec) {
+  const HubDev md = with_shape(md0, prec);
+  const int b = prec == HPHI_FP64 ? 8 * pick_kq(md) : 4 * pick_k<float>(md);
+  return b >= 16 ? 2 : (b >= 8 ? 1 : 0);
 }
 
 int hub_up_grid(const HubDev& md0, int prec, Epi epi) {

@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(kThreads) k_hv_spin(const SpinDev md, const S*
   __shared__ LinGroup s_lin[kMaxLin];
   __shared__ PairEntry s_pair[kMaxPairs];
   __shared__ double s_pcoef[kMaxPairGroups];
-  __shared__ double s_inv[kMaxNvec];
+  __shared__ R s_inv[kMaxNvec];
   __shared__ uint64_t s_hi[2];
   __shared__ double s_red[(E == Epi::kStore) ? 1 : kThreads * kMaxRedQ];
 
@@ -61,16 +61,13 @@ __global__ void __launch_bounds__(kThreads) k_hv_spin(const SpinDev md, const S*
   for (int k = tid; k < md.n_pairs; k += kThreads) s_pair[k] = md.pairs[k];
   for (int k = tid; k < md.n_pair_groups; k += kThreads) s_pcoef[k] = md.pair_coef[k];
   if constexpr (E == Epi::kTpq) {
-    for (int k = tid; k < nvec; k += kThreads) s_inv[k] = fa.scal[k];
+    for (int k = tid; k < nvec; k += kThreads) s_inv[k] = (R)fa.scal[k];
   }
-  EpiScalars es{0.0, 0.0};
-  if constexpr (E == Epi::kLanczos1) {
-    es.c1 = fa.scal[0];
-    es.c2 = fa.scal[1];
-  }
+  const EpiScalars<R> es = epi_scalars<R, E>(fa);
   __syncthreads();
 
-  Red<F64> red;
+  constexpr int kNQ = n_red<E>() > 0 ? n_red<E>() : 1;
+  Red<F64, kNQ> red;
   red.zero();
   const int64_t total = md.dim * (int64_t)nvec;
   __shared__ int64_t s_item;
@@ -222,9 +219,9 @@ __global__ void __launch_bounds__(kThreads) k_hv_spin(const SpinDev md, const S*
         hr += (R)cc.x * vr;
       }
     }
-    epilogue<S, E>(idx, c, sr, si, hr, hi, w, fa, es, s_inv, red);
+    epilogue<S, E, kNQ>(idx, sr, si, hr, hi, w, fa, es, E == Epi::kTpq ? s_inv[c] : R(0), red);
   }
-  if constexpr (E != Epi::kStore) block_finish<F64>(red, n_red<E>(), nvec, fa.partials, s_red);
+  if constexpr (E != Epi::kStore) block_finish<F64, kThreads, kNQ>(red, n_red<E>(), nvec, fa.partials, s_red);
 }
 
 // ------------------------------------------------------------------ Hubbard kernel
@@ -246,7 +243,7 @@ __global__ void __launch_bounds__(kThreads) k_hv_hub(const HubDev md, const S* _
   __shared__ LinGroup s_mlin[kMaxLin];
   __shared__ PairEntry s_pair[kMaxPairs];
   __shared__ double s_pcoef[kMaxPairGroups];
-  __shared__ double s_inv[kMaxNvec];
+  __shared__ R s_inv[kMaxNvec];
   __shared__ int64_t s_dl_src[kMaxHops];   // source element offset of neighbour row d'
   __shared__ uint32_t s_dl_meta[kMaxHops];  // bit 0 negative sign, bit 1 direction b, class << 2
   __shared__ int s_dl_n;
@@ -263,16 +260,13 @@ __global__ void __launch_bounds__(kThreads) k_hv_hub(const HubDev md, const S* _
   for (int k = tid; k < md.n_pairs; k += kThreads) s_pair[k] = md.pairs[k];
   for (int k = tid; k < md.n_pair_groups; k += kThreads) s_pcoef[k] = md.pair_coef[k];
   if constexpr (E == Epi::kTpq) {
-    for (int k = tid; k < nvec; k += kThreads) s_inv[k] = fa.scal[k];
+    for (int k = tid; k < nvec; k += kThreads) s_inv[k] = (R)fa.scal[k];
   }
-  EpiScalars es{0.0, 0.0};
-  if constexpr (E == Epi::kLanczos1) {
-    es.c1 = fa.scal[0];
-    es.c2 = fa.scal[1];
-  }
+  const EpiScalars<R> es = epi_scalars<R, E>(fa);
   __syncthreads();
 
-  Red<F64> red;
+  constexpr int kNQ = n_red<E>() > 0 ? n_red<E>() : 1;
+  Red<F64, kNQ> red;
   red.zero();
   const int64_t row_elems = md.dim_up * (int64_t)nvec;
   const int64_t nchunk = (row_elems + kThreads - 1) / kThreads;
@@ -461,9 +455,9 @@ __global__ void __launch_bounds__(kThreads) k_hv_hub(const HubDev md, const S* _
       }
     }
     if (ndl) flush(cur);
-    epilogue<S, E>(idx, c, sr, si, hr, hi, w, fa, es, s_inv, red);
+    epilogue<S, E, kNQ>(idx, sr, si, hr, hi, w, fa, es, E == Epi::kTpq ? s_inv[c] : R(0), red);
   }
-  if constexpr (E != Epi::kStore) block_finish<F64>(red, n_red<E>(), nvec, fa.partials, s_red);
+  if constexpr (E != Epi::kStore) block_finish<F64, kThreads, kNQ>(red, n_red<E>(), nvec, fa.partials, s_red);
 }
 
 template <class S, Epi E>

@@ -725,13 +725,6 @@ __global__ void __launch_bounds__(kThreads) k_sec_hi(const SecDev d, const T* __
   }
 }
 
-// a 128-bit integer as the nearest-ish fp64 (two roundings: relative error below 2^-52)
-__device__ __forceinline__ double i128_to_double(__int128 v) {
-  const long long hi = (long long)(v >> 64);
-  const unsigned long long lo = (unsigned long long)v;
-  return fma(__ll2double_rn(hi), 18446744073709551616.0, __ull2double_rn(lo));
-}
-
 // K consecutive values of an interleaved shared-memory tile with the widest aligned loads
 template <class T, int K>
 __device__ __forceinline__ void tile_load(const T* p, T* out) {
@@ -780,7 +773,6 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
   __shared__ int s_nk;
   __shared__ unsigned long long s_t;
   __shared__ T s_w[kSecMaxCls];
-  __shared__ double s_inv[1];
   __shared__ double s_red[(NT / 32) * kMaxRedQ];
 
   if (fa.done != nullptr && *fa.done) return;
@@ -813,15 +805,9 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
   if (tid < d.n_str)
     s_sb[tid] = make_uint2((uint32_t)d.str_b[tid] | ((uint32_t)d.str_cls[tid] << 16), (uint32_t)d.str_t[tid] * nJ);
   if (tid < K) tile[(size_t)d.nq_max * K + tid] = (T)0;  // the zero entry unused neighbour slots point at
-  if constexpr (E == Epi::kTpq) {
-    if (tid == 0) s_inv[0] = fa.scal[0];
-  }
-  EpiScalars es{0.0, 0.0};
-  if constexpr (E == Epi::kLanczos1) {
-    es.c1 = fa.scal[0];
-    es.c2 = fa.scal[1];
-  }
-  const R coef0 = (R)d.coef[0];
+  const EpiScalars<R> es = epi_scalars<R, E>(fa);
+  const R inv = E == Epi::kTpq ? opaque((R)fa.scal[0]) : (R)0;
+  const R coef0 = opaque((R)d.coef[0]);
   const int n_str = d.n_str;
   const uint32_t pad2 = (uint32_t)d.nq_max | ((uint32_t)d.nq_max << 16);
   constexpr int NQ = n_red<E>() > 0 ? n_red<E>() : 1;  // reduced quantities of the epilogue
@@ -1000,7 +986,7 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
           const R dg = s_dtab[ci];
           if constexpr (!FIX) {
             const R hv = ONE ? dg * xq + coef0 * (acc[e][m] + wv) : dg * xq + (acc[e][m] + wv);
-            epilogue<float, E, NQ>(idx, 0, xq, 0.f, hv, 0.f, reinterpret_cast<float*>(w), fa, es, s_inv, red);
+            epilogue<float, E, NQ>(idx, xq, 0.f, hv, 0.f, reinterpret_cast<float*>(w), fa, es, inv, red);
           } else {
             const long long S = acc[e][m] + wv;
             if constexpr (E == Epi::kLanczos1) {
@@ -1047,7 +1033,7 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
                 red.add(0, x, hv);
                 red.tick();
               } else {
-                epilogue<double, E, NQ>(idx, 0, x, 0.0, hv, 0.0, reinterpret_cast<double*>(w), fa, es, s_inv, red);
+                epilogue<double, E, NQ>(idx, x, 0.0, hv, 0.0, reinterpret_cast<double*>(w), fa, es, inv, red);
               }
             }
           }

@@ -29,9 +29,8 @@ template <int NQ> struct Red<true, NQ> {
 // fp32 products accumulated in (hi, lo) pairs: TwoProduct by FMA and TwoSum (Knuth), exact per
 // product; every 16 products the pair is folded into a second pair (h2, l2) by a double-float
 // addition (TwoSum of the high parts, then a fast renormalisation; relative error about 2^-46
-// per fold), and the fp64 value is formed once, in get().  The fold is fp32-only on purpose:
-// the compiler if-converts the every-16th branch, so the fold's instructions issue on every
-// product, and fp64 conversions there would saturate GB300's 1/64-rate fp64 pipe.
+// per fold), and the fp64 value is formed once, in get().  The opaque statement in the fold's
+// branch keeps the compiler from if-converting it, which made every product issue the fold.
 template <int NQ> struct Red<false, NQ> {
   float hi[NQ], lo[NQ], h2[NQ], l2[NQ];
   int n;
@@ -66,7 +65,10 @@ template <int NQ> struct Red<false, NQ> {
     n = 0;
   }
   __device__ __forceinline__ void tick() {
-    if (++n == 16) fold();
+    if (++n == 16) {
+      asm volatile("" : "+f"(hi[0]));
+      fold();
+    }
   }
   __device__ __forceinline__ double get(int q) const {
     return ((double)h2[q] + (double)l2[q]) + ((double)hi[q] + (double)lo[q]);

@@ -1118,3 +1118,34 @@ def test_autotune_full_basis_spin_model_tunes_its_sectors():
     after = m.lanczos_sectors([12, 10, 3], 12, seed=3)
     for a, b in zip(before, after):
         assert _rel(a["alpha"], b["alpha"]) < 1e-13 and _rel(a["beta"], b["beta"]) < 1e-13
+
+
+# ----------------------------------------------------------------------------- pass U gather tables
+GATHER_CASES = [
+    # (sites, n_up, n_dn, t, U, mu, V): up rows of one entry, shorter than a warp, a whole warp
+    # and remainders; the last tile part-filled (n_dn rows not a multiple of 2 or 4); integral
+    # and other diagonals, negative and non-power-of-two hopping, no U, a density term
+    (5, 0, 2, 1.0, 8.0, 0.0, 0.0), (6, 1, 3, 1.0, 8.0, 0.0, 0.0), (9, 2, 1, -2.0, 6.0, 0.0, 0.0),
+    (8, 4, 1, 0.5, 0.0, 0.0, 0.0), (11, 5, 2, 1.0, 8.0, 0.0, 0.0), (12, 6, 1, 0.7, 3.3, 0.0, 0.0),
+    (10, 3, 3, 1.0, 8.0, 0.25, 0.0), (9, 4, 2, 1.0, 8.0, 0.0, 0.5), (10, 10, 4, 1.0, 200.0, 0.0, 0.0),
+]
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("n,nu,nd,t,U,mu,V", GATHER_CASES)
+def test_hubbard_gather_tables(n, nu, nd, t, U, mu, V, prec):
+    """The product and a fused Lanczos step of the two-pass path on rows at the table's edges."""
+    import dataclasses
+    spec = wl.hubbard(n, wl.ring_bonds(n) + wl.ring_bonds(n, 2), t, U).with_basis(wl.BASIS_NUMBER, nu, nd)
+    spec = dataclasses.replace(spec, chem_pot=[(i, mu) for i in range(n)] if mu else [],
+                               density=[(0, 1, V), (2, 4, V)] if V else [])
+    m = hp.Model.from_spec(spec)
+    v = wl.gaussian_vector(5 * n + nu, m.dim)[:, 0]
+    p = hp.FP64 if prec == "fp64" else hp.FP32
+    ref = oracle.apply_H(spec, v).real
+    w = m.apply_H(_to_dev(m, v[:, None], p)).cpu().numpy()[:, 0]
+    assert _rel(w, ref) < (1e-12 if prec == "fp64" else 2e-5)
+    if m.dim > 8:
+        a, _ = oracle.lanczos(spec, v, 3)
+        r = m.lanczos(3, prec=p, v0=torch.as_tensor(v))
+        assert _rel(r["alpha"][:len(a)], a) < (1e-12 if prec == "fp64" else 2e-5)  # a: up to the breakdown
