@@ -135,13 +135,14 @@ struct hphi_model {
   std::map<int, std::unique_ptr<WinCache>> win;
   // split-row path of real S^z-sector spin models: the compiled terms, whether each precision
   // may take the path, the split asked for per precision (-1 off, 0 default, else L) and
-  // rows per tile (0 default), and the device tables built so far by (L, K)
+  // rows per tile (0 default), and the device tables built so far by (L, K, element size)
   hphi::SecTerms sec_terms;
   bool sec_ok[2] = {false, false};
   std::string sec_why;
   int sec_L[2] = {0, 0}, sec_K[2] = {0, 0};
   int sec_hi_cols[2] = {0, 0};  // pass H columns per lane per precision (0: built-in)
-  std::map<std::pair<int, int>, std::unique_ptr<hphi::SecTables, hphi::SecTablesDeleter>> sec_tab;
+  int sec_L0[2] = {0, 0};  // the default split of each precision
+  std::map<std::array<int, 3>, std::unique_ptr<hphi::SecTables, hphi::SecTablesDeleter>> sec_tab;
 };
 
 namespace {
@@ -565,24 +566,24 @@ hphi::Status build_hub_fast(hphi_model* m, cudaStream_t st) {
 }
 
 // ------------------------------------------------------------------ split-row spin path
-// The split (L, K) precision prec runs with: the one asked for, else the default (largest
-// low part whose rows fit one tile, widest tile that fits); (0, 0) when the path is off.
-std::pair<int, int> sec_shape(const hphi_model* m, int prec) {
+// The split (L, K, element size) precision prec runs with: the one asked for, else the default;
+// L = 0 when the path is off.
+std::array<int, 3> sec_shape(const hphi_model* m, int prec) {
   const int pi = prec == HPHI_FP64 ? 0 : 1;
-  if (!m->sec_ok[pi] || m->sec_L[pi] < 0) return {0, 0};
   const int esz = prec == HPHI_FP64 ? 8 : 4;
-  const int L = m->sec_L[pi] > 0 ? m->sec_L[pi] : hphi::sec_default_L(m->sec_terms, esz);
-  if (L <= 0) return {0, 0};
+  if (!m->sec_ok[pi] || m->sec_L[pi] < 0) return {0, 0, esz};
+  const int L = m->sec_L[pi] > 0 ? m->sec_L[pi] : m->sec_L0[pi];
+  if (L <= 0) return {0, 0, esz};
   const int K = m->sec_K[pi] > 0 ? m->sec_K[pi] : hphi::sec_default_K(m->sec_terms, L, esz);
-  return {L, K};
+  return {L, K, esz};
 }
 
 // Builds (once) the tables of the shape prec runs with.  Never called inside a stream capture.
 hphi::Status sec_ensure(hphi_model* m, int prec, cudaStream_t st) {
-  const std::pair<int, int> sh = sec_shape(m, prec);
-  if (sh.first == 0 || m->sec_tab.count(sh)) return {};
+  const std::array<int, 3> sh = sec_shape(m, prec);
+  if (sh[0] == 0 || m->sec_tab.count(sh)) return {};
   hphi::SecTables* t = nullptr;
-  hphi::Status s = hphi::sec_build(m->sec_terms, sh.first, sh.second, &t, st);
+  hphi::Status s = hphi::sec_build(m->sec_terms, sh[0], sh[1], sh[2], &t, st);
   if (s.code) return s;
   m->sec_tab[sh].reset(t);
   return {};
@@ -602,7 +603,9 @@ hphi::Status sec_prepare(hphi_model* m, cudaStream_t st) {
   }
   for (int prec : {HPHI_FP64, HPHI_FP32}) {
     std::string why;
-    m->sec_ok[prec == HPHI_FP64 ? 0 : 1] = hphi::sec_applicable(m->sec_terms, prec, &why);
+    const int pi = prec == HPHI_FP64 ? 0 : 1;
+    m->sec_ok[pi] = hphi::sec_applicable(m->sec_terms, prec, &why);
+    m->sec_L0[pi] = m->sec_ok[pi] ? hphi::sec_default_L(m->sec_terms, prec == HPHI_FP64 ? 8 : 4) : 0;
     if (!why.empty()) m->sec_why = why;
     hphi::Status s = sec_ensure(m, prec, st);
     if (s.code) return s;
@@ -831,13 +834,15 @@ hphi::Status sec_autotune(hphi_model* m, int prec, hphi_tune_result* res, cudaSt
   const int pi = prec == HPHI_FP64 ? 0 : 1;
   const int esz = prec == HPHI_FP64 ? 8 : 4;
   const int saved_L = m->sec_L[pi], saved_K = m->sec_K[pi];
-  const int L0 = hphi::sec_default_L(m->sec_terms, esz);
+  const int L0 = m->sec_L0[pi];
   if (L0 <= 0) return {};
-  std::vector<std::pair<int, int>> cand;
-  for (int L = L0; L >= std::max(1, L0 - 2); --L) {
+  const std::array<int, 3> dflt = sec_shape(m, prec);
+  std::vector<std::array<int, 3>> cand = {dflt};
+  for (int L = L0 + 1; L >= std::max(1, L0 - 2); --L) {
     if (m->n_sites - L > hphi::kSecMaxH) break;
-    const int kmax = hphi::sec_default_K(m->sec_terms, L, esz);
-    for (int K = 1; K <= kmax; K *= 2) cand.emplace_back(L, K);
+    const int kmax = hphi::sec_tallest_K(m->sec_terms, L, esz);
+    for (int K = 1; K <= kmax; K *= 2)
+      if (hphi::sec_fits(m->sec_terms, L, K, esz) && std::array<int, 3>{L, K, esz} != dflt) cand.push_back({L, K, esz});
   }
   hphi::Status s;
   if ((s = m->ws.vecA.ensure((size_t)esz * (size_t)m->dim)).code) return s;
@@ -852,18 +857,17 @@ hphi::Status sec_autotune(hphi_model* m, int prec, hphi_tune_result* res, cudaSt
   } tm;
   HPHI_CUDA_TRY(cudaEventCreate(&tm.a));
   HPHI_CUDA_TRY(cudaEventCreate(&tm.b));
-  const std::pair<int, int> dflt = sec_shape(m, prec);
   m->sec_hi_cols[pi] = 0;  // the shapes are compared at the built-in pass-H columns
   float best = 1e30f, worst = 0.f, dms = 0.f;
-  std::pair<int, int> best_sh = dflt;
+  std::array<int, 3> best_sh = dflt;
   hphi::FusedArgs fa;
   for (const auto& sh : cand) {
-    m->sec_L[pi] = sh.first;
-    m->sec_K[pi] = sh.second;
+    m->sec_L[pi] = sh[0];
+    m->sec_K[pi] = sh[1];
     if ((s = sec_ensure(m, prec, st)).code) {
-      if (s.code != HPHI_ERR_OUT_OF_MEMORY) break;
+      if (sh == dflt || (s.code != HPHI_ERR_OUT_OF_MEMORY && s.code != HPHI_ERR_UNSUPPORTED)) break;
       s = {};
-      continue;  // a candidate whose tables do not fit is skipped
+      continue;  // a candidate whose tables do not fit, or whose split has too many straddling terms, is skipped
     }
     const size_t need = hv_scratch_bytes(m, prec, 1, hphi::Epi::kStore);
     if ((s = m->ws.work.ensure(need)).code) break;
@@ -888,7 +892,7 @@ hphi::Status sec_autotune(hphi_model* m, int prec, hphi_tune_result* res, cudaSt
     }
     // keep only the tables of this precision's default and best so far, and of the shape the
     // other precision runs with
-    const std::pair<int, int> other = sec_shape(m, pi == 0 ? HPHI_FP32 : HPHI_FP64);
+    const std::array<int, 3> other = sec_shape(m, pi == 0 ? HPHI_FP32 : HPHI_FP64);
     for (auto it = m->sec_tab.begin(); it != m->sec_tab.end();) {
       if (it->first != dflt && it->first != best_sh && it->first != other) it = m->sec_tab.erase(it);
       else ++it;
@@ -899,8 +903,8 @@ hphi::Status sec_autotune(hphi_model* m, int prec, hphi_tune_result* res, cudaSt
     m->sec_K[pi] = saved_K;
     return s;
   }
-  m->sec_L[pi] = best_sh.first;
-  m->sec_K[pi] = best_sh.second;
+  m->sec_L[pi] = best_sh[0];
+  m->sec_K[pi] = best_sh[1];
   // pass H at half the columns per lane on the chosen shape (narrower stripes keep a large
   // class's stripe nearer L2's size, at more instructions per output)
   {
@@ -936,8 +940,8 @@ hphi::Status sec_autotune(hphi_model* m, int prec, hphi_tune_result* res, cudaSt
     }
     res->best_split_hi_cols = m->sec_hi_cols[pi] ? full / 2 : full;
   }
-  res->best_split_L = best_sh.first;
-  res->best_split_K = best_sh.second;
+  res->best_split_L = best_sh[0];
+  res->best_split_K = best_sh[1];
   res->best_ms = best;
   res->default_ms = dms;
   res->worst_ms = worst;
@@ -1160,8 +1164,8 @@ int hphi_set_sector_split(hphi_model* m, int prec, int L, int K, void* stream) {
   m->sec_hi_cols[pi] = 0;
   if (L >= 0) {
     const int esz = prec == HPHI_FP64 ? 8 : 4;
-    const std::pair<int, int> sh = sec_shape(m, prec);
-    if (sh.first == 0 || !hphi::sec_fits(m->sec_terms, sh.first, sh.second, esz)) {
+    const std::array<int, 3> sh = sec_shape(m, prec);
+    if (sh[0] == 0 || !hphi::sec_fits(m->sec_terms, sh[0], sh[1], esz)) {
       m->sec_L[pi] = oldL;
       m->sec_K[pi] = oldK;
       return fail(m, HPHI_ERR_INVALID_ARG,

@@ -135,6 +135,7 @@ constexpr int kSecMaxSp = 24;    // straddling S^z S^z pairs
 constexpr int kSecMaxSl = 8;     // layers of straddling pairs
 constexpr int kSecMaxL = 20;
 constexpr int kSecMaxH = 22;
+constexpr int kSecMaxHH = 24;    // high bits of pass H's split (12 bytes of tables per high part)
 constexpr int kSecDtab = 2048;   // diagonal table entries
 
 struct SecDev {
@@ -152,29 +153,23 @@ struct SecDev {
   double unit;
   int qextra;                   // extra headroom bits of the quantised copy
   int dint;                     // the diagonal is an integer multiple of `unit` everywhere
-  // low side
-  // low-part tables cover the classes present: entry j - jbase for list position j, nJ of them
-  uint32_t lo_off[kSecMaxL + 2];     // start of popcount class q in the list of all 2^L low parts
-  uint32_t jbase, nJ;
-  const uint32_t* lo_list;      // [nJ] low parts grouped by popcount, ascending
-  // low neighbours in groups of four 16-bit slots: group g of entry j is lo_nbr4[g * nJ + j];
-  // slot 4g + t holds the rank (in its class) of neighbour 4g + t, unused slots hold nq_max,
-  // the index of a zero entry placed after the staged rows
-  int lo_groups;
-  const uint2* lo_nbr4;         // [lo_groups][nJ]
-  const uint8_t* lo_cnt;        // [nJ] neighbours; entries are class-sorted
-  const uint32_t* lo_cls4;      // [lo_groups][nJ] class byte of each slot (multi-class only)
-  const uint16_t* lo_diag;      // [nJ] packed diagonal counts of the low part
+  // low side: class q has lo_off[q + 1] - lo_off[q] low parts, ascending; its tables start at
+  // padded entry lo_pad[q] (whole warps per class), lo_stride entries in all
+  uint32_t lo_off[kSecMaxL + 2];
+  uint32_t lo_pad[kSecMaxL + 2];
+  int64_t lo_stride;
+  const uint2* lo_rec;          // gather table of the low-low bonds (gather.cuh), phases = classes
+  const uint4* lo_hdr;
+  // per low part: x = bits | diagonal count field 0 << 20, y = low bits of the straddling bonds
+  // (bit n: the bit of bond n's low site) | diagonal count field 1 << 24
+  const uint2* lo_info;
   // high side
   const uint64_t* hi_off;       // [2^H] first row element of each high part
-  int hi_slots;
-  const uint32_t* hi_nbr;       // [hi_slots][2^H] neighbour high part | class << 24
-  const uint8_t* hi_cnt;        // [2^H]
   const uint16_t* hi_diag;      // [2^H] packed diagonal counts of the high part
-  // straddling exchange: high bit a, low bit b, class, index of b's rank table
+  // straddling exchange: high bit a, class; ranks (in its class) of lo ^ 2^b, four bonds a record
   int n_str;
-  uint8_t str_a[kSecMaxStr], str_b[kSecMaxStr], str_cls[kSecMaxStr], str_t[kSecMaxStr];
-  const uint16_t* str_rank;     // [sites][nJ] rank (in its class) of lo ^ 2^b
+  uint8_t str_a[kSecMaxStr], str_cls[kSecMaxStr];
+  const uint2* str_rank4;       // [(n_str + 3) / 4][lo_stride]
   // straddling S^z S^z pairs: high bit a, low bit b, layer l.  Pairs of one layer have
   // distinct low bits, so per row the pairs whose high bit is set give one mask of low bits
   // per layer and the count is a popcount per layer; layer l counts into diagonal field sp_lg[l]
@@ -190,11 +185,17 @@ struct SecDev {
   int64_t n_tiles;
   const uint32_t* hi_seq;       // [2^H] high parts in processing order
   const uint32_t* tiles;        // [n_tiles] start in hi_seq | (rows - 1) << 24
-  // high pass work: classes p ascending, stripes, rows of class p
+  // high pass: its own split hL <= L, so that every bond above hL is a combination of whole
+  // (shorter) rows.  Work: classes p ascending, stripes, rows of class p
+  int hL, hH;
+  int hh_c0[kSecMaxCls + 1];    // bonds of class c: hh_mask[hh_c0[c]] .. hh_mask[hh_c0[c + 1] - 1]
+  const uint32_t* hh_mask;      // the two bits a bond flips in the high part
+  const uint64_t* h_off;        // [2^hH] first row element of each high part
+  const uint32_t* h_cls;        // [2^hH] high parts grouped by popcount, ascending
   int n_pc;                     // classes present
-  int pc_p[kSecMaxH + 1];       // popcount of each class present
-  uint32_t pc_row0[kSecMaxH + 2];   // start of the class in hi_cls
-  const uint32_t* hi_cls;       // [2^H] high parts grouped by popcount, ascending
+  uint32_t pc_row0[kSecMaxHH + 1];  // start of the class in h_cls
+  uint32_t pc_rows[kSecMaxHH + 1];  // its high parts
+  uint32_t pc_nq[kSecMaxHH + 1];    // entries of each of its rows
 };
 
 // ------------------------------------------------------------------ scalar traits
@@ -357,21 +358,22 @@ struct SecTerms {
   std::vector<PairEntry> pairs;
   std::vector<double> pcoef;
 };
-struct SecTables;  // device tables of one split (L, K); defined in k_sector.cu
+struct SecTables;  // device tables of one split (L, K) and element size; defined in k_sector.cu
 void sec_free(SecTables* t);
 struct SecTablesDeleter {
   void operator()(SecTables* t) const { sec_free(t); }
 };
 // true when the model takes the split-row path (empty *why), else the reason
 bool sec_applicable(const SecTerms& t, int prec, std::string* why);
-// the split used when nothing else is asked: the largest L whose longest row fits one tile
-// of K = 1 rows of element size esz (0: none fits)
+// the split used when nothing else is asked for element size esz (0: no row fits a tile)
 int sec_default_L(const SecTerms& t, int esz);
-// tile rows K for low-part length L at element size esz (largest power of two that fits)
+// tile rows K for low-part length L at element size esz: 16-byte tile entries if they fit, and
+// the tallest tile the autotuner tries
 int sec_default_K(const SecTerms& t, int L, int esz);
+int sec_tallest_K(const SecTerms& t, int L, int esz);
 // K rows of the longest row of split L fit one tile at element size esz
 bool sec_fits(const SecTerms& t, int L, int K, int esz);
-Status sec_build(const SecTerms& t, int L, int K, SecTables** out, cudaStream_t st);
+Status sec_build(const SecTerms& t, int L, int K, int esz, SecTables** out, cudaStream_t st);
 const SecDev& sec_dev(const SecTables* t);
 size_t sec_scratch_bytes(const SecDev& d, int prec, Epi epi);
 int sec_grid(const SecDev& d, int prec, Epi epi);

@@ -67,6 +67,14 @@ __device__ __forceinline__ double i128_to_double(__int128 v) {
   return fma(__ll2double_rn(hi), 18446744073709551616.0, __ull2double_rn(lo));
 }
 
+// 4- or 8-byte asynchronous copy to shared memory, and 16-byte ones past L1
+template <int B>
+__device__ __forceinline__ void copy_async(void* dst, const void* src) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  if constexpr (B == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(B) : "memory");
+}
+
 // ------------------------------------------------------------------ gather sums
 // fp64 terms are summed in an exact-alignment fixed-point accumulator: every term's
 // 53-bit significand is shifted to the running largest exponent and added as a 64-bit
@@ -218,6 +226,23 @@ __device__ __forceinline__ void epilogue(int64_t idx, typename Traits<S>::R sr, 
     }
     red.tick();
   }
+}
+
+// The refinement's element in folded units (x = xr 2^eoff, hv = hvu 2^e2): two fp64 conversions,
+// one scale and three multiply-adds an element instead of about ten operations.
+template <int NQ>
+__device__ __forceinline__ void refine_folded(double hvu, double xr, double s_e2, int64_t idx, const FusedArgs& fa,
+                                              Red<true, NQ>& red) {
+  reinterpret_cast<double*>(fa.out)[idx] = hvu * s_e2;
+  red.add(0, xr, hvu);
+  red.add(1, xr, xr);
+  red.add(2, hvu, hvu);
+}
+
+// A sum of folded products back in plain units: quantity 0 is x hv, 1 x x and 2 hv hv.
+__device__ __forceinline__ double folded_sum(double x, int q, double s_eoff, double s_e2) {
+  const double a = q == 2 ? s_e2 : s_eoff, b = q == 1 ? s_eoff : s_e2;
+  return (x * a) * b;
 }
 
 template <Epi E> __host__ __device__ constexpr int n_red() {

@@ -22,10 +22,19 @@
 namespace hphi {
 
 constexpr int kGatherPhases = 8;
-// zero entries after a staged row: one per 4 bytes (or fewer, wider ones) of a 128-byte bank row
-constexpr int kGatherZeroBytes = 128;
+// lanes that share one pass over the banks for entries of the given width, which is also the
+// number of zero entries after a staged row
+__host__ __device__ constexpr int gather_lanes(int entry_bytes) {
+  return entry_bytes <= 4 ? 32 : (entry_bytes <= 8 ? 16 : 8);
+}
 
 // records are read in chunks of this many groups; a table has whole chunks allocated
 constexpr int kGatherChunk = 4;
+
+// end of phase f from a warp's header
+__device__ __forceinline__ int gather_end(const uint4& h, int f) {
+  const uint32_t w = f < 2 ? h.x : f < 4 ? h.y : f < 6 ? h.z : h.w;
+  return (int)((f & 1) ? (w >> 16) : (w & 0xffffu));
+}
 
 }  // namespace hphi

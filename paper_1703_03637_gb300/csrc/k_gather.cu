@@ -96,19 +96,15 @@ Status build_gather_table(const uint32_t* nbr, int64_t nbr_stride, const uint8_t
   if (n <= 0) return {};
   const int g = (n + 32 * kGtWarps - 1) / (32 * kGtWarps);
   uint16_t* r = reinterpret_cast<uint16_t*>(rec);
-  switch (entry_bytes) {
-    case 4:
-      k_gather_table<32><<<g, kGtWarps * 32, 0, st>>>(nbr, nbr_stride, deg, n, shift, n_phase, (uint32_t)zero0, r,
-                                                      stride, out0, max_slots, hdr);
-      break;
-    case 8:
-      k_gather_table<16><<<g, kGtWarps * 32, 0, st>>>(nbr, nbr_stride, deg, n, shift, n_phase, (uint32_t)zero0, r,
-                                                      stride, out0, max_slots, hdr);
-      break;
-    default:  // 16 bytes and wider entries: eight lanes a pass
-      k_gather_table<8><<<g, kGtWarps * 32, 0, st>>>(nbr, nbr_stride, deg, n, shift, n_phase, (uint32_t)zero0, r,
-                                                     stride, out0, max_slots, hdr);
+#define HPHI_GT(WW)                                                                                           \
+  k_gather_table<WW><<<g, kGtWarps * 32, 0, st>>>(nbr, nbr_stride, deg, n, shift, n_phase, (uint32_t)zero0, r, \
+                                                  stride, out0, max_slots, hdr)
+  switch (gather_lanes(entry_bytes)) {
+    case 32: HPHI_GT(32); break;
+    case 16: HPHI_GT(16); break;
+    default: HPHI_GT(8);
   }
+#undef HPHI_GT
   HPHI_CUDA_TRY(cudaGetLastError());
   return {};
 }

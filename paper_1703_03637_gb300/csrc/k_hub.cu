@@ -65,6 +65,7 @@ __device__ __forceinline__ void load_k(const R* p, R* out) {
   }
 }
 
+constexpr int kZeroBytes = 128;      // gather_lanes(4 .. 16) entries
 constexpr int kSmemBudget = 208000;  // shared-memory bytes of the row tile (plus its zero entries and ~7 KB static)
 
 // neighbour table of one species, hop-slot major: nbr[q * n + k] is the q-th active hop
@@ -241,14 +242,6 @@ __global__ void __launch_bounds__(kThreads) k_quant(const double* __restrict__ X
   }
 }
 
-// 4- or 8-byte asynchronous copy to shared memory, and 16-byte ones past L1
-template <int B>
-__device__ __forceinline__ void copy_async(void* dst, const void* src) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-  if constexpr (B == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
-  else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(B) : "memory");
-}
-
 // Pass U: up-spin hops on K rows staged in shared memory, the diagonal, + c_dn W and the fused
 // epilogue.  T is float (fp32 vectors) or long long (fp64 vectors on the fixed-point copy; the
 // diagonal term and the reductions take the row's own value from the same quantised tile).
@@ -304,7 +297,7 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_hub_up(const HubDe
   const int c_l2 = cexp - 1023;
   const int e2 = eoff + c_l2;
   const bool fold = c_p2 && eoff >= -1022 && eoff <= 1023 && e2 >= -1022 && e2 <= 1023 &&
-                    (E == Epi::kStore || E == Epi::kLanczos1);
+                    E != Epi::kTpq;
   const double s_eoff = fold ? __longlong_as_double((long long)(eoff + 1023) << 52) : 1.0;
   const double s_e2 = fold ? __longlong_as_double((long long)(e2 + 1023) << 52) : 1.0;
   const double r_k = fold ? __longlong_as_double((long long)(1023 - c_l2) << 52) : 1.0;  // 2^-k
@@ -323,7 +316,7 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_hub_up(const HubDe
   const int dim_up = (int)md.dim_up;
   const int64_t dim_dn = md.dim_dn;
   // the zero entries after the row that unused slots read
-  for (int k = tid; k < kGatherZeroBytes / (int)sizeof(T); k += NT) tile[(size_t)dim_up * K + k] = (T)0;
+  for (int k = tid; k < gather_lanes(K * (int)sizeof(T)) * K; k += NT) tile[(size_t)dim_up * K + k] = (T)0;
   constexpr int NQ = n_red<E>() > 0 ? n_red<E>() : 1;
   Red<FIX, NQ> red;
   red.zero();
@@ -446,6 +439,8 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_hub_up(const HubDe
                 ia = 0;
                 ic = 0;
               }
+            } else if constexpr (E == Epi::kRefine) {
+              refine_folded(hvu, __ll2double_rn(xq), s_e2, idx, fa, red);
             }
             continue;
           }
@@ -494,6 +489,8 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_hub_up(const HubDe
             pmx = max(pmx, (int)((__double_as_longlong(pv) >> 52) & 0x7ff));
             red.add(0, xr, hvu);
             red.tick();
+          } else if constexpr (E == Epi::kRefine) {
+            refine_folded(hvu, xr, s_e2, idx, fa, red);
           }
         } else {
           const double x = fix_to_double(xq, eoff);
@@ -528,7 +525,7 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_hub_up(const HubDe
 #pragma unroll
     for (int q = 0; q < nq; ++q) {
       double x = red.get(q);
-      if (fold) x = (x * s_eoff) * s_e2;  // back from units of 2^(eoff + e2)
+      if (fold) x = folded_sum(x, q, s_eoff, s_e2);
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(0xffffffffu, x, off);
       if (lane == 0) s_red[wid * kMaxRedQ + q] = x;
@@ -581,7 +578,7 @@ inline int up_threads(size_t tile_bytes) { return tile_bytes > 110000 ? 1024 : 5
 template <class KernelT>
 int occupancy_for(KernelT kern, int nt, size_t smem) {
   int n = 0;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + kGatherZeroBytes);
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + kZeroBytes);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, nt, smem) != cudaSuccess || n < 1) {
     cudaGetLastError();
     n = 1;
@@ -590,7 +587,9 @@ int occupancy_for(KernelT kern, int nt, size_t smem) {
 }
 
 template <class T, int K>
-size_t up_smem(const HubDev& md) { return (size_t)K * md.dim_up * sizeof(T) + kGatherZeroBytes; }
+size_t up_smem(const HubDev& md) {
+  return (size_t)K * sizeof(T) * (size_t)(md.dim_up + gather_lanes(K * (int)sizeof(T)));
+}
 
 template <class T, int K, Epi E>
 int up_occupancy(const HubDev& md) {
@@ -603,7 +602,7 @@ template <class T, int K, Epi E>
 Status launch_up(const HubDev& md, const T* X, const T* W, const int* Ep, void* w, const FusedArgs& fa, int grid,
                  cudaStream_t st) {
   const size_t smem = up_smem<T, K>(md);
-  const int most = kSmemBudget + kGatherZeroBytes;
+  const int most = kSmemBudget + kZeroBytes;
   if (up_threads(smem) == 1024) {
     HPHI_CUDA_TRY(cudaFuncSetAttribute(k_hub_up<T, K, E, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     k_hub_up<T, K, E, 1024><<<grid, 1024, smem, st>>>(md, X, W, Ep, w, fa);

@@ -9,16 +9,20 @@
 //   high-high bonds  combine whole rows:      row hi    <- row hi ^ m, same column
 //   straddling bonds gather from one row:     (hi, lo)  <- (hi ^ 2^a, lo ^ 2^b)
 // (section 4.3's point, terms acting on data that is already local, with the row as the
-// local unit).  Two passes:
-//   pass H  (k_sec_hi)  the high-high row combinations, stripe-major per popcount class so
-//           one column stripe of every row of the class is the L2 working set; the plain
-//           sums go to W (a scratch vector for Lanczos, else the output buffer itself).
-//   pass R  (k_sec_lo)  stages K rows of one class in shared memory, applies the low-low
-//           bonds from a per-class neighbour table, gathers the straddling bonds from the
-//           partner rows (for one bond the column map lo -> rank(lo ^ 2^b) is increasing,
-//           so a warp's gathers stay close together), adds the diagonal from integer bond
-//           counts and a small table, adds W and runs the fused Lanczos / mTPQ / refine
-//           epilogue.
+// local unit).  Two passes, each with its own split:
+//   pass H  (k_sec_hi)  the row combinations of every bond above its split hL, stripe-major per
+//           popcount class so one column stripe of every row of the class is the L2 working
+//           set; the plain sums go to W (a scratch vector for Lanczos, else the output itself).
+//   pass R  (k_sec_lo)  stages K rows of one class in shared memory, applies the bonds inside
+//           the row that pass H left (those with a site below hL) from a gather table, gathers
+//           the straddling ones from the partner rows (for one bond the column map
+//           lo -> rank(lo ^ 2^b) is increasing, so a warp's gathers stay close together), adds
+//           the diagonal from integer bond counts and a small table, adds W and runs the fused
+//           Lanczos / mTPQ / refine epilogue.
+// Pass H costs a third of pass R per active bond (coalesced, no tables), so hL is as small as
+// rows of a few hundred entries allow: it takes the bonds of the sites hL .. L - 1 among
+// themselves, which would be gathers of pass R, and those of these sites with the high part,
+// which would straddle.
 // fp64 vectors run on the 64-bit fixed-point copy (integer sums, one conversion per
 // element); fp32 vectors sum in fp32.
 #include <math.h>
@@ -32,6 +36,7 @@
 
 #include "common.cuh"
 #include "epilogue.cuh"
+#include "gather.cuh"
 #include "reduce.cuh"
 
 namespace hphi {
@@ -234,7 +239,8 @@ Analysis analyse(const SecTerms& t) {
   return a;
 }
 
-constexpr int kTileBudget = 200000;  // shared-memory bytes of one row tile
+constexpr int kTileBudget = 200000;  // shared-memory bytes of one row tile (without its zero entries)
+constexpr int kSecHighL = 12;        // pass H split where the number of high bits allows it
 
 // longest row of a class present in the sector for low-part length L
 uint64_t longest_row(int N, int n_ones, int L) {
@@ -270,7 +276,10 @@ bool sec_applicable(const SecTerms& t, int prec, std::string* why) {
   return true;
 }
 
-int sec_default_L(const SecTerms& t, int esz) {
+namespace {
+
+// largest low part whose longest row fits one tile of one row (0: none)
+int largest_L(const SecTerms& t, int esz) {
   const int N = t.n_sites;
   for (int L = std::min(kSecMaxL, N - 1); L >= 1; --L) {
     if (!split_ok(N, L)) continue;
@@ -280,20 +289,75 @@ int sec_default_L(const SecTerms& t, int esz) {
   return 0;
 }
 
+// why split L cannot be built (empty: it can): the limits on bonds and pairs across it
+std::string straddle_limits(const Analysis& a, int L) {
+  int n_str = 0, n_sp = 0;
+  uint64_t sites = 0;
+  for (const Bond& b : a.bonds)
+    if (b.i < L && b.j >= L) {
+      ++n_str;
+      sites |= 1ull << b.i;
+    }
+  if (n_str > kSecMaxStr) return "split-row path: too many straddling bonds";
+  if (__builtin_popcountll(sites) > kSecMaxStrSites) return "split-row path: too many straddling sites";
+  std::vector<std::pair<int, uint64_t>> layers;  // diagonal group, low sites used
+  for (int g = 0; g < a.n_dg; ++g)
+    for (const auto& pr : a.gpairs[g]) {
+      if (!(pr.first < L && pr.second >= L)) continue;
+      if (++n_sp > kSecMaxSp) return "split-row path: too many straddling S^z S^z pairs";
+      const uint64_t bit = 1ull << pr.first;
+      size_t l = 0;
+      while (l < layers.size() && (layers[l].first != g || (layers[l].second & bit))) ++l;
+      if (l == layers.size()) layers.emplace_back(g, 0);
+      layers[l].second |= bit;
+    }
+  return layers.size() > (size_t)kSecMaxSl ? "split-row path: too many straddling pair layers" : "";
+}
+
+// Pass H's split.  Rows of C(12, 6) = 924 entries fill 128-column stripes to nine tenths; fp64
+// Lanczos group (pass H + pass R) at hL = 9 / 10 / 11 / 12 / 13 on GB300: 6x5 torus, S^z = 0
+// 4.69 / 4.18 / 3.98 / 3.98 / 3.95 ms; 28-site J1-J2 ring, 9 up 0.50 / 0.40 / 0.36 / 0.33 ms
+// (at 9 bits a row's part-filled stripes cost more than the bonds it takes over).
+int high_L(int N, int L) { return std::min(L, std::max(kSecHighL, N - kSecMaxHH)); }
+
+}  // namespace
+
+// The low part used when nothing else is asked: rows of C(14, 7) = 3,432 entries in fp64, two a
+// tile (55 KB), and C(15, 7) = 6,435 in fp32, four a tile (103 KB), so two CTAs share an SM;
+// below 24 sites N - 10 bits (at least 12) keep enough tiles for every SM.  fp64 Lanczos group
+// at (L, K) on GB300: 6x5 torus (13, 2) 4.68, (14, 2) 3.98, (15, 2) 4.06, (16, 1) 4.29,
+// (17, 1) 4.43 ms; 28-site J1-J2 ring, S^z = 0 (13, 2) 1.31, (14, 2) 1.19, (15, 2) 1.24,
+// (17, 1) 1.49 ms; 6x4 torus (12, 2) 0.108, (13, 2) 0.101, (14, 2) 0.099 ms.  A split that the
+// limits above rule out gives way to the next larger.
+int sec_default_L(const SecTerms& t, int esz) {
+  const int most = largest_L(t, esz);
+  if (most == 0) return 0;
+  const Analysis a = analyse(t);
+  if (!a.ok || !straddle_limits(a, most).empty()) return most;
+  for (int L = std::min(most, std::min(esz >= 8 ? 14 : 15, std::max(12, t.n_sites - 10))); L < most; ++L)
+    if (split_ok(t.n_sites, L) && straddle_limits(a, L).empty()) return L;
+  return most;
+}
+
 bool sec_fits(const SecTerms& t, int L, int K, int esz) {
   if (!split_ok(t.n_sites, L) || K < 1) return false;
   const uint64_t r = longest_row(t.n_sites, t.n_ones, L);
   return r >= 1 && r <= 65535 && r * (uint64_t)esz * (uint64_t)K <= (uint64_t)kTileBudget;
 }
 
-int sec_default_K(const SecTerms& t, int L, int esz) {
+// tallest tile that fits, up to kmax rows
+static int tallest(const SecTerms& t, int L, int esz, int kmax) {
   const uint64_t r = std::max<uint64_t>(1, longest_row(t.n_sites, t.n_ones, L));
-  // 8-byte elements stop at 4 rows (8 int64 rows run out of registers)
-  const int kmax = esz >= 8 ? 4 : 8;
   int K = 1;
   while (K < kmax && r * esz * (uint64_t)(2 * K) <= (uint64_t)kTileBudget) K *= 2;
   return K;
 }
+
+// rows per tile: 16-byte tile entries (two int64 or four fp32 rows) take one shared-memory load
+// a neighbour; taller tiles are left to the autotuner (8-byte elements stop at 4 rows: 8 int64
+// rows run out of registers)
+int sec_default_K(const SecTerms& t, int L, int esz) { return tallest(t, L, esz, 16 / esz); }
+int sec_tallest_K(const SecTerms& t, int L, int esz) { return tallest(t, L, esz, esz >= 8 ? 4 : 8); }
 
 // ====================================================================== device tables
 struct SecTables {
@@ -328,9 +392,40 @@ Status up(SecTables* T, const std::vector<X>& v, const X** out, cudaStream_t st)
   return {};
 }
 
+// device room for n values, owned by T
+template <class X>
+Status room(SecTables* T, size_t n, X** out) {
+  void* p = nullptr;
+  const size_t b = sizeof(X) * std::max<size_t>(1, n);
+  const cudaError_t e = cudaMalloc(&p, b);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return {e == cudaErrorMemoryAllocation ? HPHI_ERR_OUT_OF_MEMORY : HPHI_ERR_CUDA,
+            std::string("split-row tables: cudaMalloc(") + std::to_string(b) + "): " + cudaGetErrorString(e)};
+  }
+  T->bufs.push_back(p);
+  *out = reinterpret_cast<X*>(p);
+  return {};
+}
+
+// neighbour lists of one low class: nbr[slot * n + u] = rank of lo ^ mask | class << 24
+__global__ void k_sec_nbr(const uint32_t* __restrict__ list, int n, const uint32_t* __restrict__ rank,
+                          const uint32_t* __restrict__ bonds, int n_bonds, uint32_t* __restrict__ nbr,
+                          uint8_t* __restrict__ deg) {
+  const int u = blockIdx.x * kThreads + threadIdx.x;
+  if (u >= n) return;
+  const uint32_t lo = list[u];
+  int c = 0;
+  for (int k = 0; k < n_bonds; ++k) {
+    const uint32_t m = bonds[k] & 0xffffffu;
+    if (__popc(lo & m) == 1) nbr[(int64_t)(c++) * n + u] = rank[lo ^ m] | (bonds[k] & 0xff000000u);
+  }
+  deg[u] = (uint8_t)c;
+}
+
 }  // namespace
 
-Status sec_build(const SecTerms& t, int L, int K, SecTables** out, cudaStream_t st) {
+Status sec_build(const SecTerms& t, int L, int K, int esz, SecTables** out, cudaStream_t st) {
   *out = nullptr;
   Analysis a = analyse(t);
   if (!a.ok) return {HPHI_ERR_UNSUPPORTED, a.why};
@@ -361,6 +456,10 @@ Status sec_build(const SecTerms& t, int L, int K, SecTables** out, cudaStream_t 
   d.qextra = a.qextra;
   d.dint = a.dint ? 1 : 0;
 
+  {
+    const std::string why = straddle_limits(a, L);
+    if (!why.empty()) return {HPHI_ERR_UNSUPPORTED, why};
+  }
   // low side: popcount-grouped list and ranks
   std::vector<uint32_t> lo_rank(nL), lo_list(nL);
   {
@@ -376,76 +475,37 @@ Status sec_build(const SecTerms& t, int L, int K, SecTables** out, cudaStream_t 
   }
   // the low-part tables cover the classes present, q in [n1 - H, n1] within [0, L]
   const int qmin = std::max(0, n1 - H), qmax = std::min(L, n1);
-  const uint32_t j0 = d.lo_off[qmin], nJ = d.lo_off[qmax + 1] - j0;
-  d.jbase = j0;
-  d.nJ = nJ;
-  // bonds by group
-  std::vector<int> llb, hhb, stb;
-  for (size_t k = 0; k < a.bonds.size(); ++k) {
+  d.lo_stride = 0;
+  for (int q = qmin; q <= qmax; ++q) {
+    d.lo_pad[q] = (uint32_t)d.lo_stride;
+    d.lo_stride += (d.lo_off[q + 1] - d.lo_off[q] + 31) / 32 * 32;
+  }
+  // bonds by pass, class by class
+  d.hL = high_L(N, L);
+  d.hH = N - d.hL;
+  std::vector<int> order(a.bonds.size());
+  for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return a.bond_cls[x] < a.bond_cls[y]; });
+  std::vector<uint32_t> ll, hh;  // ll: the two low bits | class << 24
+  std::vector<int> stb;
+  for (int c = 0; c <= kSecMaxCls; ++c) d.hh_c0[c] = 0;
+  for (int k : order) {
     const Bond& b = a.bonds[k];
-    if (b.j < L) llb.push_back((int)k);
-    else if (b.i >= L) hhb.push_back((int)k);
-    else stb.push_back((int)k);
-  }
-  if ((int)stb.size() > kSecMaxStr) return {HPHI_ERR_UNSUPPORTED, "split-row path: too many straddling bonds"};
-  // low neighbour table, class-sorted per entry
-  std::vector<int> ll_sorted = llb;
-  std::stable_sort(ll_sorted.begin(), ll_sorted.end(), [&](int x, int y) { return a.bond_cls[x] < a.bond_cls[y]; });
-  int lo_slots = 0;
-  std::vector<uint8_t> lo_cnt(nJ, 0);
-  std::vector<uint16_t> lo_diag(nJ, 0);
-  for (uint32_t j = 0; j < nJ; ++j) {
-    const uint32_t lo = lo_list[j0 + j];
-    int c = 0;
-    for (int k : ll_sorted) {
-      const Bond& b = a.bonds[k];
-      if (((lo >> b.i) ^ (lo >> b.j)) & 1u) ++c;
-    }
-    if (c > 255) return {HPHI_ERR_UNSUPPORTED, "split-row path: more than 255 low-part neighbours"};
-    lo_cnt[j] = (uint8_t)c;
-    lo_slots = std::max(lo_slots, c);
-  }
-  // groups of four slots; slots past an entry's count point at the zero entry (index nq_max)
-  const int G = std::max(1, (lo_slots + 3) / 4);
-  std::vector<uint16_t> lo_nbr((size_t)G * nJ * 4, (uint16_t)nqmax);
-  std::vector<uint8_t> lo_cls(d.one_cls ? 4 : (size_t)G * nJ * 4, 0);
-  for (uint32_t j = 0; j < nJ; ++j) {
-    const uint32_t lo = lo_list[j0 + j];
-    int s = 0;
-    for (int k : ll_sorted) {
-      const Bond& b = a.bonds[k];
-      if (!(((lo >> b.i) ^ (lo >> b.j)) & 1u)) continue;
-      const uint32_t lo2 = lo ^ ((1u << b.i) | (1u << b.j));
-      const size_t o = ((size_t)(s / 4) * nJ + j) * 4 + (s % 4);
-      lo_nbr[o] = (uint16_t)lo_rank[lo2];  // same class: rank < C(L, q) <= 65535
-      if (!d.one_cls) lo_cls[o] = (uint8_t)a.bond_cls[k];
-      ++s;
+    const int c = a.bond_cls[k];
+    if (b.i >= d.hL) {
+      hh.push_back((1u << (b.i - d.hL)) | (1u << (b.j - d.hL)));
+      for (int e = c + 1; e <= kSecMaxCls; ++e) ++d.hh_c0[e];
+    } else if (b.j < L) {
+      ll.push_back((1u << b.i) | (1u << b.j) | ((uint32_t)c << 24));
+    } else {
+      stb.push_back(k);
     }
   }
-  d.lo_groups = G;
-  // straddling bonds (a = high site - L, b = low site) and one rank table per distinct low site
-  std::vector<int> str_sites;
   d.n_str = (int)stb.size();
   for (int n = 0; n < d.n_str; ++n) {
-    const Bond& b = a.bonds[stb[n]];
-    d.str_a[n] = (uint8_t)(b.j - L);
-    d.str_b[n] = (uint8_t)b.i;
+    d.str_a[n] = (uint8_t)(a.bonds[stb[n]].j - L);
     d.str_cls[n] = (uint8_t)a.bond_cls[stb[n]];
-    auto it = std::find(str_sites.begin(), str_sites.end(), b.i);
-    if (it == str_sites.end()) {
-      str_sites.push_back(b.i);
-      it = str_sites.end() - 1;
-    }
-    d.str_t[n] = (uint8_t)(it - str_sites.begin());
   }
-  if ((int)str_sites.size() > kSecMaxStrSites) return {HPHI_ERR_UNSUPPORTED, "split-row path: too many straddling sites"};
-  std::vector<uint16_t> str_rank((size_t)std::max<size_t>(1, str_sites.size()) * nJ, 0);
-  for (size_t u = 0; u < str_sites.size(); ++u)
-    for (uint32_t j = 0; j < nJ; ++j) {
-      const uint32_t r = lo_rank[lo_list[j0 + j] ^ (1u << str_sites[u])];
-      // ranks in classes that never receive a straddling gather may exceed 16 bits; unused
-      str_rank[u * nJ + j] = (uint16_t)(r <= 65535 ? r : 0);
-    }
   // diagonal counts: field g of 8 bits
   auto counts = [&](uint64_t s, int side) -> uint16_t {  // side 0: low part only, 1: high part only
     uint32_t packed = 0;
@@ -461,7 +521,24 @@ Status sec_build(const SecTerms& t, int L, int K, SecTables** out, cudaStream_t 
     }
     return (uint16_t)packed;
   };
-  for (uint32_t j = 0; j < nJ; ++j) lo_diag[j] = counts(lo_list[j0 + j], 0);
+  std::vector<uint2> lo_info((size_t)d.lo_stride, make_uint2(0u, 0u));
+  const int n_sg = (d.n_str + 3) / 4;
+  std::vector<uint16_t> str_rank((size_t)std::max(1, n_sg) * 4 * (size_t)d.lo_stride, 0);
+  for (int q = qmin; q <= qmax; ++q)
+    for (uint32_t u = 0; u < d.lo_off[q + 1] - d.lo_off[q]; ++u) {
+      const uint32_t lo = lo_list[d.lo_off[q] + u];
+      const size_t j = d.lo_pad[q] + u;
+      const uint32_t dc = counts(lo, 0);
+      uint32_t bits = 0;
+      for (int n = 0; n < d.n_str; ++n) {
+        const int b = a.bonds[stb[n]].i;
+        bits |= ((lo >> b) & 1u) << n;
+        // ranks in classes that never receive a straddling gather may exceed 16 bits; unused
+        const uint32_t r = lo_rank[lo ^ (1u << b)];
+        str_rank[((size_t)(n / 4) * (size_t)d.lo_stride + j) * 4 + (n % 4)] = (uint16_t)(r <= 65535 ? r : 0);
+      }
+      lo_info[j] = make_uint2(lo | ((dc & 0xffu) << 20), bits | ((dc >> 8) << 24));
+    }
   // straddling S^z S^z pairs in layers: a pair joins the first layer of its group that has
   // no pair on the same low site yet (one low bit counts one pair per layer)
   d.n_sp = 0;
@@ -470,12 +547,10 @@ Status sec_build(const SecTerms& t, int L, int K, SecTables** out, cudaStream_t 
   for (int g = 0; g < a.n_dg; ++g)
     for (const auto& pr : a.gpairs[g]) {
       if (pr.first < L && pr.second >= L) {
-        if (d.n_sp >= kSecMaxSp) return {HPHI_ERR_UNSUPPORTED, "split-row path: too many straddling S^z S^z pairs"};
         const uint32_t bit = 1u << pr.first;
         int l = 0;
         while (l < d.n_sl && (d.sp_lg[l] != g || (layer_bits[l] & bit))) ++l;
         if (l == d.n_sl) {
-          if (d.n_sl >= kSecMaxSl) return {HPHI_ERR_UNSUPPORTED, "split-row path: too many straddling pair layers"};
           d.sp_lg[d.n_sl++] = (uint8_t)g;
           layer_bits.push_back(0u);
         }
@@ -502,46 +577,24 @@ Status sec_build(const SecTerms& t, int L, int K, SecTables** out, cudaStream_t 
     }
     if (run != (uint64_t)d.dim) return {HPHI_ERR_CUDA, "split-row path: row offsets do not add up to the dimension"};
   }
-  std::vector<int> hh_sorted = hhb;
-  std::stable_sort(hh_sorted.begin(), hh_sorted.end(), [&](int x, int y) { return a.bond_cls[x] < a.bond_cls[y]; });
-  int hi_slots = 0;
-  std::vector<uint8_t> hi_cnt(nH, 0);
   std::vector<uint16_t> hi_diag(nH, 0);
-  for (uint32_t hi = 0; hi < nH; ++hi) {
-    int c = 0;
-    for (int k : hh_sorted) {
-      const Bond& b = a.bonds[k];
-      if (((hi >> (b.i - L)) ^ (hi >> (b.j - L))) & 1u) ++c;
-    }
-    hi_cnt[hi] = (uint8_t)c;
-    hi_slots = std::max(hi_slots, c);
-    hi_diag[hi] = counts((uint64_t)hi << L, 1);
-  }
-  std::vector<uint32_t> hi_nbr((size_t)std::max(1, hi_slots) * nH, 0);
-  for (uint32_t hi = 0; hi < nH; ++hi) {
-    int s = 0;
-    for (int k : hh_sorted) {
-      const Bond& b = a.bonds[k];
-      if (!(((hi >> (b.i - L)) ^ (hi >> (b.j - L))) & 1u)) continue;
-      const uint32_t h2 = hi ^ ((1u << (b.i - L)) | (1u << (b.j - L)));
-      hi_nbr[(size_t)s * nH + hi] = h2 | ((uint32_t)a.bond_cls[k] << 24);
-      ++s;
-    }
-  }
-  d.hi_slots = hi_slots;
-  // classes present, high parts grouped by popcount
-  std::vector<uint32_t> hi_cls;
+  for (uint32_t hi = 0; hi < nH; ++hi) hi_diag[hi] = counts((uint64_t)hi << L, 1);
+  // classes of pass H: high parts grouped by popcount
   d.n_pc = 0;
-  for (int p = 0; p <= H; ++p) {
-    const int q = n1 - p;
-    if (q < 0 || q > L) continue;
-    d.pc_p[d.n_pc] = p;
-    d.pc_row0[d.n_pc] = (uint32_t)hi_cls.size();
-    for (uint32_t hi = 0; hi < nH; ++hi)
-      if (__builtin_popcount(hi) == p) hi_cls.push_back(hi);
-    ++d.n_pc;
+  {
+    uint32_t row0 = 0;
+    for (int p = 0; p <= d.hH; ++p) {
+      const uint32_t rows = (uint32_t)binom_u(d.hH, p);
+      const int q = n1 - p;
+      if (q >= 0 && q <= d.hL) {
+        d.pc_row0[d.n_pc] = row0;
+        d.pc_rows[d.n_pc] = rows;
+        d.pc_nq[d.n_pc] = (uint32_t)binom_u(d.hL, q);
+        ++d.n_pc;
+      }
+      row0 += rows;
+    }
   }
-  d.pc_row0[d.n_pc] = (uint32_t)hi_cls.size();
   // row-pass tiles.  A row is read three times: staged by its own tile, and gathered by the
   // tiles of its straddling partners hi ^ 2^a (a in S, the high bits of the straddling bonds),
   // which lie one class above or below.  Blocks of high parts that agree outside S are closed
@@ -563,8 +616,7 @@ Status sec_build(const SecTerms& t, int L, int K, SecTables** out, cudaStream_t 
     std::sort(sv.begin(), sv.end());
     std::vector<uint32_t> in_cls;
     for (uint32_t o = 0;; o = ((o | S) + 1) & nonS) {  // the settings of the other bits, ascending
-      for (int i = 0; i < d.n_pc; ++i) {
-        const int p = d.pc_p[i];
+      for (int p = std::max(0, n1 - L); p <= std::min(H, n1); ++p) {
         in_cls.clear();
         for (uint32_t x : sv)
           if (__builtin_popcount(o | x) == p) in_cls.push_back(o | x);
@@ -580,29 +632,68 @@ Status sec_build(const SecTerms& t, int L, int K, SecTables** out, cudaStream_t 
   d.n_tiles = (int64_t)tiles.size();
 
   Status s;
-  const std::vector<uint32_t> lo_used(lo_list.begin() + j0, lo_list.begin() + j0 + nJ);
-  if ((s = up(T.get(), lo_used, &d.lo_list, st)).code) return s;
+  if ((s = up(T.get(), lo_info, &d.lo_info, st)).code) return s;
   {
     const uint16_t* p16 = nullptr;
-    if ((s = up(T.get(), lo_nbr, &p16, st)).code) return s;
-    d.lo_nbr4 = reinterpret_cast<const uint2*>(p16);
+    if ((s = up(T.get(), str_rank, &p16, st)).code) return s;
+    d.str_rank4 = reinterpret_cast<const uint2*>(p16);
   }
-  if ((s = up(T.get(), lo_cnt, &d.lo_cnt, st)).code) return s;
-  {
-    const uint8_t* p8 = nullptr;
-    if ((s = up(T.get(), lo_cls, &p8, st)).code) return s;
-    d.lo_cls4 = reinterpret_cast<const uint32_t*>(p8);
-  }
-  if ((s = up(T.get(), lo_diag, &d.lo_diag, st)).code) return s;
+  if ((s = up(T.get(), hh, &d.hh_mask, st)).code) return s;
   if ((s = up(T.get(), hi_off, &d.hi_off, st)).code) return s;
-  if ((s = up(T.get(), hi_nbr, &d.hi_nbr, st)).code) return s;
-  if ((s = up(T.get(), hi_cnt, &d.hi_cnt, st)).code) return s;
   if ((s = up(T.get(), hi_diag, &d.hi_diag, st)).code) return s;
-  if ((s = up(T.get(), str_rank, &d.str_rank, st)).code) return s;
   if ((s = up(T.get(), dtab, &d.dtab, st)).code) return s;
   if ((s = up(T.get(), hi_seq, &d.hi_seq, st)).code) return s;
   if ((s = up(T.get(), tiles, &d.tiles, st)).code) return s;
-  if ((s = up(T.get(), hi_cls, &d.hi_cls, st)).code) return s;
+  // the gather table (per class, in its padded place) and pass H's row offsets and class lists
+  // are built on the device; what only the builders read is freed with `tmp`
+  SecTables tmp;
+  struct Free {
+    SecTables& t;
+    ~Free() {
+      for (void* p : t.bufs) cudaFree(p);
+    }
+  } free_tmp{tmp};
+  const uint32_t *g_rank = nullptr, *g_list = nullptr, *g_ll = nullptr, *g_off = nullptr;
+  if ((s = up(&tmp, lo_rank, &g_rank, st)).code) return s;
+  if ((s = up(&tmp, lo_list, &g_list, st)).code) return s;
+  if ((s = up(&tmp, ll, &g_ll, st)).code) return s;
+  const int n_ll = (int)ll.size();
+  const int slots = std::max(1, (n_ll + 4 * kGatherChunk - 1) / (4 * kGatherChunk)) * 4 * kGatherChunk;
+  uint32_t* g_nbr = nullptr;
+  uint8_t* g_deg = nullptr;
+  uint2* rec = nullptr;
+  uint4* hdr = nullptr;
+  uint32_t *h_cls = nullptr, *h_rank = nullptr;
+  uint64_t* h_off = nullptr;
+  const size_t n_h = (size_t)1 << d.hH;
+  if ((s = room(&tmp, (size_t)std::max(1, n_ll) * nqmax, &g_nbr)).code) return s;
+  if ((s = room(&tmp, nqmax, &g_deg)).code) return s;
+  if ((s = room(&tmp, n_h, &h_rank)).code) return s;
+  if ((s = room(T.get(), (size_t)(slots / 4) * (size_t)d.lo_stride, &rec)).code) return s;
+  if ((s = room(T.get(), (size_t)d.lo_stride / 32, &hdr)).code) return s;
+  if ((s = room(T.get(), n_h, &h_cls)).code) return s;
+  if ((s = room(T.get(), n_h, &h_off)).code) return s;
+  const int entry = (int)(K * esz);
+  for (int q = qmin; q <= qmax; ++q) {
+    const int n = (int)(d.lo_off[q + 1] - d.lo_off[q]);
+    k_sec_nbr<<<(n + kThreads - 1) / kThreads, kThreads, 0, st>>>(g_list + d.lo_off[q], n, g_rank, g_ll, n_ll, g_nbr, g_deg);
+    HPHI_CUDA_TRY(cudaGetLastError());
+    if ((s = build_gather_table(g_nbr, n, g_deg, n, 24, std::max(1, d.n_cls), d.nq_max, entry, rec, d.lo_stride,
+                                d.lo_pad[q], slots, hdr, st)).code)
+      return s;
+  }
+  {
+    std::vector<uint32_t> off(d.hH + 2, 0);
+    for (int p = 0; p <= d.hH; ++p) off[p + 1] = off[p] + (uint32_t)binom_u(d.hH, p);
+    if ((s = up(&tmp, off, &g_off, st)).code) return s;
+    HPHI_CUDA_TRY(cudaStreamSynchronize(st));  // `off` dies here
+    if ((s = build_popcount_tables(d.hH, h_rank, h_cls, g_off, st)).code) return s;
+    if ((s = build_hi_offsets(d.hL, d.hH, n1, h_off, st)).code) return s;
+  }
+  d.lo_rec = rec;
+  d.lo_hdr = hdr;
+  d.h_cls = h_cls;
+  d.h_off = h_off;
   HPHI_CUDA_TRY(cudaStreamSynchronize(st));  // host vectors die here
   *out = T.release();
   return {};
@@ -626,43 +717,43 @@ __device__ __forceinline__ float sec_w<float>(const SecDev& d, int c) { return (
 template <>
 __device__ __forceinline__ long long sec_w<long long>(const SecDev& d, int c) { return (long long)d.mult[c]; }
 
-// pass H: W[row hi][col] = sum over active high-high bonds of w X[row hi'][col].  Warp items
-// (class, stripe of 32 * EPT columns, row) run class by class and stripe by stripe, claimed in
-// order from a counter, so the stripe of all rows of the class stays in L2 while it is used.
+// pass H: W[row hi][col] = sum over active bonds above the split hL of w X[row hi'][col].  Warp
+// items (class, stripe of 32 * EPT columns, row) run class by class and stripe by stripe,
+// claimed in order from a counter, so the stripe of all rows of the class stays in L2 while it
+// is used.  Lane k of the warp tests bond k and fetches its partner row's offset; the active
+// ones are compacted into shared memory and read back as broadcasts.  Bonds of one coefficient
+// class are summed plainly and weighted once.  6x5 torus, S^z = 0 (155,117,520 rows), int64, 30
+// bonds at hL = 12 (25 lie above pass R's L = 14): 1.09 ms, bound by the loads' L1
+// wavefronts (84 %), the integer pipe (65 %) and L2 (69 %).
 template <class T, int EPT, bool ONE>
 __global__ void __launch_bounds__(kThreads) k_sec_hi(const SecDev d, const T* __restrict__ X, T* W,
                                                      const int* __restrict__ done,
                                                      unsigned long long* __restrict__ counter) {
   if (done != nullptr && *done) return;
   constexpr int SW = 32 * EPT;
-  __shared__ long long s_item0[kSecMaxH + 2];
-  __shared__ uint32_t s_nrow[kSecMaxH + 1], s_nq[kSecMaxH + 1], s_nstr[kSecMaxH + 1];
+  __shared__ long long s_item0[kSecMaxHH + 2];
+  __shared__ uint32_t s_nrow[kSecMaxHH + 1], s_nq[kSecMaxHH + 1], s_row0[kSecMaxHH + 1];
+  __shared__ int s_c0[kSecMaxCls + 1];
   __shared__ T s_w[kSecMaxCls];
   __shared__ unsigned long long s_claim;
-  // per warp: the current batch of neighbour rows (first element, weight), read back as
-  // shared-memory broadcasts by every lane
-  __shared__ uint64_t s_src[kHiWarps][32];
-  __shared__ T s_wt[kHiWarps][32];
+  __shared__ uint64_t s_src[kHiWarps][32];  // per warp: first element of each active partner row
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) {
     long long acc = 0;
     for (int i = 0; i < d.n_pc; ++i) {
-      const int q = d.n_ones - d.pc_p[i];
-      const uint32_t nrow = d.pc_row0[i + 1] - d.pc_row0[i];
-      const uint32_t nq = d.lo_off[q + 1] - d.lo_off[q];
-      const uint32_t ns = (nq + SW - 1) / SW;
       s_item0[i] = acc;
-      s_nrow[i] = nrow;
-      s_nq[i] = nq;
-      s_nstr[i] = ns;
-      acc += (long long)nrow * ns;
+      s_nrow[i] = d.pc_rows[i];
+      s_nq[i] = d.pc_nq[i];
+      s_row0[i] = d.pc_row0[i];
+      acc += (long long)d.pc_rows[i] * ((d.pc_nq[i] + SW - 1) / SW);
     }
     s_item0[d.n_pc] = acc;
   }
   if (tid < kSecMaxCls) s_w[tid] = tid < d.n_cls ? sec_w<T>(d, tid) : (T)0;
+  if (tid <= kSecMaxCls) s_c0[tid] = d.hh_c0[tid];
   __syncthreads();
   const long long total = s_item0[d.n_pc];
-  const size_t nH = (size_t)1 << d.H;
+  const int n_cls = ONE ? 1 : d.n_cls;
   for (;;) {
     if (tid == 0) s_claim = atomicAdd(counter, (unsigned long long)(kHiWarps * kHiClaim));
     __syncthreads();
@@ -676,50 +767,57 @@ __global__ void __launch_bounds__(kThreads) k_sec_hi(const SecDev d, const T* __
       while (item >= s_item0[pc + 1]) ++pc;
       const long long k = item - s_item0[pc];
       const uint32_t nrow = s_nrow[pc];
-      const uint32_t sidx = (uint32_t)(k / nrow);
-      const uint32_t r = (uint32_t)(k - (long long)sidx * nrow);
+      const uint32_t sidx = (uint32_t)k / nrow;  // fewer than 2^32 items a class
+      const uint32_t r = (uint32_t)k - sidx * nrow;
       const int nq = (int)s_nq[pc];
-      const uint32_t hi = __ldg(d.hi_cls + d.pc_row0[pc] + r);
-      const uint64_t o = __ldg(d.hi_off + hi);
-      const int cnt = __ldg(d.hi_cnt + hi);
+      const uint32_t hi = __ldg(d.h_cls + s_row0[pc] + r);
+      const uint64_t o = __ldg(d.h_off + hi);
       const int col0 = (int)sidx * SW + lane;
       const bool full = (int)sidx * SW + SW <= nq;  // the whole stripe lies inside the row
-      T acc[EPT];
+      T tot[EPT];
 #pragma unroll
-      for (int j = 0; j < EPT; ++j) acc[j] = (T)0;
-      for (int qb = 0; qb < cnt; qb += 32) {
-        const int nn = min(32, cnt - qb);
-        __syncwarp();  // the previous batch's entries have been read
-        if (lane < nn) {
-          const uint32_t e = __ldg(d.hi_nbr + (size_t)(qb + lane) * nH + hi);
-          s_src[warp][lane] = __ldg(d.hi_off + (e & 0xffffffu));
-          if constexpr (!ONE) s_wt[warp][lane] = s_w[e >> 24];
-        }
-        __syncwarp();
-        for (int q0 = 0; q0 < nn; q0 += 4) {
-          T x[4][EPT];
+      for (int j = 0; j < EPT; ++j) tot[j] = (T)0;
+      for (int c = 0; c < n_cls; ++c) {
+        T acc[EPT];
 #pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const bool on = q0 + t < nn;
-            const T* p = X + s_src[warp][(q0 + t) & 31] + col0;
+        for (int j = 0; j < EPT; ++j) acc[j] = (T)0;
+        const int b1 = s_c0[c + 1];
+        for (int qb = s_c0[c]; qb < b1; qb += 32) {
+          const uint32_t m = qb + lane < b1 ? __ldg(d.hh_mask + qb + lane) : 0u;
+          const bool on = __popc(hi & m) == 1;
+          const unsigned bal = __ballot_sync(0xffffffffu, on);  // the previous batch has been read
+          if (on) s_src[warp][__popc(bal & ((1u << lane) - 1u))] = __ldg(d.h_off + (hi ^ m));
+          const int nn = __popc(bal);
+          __syncwarp();
+          for (int q0 = 0; q0 < nn; q0 += 4) {
+            T x[4][EPT];
 #pragma unroll
-            for (int j = 0; j < EPT; ++j) x[t][j] = (on && (full || col0 + j * 32 < nq)) ? __ldg(p + j * 32) : (T)0;
-          }
+            for (int t = 0; t < 4; ++t) {
+              const bool live = q0 + t < nn;
+              const T* p = X + s_src[warp][(q0 + t) & 31] + col0;
 #pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const T wt = ONE ? (T)1 : ((q0 + t < nn) ? s_wt[warp][(q0 + t) & 31] : (T)0);
-#pragma unroll
-            for (int j = 0; j < EPT; ++j) {
-              if constexpr (ONE) acc[j] += x[t][j];
-              else acc[j] += wt * x[t][j];
+              for (int j = 0; j < EPT; ++j) x[t][j] = (live && (full || col0 + j * 32 < nq)) ? __ldg(p + j * 32) : (T)0;
             }
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+#pragma unroll
+              for (int j = 0; j < EPT; ++j) acc[j] += x[t][j];
           }
+          __syncwarp();
+        }
+        if constexpr (ONE) {
+#pragma unroll
+          for (int j = 0; j < EPT; ++j) tot[j] = acc[j];
+        } else {
+          const T wt = s_w[c];
+#pragma unroll
+          for (int j = 0; j < EPT; ++j) tot[j] += wt * acc[j];
         }
       }
 #pragma unroll
       for (int j = 0; j < EPT; ++j) {
         const int col = col0 + j * 32;
-        if (col < nq) W[o + col] = acc[j];
+        if (col < nq) W[o + col] = tot[j];
       }
     }
   }
@@ -743,13 +841,18 @@ __device__ __forceinline__ void tile_load(const T* p, T* out) {
   }
 }
 
-// pass R: K rows of one class in shared memory; low-low exchange from the grouped neighbour
-// table, straddling exchange gathered from the partner rows, diagonal from packed counts, plus
-// the pass-H sums Wh, then the fused epilogue.  X is the input (fp32) or its fixed-point copy.
-// Every thread owns E elements of the tile at a time (E * K values); the straddling bonds run
-// in an outer loop that is the same for all threads, so each bond's constants (low bit, rank
-// table, partner row pointers, activating bit values) are read once per thread and used for
-// all its elements, and the loads of the E elements are independent.
+// pass R: K rows of one class in shared memory; the bonds inside the row from the gather table,
+// straddling exchange gathered from the partner rows, diagonal from packed counts, plus the
+// pass-H sums Wh, then the fused epilogue.  X is the input (fp32) or its fixed-point copy.  A
+// thread owns one column of the K rows at a time: the table's records are streamed a chunk
+// ahead across columns, W and the previous Lanczos vector are requested before the straddling
+// gathers, which run four bonds (4 K loads) at a time.
+//
+// 6x5 torus, S^z = 0 (155,117,520 rows), Lanczos step on GB300: fp64 2.77 ms (L = 14, two rows a
+// tile), bound by instruction issue (65 %) and shared-memory wavefronts (59 %); fp32 1.88 ms
+// (L = 15, four rows).  One row a tile at L = 17, every bond below L in state order and all
+// bonds across L gathered here, took 5.82 and 5.29 ms (pass H then 0.78 and 0.49 ms instead of
+// 1.09 and 0.76 ms).
 template <class T, int K, Epi E, int NT, bool ONE>
 __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDev d, const T* __restrict__ X,
                                                                     const T* Wh, void* w, FusedArgs fa,
@@ -757,29 +860,28 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
                                                                     unsigned long long* __restrict__ claim) {
   using R = std::conditional_t<sizeof(T) == 4, float, double>;
   constexpr bool FIX = sizeof(T) == 8;
-  constexpr int EL = (K >= 4) ? 1 : 4 / K;  // elements per thread
+  constexpr int kZero = gather_lanes(K * (int)sizeof(T));
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tile = reinterpret_cast<T*>(smem_raw);
-  R* s_dtab = reinterpret_cast<R*>(smem_raw + (((size_t)(d.nq_max + 1) * K * sizeof(T) + 15) / 16) * 16);
+  R* s_dtab = reinterpret_cast<R*>(smem_raw + (((size_t)(d.nq_max + kZero) * K * sizeof(T) + 15) / 16) * 16);
   int* s_dti = reinterpret_cast<int*>(s_dtab + d.dtab_n);  // fp64 with d.dint: the table in units
   __shared__ uint64_t s_roff[K];
   __shared__ uint32_t s_hrow[K];
   __shared__ uint32_t s_hdiag[K];
+  __shared__ uint32_t s_hb[K];               // bit n: the high bit of straddling bond n
   __shared__ uint32_t s_spm[K][kSecMaxSl];
-  __shared__ uint2 s_sb[kSecMaxStr];         // low bit | class << 16, offset of the bond's rank table
-  __shared__ uint32_t s_need[kSecMaxStr];    // bit m: low-bit value that activates the bond in row m
   __shared__ const T* s_ptr[kSecMaxStr][K];  // partner row of row m through the bond
   __shared__ uint32_t s_hi0;
   __shared__ int s_nk;
   __shared__ unsigned long long s_t;
   __shared__ T s_w[kSecMaxCls];
+  __shared__ T s_sw[kSecMaxStr];             // weight of each straddling bond
   __shared__ double s_red[(NT / 32) * kMaxRedQ];
 
   if (fa.done != nullptr && *fa.done) return;
   const int tid = threadIdx.x;
-  const uint32_t nJ = d.nJ;
   // fixed point: element = q 2^eoff; a power-of-two unit 2^k folds into the scales (see
-  // k_hub_up_q): hv = (dg 2^-k xr + (+-S)) 2^(eoff + k)
+  // k_hub_up): hv = (dg 2^-k xr + (+-S)) 2^(eoff + k)
   const int eoff = FIX ? (*Ep + d.qextra - 1078) : 0;
   const long long ubits = __double_as_longlong(d.unit);
   const int uexp = (int)((ubits >> 52) & 0x7ff);
@@ -788,47 +890,52 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
   const int u_l2 = uexp - 1023;
   const int e2 = eoff + u_l2;
   const bool fold = u_p2 && eoff >= -1022 && eoff <= 1023 && e2 >= -1022 && e2 <= 1023 &&
-                    (E == Epi::kStore || E == Epi::kLanczos1);
+                    E != Epi::kTpq;
   const double s_eoff = fold ? __longlong_as_double((long long)(eoff + 1023) << 52) : 1.0;
   const double s_e2 = fold ? __longlong_as_double((long long)(e2 + 1023) << 52) : 1.0;
   const double r_k = fold ? __longlong_as_double((long long)(1023 - u_l2) << 52) : 1.0;
   for (int k = tid; k < d.dtab_n; k += NT) s_dtab[k] = (R)(d.dtab[k] * r_k);
-  // integral diagonal (in units of `unit`): in the folded fp64 Lanczos step the element is one
-  // exact int64 sum d q + (+-S), so its conversion is the only rounding, and <x, H x> adds the
-  // exact products q (d q +- S) in 128 bits, moved to fp64 every 64 elements
-  const bool dint = FIX && fold && d.dint && E == Epi::kLanczos1;
+  // integral diagonal (in units of `unit`): in the folded fp64 product and Lanczos step the
+  // element is one exact int64 sum d q + (+-S), so its conversion is the only rounding, and
+  // <x, H x> adds the exact products q (d q +- S) in 128 bits, moved to fp64 every 64 elements
+  const bool dint = fold && d.dint;
   if (dint)
     for (int k = tid; k < d.dtab_n; k += NT) s_dti[k] = (int)__double2ll_rn(d.dtab[k] * r_k);
   __int128 ia = 0;
   int ic = 0;
   if (tid < kSecMaxCls) s_w[tid] = tid < d.n_cls ? sec_w<T>(d, tid) : (T)0;
-  if (tid < d.n_str)
-    s_sb[tid] = make_uint2((uint32_t)d.str_b[tid] | ((uint32_t)d.str_cls[tid] << 16), (uint32_t)d.str_t[tid] * nJ);
-  if (tid < K) tile[(size_t)d.nq_max * K + tid] = (T)0;  // the zero entry unused neighbour slots point at
+  if (tid < d.n_str) s_sw[tid] = sec_w<T>(d, d.str_cls[tid]);
+  for (int k = tid; k < kZero * K; k += NT) tile[(size_t)d.nq_max * K + k] = (T)0;  // entries unused slots read
   const EpiScalars<R> es = epi_scalars<R, E>(fa);
   const R inv = E == Epi::kTpq ? opaque((R)fa.scal[0]) : (R)0;
+  const double c1e = FIX ? (double)es.c1 * s_e2 : 0.0;
   const R coef0 = opaque((R)d.coef[0]);
-  const int n_str = d.n_str;
-  const uint32_t pad2 = (uint32_t)d.nq_max | ((uint32_t)d.nq_max << 16);
+  const int n_str = d.n_str, n_cls = d.n_cls;
+  const int64_t stride = d.lo_stride;
   constexpr int NQ = n_red<E>() > 0 ? n_red<E>() : 1;  // reduced quantities of the epilogue
   Red<FIX, NQ> red;
   red.zero();
   int pmx = 0;  // fp64 Lanczos: largest exponent field of the P values written (fa.pexp)
 
   // tiles are claimed in order from a counter, so the tiles in flight stay a narrow window of
-  // the processing order (a fixed stride would let CTAs drift apart over thousands of tiles)
-  for (;;) {
+  // the processing order (a fixed stride would let CTAs drift apart over thousands of tiles);
+  // with a CTA for every tile each takes its own, so the partial sums keep their places
+  const bool own = d.n_tiles <= (int64_t)gridDim.x;
+  for (bool first = true;; first = false) {
+    int64_t t = blockIdx.x;
     __syncthreads();  // the previous tile's rows are no longer read
-    if (tid == 0) s_t = atomicAdd(claim, 1ull);
-    __syncthreads();
-    const int64_t t = (int64_t)s_t;
-    if (t >= d.n_tiles) break;
+    if (!own) {
+      if (tid == 0) s_t = atomicAdd(claim, 1ull);
+      __syncthreads();
+      t = (int64_t)s_t;
+    }
+    if (t >= d.n_tiles || (own && !first)) break;
     if (tid < K) {
       const uint32_t tw = __ldg(d.tiles + t);
       const uint32_t start = tw & 0xffffffu;
       const int nk = (int)(tw >> 24) + 1;
       uint64_t roff = 0;
-      uint32_t hd = 0, hi = 0;
+      uint32_t hd = 0, hi = 0, hb = 0;
       for (int l = 0; l < kSecMaxSl; ++l) s_spm[tid][l] = 0u;
       if (tid < nk) {
         hi = __ldg(d.hi_seq + start + tid);
@@ -837,204 +944,211 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
         hd = __ldg(d.hi_diag + hi);
         for (int n = 0; n < d.n_sp; ++n)
           if ((hi >> d.sp_a[n]) & 1u) s_spm[tid][d.sp_l[n]] |= 1u << d.sp_b[n];
+        for (int n = 0; n < n_str; ++n) hb |= ((hi >> d.str_a[n]) & 1u) << n;
       }
       if (tid == 0) s_nk = nk;
       s_roff[tid] = roff;
       s_hrow[tid] = hi;
       s_hdiag[tid] = hd;
+      s_hb[tid] = hb;
     }
     __syncthreads();
     const int nk = s_nk;
-    // straddling bonds of this tile's rows, one bond per thread (read after the staging barrier)
-    if (tid < n_str) {
+    if (tid < n_str) {  // partner rows, one bond per thread (read after the staging barrier)
       const uint32_t a = d.str_a[tid];
-      uint32_t need = 0u;
 #pragma unroll
-      for (int m = 0; m < K; ++m) {
-        const uint32_t hi = s_hrow[m];
-        // active when bit b of lo differs from bit a of hi
-        need |= (1u - ((hi >> a) & 1u)) << m;
-        s_ptr[tid][m] = X + (m < nk ? __ldg(d.hi_off + (hi ^ (1u << a))) : 0ull);
-      }
-      s_need[tid] = need;
+      for (int m = 0; m < K; ++m) s_ptr[tid][m] = X + (m < nk ? __ldg(d.hi_off + (s_hrow[m] ^ (1u << a))) : 0ull);
     }
     const int q = d.n_ones - __popc(s_hi0);
-    const uint32_t loff = d.lo_off[q] - d.jbase;  // the class in the tables of the present classes
+    const uint32_t lpad = d.lo_pad[q];
     const int nq = (int)(d.lo_off[q + 1] - d.lo_off[q]);
-    // stage the rows, tile[u * K + m] = X[row m][u], with kStage elements per thread in flight
-    constexpr int kStage = (K >= 8) ? 1 : 8 / K;
-    for (int u0 = tid; u0 < nq; u0 += NT * kStage) {
-      T tmp[kStage][K];
+    const int nqp = (nq + 31) & ~31;
+    // stage the rows, tile[u * K + m] = X[row m][u]
+    for (int u = tid; u < nq; u += NT) {
 #pragma unroll
-      for (int e = 0; e < kStage; ++e) {
-        const int u = u0 + e * NT;
-#pragma unroll
-        for (int m = 0; m < K; ++m) tmp[e][m] = (u < nq && m < nk) ? __ldg(X + s_roff[m] + u) : (T)0;
-      }
-#pragma unroll
-      for (int e = 0; e < kStage; ++e) {
-        const int u = u0 + e * NT;
-        if (u < nq) {
-#pragma unroll
-          for (int m = 0; m < K; ++m) tile[u * K + m] = tmp[e][m];
-        }
+      for (int m = 0; m < K; ++m) {
+        if (m < nk) copy_async<(int)sizeof(T)>(tile + u * K + m, X + s_roff[m] + u);
+        else tile[u * K + m] = (T)0;
       }
     }
+    // whole warps run to the padded row length: the table's padding reads zero entries
+    const uint2* rec = d.lo_rec + lpad;
+    const uint4* hdr = d.lo_hdr + (lpad >> 5);
+    uint2 cur[kGatherChunk];
+    uint4 hd = make_uint4(0u, 0u, 0u, 0u);
+    if (tid < nqp) {
+      if constexpr (ONE) hd.x = __ldg(&hdr[tid >> 5].x);
+      else hd = __ldg(hdr + (tid >> 5));
+#pragma unroll
+      for (int j = 0; j < kGatherChunk; ++j) cur[j] = __ldg(rec + tid + j * stride);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    const uint32_t kmask = (1u << nk) - 1u;
-    for (int u0 = tid; u0 < nq; u0 += NT * EL) {
-      uint32_t lo[EL], jj[EL];
-      int ng[EL];
-      T acc[EL][K];
-      int gmax = 0;
+    for (int u = tid; u < nqp; u += NT) {
+      const bool on = u < nq;
+      const uint4 h = hd;
+      const int ng = ((int)(ONE ? h.x & 0xffffu : h.w >> 16) + 3) >> 2;
+      const int un = u + NT < nqp ? u + NT : u;
+      if constexpr (ONE) hd.x = __ldg(&hdr[un >> 5].x);
+      else hd = __ldg(hdr + (un >> 5));
+      const uint2 info = __ldg(d.lo_info + lpad + u);
+      uint2 rk = n_str > 0 ? __ldg(d.str_rank4 + lpad + u) : make_uint2(0u, 0u);
+      T acc[K];
 #pragma unroll
-      for (int e = 0; e < EL; ++e) {
-        const int u = u0 + e * NT;
-        const bool ok = u < nq;
-        jj[e] = loff + (uint32_t)(ok ? u : 0);
-        lo[e] = __ldg(d.lo_list + jj[e]);
-        ng[e] = ok ? ((int)__ldg(d.lo_cnt + jj[e]) + 3) >> 2 : 0;
-        gmax = max(gmax, ng[e]);
+      for (int m = 0; m < K; ++m) acc[m] = (T)0;
+      int f = 0, fe = ONE ? 0 : gather_end(h, 0);  // class of the current slots and its end
+      int c0 = 0;
+      do {
+        const uint2* src = c0 + kGatherChunk < ng ? rec + u + (int64_t)(c0 + kGatherChunk) * stride : rec + un;
+        uint2 nxt[kGatherChunk];
 #pragma unroll
-        for (int m = 0; m < K; ++m) acc[e][m] = (T)0;
-      }
-      // Lanczos: ask L2 for this thread's W and P elements now, so the epilogue's loads find
-      // them there instead of in DRAM (measured 1 to 3 % faster on the 6x6 sector)
-      if constexpr (E == Epi::kLanczos1) {
-        const char* pin = reinterpret_cast<const char*>(fa.in ? fa.in : fa.out);
+        for (int j = 0; j < kGatherChunk; ++j) nxt[j] = __ldg(src + j * stride);
 #pragma unroll
-        for (int e = 0; e < EL; ++e) {
-          const int u = u0 + e * NT;
-          if (u < nq) {
+        for (int j = 0; j < kGatherChunk; ++j) {
+          if (c0 + j < ng) {
+            const uint2 r = cur[j];
+            T v[4][K];
+            tile_load<T, K>(tile + (r.x & 0xffffu) * K, v[0]);
+            tile_load<T, K>(tile + (r.x >> 16) * K, v[1]);
+            tile_load<T, K>(tile + (r.y & 0xffffu) * K, v[2]);
+            tile_load<T, K>(tile + (r.y >> 16) * K, v[3]);
+            if constexpr (ONE) {
 #pragma unroll
-            for (int m = 0; m < K; ++m) {
-              if (m < nk) {
-                const int64_t idx = (int64_t)s_roff[m] + u;
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(Wh + idx));
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(pin + idx * (int64_t)sizeof(T)));
+              for (int m = 0; m < K; ++m) acc[m] += (v[0][m] + v[1][m]) + (v[2][m] + v[3][m]);
+            } else {
+              const int s0 = 4 * (c0 + j);
+              while (f + 1 < n_cls && s0 >= fe) fe = gather_end(h, ++f);
+              if (s0 + 4 <= fe || f + 1 == n_cls) {  // one class, or padding after the last
+                const T wf = s_w[f];
+#pragma unroll
+                for (int m = 0; m < K; ++m) acc[m] += wf * ((v[0][m] + v[1][m]) + (v[2][m] + v[3][m]));
+              } else {
+                int ff = f, ffe = fe;
+#pragma unroll
+                for (int t4 = 0; t4 < 4; ++t4) {
+                  while (ff + 1 < n_cls && s0 + t4 >= ffe) ffe = gather_end(h, ++ff);
+                  const T wf = s_w[ff];
+#pragma unroll
+                  for (int m = 0; m < K; ++m) acc[m] += wf * v[t4][m];
+                }
               }
             }
           }
         }
+#pragma unroll
+        for (int j = 0; j < kGatherChunk; ++j) cur[j] = nxt[j];
+        c0 += kGatherChunk;
+      } while (c0 < ng);
+      // this column's W and (Lanczos) previous vector, then the straddling gathers
+      T wv[K];
+      R pin[K];
+#pragma unroll
+      for (int m = 0; m < K; ++m) {
+        const int64_t idx = (int64_t)s_roff[m] + u;
+        wv[m] = (on && m < nk) ? Wh[idx] : (T)0;
+        if constexpr (E == Epi::kLanczos1)
+          pin[m] = (on && m < nk) ? reinterpret_cast<const R*>(fa.in ? fa.in : fa.out)[idx] : (R)0;
       }
-      // low-low exchange: four neighbours per table load, unused slots read the zero entry
-      for (int g = 0; g < gmax; ++g) {
-        uint2 rec[EL];
-        uint32_t cw[EL];
+      uint32_t act[K];  // bond n acts on row m: its low bit differs from its high bit
 #pragma unroll
-        for (int e = 0; e < EL; ++e) {
-          const uint32_t o = (uint32_t)g * nJ + jj[e];  // < 2^28
-          rec[e] = g < ng[e] ? __ldg(d.lo_nbr4 + o) : make_uint2(pad2, pad2);
-          if constexpr (!ONE) cw[e] = g < ng[e] ? __ldg(d.lo_cls4 + o) : 0u;
-        }
+      for (int m = 0; m < K; ++m) act[m] = (on && m < nk) ? info.y ^ s_hb[m] : 0u;
+      for (int n0 = 0; n0 < n_str; n0 += 4) {
+        const uint2 r = rk;
+        if (n0 + 4 < n_str) rk = __ldg(d.str_rank4 + (int64_t)(n0 / 4 + 1) * stride + lpad + u);
+        T x[4][K];
 #pragma unroll
-        for (int e = 0; e < EL; ++e) {
-#pragma unroll
-          for (int t4 = 0; t4 < 4; ++t4) {
-            const uint32_t word = (t4 < 2) ? rec[e].x : rec[e].y;
-            const uint32_t nb = (t4 & 1) ? (word >> 16) : (word & 0xffffu);
-            T v[K];
-            tile_load<T, K>(tile + nb * K, v);
-#pragma unroll
-            for (int m = 0; m < K; ++m) {
-              if constexpr (ONE) acc[e][m] += v[m];
-              else acc[e][m] += s_w[(cw[e] >> (8 * t4)) & (kSecMaxCls - 1)] * v[m];
-            }
-          }
-        }
-      }
-      // straddling exchange, one bond at a time for all elements of the thread
-      for (int n = 0; n < n_str; ++n) {
-        const uint2 sb = s_sb[n];
-        const uint32_t b = sb.x & 31u;
-        const uint32_t need = s_need[n];
-        const T wn = ONE ? (T)1 : s_w[(sb.x >> 16) & (kSecMaxCls - 1)];
-        const T* pm[K];
-#pragma unroll
-        for (int m = 0; m < K; ++m) pm[m] = s_ptr[n][m];
-        uint32_t col[EL], act[EL];
-#pragma unroll
-        for (int e = 0; e < EL; ++e) {
-          const uint32_t lb = (lo[e] >> b) & 1u;
-          act[e] = (lb ? need : ~need) & kmask & (ng[e] >= 0 && u0 + e * NT < nq ? 0xffffffffu : 0u);
-          col[e] = act[e] ? (uint32_t)__ldg(d.str_rank + sb.y + jj[e]) : 0u;
-        }
-#pragma unroll
-        for (int e = 0; e < EL; ++e)
+        for (int t4 = 0; t4 < 4; ++t4) {
+          const int n = n0 + t4;
+          const uint32_t word = t4 < 2 ? r.x : r.y;
+          const uint32_t col = (t4 & 1) ? word >> 16 : word & 0xffffu;
 #pragma unroll
           for (int m = 0; m < K; ++m) {
-            const T x = ((act[e] >> m) & 1u) ? __ldg(pm[m] + col[e]) : (T)0;
-            if constexpr (ONE) acc[e][m] += x;
-            else acc[e][m] += wn * x;
+            x[t4][m] = (T)0;
+            if (n < n_str && ((act[m] >> n) & 1u)) x[t4][m] = __ldg(s_ptr[n][m] + col);
           }
+        }
+        if constexpr (ONE) {
+#pragma unroll
+          for (int m = 0; m < K; ++m) acc[m] += (x[0][m] + x[1][m]) + (x[2][m] + x[3][m]);
+        } else {
+#pragma unroll
+          for (int t4 = 0; t4 < 4; ++t4) {
+            const T wn = n0 + t4 < n_str ? s_sw[n0 + t4] : (T)0;
+#pragma unroll
+            for (int m = 0; m < K; ++m) acc[m] += wn * x[t4][m];
+          }
+        }
       }
-      // diagonal, pass-H sums and the epilogue
+      if (!on) continue;
+      // diagonal and the epilogue
+      const uint32_t lo = info.x & 0xfffffu;
+      const uint32_t ldc = (info.x >> 20) | ((info.y >> 24) << 8);
 #pragma unroll
-      for (int e = 0; e < EL; ++e) {
-        const int u = u0 + e * NT;
-        if (u >= nq) break;
-        const uint32_t ld = __ldg(d.lo_diag + jj[e]);
-#pragma unroll
-        for (int m = 0; m < K; ++m) {
-          if (m >= nk) break;
-          uint32_t c = ld + s_hdiag[m];
-          for (int l = 0; l < d.n_sl; ++l) c += (uint32_t)__popc(lo[e] & s_spm[m][l]) << (8 * d.sp_lg[l]);
-          const int ci = (int)(c & 0xffu) + d.dstride * (int)(c >> 8);
-          const int64_t idx = (int64_t)s_roff[m] + u;
-          const T xq = tile[u * K + m];
-          const T wv = Wh[idx];
+      for (int m = 0; m < K; ++m) {
+        if (m >= nk) break;
+        uint32_t c = ldc + s_hdiag[m];
+        for (int l = 0; l < d.n_sl; ++l) c += (uint32_t)__popc(lo & s_spm[m][l]) << (8 * d.sp_lg[l]);
+        const int ci = (int)(c & 0xffu) + d.dstride * (int)(c >> 8);
+        const int64_t idx = (int64_t)s_roff[m] + u;
+        const T xq = tile[u * K + m];
+        const T S = acc[m] + wv[m];
+        if constexpr (!FIX) {
           const R dg = s_dtab[ci];
-          if constexpr (!FIX) {
-            const R hv = ONE ? dg * xq + coef0 * (acc[e][m] + wv) : dg * xq + (acc[e][m] + wv);
-            epilogue<float, E, NQ>(idx, xq, 0.f, hv, 0.f, reinterpret_cast<float*>(w), fa, es, inv, red);
+          const float hv = ONE ? dg * xq + coef0 * S : dg * xq + S;
+          if constexpr (E == Epi::kLanczos1) {
+            reinterpret_cast<float*>(fa.out)[idx] = es.c1 * hv - es.c2 * pin[m];
+            red.add(0, xq, hv);
+            red.tick();
           } else {
-            const long long S = acc[e][m] + wv;
-            if constexpr (E == Epi::kLanczos1) {
-              if (dint) {
-                const long long hq = (long long)s_dti[ci] * xq + (u_neg ? -S : S);  // hv = hq 2^e2
-                const double hvu = __ll2double_rn(hq);
-                double* P = reinterpret_cast<double*>(fa.out);
-                const double* Pin = fa.in ? reinterpret_cast<const double*>(fa.in) : P;
-                const double pv = fma(es.c1 * s_e2, hvu, -(es.c2 * Pin[idx]));
-                P[idx] = pv;
-                pmx = max(pmx, (int)((__double_as_longlong(pv) >> 52) & 0x7ff));
-                ia += (__int128)xq * (__int128)hq;
-                if (++ic == 64) {
-                  red.add(0, i128_to_double(ia), 1.0);
-                  ia = 0;
-                  ic = 0;
-                }
-                continue;
+            epilogue<float, E, NQ>(idx, xq, 0.f, hv, 0.f, reinterpret_cast<float*>(w), fa, es, inv, red);
+          }
+        } else {
+          if (dint) {
+            const long long hq = (long long)s_dti[ci] * xq + (u_neg ? -S : S);  // hv = hq 2^e2
+            const double hvu = __ll2double_rn(hq);
+            if constexpr (E == Epi::kStore) {
+              reinterpret_cast<double*>(w)[idx] = hvu * s_e2;
+            } else if constexpr (E == Epi::kLanczos1) {
+              const double pv = fma(c1e, hvu, -(es.c2 * pin[m]));
+              reinterpret_cast<double*>(fa.out)[idx] = pv;
+              pmx = max(pmx, (int)((__double_as_longlong(pv) >> 52) & 0x7ff));
+              ia += (__int128)xq * (__int128)hq;
+              if (++ic == 64) {
+                red.add(0, i128_to_double(ia), 1.0);
+                ia = 0;
+                ic = 0;
               }
+            } else if constexpr (E == Epi::kRefine) {
+              refine_folded(hvu, __ll2double_rn(xq), s_e2, idx, fa, red);
             }
-            const double xr = __ll2double_rn(xq);
-            if (fold) {
-              const double hvu = fma(dg, xr, __ll2double_rn(u_neg ? -S : S));  // hv = hvu 2^e2
-              if constexpr (E == Epi::kStore) {
-                reinterpret_cast<double*>(w)[idx] = hvu * s_e2;
-              } else if constexpr (E == Epi::kLanczos1) {
-                double* P = reinterpret_cast<double*>(fa.out);
-                const double* Pin = fa.in ? reinterpret_cast<const double*>(fa.in) : P;
-                const double pv = fma(es.c1 * s_e2, hvu, -(es.c2 * Pin[idx]));
-                P[idx] = pv;
-                pmx = max(pmx, (int)((__double_as_longlong(pv) >> 52) & 0x7ff));
-                red.add(0, xr, hvu);
-                red.tick();
-              }
+            continue;
+          }
+          const R dg = s_dtab[ci];
+          const double xr = __ll2double_rn(xq);
+          if (fold) {
+            const double hvu = fma(dg, xr, __ll2double_rn(u_neg ? -S : S));  // hv = hvu 2^e2
+            if constexpr (E == Epi::kStore) {
+              reinterpret_cast<double*>(w)[idx] = hvu * s_e2;
+            } else if constexpr (E == Epi::kLanczos1) {
+              const double pv = fma(c1e, hvu, -(es.c2 * pin[m]));
+              reinterpret_cast<double*>(fa.out)[idx] = pv;
+              pmx = max(pmx, (int)((__double_as_longlong(pv) >> 52) & 0x7ff));
+              red.add(0, xr, hvu);
+              red.tick();
+            } else if constexpr (E == Epi::kRefine) {
+              refine_folded(hvu, xr, s_e2, idx, fa, red);
+            }
+          } else {
+            const double x = fix_to_double(xq, eoff);
+            const double hv = fma((double)dg, x, d.unit * fix_to_double(S, eoff));
+            if constexpr (E == Epi::kLanczos1) {  // the epilogue's Lanczos step, with the exponent kept
+              const double pv = es.c1 * hv - es.c2 * pin[m];
+              reinterpret_cast<double*>(fa.out)[idx] = pv;
+              pmx = max(pmx, (int)((__double_as_longlong(pv) >> 52) & 0x7ff));
+              red.add(0, x, hv);
+              red.tick();
             } else {
-              const double x = fix_to_double(xq, eoff);
-              const double hv = fma((double)dg, x, d.unit * fix_to_double(S, eoff));
-              if constexpr (E == Epi::kLanczos1) {  // the epilogue's Lanczos step, with the exponent kept
-                double* P = reinterpret_cast<double*>(fa.out);
-                const double* Pin = fa.in ? reinterpret_cast<const double*>(fa.in) : P;
-                const double pv = es.c1 * hv - es.c2 * Pin[idx];
-                P[idx] = pv;
-                pmx = max(pmx, (int)((__double_as_longlong(pv) >> 52) & 0x7ff));
-                red.add(0, x, hv);
-                red.tick();
-              } else {
-                epilogue<double, E, NQ>(idx, x, 0.0, hv, 0.0, reinterpret_cast<double*>(w), fa, es, inv, red);
-              }
+              epilogue<double, E, NQ>(idx, x, 0.0, hv, 0.0, reinterpret_cast<double*>(w), fa, es, inv, red);
             }
           }
         }
@@ -1054,7 +1168,7 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
 #pragma unroll
     for (int qq = 0; qq < nq; ++qq) {
       double x = red.get(qq);
-      if (fold) x = (x * s_eoff) * s_e2;  // back from units of 2^(eoff + e2)
+      if (fold) x = folded_sum(x, qq, s_eoff, s_e2);
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(0xffffffffu, x, off);
       if (lane == 0) s_red[wid * kMaxRedQ + qq] = x;
@@ -1069,8 +1183,8 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
 }
 
 // ---------------------------------------------------------------- launch helpers
-size_t lo_smem(const SecDev& d, int esz) {  // the rows, their zero entry, the diagonal table(s)
-  return (((size_t)(d.nq_max + 1) * d.K * esz + 15) / 16) * 16 + (size_t)d.dtab_n * esz +
+size_t lo_smem(const SecDev& d, int esz) {  // the rows, their zero entries, the diagonal table(s)
+  return (((size_t)(d.nq_max + gather_lanes(d.K * esz)) * d.K * esz + 15) / 16) * 16 + (size_t)d.dtab_n * esz +
          (esz == 8 && d.dint ? (size_t)d.dtab_n * 4 : 0);
 }
 
@@ -1092,7 +1206,7 @@ template <class T, int K, Epi E, bool ONE>
 Status launch_lo_t(const SecDev& d, const T* X, const T* Wh, void* w, const FusedArgs& fa, const int* Ep, int grid,
                    unsigned long long* claim, cudaStream_t st) {
   const size_t smem = lo_smem(d, (int)sizeof(T));
-  HPHI_CUDA_TRY(cudaMemsetAsync(claim, 0, sizeof(unsigned long long), st));
+  if (d.n_tiles > grid) HPHI_CUDA_TRY(cudaMemsetAsync(claim, 0, sizeof(unsigned long long), st));
 #define HPHI_SECLO(NN)                                                                                        \
   HPHI_CUDA_TRY(cudaFuncSetAttribute(k_sec_lo<T, K, E, NN, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                      (int)smem));                                                             \

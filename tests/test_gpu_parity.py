@@ -1149,3 +1149,27 @@ def test_hubbard_gather_tables(n, nu, nd, t, U, mu, V, prec):
         a, _ = oracle.lanczos(spec, v, 3)
         r = m.lanczos(3, prec=p, v0=torch.as_tensor(v))
         assert _rel(r["alpha"][:len(a)], a) < (1e-12 if prec == "fp64" else 2e-5)  # a: up to the breakdown
+
+
+# ----------------------------------------------------------------------------- pass H with its own split
+@pytest.mark.parametrize("mk,n_up,L,K", [
+    (lambda: wl.heisenberg_square(6, 3), 9, 13, 2), (lambda: wl.heisenberg_square(6, 3), 5, 14, 4),
+    (lambda: wl.j1j2_ring(18), 9, 14, 2), (lambda: wl.j1j2_ring(18), 15, 13, 4), (lambda: wl.j1j2_ring(19), 7, 16, 1),
+    (lambda: wl.heisenberg_ring(22), 4, 0, 0),
+], ids=["6x3-L13-K2", "6x3-L14-K4", "j1j2-L14-K2", "j1j2-L13-K4", "j1j2_19-L16-K1", "ring22-default"])
+def test_sector_two_splits(mk, n_up, L, K):
+    """Splits whose low part is longer than pass H's 12 bits: bonds of the sites between the two
+    splits run in pass H, bonds below them in pass R; one and several coefficient classes, a
+    part-filled last tile, more tiles than CTAs (ring22) and fewer."""
+    spec = mk().with_basis(wl.BASIS_SZ, n_up)
+    m = hp.Model.from_spec(spec)
+    v = wl.gaussian_vector(151 + n_up, m.dim)
+    ref = oracle.apply_H(spec, v).real
+    a, b = oracle.lanczos(spec, v[:, 0], 4)
+    for prec, tol in ((hp.FP64, 1e-12), (hp.FP32, 2e-5)):
+        m.set_sector_split(prec, L, K)
+        assert _rel(m.apply_H(_to_dev(m, v, prec)).cpu().numpy(), ref) < tol
+        r = m.lanczos(4, prec=prec, v0=torch.as_tensor(v[:, 0]), refine=True)
+        assert _rel(r["alpha"], a) < tol and _rel(r["beta"], b) < tol
+        # 4 steps: the Ritz value is the Rayleigh quotient of the refined vector
+        assert abs(r["e_refined"] - oracle.ritz_values(a, b)[0]) <= 10 * tol * abs(a[0]) + 10 * tol
