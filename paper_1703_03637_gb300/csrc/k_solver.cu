@@ -42,25 +42,27 @@ template <class R>
 __global__ void __launch_bounds__(kThreads) k_lz_init(const double* __restrict__ v0, R* __restrict__ C, R* __restrict__ P,
                                                        int64_t n_real, double* __restrict__ partials) {
   __shared__ double sm[kThreads];
+  constexpr int U = sizeof(R) == 8 ? 4 : 8;
   double acc = 0.0;
-  // four elements per thread and iteration, one grid stride apart (coalesced, loads first)
+  // U elements per thread and iteration, one grid stride apart (coalesced, loads first)
   const int64_t stride = (int64_t)gridDim.x * kThreads;
-  for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < n_real; i += 4 * stride) {
-    R x[4];
+  for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < n_real; i += U * stride) {
+    R x[U];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < U; ++u) {
       const int64_t k = i + u * stride;
       x[u] = k < n_real ? (v0 != nullptr ? (R)v0[k] : C[k]) : (R)0;
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < U; ++u) {
       const int64_t k = i + u * stride;
       if (k < n_real) {
         if (v0 != nullptr) C[k] = x[u];
         P[k] = (R)0;
-        acc = fma((double)x[u], (double)x[u], acc);
+        if constexpr (sizeof(R) == 8) acc = fma(x[u], x[u], acc);
       }
     }
+    if constexpr (sizeof(R) == 4) acc += sum_squares<U>(x);
   }
   const double t = block_sum(acc, sm);
   if (threadIdx.x == 0) partials[(size_t)blockIdx.x * kMaxRedQ] = t;
@@ -368,7 +370,9 @@ __global__ void k_tridiag(LzDev lz, int n_eig, int want_vec, double tail_tol, do
 
 // ------------------------------------------------------------------ Ritz vector from a stored basis
 // x = sum_{k < n} coef_k sigma_k V_k, V_k the unnormalised Lanczos vectors kept in HBM
-// (stride_real reals apart); fp64 accumulation, one streaming read of the basis.
+// (stride_real reals apart); fp64 accumulation, one streaming read of the basis.  fp32 vectors
+// are widened by integer operations, which leaves the fp64 pipe one multiply-add a number: 8
+// vectors of 155,117,520 numbers 2.22 ms instead of 4.48 ms.
 template <class R>
 __global__ void __launch_bounds__(kThreads) k_lz_combine(LzDev lz, const R* __restrict__ V, int64_t n_real,
                                                           int64_t stride_real, double* __restrict__ x) {
@@ -378,7 +382,15 @@ __global__ void __launch_bounds__(kThreads) k_lz_combine(LzDev lz, const R* __re
   __syncthreads();
   for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < n_real; i += (int64_t)gridDim.x * kThreads) {
     double acc = 0.0;
-    for (int k = 0; k < n; ++k) acc = fma(s_c[k], (double)V[(int64_t)k * stride_real + i], acc);
+    int k = 0;
+    for (; k + 4 <= n; k += 4) {  // four vectors' loads in flight
+      R v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = V[(int64_t)(k + u) * stride_real + i];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) acc = fma(s_c[k + u], widen(v[u]), acc);
+    }
+    for (; k < n; ++k) acc = fma(s_c[k], widen(V[(int64_t)k * stride_real + i]), acc);
     x[i] = acc;
   }
 }
@@ -524,25 +536,42 @@ __global__ void __launch_bounds__(kThreads) k_refine_resid(const double* __restr
 
 // ------------------------------------------------------------------ mTPQ
 // X <- (storage precision) psi0 (if given); per-column partial |X|^2.  nvec divides kThreads.
+// fp64 operations of the norm bounded the fp32 kernel (2^24 rows of 64 complex starts: 7.72 ms
+// with one conversion and one multiply-add a number; see sum_squares for what replaced them: 2.10 ms).
 template <class R, bool CPLX>
 __global__ void __launch_bounds__(kThreads) k_tpq_init(const double* __restrict__ psi0, R* __restrict__ X,
                                                         int64_t n_rows, int nvec, double* __restrict__ partials) {
   __shared__ double sm[kThreads];
-  const int W = CPLX ? 2 : 1;
+  constexpr int W = CPLX ? 2 : 1;
+  constexpr bool F64 = sizeof(R) == 8;
   const int64_t n_elem = n_rows * nvec;
+  constexpr int U = 8 / W;  // numbers per group of sum_squares: 8
   double acc = 0.0;
   const int c = threadIdx.x % nvec;
-  for (int64_t e = blockIdx.x * (int64_t)kThreads + threadIdx.x; e < n_elem; e += (int64_t)gridDim.x * kThreads) {
-    for (int w = 0; w < W; ++w) {
-      const int64_t i = e * W + w;
-      R x;
-      if (psi0 != nullptr) {
-        x = (R)psi0[i];
-        X[i] = x;
-      } else {
-        x = X[i];
+  const int64_t stride = (int64_t)gridDim.x * kThreads;  // a multiple of nvec: the column stays
+  for (int64_t e = blockIdx.x * (int64_t)kThreads + threadIdx.x; e < n_elem; e += U * stride) {
+    R x[U * W];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t k = e + u * stride;
+#pragma unroll
+      for (int w = 0; w < W; ++w)
+        x[u * W + w] = k < n_elem ? (psi0 != nullptr ? (R)psi0[k * W + w] : X[k * W + w]) : (R)0;
+    }
+    if (psi0 != nullptr) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t k = e + u * stride;
+#pragma unroll
+        for (int w = 0; w < W; ++w)
+          if (k < n_elem) X[k * W + w] = x[u * W + w];
       }
-      acc = fma((double)x, (double)x, acc);
+    }
+    if constexpr (F64) {
+#pragma unroll
+      for (int u = 0; u < U * W; ++u) acc = fma(x[u], x[u], acc);
+    } else {
+      acc += sum_squares<U * W>(x);
     }
   }
   sm[threadIdx.x] = acc;

@@ -1173,3 +1173,23 @@ def test_sector_two_splits(mk, n_up, L, K):
         assert _rel(r["alpha"], a) < tol and _rel(r["beta"], b) < tol
         # 4 steps: the Ritz value is the Rayleigh quotient of the refined vector
         assert abs(r["e_refined"] - oracle.ritz_values(a, b)[0]) <= 10 * tol * abs(a[0]) + 10 * tol
+
+
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -45, 2.0 ** 50])
+@pytest.mark.parametrize("mk,nv", [(lambda: wl.kitaev_honeycomb(2, 2), 4), (lambda: wl.heisenberg_ring(9), 1)],
+                         ids=["complex4", "real1"])
+def test_fp32_start_norms_at_any_scale(mk, nv, scale):
+    """The fp32 start norms (mTPQ and Lanczos) do not depend on the start vector's scale: inside
+    the range where squares are summed in fp32 pairs and outside it, and in the last, part-filled
+    group of eight numbers."""
+    spec = mk()
+    m = hp.Model.from_spec(spec)
+    psi0 = wl.gaussian_vector(17, m.dim, nv, complex_=m.is_complex)
+    r = m.tpq(nv, 3, l=2.0, prec=hp.FP32, psi0=torch.as_tensor(psi0 * scale))
+    for c in range(nv):
+        u, h2, nrm = oracle.tpq(spec, psi0[:, c], 3, 2.0)
+        assert _rel(r["u"][:, c], u) < 2e-5 and _rel(r["h2"][:, c], h2) < 2e-5 and _rel(r["norm"][:, c], nrm) < 2e-5
+    if nv == 1:
+        a, b = oracle.lanczos(spec, psi0[:, 0], 3)
+        q = m.lanczos(3, prec=hp.FP32, v0=torch.as_tensor(psi0[:, 0] * scale))
+        assert _rel(q["alpha"], a) < 2e-5 and _rel(q["beta"], b) < 2e-5
