@@ -174,7 +174,7 @@ typedef struct {
  * hphi_lanczos_run / hphi_tpq_run on this model.  The two-pass Hubbard path is tuned over
  * columns per thread of the down-spin pass x rows per tile of the up-spin pass.  Real spin
  * models in an S^z sector that take the split-row path (see hphi_set_sector_split) are tuned
- * over the split: the default low part and up to two bits fewer, each with every tile height
+ * over the split: the default low part, one bit more and up to two fewer, each with every tile height
  * that fits, and then over the high pass's columns per lane on the chosen split.  A real spin model in its full basis has every S^z sector of at least 2^20 rows
  * tuned that way: hphi_lanczos_run_sectors keeps those sectors' shapes; the result then
  * counts the candidates of all of them and reports the timings of the largest.  Other models
@@ -193,9 +193,10 @@ int hphi_autotune(hphi_model* m, int prec, hphi_tune_result* out, void* stream);
  * coefficient groups beyond a constant (Heisenberg, XXZ and J1-J2 models on regular lattices);
  * fp64 also needs the exchange couplings to be small integer multiples of one power of two.
  * Other models use the generic gather kernel.  This call chooses the split used for prec:
- * L = -1 turns the path off (generic kernel), L = 0 restores the default (the largest low
- * part whose rows fit one shared-memory tile), 1..20 forces the low part's length; K = 0
- * picks the widest tile that fits, 1/2/4/8 forces the rows per tile.  The device tables of
+ * L = -1 turns the path off (generic kernel), L = 0 restores the default (14 bits in fp64, 15
+ * in fp32, fewer on small clusters), 1..20 forces the low part's length; K = 0 picks 16-byte
+ * tile entries (two fp64 or four fp32 rows) if they fit, 1/2/4/8 forces the rows per tile.  The
+ * high-part combinations use a shorter split of their own (12 bits where the tables allow).  The device tables of
  * the split are built here (a host loop over 2^L low and 2^(N-L) high parts, then an upload
  * on `stream`, which is synchronised).  Results agree with the generic kernel to rounding
  * (fp32) or exactly up to the final conversion (fp64 fixed-point sums).  Returns
@@ -208,12 +209,13 @@ int hphi_set_sector_split(hphi_model* m, int prec, int L, int K, void* stream);
  * flipped sites lie in one cyclic window of `bits` sites and visits the rows with that
  * window's bits varying fastest, so a pass's gathers hit a block of rows small enough to
  * stay in L2 instead of reaching across the whole vector in HBM.  bits = -1 (the default)
- * runs one pass, 0 sizes the window so that a block of input rows fills about a quarter of
- * L2, 1..32 forces a window size (a window covering all sites means one pass).  At most 8
- * passes; a plan that needs more falls back to one pass.  The passes cut HBM traffic about
- * threefold on the 2^24-row Kitaev cluster but add instructions, and one pass is already
- * bound by instruction issue there, hence the default.  The Lanczos step (one vector) is not
- * affected.  Results agree with one pass up to floating-point summation order. */
+ * leaves the choice to the library: tiles of rows in shared memory, a few passes, each over the
+ * terms inside one set of sites, for nvec a power of two from 64 bytes a row where there are
+ * enough tiles, else one gather pass.  0 sizes the window so that a block of input rows fills
+ * about a quarter of L2, 1..32 forces a window size (a window covering all sites means one
+ * gather pass).  At most 8 window passes; a plan that needs more falls back to one gather pass.
+ * The Lanczos step (one vector) is not affected.  Results agree with one pass up to
+ * floating-point summation order. */
 int hphi_set_window_bits(hphi_model* m, int bits);
 
 /* ---------------------------------------------------------------- start vectors */

@@ -133,6 +133,9 @@ struct hphi_model {
     hphi::BatchPlan plan;
   };
   std::map<int, std::unique_ptr<WinCache>> win;
+  // tile plans of the full basis for t = 7 .. 10 sites (built with the sector tables)
+  hphi::TilePlan tile[4];
+  DBuf d_tile_ents[4], d_tile_dep[4];
   // split-row path of real S^z-sector spin models: the compiled terms, whether each precision
   // may take the path, the split asked for per precision (-1 off, 0 default, else L) and
   // rows per tile (0 default), and the device tables built so far by (L, K, element size)
@@ -342,6 +345,24 @@ hphi::Status compile_spin(hphi_model* m, cudaStream_t st) {
   d.max_run = max_run;
   m->host_entries = ents;
   m->win.clear();
+  for (int k = 0; k < 4; ++k) {
+    m->tile[k] = hphi::TilePlan{};
+    hphi::TileHost th;
+    if (sector || !hphi::batch_tile_plan(N, 7 + k, ents, cls, &th)) continue;
+    if ((s = upload(m->d_tile_ents[k], th.ents, st)).code) return s;
+    if ((s = upload(m->d_tile_dep[k], th.dep, st)).code) return s;
+    HPHI_CUDA_TRY(cudaStreamSynchronize(st));  // th dies here
+    hphi::TilePlan& tp = m->tile[k];
+    tp.n_pass = th.n_pass;
+    tp.max_run = th.max_run;
+    for (int p = 0; p < th.n_pass; ++p) {
+      tp.pass[p].ents = m->d_tile_ents[k].as<hphi::TileEntry>() + th.e0[p];
+      tp.pass[p].n_ent = th.e0[p + 1] - th.e0[p];
+      tp.pass[p].dep = m->d_tile_dep[k].as<uint32_t>() + (size_t)p * 1024;
+      tp.pass[p].t = 7 + k;
+      memcpy(tp.pass[p].pos, th.pos[p], sizeof(th.pos[p]));
+    }
+  }
   d.n_classes = (int)cls.size();
   d.n_lin = (int)lg.size();
   d.n_pairs = (int)pe.size();
@@ -695,6 +716,13 @@ bool use_hub_fast(hphi_model* m, int prec, int nvec, hphi::Epi epi) {
 
 bool use_batch(hphi_model* m, int nvec) { return m->kind == HPHI_SPIN_HALF && hphi::batch_applies(m->sdev, nvec); }
 
+// The tile plan of this launch, or null (gather kernels; also when the window setting asks for
+// their passes)
+const hphi::TilePlan* use_tile(hphi_model* m, int prec, int nvec, hphi::Epi epi) {
+  if (m->kind != HPHI_SPIN_HALF || m->win_bits_opt >= 0) return nullptr;
+  return hphi::tile_choose(m->tile, m->sdev, prec, m->cplx_model, nvec, epi);
+}
+
 // Split-row tables when the split-row path applies to this launch (one real vector of an
 // S^z-sector spin model), else null.  The path also needs its scratch (sec_scratch_bytes).
 const hphi::SecDev* use_sec(hphi_model* m, int prec, int nvec, hphi::Epi epi) {
@@ -740,6 +768,7 @@ int hv_kernels(hphi_model* m, int prec, int nvec, hphi::Epi epi) {
   if (use_sec(m, prec, nvec, epi) && m->ws.work.p != nullptr &&
       m->ws.work.bytes >= hphi::sec_scratch_bytes(*use_sec(m, prec, nvec, epi), prec, epi))
     return prec == HPHI_FP64 ? 4 : 2;  // (max-exponent, quantise,) pass H, pass R
+  if (const hphi::TilePlan* tp = use_tile(m, prec, nvec, epi)) return tp->n_pass + (prec == HPHI_FP64 ? 1 : 0);
   if (use_batch(m, nvec)) {
     const hphi::BatchPlan* plan = epi == hphi::Epi::kLanczos1 ? nullptr : batch_plan(m, prec, nvec);
     const int passes = plan ? plan->n_pass : 1;
@@ -753,10 +782,11 @@ int hv_kernels(hphi_model* m, int prec, int nvec, hphi::Epi epi) {
   return 1;
 }
 
-// scratch an H v launch needs beyond its vectors (0: none)
-size_t hv_scratch_bytes(hphi_model* m, int prec, int nvec, hphi::Epi epi) {
+// scratch an H v launch needs beyond its vectors (0: none); aligned: they start on 32 bytes
+size_t hv_scratch_bytes(hphi_model* m, int prec, int nvec, hphi::Epi epi, bool aligned = true) {
   if (use_hub_fast(m, prec, nvec, epi)) return hphi::hub_scratch_bytes(m->hdev, prec, epi);
   if (const hphi::SecDev* sd = use_sec(m, prec, nvec, epi)) return hphi::sec_scratch_bytes(*sd, prec, epi);
+  if (aligned && use_tile(m, prec, nvec, epi)) return hphi::tile_scratch_bytes(prec, nvec);
   if (use_batch(m, nvec))
     return hphi::batch_scratch_bytes(m->sdev, epi == hphi::Epi::kLanczos1 ? nullptr : batch_plan(m, prec, nvec), prec,
                                      m->cplx_model, nvec);
@@ -788,6 +818,8 @@ int hv_grid_for(hphi_model* m, int nvec, int prec, hphi::Epi epi) {
     if (m->ws.work.p != nullptr && m->ws.work.bytes >= hphi::sec_scratch_bytes(*sd, prec, epi))
       return hphi::sec_grid(*sd, prec, epi);
   }
+  if (const hphi::TilePlan* tp = use_tile(m, prec, nvec, epi))
+    return hphi::tile_grid(*tp, m->sdev, prec, m->cplx_model, nvec);
   if (use_batch(m, nvec)) return hphi::batch_grid(prec, m->cplx_model, nvec, epi, m->dim);
   const bool hub = m->kind == HPHI_HUBBARD;
   const int64_t cap = hphi::hv_resident_grid(hub, prec, m->cplx_model, epi);
@@ -809,6 +841,11 @@ hphi::Status hv_launch(hphi_model* m, int prec, const void* v, void* w, int nvec
     hphi::SecDev dd = *use_sec(m, prec, nvec, epi);
     dd.hi_cols = m->sec_hi_cols[prec == HPHI_FP64 ? 0 : 1];
     return hphi::launch_sec(dd, prec, v, w, scratch, epi, fa, grid, st);
+  }
+  if (const hphi::TilePlan* tp = use_tile(m, prec, nvec, epi)) {
+    if (hphi::batch_aligned(v, epi == hphi::Epi::kTpq ? fa.out : w) &&
+        (scratch != nullptr || hphi::tile_scratch_bytes(prec, nvec) == 0))
+      return hphi::launch_tile(m->sdev, *tp, prec, m->cplx_model, v, w, scratch, nvec, epi, fa, grid, st);
   }
   if (use_batch(m, nvec) && hphi::batch_aligned(v, w)) {
     const hphi::BatchPlan* plan = epi == hphi::Epi::kLanczos1 ? nullptr : batch_plan(m, prec, nvec);
@@ -1117,7 +1154,7 @@ int hphi_apply_H(hphi_model* m, const void* v, void* w, int nvec, int prec, void
   if (v == w) return fail(m, HPHI_ERR_INVALID_ARG, "apply_H: v and w must not overlap");
   hphi::FusedArgs fa;
   void* scratch = nullptr;
-  const size_t need = hv_scratch_bytes(m, prec, nvec, hphi::Epi::kStore);
+  const size_t need = hv_scratch_bytes(m, prec, nvec, hphi::Epi::kStore, hphi::batch_aligned(v, w));
   if (need && m->kind == HPHI_SPIN_HALF && !use_batch(m, nvec)) {
     scratch = optional_scratch(m, need);
   } else if (need) {

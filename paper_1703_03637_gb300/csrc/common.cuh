@@ -342,6 +342,48 @@ int batch_grid(int prec, bool cplx, int nvec, Epi epi, int64_t dim);
 Status launch_batch(const SpinDev& md, const BatchPlan* plan, int prec, bool cplx, const void* v, void* w,
                     void* scratch, int nvec, Epi epi, const FusedArgs& fa, int grid, cudaStream_t st);
 
+// Tiled H v of many vectors in the full basis (k_tile.cu): passes over tiles of 2^t rows that a
+// set of t sites closes.
+constexpr int kTileMaxEntries = 128;  // terms of one pass
+constexpr int kTilePerRow4 = 1;       // TileEntry::flags: the phase depends on which of 4 rows,
+constexpr int kTilePerRow8 = 2;       // or of 8 rows, of a thread,
+constexpr int kTileReal = 4;          // the class coefficient and the phase are real
+struct TileEntry {
+  uint32_t lmask;    // flipped sites as local row bits
+  uint16_t phases;   // as in SpinEntry
+  uint16_t cls;
+  uint8_t i, j;      // sites whose row bits select the phase
+  uint16_t flags;
+  uint32_t flip;     // two bits per row bit: which of the sites i, j that bit is
+};
+static_assert(sizeof(TileEntry) == 16, "TileEntry layout");
+struct TilePass {
+  const TileEntry* ents = nullptr;
+  const uint32_t* dep = nullptr;  // [4][256] visit-index byte -> row bits (the set's sites first)
+  int n_ent = 0, t = 0, first = 0;
+  uint8_t pos[12] = {};           // local row bit -> site
+};
+struct TilePlan {
+  int n_pass = 0, max_run = 0;
+  TilePass pass[kMaxPasses];
+};
+struct TileHost {                 // a plan's tables before their upload
+  int n_pass = 0, max_run = 0;
+  int e0[kMaxPasses + 1] = {};
+  uint8_t pos[kMaxPasses][12] = {};
+  std::vector<TileEntry> ents;
+  std::vector<uint32_t> dep;
+};
+bool batch_tile_plan(int n_sites, int t, const std::vector<SpinEntry>& ents, const std::vector<double2>& cls,
+                     TileHost* out);
+// plans[t - 7], t = 7 .. 10 (n_pass 0: none); null when the gather kernels run the launch
+const TilePlan* tile_choose(const TilePlan* plans, const SpinDev& md, int prec, bool cplx, int nvec, Epi epi);
+int tile_grid(const TilePlan& plan, const SpinDev& md, int prec, bool cplx, int nvec);
+size_t tile_scratch_bytes(int prec, int nvec);  // column exponents (fp64)
+Status launch_tile(const SpinDev& md, const TilePlan& plan, int prec, bool cplx, const void* v, void* w, void* scratch,
+                   int nvec, Epi epi, const FusedArgs& fa, int grid, cudaStream_t st);
+Status launch_maxexp_cols(const double* v, int64_t rows, int nvec, int ncomp, int* E, cudaStream_t st);
+
 // fp64 -> 64-bit fixed point at one scale per vector (k_hub.cu): q = round(x 2^(1078 - E - extra)),
 // E the largest exponent field of x (computed into *Ep unless exp_ready), |q| < 2^(56 - extra)
 Status launch_quant_vec(const double* X, long long* Q, int64_t n, int* Ep, const int* done, bool exp_ready, int extra,

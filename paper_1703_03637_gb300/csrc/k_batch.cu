@@ -599,17 +599,26 @@ bool batch_plan_windows(int n_sites, int wbits, const std::vector<SpinEntry>& en
   return true;
 }
 
+Status launch_maxexp_cols(const double* v, int64_t rows, int nvec, int ncomp, int* E, cudaStream_t st) {
+  const int rowlen = nvec * ncomp;
+  HPHI_CUDA_TRY(cudaMemsetAsync(E, 0, sizeof(int) * nvec, st));
+  const int gv = (int)std::max<int64_t>(
+      1, std::min<int64_t>((rows * rowlen + kThreads - 1) / kThreads, (int64_t)num_sms() * 8));
+  k_maxexp_cols<<<gv, kThreads, 0, st>>>(v, rows, rowlen, ncomp, E);
+  HPHI_CUDA_TRY(cudaGetLastError());
+  return {};
+}
+
 Status launch_quant_cols(const double* v, int64_t rows, int nvec, int ncomp, long long* Q, int* E, cudaStream_t st) {
   const int rowlen = nvec * ncomp;
   if ((rowlen & (rowlen - 1)) != 0 || nvec > kMaxNvec)
     return {HPHI_ERR_INVALID_ARG, "quantised copy: nvec must be a power of two up to 256"};
   int lg_row = 0;
   while ((1 << lg_row) < rowlen) ++lg_row;
-  HPHI_CUDA_TRY(cudaMemsetAsync(E, 0, sizeof(int) * nvec, st));
+  Status s = launch_maxexp_cols(v, rows, nvec, ncomp, E, st);
+  if (s.code) return s;
   const int gv = (int)std::max<int64_t>(
       1, std::min<int64_t>((rows * rowlen + kThreads - 1) / kThreads, (int64_t)num_sms() * 8));
-  k_maxexp_cols<<<gv, kThreads, 0, st>>>(v, rows, rowlen, ncomp, E);
-  HPHI_CUDA_TRY(cudaGetLastError());
   k_quant_cols<<<gv, kThreads, 0, st>>>(v, Q, rows * rowlen, lg_row, ncomp == 2 ? 1 : 0, E);
   HPHI_CUDA_TRY(cudaGetLastError());
   return {};

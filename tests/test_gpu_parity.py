@@ -1193,3 +1193,63 @@ def test_fp32_start_norms_at_any_scale(mk, nv, scale):
         a, b = oracle.lanczos(spec, psi0[:, 0], 3)
         q = m.lanczos(3, prec=hp.FP32, v0=torch.as_tensor(psi0[:, 0] * scale))
         assert _rel(q["alpha"], a) < 2e-5 and _rel(q["beta"], b) < 2e-5
+
+
+# ----------------------------------------------------------------------------- tiled rows of many vectors
+def _mixed_ring(n, complex_):
+    """One 3x3 coupling with S^x S^z and S^x S^y parts on every bond and a tilted field: phases
+    that read sites outside the flipped ones, real and imaginary class coefficients."""
+    J = np.array([[1.0, 0.3, 0.2], [-0.3, 0.5, 0.0], [0.1, 0.0, 0.7]])
+    if not complex_:
+        J[0, 1] = J[1, 0] = 0.0
+    h = (0.1, 0.2 if complex_ else 0.0, 0.3)
+    return wl.ModelSpec(kind=wl.SPIN, n_sites=n, couplings=[(i, (i + 1) % n, J) for i in range(n)],
+                        fields=[(i, h) for i in range(n)], name=f"mixed_ring_{n}")
+
+
+TILE_CASES = [
+    ("kitaev_4x2_64", lambda: wl.kitaev_honeycomb(4, 2), 64),
+    ("kitaev_3x3_16", lambda: wl.kitaev_honeycomb(3, 3), 16),
+    ("mixed_complex_16_64", lambda: _mixed_ring(16, True), 64),
+    ("mixed_real_17_64", lambda: _mixed_ring(17, False), 64),
+    ("heisenberg_ring16_128", lambda: wl.heisenberg_ring(16), 128),
+    ("random_complex_16_64", lambda: wl.random_spin_model(16, 12, seed=21), 64),
+]
+
+
+@pytest.mark.parametrize("name,mk,nvec", TILE_CASES, ids=[c[0] for c in TILE_CASES])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_tiled_rows(name, mk, nvec, prec):
+    """Products and mTPQ steps of the tile passes against the oracle on the first, a middle and
+    the last column; another order of magnitude in every column (fp64 scales are per column)."""
+    spec = mk()
+    m = hp.Model.from_spec(spec)
+    p, tol = (hp.FP64, 1e-12) if prec == "fp64" else (hp.FP32, 2e-5)
+    cols = [0, nvec // 2 - 1, nvec - 1]
+    g = torch.Generator().manual_seed(31)
+    v = torch.randn((m.dim, nvec), dtype=torch.complex128 if m.is_complex else torch.float64, generator=g)
+    v = v * (10.0 ** torch.linspace(-6, 6, nvec, dtype=torch.float64))[None, :]
+    w = m.apply_H(v.to(device="cuda", dtype=m.dtype(p)))
+    for c in cols:
+        ref = oracle.apply_H(spec, v[:, c].numpy())
+        assert _rel(w[:, c].cpu().numpy(), ref if m.is_complex else ref.real) < tol
+    r = m.tpq(nvec, 3, l=2.0, prec=p, psi0=v)
+    for c in cols:
+        u, h2, nrm = oracle.tpq(spec, v[:, c].numpy(), 3, 2.0)
+        for k, x in (("u", u), ("h2", h2), ("norm", nrm)):
+            assert _rel(r[k][:, c], x) < (1e-11 if prec == "fp64" else 2e-5), k
+
+
+def test_tiled_rows_wide_dynamic_range():
+    """fp64 columns at both ends of the exponent range: scales whose class coefficients leave the
+    normal range take the two-step conversion."""
+    spec = wl.kitaev_honeycomb(4, 2)
+    m = hp.Model.from_spec(spec)
+    g = torch.Generator().manual_seed(33)
+    v = torch.randn((m.dim, 64), dtype=torch.complex128, generator=g)
+    scale = torch.ones(64, dtype=torch.float64)
+    scale[0], scale[1], scale[2] = 1e-290, 1e-300, 1e300
+    w = m.apply_H((v * scale[None, :]).cuda()).cpu()
+    for c in (0, 1, 2, 3):
+        ref = oracle.apply_H(spec, v[:, c].numpy())
+        assert _rel((w[:, c] / scale[c]).numpy(), ref) < 1e-12
