@@ -158,7 +158,7 @@ int hphi_release_workspace(hphi_model* m);
 
 typedef struct {
   int n_candidates;    /* launch configurations timed (0: nothing to tune for this model)      */
-  int best_dn_ept;     /* chosen columns per thread of the down-spin pass                       */
+  int best_dn_ept;     /* chosen 16-byte pieces per lane of the down-spin pass                  */
   int best_up_k;       /* chosen rows per shared-memory tile of the up-spin pass                */
   float best_ms;       /* H v time of the chosen configuration                                  */
   float default_ms;    /* H v time of the built-in default                                      */
@@ -172,7 +172,7 @@ typedef struct {
 /* Times the launch configurations of the model's H v at precision prec (HPHI_FP64 or
  * HPHI_FP32) on a seeded vector and keeps the fastest for every later hphi_apply_H /
  * hphi_lanczos_run / hphi_tpq_run on this model.  The two-pass Hubbard path is tuned over
- * columns per thread of the down-spin pass x rows per tile of the up-spin pass.  Real spin
+ * 16-byte pieces per lane of the down-spin pass x rows per tile of the up-spin pass.  Real spin
  * models in an S^z sector that take the split-row path (see hphi_set_sector_split) are tuned
  * over the split: the default low part, one bit more and up to two fewer, each with every tile height
  * that fits, and then over the high pass's columns per lane on the chosen split.  A real spin model in its full basis has every S^z sector of at least 2^20 rows

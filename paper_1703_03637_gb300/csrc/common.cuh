@@ -101,9 +101,9 @@ struct HubDev {
   const uint32_t* list_dn;   // [dim_dn]
   unsigned long long* counter;  // work-item counter of the generic kernel
   // two-pass path (real model, one hopping value per species): neighbour tables
-  // nbr[k * maxdeg + q] = rank of the q-th hop target of species state k | sign << 31
+  // rank of the q-th hop target of species state k | sign << 31 (layouts at k_hub_nbr)
   int fast;
-  int dn_ept;                // pass D columns per thread (0: default)
+  int dn_ept;                // pass D 16-byte pieces per lane (0: default)
   int up_k;                  // pass U rows per tile (0: largest that fits)
   int tuned_ept[2], tuned_k[2];  // autotuner choices per precision (HPHI_FP64, HPHI_FP32)
   int maxdeg_up, maxdeg_dn;

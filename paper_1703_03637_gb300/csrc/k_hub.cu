@@ -35,15 +35,10 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratch
 
 namespace {
 
-// columns per thread in pass D (stripe = kThreads * EPT columns); the stripe of all rows is
-// the L2 working set of pass D
-// built-in pass-D columns per thread per precision (hphi_autotune replaces them per model)
-#ifndef HPHI_DN_EPT32
-#define HPHI_DN_EPT32 4
-#endif
-#ifndef HPHI_DN_EPT64
-#define HPHI_DN_EPT64 1
-#endif
+// 16-byte pieces per lane of pass D unless hphi_autotune has chosen (a warp's stripe is 32 times
+// that wide): two, or one where wider stripes would leave fewer than two rounds of warps (4x3
+// torus, 6 + 5 electrons, fp64 product 0.052 against 0.057 ms)
+constexpr int kDnPieces = 2;
 
 // K consecutive values of a shared-memory row tile with the widest aligned accesses
 template <class R, int K>
@@ -68,9 +63,9 @@ __device__ __forceinline__ void load_k(const R* p, R* out) {
 constexpr int kZeroBytes = 128;      // gather_lanes(4 .. 16) entries
 constexpr int kSmemBudget = 208000;  // shared-memory bytes of the row tile (plus its zero entries and ~7 KB static)
 
-// neighbour table of one species, hop-slot major: nbr[q * n + k] is the q-th active hop
-// target of state k (rank | sign << 31), so threads of consecutive states read
-// consecutive words
+// neighbour table of one species: the q-th active hop target of state k (rank | sign << 31) at
+// nbr[q * n + k] for the up species (threads of consecutive states read consecutive words) and
+// at nbr[k * maxdeg_dn + q] for the down species (a warp reads one state's list)
 __global__ void k_hub_nbr(const HubDev md, int species, uint32_t* __restrict__ nbr, uint8_t* __restrict__ deg,
                           uint8_t* __restrict__ npos) {
   const int64_t n = species ? md.dim_dn : md.dim_up;
@@ -89,7 +84,7 @@ __global__ void k_hub_nbr(const HubDev md, int species, uint32_t* __restrict__ n
           if ((int)sg != pass) continue;
           const uint32_t b2 = b ^ h.mask;
           const uint32_t r2 = md.sector ? md.rank[b2] : b2;
-          nbr[(int64_t)cnt * n + k] = r2 | (sg << 31);
+          nbr[species ? k * md.maxdeg_dn + cnt : (int64_t)cnt * n + k] = r2 | (sg << 31);
           ++cnt;
         }
       }
@@ -100,103 +95,100 @@ __global__ void k_hub_nbr(const HubDev md, int species, uint32_t* __restrict__ n
   }
 }
 
-// difference of two accumulated sums (pass D keeps positive and negative terms apart)
-__device__ __forceinline__ IntAcc diff_acc(const IntAcc& p, const IntAcc& n) {
-  IntAcc r;
-  r.s = p.s - n.s;
-  return r;
-}
-__device__ __forceinline__ F32Acc diff_acc(const F32Acc& p, const F32Acc& n) {
-  F32Acc r;
-  r.s = p.s - n.s;
-  return r;
-}
-
-// pass D: W[d][u] = sum over down-spin neighbours d' of d of +-X[d'][u].  Items run
-// stripe-major (stripe = kThreads * EPT columns) so one stripe of all rows is the L2
-// working set.  Each warp loads the row's neighbour list once (lane q holds entry q) and
-// broadcasts it with shuffles, so the data loads of four neighbours issue back to back.
-template <class R, int EPT>
+// Pass D: W[d][u] = sum over down-spin neighbours d' of d of +-X[d'][u].  A warp item is one row
+// and a stripe of 32 * P 16-byte pieces; items run stripe by stripe, claimed in order from a
+// counter, so all CTAs stay on neighbouring rows of one stripe and that stripe of all rows stays
+// in L2.  Lane q holds the row's neighbour q and shuffles broadcast it; the list is sign-sorted,
+// entries [0, npos) add and the rest subtract.  VEC: rows start on 16 bytes, one load a piece;
+// otherwise element by element.
+//
+// Bound by the loads from L2 (17 neighbours a row on average: 13.6 TB/s).  Measured on GB300
+// against 256 single elements a CTA and claim: 16 sites, 8 + 8 electrons, int64 1.65 ms instead of
+// 2.37 ms; 7 + 6 electrons, fp32 0.37 instead of 0.50 ms; 18 sites, 9 + 9, fp32 11.8 instead of
+// 16.1 ms.
+template <class R, int P, bool VEC>
 __global__ void __launch_bounds__(kThreads) k_hub_dn(const HubDev md, const R* __restrict__ X, R* __restrict__ W,
                                                      const int* __restrict__ done,
-                                                     unsigned long long* __restrict__ next_item) {
-  using A = typename SumAcc<R>::T;
+                                                     unsigned long long* __restrict__ next_item, int claim) {
   if (done != nullptr && *done) return;
-  const int tid = threadIdx.x, lane = tid & 31;
-  constexpr int SW = kThreads * EPT;
+  constexpr int PV = 16 / (int)sizeof(R), NE = P * PV, SW = 32 * NE;
+  constexpr int kWarps = kThreads / 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t dim_up = md.dim_up, dim_dn = md.dim_dn;
-  const int n_str = (int)((dim_up + SW - 1) / SW);
-  const int64_t n_items = (int64_t)n_str * dim_dn;
-  const int last_full = (int)(dim_up / SW);  // stripes [0, last_full) need no bounds checks
-  // items are handed out in order from a counter, so all CTAs stay on neighbouring rows of
-  // one stripe and the stripe of X they gather stays in L2 (static round-robin lets CTAs
-  // drift over several stripes)
+  const int64_t n_items = ((dim_up + SW - 1) / SW) * dim_dn;
   __shared__ int64_t s_item;
   for (;;) {
     __syncthreads();
-    if (tid == 0) s_item = (int64_t)atomicAdd(next_item, 1ull);
+    if (tid == 0) s_item = (int64_t)atomicAdd(next_item, (unsigned long long)(kWarps * claim));
     __syncthreads();
-    const int64_t item = s_item;
-    if (item >= n_items) break;
-    const int s = (int)(item / dim_dn);
-    const int64_t d = item - (int64_t)s * dim_dn;
-    const int deg = md.deg_dn[d];
-    const int npos = md.npos_dn[d];
-    const int u0 = s * SW + tid;
-    const bool full = s < last_full;
-    // the list is sign-sorted: entries [0, npos) add, [npos, deg) subtract; each group is
-    // summed without per-term sign handling and the two sums are subtracted once
-    A accp[EPT], accn[EPT];
+    const int64_t base = s_item;
+    if (base >= n_items) break;
+    int64_t s = base / dim_dn, d = base - s * dim_dn + warp;  // the CTA's warps on neighbouring rows
+    for (int it = 0; it < claim; ++it, d += kWarps) {
+      while (d >= dim_dn) {
+        d -= dim_dn;
+        ++s;
+      }
+      const int64_t u0 = s * SW;
+      if (u0 >= dim_up) break;
+      const int deg = __ldg(md.deg_dn + d), npos = __ldg(md.npos_dn + d);
+      const bool full = u0 + SW <= dim_up;
+      // first column of element j of this lane
+      auto col = [&](int j) -> int64_t { return u0 + (VEC ? ((j / PV) * 32 + lane) * PV + j % PV : j * 32 + lane); };
+      R acc[NE];
 #pragma unroll
-    for (int j = 0; j < EPT; ++j) {
-      accp[j].zero();
-      accn[j].zero();
-    }
-    for (int qb = 0; qb < deg; qb += 32) {
-      const int nq = (deg - qb < 32) ? (deg - qb) : 32;
-      const uint32_t mine = (lane < nq) ? __ldg(md.nbr_dn + (int64_t)(qb + lane) * dim_dn + d) : 0u;
-      for (int q0 = 0; q0 < nq; q0 += 4) {
-        R x[4][EPT];
+      for (int j = 0; j < NE; ++j) acc[j] = (R)0;
+      for (int qb = 0; qb < deg; qb += 32) {
+        const int nq = min(32, deg - qb);
+        const uint32_t mine = lane < nq ? __ldg(md.nbr_dn + d * md.maxdeg_dn + qb + lane) : 0u;
+        for (int q0 = 0; q0 < nq; q0 += 4) {
+          R x[4][NE];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          const uint32_t e = __shfl_sync(0xffffffffu, mine, (q0 + t) & 31);
-          const bool on = q0 + t < nq;
-          const R* src = X + (int64_t)(e & 0x7fffffffu) * dim_up + u0;
+          for (int t = 0; t < 4; ++t) {
+            const uint32_t e = __shfl_sync(0xffffffffu, mine, (q0 + t) & 31);
+            const bool on = q0 + t < nq;
+            const R* src = X + (int64_t)(e & 0x7fffffffu) * dim_up;
+            if constexpr (VEC) {
 #pragma unroll
-          for (int j = 0; j < EPT; ++j) {
-            x[t][j] = (R)0;
-            if (on && (full || u0 + j * kThreads < dim_up)) x[t][j] = __ldg(src + j * kThreads);
+              for (int j = 0; j < P; ++j) {
+                uint4 p = make_uint4(0u, 0u, 0u, 0u);
+                if (on && (full || col(j * PV) < dim_up)) p = __ldg(reinterpret_cast<const uint4*>(src + col(j * PV)));
+                memcpy(&x[t][j * PV], &p, 16);
+              }
+            } else {
+#pragma unroll
+              for (int j = 0; j < NE; ++j) x[t][j] = (on && (full || col(j) < dim_up)) ? __ldg(src + col(j)) : (R)0;
+            }
+          }
+          const int left = npos - (qb + q0);  // of these four, so many add
+          if (left >= 4) {
+#pragma unroll
+            for (int j = 0; j < NE; ++j) acc[j] += (x[0][j] + x[1][j]) + (x[2][j] + x[3][j]);
+          } else if (left <= 0) {
+#pragma unroll
+            for (int j = 0; j < NE; ++j) acc[j] -= (x[0][j] + x[1][j]) + (x[2][j] + x[3][j]);
+          } else {
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+#pragma unroll
+              for (int j = 0; j < NE; ++j) acc[j] += t < left ? x[t][j] : -x[t][j];
           }
         }
-        const int qn = qb + q0;  // list position of t = 0
-        if (qn + 4 <= npos) {
-#pragma unroll
-          for (int t = 0; t < 4; ++t)
-#pragma unroll
-            for (int j = 0; j < EPT; ++j) accp[j].add(x[t][j], false);
-        } else if (qn >= npos) {
-#pragma unroll
-          for (int t = 0; t < 4; ++t)
-#pragma unroll
-            for (int j = 0; j < EPT; ++j) accn[j].add(x[t][j], false);
-        } else {
-#pragma unroll
-          for (int t = 0; t < 4; ++t)
-#pragma unroll
-            for (int j = 0; j < EPT; ++j) {
-              if (qn + t < npos) accp[j].add(x[t][j], false);
-              else accn[j].add(x[t][j], false);
-            }
-        }
       }
-    }
-    A acc[EPT];
+      R* dst = W + d * dim_up;
+      if constexpr (VEC) {
 #pragma unroll
-    for (int j = 0; j < EPT; ++j) acc[j] = diff_acc(accp[j], accn[j]);
-    R* dst = W + d * dim_up + u0;
+        for (int j = 0; j < P; ++j)
+          if (full || col(j * PV) < dim_up) {
+            uint4 p;
+            memcpy(&p, &acc[j * PV], 16);
+            __stcs(reinterpret_cast<uint4*>(dst + col(j * PV)), p);
+          }
+      } else {
 #pragma unroll
-    for (int j = 0; j < EPT; ++j) {
-      if (full || u0 + j * kThreads < dim_up) __stcs(dst + j * kThreads, (R)acc[j].value());
+        for (int j = 0; j < NE; ++j)
+          if (full || col(j) < dim_up) __stcs(dst + col(j), acc[j]);
+      }
     }
   }
 }
@@ -555,18 +547,33 @@ int pick_kq(const HubDev& md) {
   return k;
 }
 
-// pass D launch with the tuned (or default) columns per thread
+// pass D launch with the tuned (or default) pieces per lane
 template <class R>
 Status launch_dn(const HubDev& md, const R* X, R* W, const int* done, unsigned long long* counter, cudaStream_t st) {
-  int ept = md.dn_ept > 0 ? md.dn_ept : (sizeof(R) == 8 ? HPHI_DN_EPT64 : HPHI_DN_EPT32);
-  if (ept != 1 && ept != 2 && ept != 4) ept = 1;
-  const int64_t sw = (int64_t)kThreads * ept;
-  const int64_t items = ((md.dim_up + sw - 1) / sw) * md.dim_dn;
-  const int gd = (int)std::min<int64_t>(items, (int64_t)num_sms() * 8);
+  auto items_of = [&](int pieces) -> int64_t {
+    const int64_t sw = (int64_t)32 * pieces * 16 / (int64_t)sizeof(R);
+    return ((md.dim_up + sw - 1) / sw) * md.dim_dn;
+  };
+  const int64_t warps = (int64_t)num_sms() * 32;
+  int p = md.dn_ept;
+  if (p != 1 && p != 2 && p != 4) p = items_of(kDnPieces) >= 2 * warps ? kDnPieces : 1;
+  const int64_t items = items_of(p);
+  // items per warp and claim: four, fewer while that would leave warps without one
+  const int claim = (int)std::max<int64_t>(1, std::min<int64_t>(4, items / (2 * warps)));
+  const int gd = (int)std::min<int64_t>((items + 7) / 8, (int64_t)num_sms() * 8);
+  const bool vec = (md.dim_up * (int64_t)sizeof(R)) % 16 == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(W)) & 15u) == 0;
   HPHI_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st));
-  if (ept == 4) k_hub_dn<R, 4><<<gd, kThreads, 0, st>>>(md, X, W, done, counter);
-  else if (ept == 2) k_hub_dn<R, 2><<<gd, kThreads, 0, st>>>(md, X, W, done, counter);
-  else k_hub_dn<R, 1><<<gd, kThreads, 0, st>>>(md, X, W, done, counter);
+#define HPHI_DN(PP)                                                                    \
+  if (vec) k_hub_dn<R, PP, true><<<gd, kThreads, 0, st>>>(md, X, W, done, counter, claim);    \
+  else k_hub_dn<R, PP, false><<<gd, kThreads, 0, st>>>(md, X, W, done, counter, claim)
+  if (p == 4) {
+    HPHI_DN(4);
+  } else if (p == 1) {
+    HPHI_DN(1);
+  } else {
+    HPHI_DN(2);
+  }
+#undef HPHI_DN
   HPHI_CUDA_TRY(cudaGetLastError());
   return {};
 }

@@ -1253,3 +1253,22 @@ def test_tiled_rows_wide_dynamic_range():
     for c in (0, 1, 2, 3):
         ref = oracle.apply_H(spec, v[:, c].numpy())
         assert _rel((w[:, c] / scale[c]).numpy(), ref) < 1e-12
+
+
+@pytest.mark.parametrize("n,nu,nd", [(9, 4, 3), (10, 5, 2), (11, 3, 6), (12, 6, 6), (7, 7, 3), (13, 1, 4)])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_hubbard_down_pass_pieces(n, nu, nd, offset):
+    """Pass D on rows that start on 16 bytes and rows that do not (odd row lengths, vectors one
+    element off), one part-filled and several stripes, and 1, 2 and 4 pieces a lane."""
+    spec = wl.hubbard_ring(n, 1.0, 8.0).with_basis(wl.BASIS_NUMBER, nu, nd)
+    m = hp.Model.from_spec(spec)
+    v = wl.gaussian_vector(7 * n + nd, m.dim)[:, 0]
+    ref = oracle.apply_H(spec, v).real
+    for prec, tol in ((hp.FP64, 1e-12), (hp.FP32, 2e-5)):
+        buf = torch.zeros(2, m.dim + 1, device="cuda", dtype=m.dtype(prec))
+        x, w = buf[0, offset:offset + m.dim], buf[1, offset:offset + m.dim]
+        x.copy_(torch.as_tensor(v))
+        for _ in range(2):
+            m.apply_H(x, w)
+            assert _rel(w.cpu().numpy(), ref) < tol
+            m.autotune(prec)
