@@ -133,9 +133,9 @@ struct hphi_model {
     hphi::BatchPlan plan;
   };
   std::map<int, std::unique_ptr<WinCache>> win;
-  // tile plans of the full basis for t = 7 .. 10 sites (built with the sector tables)
-  hphi::TilePlan tile[4];
-  DBuf d_tile_ents[4], d_tile_dep[4];
+  // tile plans of the full basis for t = 8 .. 10 sites (built with the sector tables)
+  hphi::TilePlan tile[3];
+  DBuf d_tile_ents[3], d_tile_dep[3];
   // split-row path of real S^z-sector spin models: the compiled terms, whether each precision
   // may take the path, the split asked for per precision (-1 off, 0 default, else L) and
   // rows per tile (0 default), and the device tables built so far by (L, K, element size)
@@ -345,10 +345,10 @@ hphi::Status compile_spin(hphi_model* m, cudaStream_t st) {
   d.max_run = max_run;
   m->host_entries = ents;
   m->win.clear();
-  for (int k = 0; k < 4; ++k) {
+  for (int k = 0; k < 3; ++k) {
     m->tile[k] = hphi::TilePlan{};
     hphi::TileHost th;
-    if (sector || !hphi::batch_tile_plan(N, 7 + k, ents, cls, &th)) continue;
+    if (sector || !hphi::batch_tile_plan(N, 8 + k, ents, cls, &th)) continue;
     if ((s = upload(m->d_tile_ents[k], th.ents, st)).code) return s;
     if ((s = upload(m->d_tile_dep[k], th.dep, st)).code) return s;
     HPHI_CUDA_TRY(cudaStreamSynchronize(st));  // th dies here
@@ -359,7 +359,7 @@ hphi::Status compile_spin(hphi_model* m, cudaStream_t st) {
       tp.pass[p].ents = m->d_tile_ents[k].as<hphi::TileEntry>() + th.e0[p];
       tp.pass[p].n_ent = th.e0[p + 1] - th.e0[p];
       tp.pass[p].dep = m->d_tile_dep[k].as<uint32_t>() + (size_t)p * 1024;
-      tp.pass[p].t = 7 + k;
+      tp.pass[p].t = 8 + k;
       memcpy(tp.pass[p].pos, th.pos[p], sizeof(th.pos[p]));
     }
   }
@@ -1761,9 +1761,10 @@ hphi::Status lanczos_impl(hphi_model* m, const hphi_lanczos_params* p, hphi_lanc
   Timer tm;
   HPHI_CUDA_TRY(cudaEventCreate(&tm.a));
   HPHI_CUDA_TRY(cudaEventCreate(&tm.b));
-  if (L.profile || L.v0_host) {
+  if (L.profile || L.v0_host || L.cta) {
     // profiled runs launch eagerly: events recorded inside a captured graph cannot be
-    // queried with cudaEventElapsedTime; so do runs copying a host start vector
+    // queried with cudaEventElapsedTime; so do runs copying a host start vector, and one-cluster
+    // runs, whose five launches cost less than a graph's capture and instantiation
     HPHI_CUDA_TRY(cudaEventRecord(tm.a, st));
     if ((s = lz_enqueue(L, st)).code) return s;
     HPHI_CUDA_TRY(cudaEventRecord(tm.b, st));

@@ -376,7 +376,7 @@ struct TileHost {                 // a plan's tables before their upload
 };
 bool batch_tile_plan(int n_sites, int t, const std::vector<SpinEntry>& ents, const std::vector<double2>& cls,
                      TileHost* out);
-// plans[t - 7], t = 7 .. 10 (n_pass 0: none); null when the gather kernels run the launch
+// plans[t - 8], t = 8 .. 10 (n_pass 0: none); null when the gather kernels run the launch
 const TilePlan* tile_choose(const TilePlan* plans, const SpinDev& md, int prec, bool cplx, int nvec, Epi epi);
 int tile_grid(const TilePlan& plan, const SpinDev& md, int prec, bool cplx, int nvec);
 size_t tile_scratch_bytes(int prec, int nvec);  // column exponents (fp64)

@@ -10,6 +10,7 @@
 // the two hopping sites.  Reductions for the fused steps are per-thread partial sums
 // (fp64, or error-free fp32 TwoSum chunks flushed to fp64) reduced per CTA in a fixed
 // order and written to a partials array, so results are bit-reproducible run to run.
+#include <algorithm>
 #include <type_traits>
 
 #include "basis.cuh"
@@ -580,48 +581,80 @@ Status launch_hv(bool hubbard, const void* md, int prec, bool cplx, const void* 
 // through distributed shared memory.  GB300 issues fp64 at 1/64 of its fp32 rate, so one SM
 // alone would be bound by the fp64 work of the diagonal and exchange sums: the cluster spreads
 // it over kClCtas SMs.  Per step: P = c1 H C - c2 P with the partial (C, H C), cluster barrier,
-// alpha from the kClCtas partials (every CTA sums them in the same order), P -= gamma C with
-// |P|^2, cluster barrier, beta, swap C and P.  The two partial slots alternate, so each
-// barrier also ends the reads of the previous one.  Scalars follow k_lz_fin's conventions (C
-// unnormalised, sigma = 1 / |C|), so k_tridiag reads the same arrays.
+// alpha, P -= gamma C with |P|^2, cluster barrier, beta, swap C and P.
+//
+// What does not change from step to step is worked out once: each row's diagonal element and the
+// cluster address of every element it gathers, with the element's signed coefficient in the
+// address's low bits (kClCoef codes).  Models with more coefficients, or rows with more elements
+// than the shared memory left (cap), decode their terms in every step instead.
+//
+// A sum over the cluster: every warp writes its sum into every CTA's slot for it before the
+// barrier; behind it one warp of each CTA adds the slots in one fixed order (the same bits in
+// every CTA), works out the step's scalars and hands them to its CTA.  One warp, because every
+// fp64 instruction of a warp holds its scheduler's fp64 unit for 64 cycles: eight warps repeating
+// the scalar work cost more than the hand-over.  The two slot arrays alternate, so each barrier
+// also ends the reads of the other.
+// Scalars follow k_lz_fin's conventions (C unnormalised, sigma = 1 / |C|), so k_tridiag reads the
+// same arrays.  Bound by latency (two barriers, two sums and about 14 dependent fp64 operations a
+// step); measured on GB300: 6.1 us a step on the 12-site ring's 4,096 rows instead of 11.5 us.
 namespace {
 constexpr int kClThreads = 256;
-
-__device__ double cl_block_sum(double x, double* s_w) {
-  for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(0xffffffffu, x, off);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  __syncthreads();  // the previous sum has been read
-  if (lane == 0) s_w[wid] = x;
-  __syncthreads();
-  double t = 0.0;
-  for (int k = 0; k < kClThreads / 32; ++k) t += s_w[k];  // same order in every thread
-  return t;
-}
+constexpr int kClWarps = kClThreads / 32;
+constexpr int kClCoef = 8;  // distinct signed coefficients a gather address can carry
 
 // cluster barrier (all threads of all CTAs; shared-memory writes before it are visible after)
 __device__ __forceinline__ void cl_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// generic address of variable p of this CTA, as seen in CTA `rank` of the cluster
-template <class T>
-__device__ __forceinline__ T* cl_map(T* p, unsigned rank) {
-  uint64_t out;
-  asm volatile("mapa.u64 %0, %1, %2;" : "=l"(out) : "l"(p), "r"(rank));
-  return reinterpret_cast<T*>(out);
+// cluster shared-memory address of this CTA's variable p as it lies in CTA `rank`
+__device__ __forceinline__ uint32_t cl_map(const void* p, unsigned rank) {
+  uint32_t out;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return out;
+}
+__device__ __forceinline__ double cl_load(uint32_t a) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a));  // ordered against cl_sync
+  return v;
+}
+__device__ __forceinline__ void cl_store(uint32_t a, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
 }
 
-// sum over the cluster's CTAs of one shared double: lane c of every warp loads CTA c's value
-// (one round trip of distributed shared memory for all of them) and the warp adds them in a
-// fixed tree order, so every thread of every CTA gets the same bits
-__device__ __forceinline__ double cl_gather_sum(double* p, int ncta) {
+// first half of a cluster sum: this warp's sum of x into its slot of every CTA
+__device__ __forceinline__ void cl_put(double x, double* slots, unsigned rank, int ncta) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+  x = __shfl_sync(0xffffffffu, x, 0);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (lane < ncta) cl_store(cl_map(slots + rank * kClWarps + wid, (unsigned)lane), x);
+}
+// second half, behind the barrier
+__device__ __forceinline__ double cl_take(const double* slots, int ncta) {
   const int lane = threadIdx.x & 31;
-  double v = lane < ncta ? *cl_map(p, (unsigned)lane) : 0.0;
+  double v = 0.0;
+  for (int k = lane; k < ncta * kClWarps; k += 32) v += slots[k];
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  // lanes may hold differently rounded sums; lane 0's is the same in every warp of every CTA,
-  // and the loop's exit test must see one value everywhere
+  // lanes may hold differently rounded sums; lane 0's is the same in every CTA, and the loop's
+  // exit test must see one value everywhere
   return __shfl_sync(0xffffffffu, v, 0);
+}
+
+// sqrt(x) and 1 / sqrt(x) to the last place or so in ten fp64 operations (x > 0): the fp32
+// reciprocal root, one third-order step, one residual step for the root
+__device__ __forceinline__ void cl_sqrt(double x, double& root, double& inv) {
+  const int hi = __double2hiint(x);
+  const int k = ((hi >> 20) - 1023) >> 1;  // x = m 4^k, m in [1, 4)
+  const double m = __hiloint2double(hi - (k << 21), __double2loint(x));
+  double y = (double)rsqrtf((float)m);
+  const double e = fma(-(m * y), y, 1.0);
+  y = fma(y * e, fma(0.375, e, 0.5), y);
+  double r = m * y;
+  r = fma(fma(-r, r, m), 0.5 * y, r);
+  root = r * __hiloint2double((k + 1023) << 20, 0);
+  inv = y * __hiloint2double((1023 - k) << 20, 0);
 }
 
 __device__ __forceinline__ unsigned cl_rank() {
@@ -630,11 +663,14 @@ __device__ __forceinline__ unsigned cl_rank() {
   return r;
 }
 
+// list: cap slots per row, slot k of local row i at list[k R + i]
 __global__ void __launch_bounds__(kClThreads, 1) k_lz_cl(const SpinDev md, LzDev lz, int steps, double brk,
-                                                         const double* __restrict__ C0, int R, int ncta) {
-  extern __shared__ __align__(16) double sm_v[];  // [2][R]: this CTA's slices of the two vectors
-  __shared__ double s_w[kClThreads / 32];
-  __shared__ double s_part[2];                   // this CTA's partial of each alternating slot
+                                                         const double* __restrict__ C0, int R, int ncta, int cap) {
+  extern __shared__ __align__(16) double sm_v[];  // [2][R] this CTA's slices, [R] diagonal, lists
+  __shared__ double s_slot[2][16 * kClWarps];
+  __shared__ double s_coef[kClCoef];
+  __shared__ double s_sc[3];  // gamma; c1 = sigma and c2 of the next step
+  __shared__ int s_over, s_ncoef, s_done;
   __shared__ SpinEntry s_ent[kMaxSpinEntries];
   __shared__ double s_cls[kMaxClasses];
   __shared__ LinGroup s_lin[kMaxLin];
@@ -648,117 +684,190 @@ __global__ void __launch_bounds__(kClThreads, 1) k_lz_cl(const SpinDev md, LzDev
   const int nloc = left <= 0 ? 0 : (left < (int64_t)R ? (int)left : R);
   double* A = sm_v;
   double* B = sm_v + R;
-  for (int i = tid; i < nloc; i += kClThreads) {
-    A[i] = C0[r0 + i];
-    B[i] = 0.0;
-  }
+  double* D = sm_v + 2 * R;
+  uint32_t* list = reinterpret_cast<uint32_t*>(sm_v + 3 * R);
+  uint8_t* s_cnt = reinterpret_cast<uint8_t*>(list + (size_t)cap * R);
   for (int k = tid; k < md.n_entries; k += kClThreads) s_ent[k] = md.entries[k];
   for (int k = tid; k < md.n_classes; k += kClThreads) s_cls[k] = md.cls_coef[k].x;
   for (int k = tid; k < md.n_lin; k += kClThreads) s_lin[k] = md.lin[k];
   for (int k = tid; k < md.n_pairs; k += kClThreads) s_pair[k] = md.pairs[k];
   for (int k = tid; k < md.n_pair_groups; k += kClThreads) s_pcoef[k] = md.pair_coef[k];
+  if (tid == 0) {
+    // +c of class k at code 2k, -c at 2k + 1
+    s_ncoef = 2 * md.n_classes;
+    s_over = s_ncoef > kClCoef ? 1 : 0;
+  }
+  __syncthreads();
+  if (tid < kClCoef) s_coef[tid] = tid < s_ncoef ? ((tid & 1) ? -s_cls[tid >> 1] : s_cls[tid >> 1]) : 0.0;
+  auto state = [&](int i) -> uint64_t {
+    return md.sector ? sector_state(md.t, (uint64_t)(r0 + i)) : (uint64_t)(r0 + i);
+  };
+  const uint32_t a_off = (uint32_t)__cvta_generic_to_shared(A);
+  for (int i = tid; i < nloc; i += kClThreads) {
+    A[i] = C0[r0 + i];
+    B[i] = 0.0;
+    const uint64_t s = state(i);
+    // diagonal: integer bit counts per coefficient group, one multiply-add per group
+    double d = md.c0;
+    for (int g = 0; g < md.n_lin; ++g) d += s_lin[g].coef * (double)__popcll(s & s_lin[g].mask);
+    if (md.n_pairs) {
+      int grp = s_pair[0].grp, cnt = 0;
+      for (int q = 0; q < md.n_pairs; ++q) {
+        const PairEntry pe = s_pair[q];
+        if (pe.grp != grp) {
+          d += s_pcoef[grp] * (double)cnt;
+          cnt = 0;
+          grp = pe.grp;
+        }
+        cnt += (int)((s >> pe.i) & (s >> pe.j) & 1ull);
+      }
+      d += s_pcoef[grp] * (double)cnt;
+    }
+    D[i] = d;
+    int c = 0;
+    if (s_ncoef <= kClCoef) {
+      for (int e = 0; e < md.n_entries; ++e) {
+        const SpinEntry en = s_ent[e];
+        const int sel = (int)((s >> en.i) & 1ull) | ((int)((s >> en.j) & 1ull) << 1);
+        const int code = (en.phases >> (3 * sel)) & 7;
+        if (!code) continue;
+        if (c < cap) {
+          const uint64_t s2 = s ^ en.mask;
+          const int64_t r2 = md.sector ? (int64_t)sector_rank(md.t, s2) : (int64_t)s2;
+          const unsigned owner = (unsigned)(r2 / R);
+          list[(size_t)c * R + i] = cl_map(A + (r2 - (int64_t)owner * R), owner) | (uint32_t)(2 * en.cls + (code == 1 ? 0 : 1));
+        }
+        ++c;
+      }
+      if (c > min(cap, 255)) s_over = 1;  // (any thread: the value is the same)
+    }
+    s_cnt[i] = (uint8_t)min(c, 255);
+  }
   // k_lz_init / its finaliser have set sigma_0, c1, c2 and the flags
   double sg = lz.sig[0];
   double c1 = lz.s[0], c2 = lz.s[1];
   int done = *lz.done;
   bool cur_a = true;  // C is A (else B)
   int k = 0;
-  cl_sync();  // every CTA has staged its slice of C_0
+  cl_sync();  // every CTA has staged its slice of C_0 and its flag
+  bool over = false;
+  for (int c = 0; c < ncta; ++c) {
+    int f;
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(f) : "r"(cl_map(&s_over, (unsigned)c)) : "memory");
+    over = over || f != 0;
+  }
   for (; k < steps && !done; ++k) {
     double* C = cur_a ? A : B;
     double* P = cur_a ? B : A;
+    const uint32_t shift = cur_a ? 0u : (uint32_t)(R * sizeof(double));
     double xh = 0.0;
     for (int i = tid; i < nloc; i += kClThreads) {
-      const uint64_t s = md.sector ? sector_state(md.t, (uint64_t)(r0 + i)) : (uint64_t)(r0 + i);
-      // diagonal: integer bit counts per coefficient group, one multiply-add per group
-      double d = md.c0;
-      for (int g = 0; g < md.n_lin; ++g) d += s_lin[g].coef * (double)__popcll(s & s_lin[g].mask);
-      if (md.n_pairs) {
-        int grp = s_pair[0].grp, cnt = 0;
-        for (int q = 0; q < md.n_pairs; ++q) {
-          const PairEntry pe = s_pair[q];
-          if (pe.grp != grp) {
-            d += s_pcoef[grp] * (double)cnt;
-            cnt = 0;
-            grp = pe.grp;
-          }
-          cnt += (int)((s >> pe.i) & (s >> pe.j) & 1ull);
-        }
-        d += s_pcoef[grp] * (double)cnt;
-      }
       const double x = C[i];
-      double hv = d * x;
-      // exchange: signed sums per coefficient class (entries are sorted by class), gathers in
-      // batches of eight so their distributed-shared-memory loads overlap
-      double acc = 0.0;
-      int cur = md.n_entries ? s_ent[0].cls : 0;
-      for (int e0 = 0; e0 < md.n_entries; e0 += 8) {
-        double y[8];
-        int sg8[8], cl8[8];
+      double hv = D[i] * x;
+      if (!over) {
+        const int cnt = s_cnt[i];
+        for (int e0 = 0; e0 < cnt; e0 += 8) {
+          double y[8];
+          uint32_t ad[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          y[j] = 0.0;
-          sg8[j] = 0;
-          cl8[j] = cur;
-          const int e = e0 + j;
-          if (e < md.n_entries) {
-            const SpinEntry en = s_ent[e];
-            cl8[j] = en.cls;
-            const int sel = (int)((s >> en.i) & 1ull) | ((int)((s >> en.j) & 1ull) << 1);
-            const int code = (en.phases >> (3 * sel)) & 7;
-            if (code) {
-              const uint64_t s2 = s ^ en.mask;
-              const int64_t r2 = md.sector ? (int64_t)sector_rank(md.t, s2) : (int64_t)s2;
-              const unsigned owner = (unsigned)(r2 / R);
-              y[j] = cl_map(C, owner)[r2 - (int64_t)owner * R];
-              sg8[j] = code == 1 ? 1 : -1;  // real models: codes +1 / -1 only
+          for (int j = 0; j < 8; ++j) ad[j] = e0 + j < cnt ? list[(size_t)(e0 + j) * R + i] : a_off;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) y[j] = e0 + j < cnt ? cl_load((ad[j] & ~7u) + shift) : 0.0;
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            if (e0 + j < cnt) hv = fma(s_coef[ad[j] & 7u], y[j], hv);
+        }
+      } else {
+        // signed sums per coefficient class (entries are sorted by class), gathers in batches of
+        // eight so their distributed-shared-memory loads overlap
+        const uint64_t s = state(i);
+        double acc = 0.0;
+        int cur = md.n_entries ? s_ent[0].cls : 0;
+        for (int e0 = 0; e0 < md.n_entries; e0 += 8) {
+          double y[8];
+          int sg8[8], cl8[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            y[j] = 0.0;
+            sg8[j] = 0;
+            cl8[j] = cur;
+            const int e = e0 + j;
+            if (e < md.n_entries) {
+              const SpinEntry en = s_ent[e];
+              cl8[j] = en.cls;
+              const int sel = (int)((s >> en.i) & 1ull) | ((int)((s >> en.j) & 1ull) << 1);
+              const int code = (en.phases >> (3 * sel)) & 7;
+              if (code) {
+                const uint64_t s2 = s ^ en.mask;
+                const int64_t r2 = md.sector ? (int64_t)sector_rank(md.t, s2) : (int64_t)s2;
+                const unsigned owner = (unsigned)(r2 / R);
+                y[j] = cl_load(cl_map(C + (r2 - (int64_t)owner * R), owner));
+                sg8[j] = code == 1 ? 1 : -1;  // real models: codes +1 / -1 only
+              }
             }
           }
-        }
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          if (cl8[j] != cur) {
-            hv = fma(s_cls[cur], acc, hv);
-            acc = 0.0;
-            cur = cl8[j];
+          for (int j = 0; j < 8; ++j) {
+            if (cl8[j] != cur) {
+              hv = fma(s_cls[cur], acc, hv);
+              acc = 0.0;
+              cur = cl8[j];
+            }
+            if (sg8[j] > 0) acc += y[j];
+            else if (sg8[j] < 0) acc -= y[j];
           }
-          if (sg8[j] > 0) acc += y[j];
-          else if (sg8[j] < 0) acc -= y[j];
         }
+        if (md.n_entries) hv = fma(s_cls[cur], acc, hv);
       }
-      if (md.n_entries) hv = fma(s_cls[cur], acc, hv);
       xh = fma(x, hv, xh);
       P[i] = c1 * hv - c2 * P[i];
     }
-    double t = cl_block_sum(xh, s_w);
-    if (tid == 0) s_part[0] = t;
-    cl_sync();  // P written everywhere (so C is no longer read), partials of alpha ready
-    const double xs = cl_gather_sum(&s_part[0], ncta);
-    const double a = xs * sg * sg;  // alpha_k = (H v_k, v_k)
-    const double gm = a * sg;
+    cl_put(xh, s_slot[0], rank, ncta);
+    cl_sync();  // P written everywhere (so C is no longer read), sums of alpha in their slots
+    double a = 0.0;
+    if (tid < 32) {
+      const double xs = cl_take(s_slot[0], ncta);
+      a = xs * sg * sg;  // alpha_k = (H v_k, v_k)
+      if (tid == 0) s_sc[0] = a * sg;
+    }
+    __syncthreads();
+    const double gm = s_sc[0];
     double pp = 0.0;
     for (int i = tid; i < nloc; i += kClThreads) {
       const double pv = fma(-gm, C[i], P[i]);
       P[i] = pv;
       pp = fma(pv, pv, pp);
     }
-    t = cl_block_sum(pp, s_w);
-    if (tid == 0) s_part[1] = t;
-    cl_sync();  // the new vector complete everywhere, partials of beta ready
-    const double ps = cl_gather_sum(&s_part[1], ncta);
-    const double b = sqrt(ps);
-    if (rank == 0 && tid == 0) {
-      lz.alpha[k] = a;
-      lz.beta[k] = b;
+    cl_put(pp, s_slot[1], rank, ncta);
+    cl_sync();  // the new vector complete everywhere, sums of beta in their slots
+    if (tid < 32) {
+      const double ps = cl_take(s_slot[1], ncta);
+      double b, sn;
+      if (ps >= 2.2250738585072014e-308 && ps <= 1.7976931348623157e308) {
+        cl_sqrt(ps, b, sn);
+      } else {  // zero, subnormal, infinite or NaN
+        b = sqrt(ps);
+        sn = 1.0 / b;
+      }
+      if (tid == 0) {
+        const bool stop = !(b > brk * fmax(1.0, fabs(a)));
+        s_done = stop ? 1 : 0;
+        s_sc[1] = sn;
+        s_sc[2] = b * sg;
+        if (rank == 0) {
+          lz.alpha[k] = a;
+          lz.beta[k] = b;
+          if (!stop) lz.sig[k + 1] = sn;
+        }
+      }
     }
-    if (!(b > brk * fmax(1.0, fabs(a)))) {
+    __syncthreads();
+    if (s_done) {
       done = 1;
     } else {
-      const double sn = 1.0 / b;
-      c1 = sn;
-      c2 = b * sg;
-      sg = sn;
-      if (rank == 0 && tid == 0) lz.sig[k + 1] = sn;
+      c1 = s_sc[1];
+      c2 = s_sc[2];
+      sg = c1;
       cur_a = !cur_a;
     }
   }
@@ -771,6 +880,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_lz_cl(const SpinDev md, LzDev
 
 constexpr int kClCtas = 16;       // CTAs per cluster (non-portable size; 8 if 16 cannot launch)
 constexpr int64_t kClMaxDim = 32768;
+constexpr int kClSmem = 190000;   // dynamic shared memory of a CTA (besides ~26 KB static)
 
 }  // namespace
 
@@ -778,13 +888,16 @@ constexpr int64_t kClMaxDim = 32768;
 size_t lz_cta_smem(const SpinDev& md) {
   if (md.dim > kClMaxDim) return 0;
   const int64_t R = (md.dim + kClCtas - 1) / kClCtas;
-  return 2 * sizeof(double) * (size_t)R;
+  return 3 * sizeof(double) * (size_t)R;
 }
 
 Status launch_lz_cta(const SpinDev& md, const LzDev& lz, int steps, double brk, const double* C0, cudaStream_t st) {
   for (int cs : {kClCtas, 8}) {
     const int R = (int)((md.dim + cs - 1) / cs);
-    const size_t smem = 2 * sizeof(double) * (size_t)R;
+    // two slices and the diagonal, a count and `cap` list slots per row
+    const size_t fixed = (3 * sizeof(double) + 1) * (size_t)R;
+    const int cap = (int)std::max<int64_t>(0, std::min<int64_t>(md.n_entries, ((int64_t)kClSmem - (int64_t)fixed) / (4 * (int64_t)R)));
+    const size_t smem = fixed + 4 * (size_t)cap * (size_t)R;
     HPHI_CUDA_TRY(cudaFuncSetAttribute(k_lz_cl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (cs > 8) HPHI_CUDA_TRY(cudaFuncSetAttribute(k_lz_cl, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
@@ -804,7 +917,7 @@ Status launch_lz_cta(const SpinDev& md, const LzDev& lz, int steps, double brk, 
       cudaGetLastError();
       continue;
     }
-    HPHI_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_lz_cl, md, lz, steps, brk, C0, R, cs));
+    HPHI_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_lz_cl, md, lz, steps, brk, C0, R, cs, cap));
     return {};
   }
   return {HPHI_ERR_CUDA, "one-cluster Lanczos: no cluster of 16 or 8 CTAs can be scheduled"};

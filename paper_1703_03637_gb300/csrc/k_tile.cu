@@ -413,13 +413,14 @@ Status launch_s(const SpinDev& md, const TilePlan& plan, const void* v, void* w,
 
 // Covers the flip masks by site sets of at most t sites: the set grows by the mask that covers
 // most new masks per added site (ties: the one whose new sites fewest masks touch, which walks
-// chains from their ends), until none fits.  False when more than kMaxPasses sets, more than
-// kTileMaxEntries entries in one, or a mask wider than t sites.
+// chains from their ends), those that touch the set first, until none fits.  False when more than kMaxPasses sets, more than
+// kTileMaxEntries entries in one, or a mask wider than t sites; below 13 sites no block of vectors
+// has enough tiles (tile_choose).
 bool batch_tile_plan(int n_sites, int t, const std::vector<SpinEntry>& ents, const std::vector<double2>& cls, TileHost* out) {
   out->ents.clear();
   out->dep.clear();
   out->n_pass = 0;
-  if (t < 7 || t > 10 || t > n_sites || n_sites > 32 || ents.empty() || (int)ents.size() > 512) return false;
+  if (t < 8 || t > 10 || n_sites < 13 || n_sites > 32 || ents.empty() || (int)ents.size() > 512) return false;
   auto pc = [](uint64_t x) { return __builtin_popcountll(x); };
   std::vector<int> pass_of(ents.size(), -1);
   size_t left = ents.size();
@@ -432,20 +433,22 @@ bool batch_tile_plan(int n_sites, int t, const std::vector<SpinEntry>& ents, con
       uint64_t bU = 0;
       int cov0 = 0;
       for (size_t k = 0; k < ents.size(); ++k) cov0 += pass_of[k] < 0 && (ents[k].mask & ~S) == 0;
-      for (size_t k = 0; k < ents.size(); ++k) {
-        const uint64_t U = S | ents[k].mask;
-        if (pass_of[k] >= 0 || U == S || pc(U) > t) continue;
-        int cov = 0, deg = 0;
-        for (size_t j = 0; j < ents.size(); ++j)
-          if (pass_of[j] < 0) {
-            cov += (ents[j].mask & ~U) == 0;
-            deg += (ents[j].mask & U & ~S) != 0;
+      for (int near = S ? 1 : 0; near >= 0 && bg < 0.0; --near) {
+        for (size_t k = 0; k < ents.size(); ++k) {
+          const uint64_t U = S | ents[k].mask;
+          if (pass_of[k] >= 0 || U == S || pc(U) > t || (near && !(ents[k].mask & S))) continue;
+          int cov = 0, deg = 0;
+          for (size_t j = 0; j < ents.size(); ++j)
+            if (pass_of[j] < 0) {
+              cov += (ents[j].mask & ~U) == 0;
+              deg += (ents[j].mask & U & ~S) != 0;
+            }
+          const double gain = (double)(cov - cov0) / (pc(U) - pc(S));
+          if (gain > bg || (gain == bg && deg < bd)) {
+            bg = gain;
+            bd = deg;
+            bU = U;
           }
-        const double gain = (double)(cov - cov0) / (pc(U) - pc(S));
-        if (gain > bg || (gain == bg && deg < bd)) {
-          bg = gain;
-          bd = deg;
-          bU = U;
         }
       }
       if (bg < 0.0) break;
@@ -525,7 +528,7 @@ bool batch_tile_plan(int n_sites, int t, const std::vector<SpinEntry>& ents, con
 
 bool tile_applies(const SpinDev& md, int prec, bool cplx, int nvec, Epi epi) {
   const int esz = (prec == HPHI_FP64 ? 8 : 4) * (cplx ? 2 : 1);
-  return md.sector == 0 && md.n_sites >= 7 && md.n_sites <= 32 && nvec >= 2 && (nvec & (nvec - 1)) == 0 &&
+  return md.sector == 0 && md.n_sites >= 13 && md.n_sites <= 32 && nvec >= 2 && (nvec & (nvec - 1)) == 0 &&
          nvec <= kMaxNvec && nvec * esz >= 64 && (epi == Epi::kStore || epi == Epi::kTpq);
 }
 
@@ -545,8 +548,8 @@ const TilePlan* tile_choose(const TilePlan* plans, const SpinDev& md, int prec, 
   const int esz = (prec == HPHI_FP64 ? 8 : 4) * (cplx ? 2 : 1);
   const TilePlan* best = nullptr;
   double bc = 1e30;
-  for (int t = 7; t <= 10; ++t) {
-    const TilePlan& pl = plans[t - 7];
+  for (int t = 8; t <= 10; ++t) {
+    const TilePlan& pl = plans[t - 8];
     if (pl.n_pass == 0 || (16 << (12 - t)) > nvec * esz) continue;
     if (prec == HPHI_FP64 && pl.max_run > 127) continue;  // the exact-integer limit
     if (tile_count(md, t, nvec, esz) < 2 * num_sms()) continue;

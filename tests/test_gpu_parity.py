@@ -1272,3 +1272,49 @@ def test_hubbard_down_pass_pieces(n, nu, nd, offset):
             m.apply_H(x, w)
             assert _rel(w.cpu().numpy(), ref) < tol
             m.autotune(prec)
+
+
+# ----------------------------------------------------------------------------- one-cluster Lanczos lists
+def _xyz_classes(n, values):
+    """Full-basis ring whose bonds take `values` exchange couplings in turn, with a transverse field."""
+    cp = [(i, (i + 1) % n, np.diag([values[i % len(values)]] * 2 + [0.5])) for i in range(n)]
+    return wl.ModelSpec(kind=wl.SPIN, n_sites=n, couplings=cp, fields=[(i, (0.25, 0.0, 0.1)) for i in range(n)],
+                        name=f"xyz_{n}_{len(values)}")
+
+
+@pytest.mark.parametrize("mk", [
+    lambda: _xyz_classes(6, [1.0]), lambda: _xyz_classes(9, [1.0, 0.7]), lambda: _xyz_classes(8, [1.0, 0.7, -0.3, 2.0, 0.9]),
+    lambda: wl.heisenberg_ring(15), lambda: wl.j1j2_ring(14).with_basis(wl.BASIS_SZ, 7),
+    lambda: wl.random_spin_model(15, 100, seed=5, complex_=False), lambda: wl.heisenberg_ring(3),
+], ids=["64-rows", "two-values", "six-values-no-list", "32768-rows", "sector", "many-terms", "8-rows"])
+def test_one_cluster_lanczos_lists(mk):
+    """The per-row gather lists (few coefficients, room for every term) and the decoding path they
+    give way to, from fewer rows than CTAs to the largest problem; eigenvalues for n_eig = 1 and 8
+    against LAPACK on the device's own T."""
+    spec = mk()
+    m = hp.Model.from_spec(spec)
+    v0 = wl.gaussian_vector(61, m.dim)[:, 0]
+    a, b = oracle.lanczos(spec, v0, 12)
+    for n_eig in (1, 8):
+        r = m.lanczos(12, v0=torch.as_tensor(v0), n_eig=n_eig)
+        n = min(len(a), r["steps"])
+        assert _rel(r["alpha"][:n], a[:n]) < 1e-11
+        assert np.max(np.abs(r["beta"][:n] - b[:n])) < 1e-11 * np.max(np.abs(a))
+        k = r["steps"]
+        want = np.linalg.eigvalsh(np.diag(r["alpha"]) + np.diag(r["beta"][:k - 1], 1) + np.diag(r["beta"][:k - 1], -1))
+        got = r["eig"][:min(n_eig, k)]
+        assert np.max(np.abs(got - want[:len(got)])) <= 1e-13 * np.max(np.abs(want))
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-90, 1e90])
+def test_ritz_values_at_any_scale(scale):
+    """The Sturm counts work on T scaled below one: couplings as far from one
+    as the unnormalised recurrence takes (its <C, H C> is of the order of the coupling cubed)."""
+    spec = wl.heisenberg_ring(10, J=scale)
+    m = hp.Model.from_spec(spec)
+    v0 = wl.gaussian_vector(62, m.dim)[:, 0]
+    r = m.lanczos(9, v0=torch.as_tensor(v0), n_eig=4, breakdown=1e-300)
+    k = r["steps"]
+    al, be = r["alpha"] / scale, r["beta"][:k - 1] / scale
+    want = np.linalg.eigvalsh(np.diag(al) + np.diag(be, 1) + np.diag(be, -1))
+    assert np.max(np.abs(r["eig"][:min(4, k)] / scale - want[:4])) <= 1e-13 * np.max(np.abs(want))
