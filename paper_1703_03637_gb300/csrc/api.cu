@@ -115,7 +115,7 @@ struct hphi_model {
   std::string err;
   int device = 0;
   // device data
-  DBuf d_entries, d_cls, d_lin, d_pairs, d_pcoef, d_hi_off, d_lo_rank, d_lo_list, d_lo_off;
+  DBuf d_entries, d_merged, d_cls, d_lin, d_pairs, d_pcoef, d_hi_off, d_lo_rank, d_lo_list, d_lo_off;
   DBuf d_nbr_up, d_deg_up, d_nbr_dn, d_deg_dn, d_npos_up, d_npos_dn, d_counter;
   DBuf d_up_rec[3], d_up_hdr[3];  // pass U gather tables by entry width
   hphi::SpinDev sdev{};
@@ -304,6 +304,37 @@ hphi::Status compile_spin(hphi_model* m, cudaStream_t st) {
     run = (k > 0 && ents[k].cls == ents[k - 1].cls) ? run + 1 : 1;
     max_run = std::max(max_run, (int)run);
   }
+  // entries of one mask and site pair with disjoint patterns, two by two, sorted by class pair
+  std::vector<hphi::SpinMerged> merged;
+  {
+    std::vector<char> used(ents.size(), 0);
+    auto live = [](const hphi::SpinEntry& e, int sel) { return ((e.phases >> (3 * sel)) & 7) != 0; };
+    std::map<std::array<uint64_t, 2>, std::vector<size_t>> same;  // by mask and sites
+    for (size_t k = 0; k < ents.size(); ++k) same[{ents[k].mask, (uint64_t)ents[k].i | ((uint64_t)ents[k].j << 8)}].push_back(k);
+    for (size_t k = 0; k < ents.size(); ++k) {
+      if (used[k]) continue;
+      used[k] = 1;
+      const hphi::SpinEntry& x = ents[k];
+      hphi::SpinMerged e{x.mask, (uint32_t)x.cls | 0xffff0000u, 0, x.i, x.j};
+      const hphi::SpinEntry* y = nullptr;
+      for (size_t o : same[{x.mask, (uint64_t)x.i | ((uint64_t)x.j << 8)}]) {
+        bool fits = !used[o] && ents[o].cls != x.cls;
+        for (int sel = 0; sel < 4; ++sel) fits = fits && !(live(x, sel) && live(ents[o], sel));
+        if (!fits) continue;
+        y = &ents[o];
+        used[o] = 1;
+        e.cls = (uint32_t)x.cls | ((uint32_t)y->cls << 16);
+        break;
+      }
+      for (int sel = 0; sel < 4; ++sel) {
+        const int a = (x.phases >> (3 * sel)) & 7, b = y ? (y->phases >> (3 * sel)) & 7 : 0;
+        e.phases |= (uint16_t)((a ? a : b ? b + 8 : 0) << (4 * sel));
+      }
+      merged.push_back(e);
+    }
+    std::stable_sort(merged.begin(), merged.end(),
+                     [](const hphi::SpinMerged& x, const hphi::SpinMerged& y) { return x.cls < y.cls; });
+  }
   std::vector<double2> cls;
   for (const cplx& c : ct.coefs) cls.push_back(make_double2(c.real(), c.imag()));
   // linear groups by value
@@ -333,6 +364,7 @@ hphi::Status compile_spin(hphi_model* m, cudaStream_t st) {
 
   hphi::Status s;
   if ((s = upload(m->d_entries, ents, st)).code) return s;
+  if ((s = upload(m->d_merged, merged, st)).code) return s;
   if ((s = upload(m->d_cls, cls, st)).code) return s;
   if ((s = upload(m->d_lin, lg, st)).code) return s;
   if ((s = upload(m->d_pairs, pe, st)).code) return s;
@@ -342,6 +374,8 @@ hphi::Status compile_spin(hphi_model* m, cudaStream_t st) {
   d.n_sites = N;
   d.sector = sector ? 1 : 0;
   d.n_entries = (int)ents.size();
+  d.n_merged = (int)merged.size();
+  d.merged = m->d_merged.as<hphi::SpinMerged>();
   d.max_run = max_run;
   m->host_entries = ents;
   m->win.clear();

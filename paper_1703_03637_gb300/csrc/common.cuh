@@ -34,6 +34,16 @@ struct SpinEntry {
 };
 static_assert(sizeof(SpinEntry) == 16, "SpinEntry layout");
 
+// Entries of one flip mask and site pair whose bit patterns exclude each other, merged two by two
+// (k_hv_spin): four 4-bit codes by b_i + 2 b_j, the phase code plus 8 for the second class.
+struct SpinMerged {
+  uint64_t mask;
+  uint32_t cls;      // first class | second << 16 (0xffff: none)
+  uint16_t phases;
+  uint8_t i, j;
+};
+static_assert(sizeof(SpinMerged) == 16, "SpinMerged layout");
+
 struct LinGroup {   // coef * popcount(bits & mask)
   uint64_t mask;
   double coef;
@@ -72,6 +82,8 @@ struct SpinDev {
   int n_entries, n_classes, n_lin, n_pairs, n_pair_groups;
   double c0;
   const SpinEntry* entries;  // sorted by class
+  int n_merged;
+  const SpinMerged* merged;  // sorted by their class pair
   const double2* cls_coef;
   const LinGroup* lin;
   const PairEntry* pairs;

@@ -30,41 +30,90 @@ namespace {
 // thread (patterns are sorted by class), so class flushes never diverge.
 constexpr int kBatch = 8;
 
+// largest hi with hi_off[hi] <= r, by one warp (32 probes a round)
+__device__ __forceinline__ uint64_t warp_find_hi(const SectorTables& t, uint64_t r, uint64_t hmax) {
+  const int lane = threadIdx.x & 31;
+  uint64_t lo = 0, hi = hmax;
+  while (lo < hi) {
+    const uint64_t step = (hi - lo + 31) >> 5;
+    const uint64_t m = lo + step * (uint64_t)(lane + 1);
+    const bool in = m <= hi && __ldg(t.hi_off + (m <= hi ? m : hi)) <= r;
+    const int c = __popc(__ballot_sync(0xffffffffu, in));  // hi_off does not decrease
+    lo += step * (uint64_t)c;
+    hi = min(hi, lo + step - 1);
+  }
+  return lo;
+}
+
+//
+// The entries are merged by flip mask (SpinMerged): one gather serves both entries of a bond
+// whose two patterns carry conjugate coefficients, which fall into two classes; a row adds the
+// value to the sums of the one class its bits select.  St is the configuration's type, 32 bits
+// up to 32 sites.
 //
 // QT (fp64): the gathers read the input quantised to 64-bit integers, one scale per vector
 // column (q = round(x 2^(1078 - E_c)), |q| < 2^56), so every class sum of at most 127 terms
 // is an exact integer sum (two integer instructions a term instead of the per-term
 // alignment of the fixed-point accumulator), converted to fp64 once per class.
-template <class S, Epi E, bool QT = false>
-__global__ void __launch_bounds__(kThreads) k_hv_spin(const SpinDev md, const S* __restrict__ v, S* __restrict__ w,
-                                                      int nvec, int lg_nvec, FusedArgs fa,
-                                                      const long long* __restrict__ Q, const int* __restrict__ Ec) {
+//
+// 22-site ring with Dzyaloshinskii-Moriya exchange, S^z = 0 (705,432 rows c128), Lanczos step on
+// GB300: 94 us instead of 173 us (one entry at a time, a binary search by one thread per 256 rows,
+// conversions per class); bound by issue (47 %), the fp64 pipe (37 %) and latency together.
+template <class S, Epi E, bool QT, class St>
+__global__ void __launch_bounds__(kThreads, (Traits<S>::kF64 && !QT) ? 2 : 3) k_hv_spin(const SpinDev md, const S* __restrict__ v, S* __restrict__ w,
+                                                         int nvec, int lg_nvec, FusedArgs fa,
+                                                         const long long* __restrict__ Q, const int* __restrict__ Ec) {
   using R = typename Traits<S>::R;
   static_assert(!QT || Traits<S>::kF64, "quantised gathers are an fp64 path");
   using A = std::conditional_t<QT, IntAcc, typename SumAcc<R>::T>;
   using T = std::conditional_t<QT, long long, R>;  // gathered scalar
   constexpr bool C = Traits<S>::kCplx;
   constexpr bool F64 = Traits<S>::kF64;
-  __shared__ SpinEntry s_ent[kMaxSpinEntries];
-  __shared__ double2 s_cls[kMaxClasses];
-  __shared__ LinGroup s_lin[kMaxLin];
+  __shared__ SpinMerged s_ent[kMaxSpinEntries];
+  __shared__ R s_cr[kMaxClasses], s_ci[kMaxClasses];
+  __shared__ St s_lm[kMaxLin];
+  __shared__ R s_lc[kMaxLin], s_pcoef[kMaxPairGroups];
   __shared__ PairEntry s_pair[kMaxPairs];
-  __shared__ double s_pcoef[kMaxPairGroups];
   __shared__ R s_inv[kMaxNvec];
   __shared__ uint64_t s_hi[2];
-  __shared__ double s_red[(E == Epi::kStore) ? 1 : kThreads * kMaxRedQ];
+  __shared__ double s_red[(E == Epi::kStore) ? 1 : kThreads * (n_red<E>() > 0 ? n_red<E>() : 1)];
 
   if (fa.done != nullptr && *fa.done) return;
   const int tid = threadIdx.x;
-  for (int k = tid; k < md.n_entries; k += kThreads) s_ent[k] = md.entries[k];
-  for (int k = tid; k < md.n_classes; k += kThreads) s_cls[k] = md.cls_coef[k];
-  for (int k = tid; k < md.n_lin; k += kThreads) s_lin[k] = md.lin[k];
+  const int n_ent = md.n_merged;
+  for (int k = tid; k < n_ent; k += kThreads) s_ent[k] = md.merged[k];
+  for (int k = tid; k < md.n_classes; k += kThreads) {
+    const double2 cc = md.cls_coef[k];
+    s_cr[k] = (R)cc.x;
+    s_ci[k] = (R)cc.y;
+  }
+  for (int k = tid; k < md.n_lin; k += kThreads) {
+    s_lm[k] = (St)md.lin[k].mask;
+    s_lc[k] = (R)md.lin[k].coef;
+  }
   for (int k = tid; k < md.n_pairs; k += kThreads) s_pair[k] = md.pairs[k];
-  for (int k = tid; k < md.n_pair_groups; k += kThreads) s_pcoef[k] = md.pair_coef[k];
+  for (int k = tid; k < md.n_pair_groups; k += kThreads) s_pcoef[k] = (R)md.pair_coef[k];
   if constexpr (E == Epi::kTpq) {
     for (int k = tid; k < nvec; k += kThreads) s_inv[k] = (R)fa.scal[k];
   }
   const EpiScalars<R> es = epi_scalars<R, E>(fa);
+  const R c0 = opaque((R)md.c0);
+  // one vector: the fixed point's scale goes into the class coefficients (an exact power of two
+  // unless a product leaves the normal range), so a sum is one conversion and its multiply-adds
+  bool pre = false;
+  if constexpr (QT) {
+    __syncthreads();
+    bool ok = nvec == 1 && Ec[0] >= 1078 - 1022;
+    const double sc = ok ? __longlong_as_double((long long)(Ec[0] - 1078 + 1023) << 52) : 1.0;
+    for (int k = tid; k < md.n_classes; k += kThreads)
+      ok = ok && (s_cr[k] == 0.0 || fabs(s_cr[k] * sc) >= 1e-290) && (s_ci[k] == 0.0 || fabs(s_ci[k] * sc) >= 1e-290);
+    pre = __syncthreads_and(ok ? 1 : 0) != 0;
+    if (pre)
+      for (int k = tid; k < md.n_classes; k += kThreads) {
+        s_cr[k] *= sc;
+        s_ci[k] *= sc;
+      }
+  }
   __syncthreads();
 
   constexpr int kNQ = n_red<E>() > 0 ? n_red<E>() : 1;
@@ -73,7 +122,8 @@ __global__ void __launch_bounds__(kThreads) k_hv_spin(const SpinDev md, const S*
   const int64_t total = md.dim * (int64_t)nvec;
   __shared__ int64_t s_item;
   const uint64_t hmax = md.sector ? ((1ull << md.t.H) - 1ull) : 0ull;
-  const int n_ent = md.n_entries;
+  const int tL = md.t.L;
+  const St lomask = (St)(((uint64_t)1 << tL) - 1);
 
   // plain H v: chunks of kThreads elements are handed out in order from a counter, so
   // resident CTAs stay on neighbouring rows and share the rows they gather through L2.
@@ -102,47 +152,99 @@ __global__ void __launch_bounds__(kThreads) k_hv_spin(const SpinDev md, const S*
       r = idx / nvec;
       c = (int)(idx - r * nvec);
     }
-    uint64_t s = (uint64_t)r;
+    uint64_t s64 = (uint64_t)r;
     if (md.sector) {
       __syncthreads();
-      if (tid == 0) s_hi[0] = sector_find_hi(md.t, (uint64_t)(base / nvec), 0, hmax);
-      if (tid == 1) {
-        const int64_t last = (base + kThreads < total ? base + kThreads : total) - 1;
-        s_hi[1] = sector_find_hi(md.t, (uint64_t)(last / nvec), 0, hmax);
+      if (tid < 64) {  // warp 0: the first row's high part, warp 1: the last row's
+        const int64_t e = tid < 32 ? base : (base + kThreads < total ? base + kThreads : total) - 1;
+        const uint64_t f = warp_find_hi(md.t, (uint64_t)(e / nvec), hmax);
+        if ((tid & 31) == 0) s_hi[tid >> 5] = f;
       }
       __syncthreads();
-      if (act) s = sector_state_in(md.t, (uint64_t)r, sector_find_hi(md.t, (uint64_t)r, s_hi[0], s_hi[1]));
+      if (act) s64 = sector_state_in(md.t, (uint64_t)r, sector_find_hi(md.t, (uint64_t)r, s_hi[0], s_hi[1]));
     }
     if (!act) continue;
+    const St s = (St)s64;
+    auto pop = [](St x) -> int {
+      if constexpr (sizeof(St) == 4) return __popc(x);
+      else return __popcll(x);
+    };
 
     // diagonal: integer bit counts per coefficient class
-    R d = (R)md.c0;
-    for (int g = 0; g < md.n_lin; ++g) d += (R)s_lin[g].coef * (R)__popcll(s & s_lin[g].mask);
+    R d = c0;
+    for (int g = 0; g < md.n_lin; ++g) d += s_lc[g] * (R)pop(s & s_lm[g]);
     if (md.n_pairs) {
       int grp = s_pair[0].grp, cnt = 0;
       for (int p = 0; p < md.n_pairs; ++p) {
         const PairEntry pe = s_pair[p];
         if (pe.grp != grp) {
-          d += (R)s_pcoef[grp] * (R)cnt;
+          d += s_pcoef[grp] * (R)cnt;
           cnt = 0;
           grp = pe.grp;
         }
-        cnt += (int)((s >> pe.i) & (s >> pe.j) & 1ull);
+        cnt += (int)((s >> pe.i) & (s >> pe.j) & (St)1);
       }
-      d += (R)s_pcoef[grp] * (R)cnt;
+      d += s_pcoef[grp] * (R)cnt;
     }
     R sr, si;
     ld<S>(v, idx, sr, si);
     R hr = d * sr, hi = d * si;
     const int eoff = QT ? Ec[c] - 1078 : 0;
 
-    A ar, ai;
-    ar.zero();
-    ai.zero();
-    int cur = n_ent ? s_ent[0].cls : 0;
+    A ar[2], ai[2];  // the sums of the two classes
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      ar[q].zero();
+      ai[q].zero();
+    }
+    uint32_t cur = n_ent ? s_ent[0].cls : 0u;
+    auto flush = [&]() {
+      if constexpr (QT && C) {
+        // the two patterns of a complex exchange: a + i b and, in its quadrant, b + i a =
+        // i (a - i b); their sums meet as integers, half the conversions' multiply-adds
+        const int p = (int)(cur & 0xffffu), o = (int)(cur >> 16);
+        if (pre && o != 0xffff && md.max_run <= 63 && s_cr[o] == s_ci[p] && s_ci[o] == s_cr[p]) {
+          const double a = s_cr[p], b = s_ci[p];
+          hr = fma(a, __ll2double_rn(ar[0].s - ai[1].s), fma(b, __ll2double_rn(ar[1].s - ai[0].s), hr));
+          hi = fma(a, __ll2double_rn(ai[0].s + ar[1].s), fma(b, __ll2double_rn(ar[0].s + ai[1].s), hi));
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            ar[q].zero();
+            ai[q].zero();
+          }
+          return;
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int cls = q ? (int)(cur >> 16) : (int)(cur & 0xffffu);
+        if (q && cls == 0xffff) break;  // no second class
+        const R cx = s_cr[cls], cy = s_ci[cls];
+        R vr, vi;
+        if constexpr (QT) {
+          vr = pre ? __ll2double_rn(ar[q].value()) : fix_to_double(ar[q].value(), eoff);
+          vi = !C ? 0.0 : pre ? __ll2double_rn(ai[q].value()) : fix_to_double(ai[q].value(), eoff);
+        } else {
+          vr = (R)ar[q].value();
+          vi = (R)ai[q].value();
+        }
+        if constexpr (C) {
+          hr += cx * vr;
+          hi += cx * vi;
+          if (cy != R(0)) {
+            hr -= cy * vi;
+            hi += cy * vr;
+          }
+        } else {
+          hr += cx * vr;
+        }
+        ar[q].zero();
+        ai[q].zero();
+      }
+    };
     for (int e0 = 0; e0 < n_ent; e0 += kBatch) {
       T xr[kBatch], xi[kBatch];
-      int code[kBatch];
+      int code[kBatch];  // phase, plus 8 for the second class
 #pragma unroll
       for (int j = 0; j < kBatch; ++j) {
         const int k = e0 + j;
@@ -150,12 +252,13 @@ __global__ void __launch_bounds__(kThreads) k_hv_spin(const SpinDev md, const S*
         xr[j] = 0;
         xi[j] = 0;
         if (k < n_ent) {
-          const SpinEntry en = s_ent[k];
-          const int sel = (int)((s >> en.i) & 1ull) | ((int)((s >> en.j) & 1ull) << 1);
-          code[j] = (en.phases >> (3 * sel)) & 7;
+          const SpinMerged en = s_ent[k];
+          const int sel = (int)((s >> en.i) & (St)1) | ((int)((s >> en.j) & (St)1) << 1);
+          code[j] = (int)((en.phases >> (4 * sel)) & 15u);
           if (code[j]) {
-            const uint64_t s2 = s ^ en.mask;
-            const uint64_t r2 = md.sector ? sector_rank(md.t, s2) : s2;
+            const St s2 = s ^ (St)en.mask;
+            uint64_t r2 = (uint64_t)s2;
+            if (md.sector) r2 = __ldg(md.t.hi_off + (s2 >> tL)) + (uint64_t)__ldg(md.t.lo_rank + (s2 & lomask));
             if constexpr (QT) {
               const int64_t o = (int64_t)r2 * nvec + c;
               if constexpr (C) {
@@ -175,51 +278,22 @@ __global__ void __launch_bounds__(kThreads) k_hv_spin(const SpinDev md, const S*
       for (int j = 0; j < kBatch; ++j) {
         const int k = e0 + j;
         if (k < n_ent) {
-          const int cls = s_ent[k].cls;
-          if (cls != cur) {
-            const double2 cc = s_cls[cur];
-            R vr, vi;
-            if constexpr (QT) {
-              vr = fix_to_double(ar.value(), eoff);
-              vi = C ? fix_to_double(ai.value(), eoff) : 0.0;
-            } else {
-              vr = (R)ar.value();
-              vi = (R)ai.value();
-            }
-            if constexpr (C) {
-              hr += (R)cc.x * vr - (R)cc.y * vi;
-              hi += (R)cc.x * vi + (R)cc.y * vr;
-            } else {
-              hr += (R)cc.x * vr;
-            }
-            ar.zero();
-            ai.zero();
+          const uint32_t cls = s_ent[k].cls;
+          if (cls != cur) {  // the entries are shared: the same for all threads
+            flush();
             cur = cls;
           }
-          if (code[j]) {
-            if constexpr (C) acc_phase<A, T>(code[j], xr[j], xi[j], ar, ai);
-            else ar.add(xr[j], code[j] != 1);
+          if (code[j] & 8) {
+            if constexpr (C) acc_phase<A, T>(code[j] & 7, xr[j], xi[j], ar[1], ai[1]);
+            else ar[1].add(xr[j], code[j] != 9);
+          } else if (code[j]) {
+            if constexpr (C) acc_phase<A, T>(code[j], xr[j], xi[j], ar[0], ai[0]);
+            else ar[0].add(xr[j], code[j] != 1);
           }
         }
       }
     }
-    if (n_ent) {
-      const double2 cc = s_cls[cur];
-      R vr, vi;
-      if constexpr (QT) {
-        vr = fix_to_double(ar.value(), eoff);
-        vi = C ? fix_to_double(ai.value(), eoff) : 0.0;
-      } else {
-        vr = (R)ar.value();
-        vi = (R)ai.value();
-      }
-      if constexpr (C) {
-        hr += (R)cc.x * vr - (R)cc.y * vi;
-        hi += (R)cc.x * vi + (R)cc.y * vr;
-      } else {
-        hr += (R)cc.x * vr;
-      }
-    }
+    if (n_ent) flush();
     epilogue<S, E, kNQ>(idx, sr, si, hr, hi, w, fa, es, E == Epi::kTpq ? s_inv[c] : R(0), red);
   }
   if constexpr (E != Epi::kStore) block_finish<F64, kThreads, kNQ>(red, n_red<E>(), nvec, fa.partials, s_red);
@@ -468,7 +542,7 @@ int occupancy_t(bool hub) {
   if (b == 0) {
     int n = 0;
     cudaError_t e = hub ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_hv_hub<S, E>, kThreads, 0)
-                        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_hv_spin<S, E>, kThreads, 0);
+                        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_hv_spin<S, E, Traits<S>::kF64, uint32_t>, kThreads, 0);
     if (e != cudaSuccess || n < 1) {
       cudaGetLastError();
       n = 2;
@@ -500,22 +574,26 @@ Status launch_t(bool hub, const void* md, const void* v, void* w, int nvec, cons
                                              reinterpret_cast<S*>(w), nvec, lg, fa);
   } else {
     const SpinDev& sd = *reinterpret_cast<const SpinDev*>(md);
-    bool qt = false;
+    const S* vs = reinterpret_cast<const S*>(v);
+    S* ws = reinterpret_cast<S*>(w);
+    const bool narrow = sd.n_sites <= 32;
+    long long* q = nullptr;
+    int* e = nullptr;
     if constexpr (Traits<S>::kF64) {
       if (spin_quantised(sd, HPHI_FP64, nvec) && scratch != nullptr) {
         constexpr int ncomp = Traits<S>::kCplx ? 2 : 1;
-        long long* q = reinterpret_cast<long long*>(scratch);
-        int* e = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(scratch) + (size_t)sd.dim * nvec * sizeof(S));
+        q = reinterpret_cast<long long*>(scratch);
+        e = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(scratch) + (size_t)sd.dim * nvec * sizeof(S));
         Status qs = launch_quant_cols(reinterpret_cast<const double*>(v), sd.dim, nvec, ncomp, q, e, st);
         if (qs.code) return qs;
-        k_hv_spin<S, E, true><<<grid, kThreads, 0, st>>>(sd, reinterpret_cast<const S*>(v), reinterpret_cast<S*>(w),
-                                                         nvec, lg, fa, q, e);
-        qt = true;
+        if (narrow) k_hv_spin<S, E, true, uint32_t><<<grid, kThreads, 0, st>>>(sd, vs, ws, nvec, lg, fa, q, e);
+        else k_hv_spin<S, E, true, uint64_t><<<grid, kThreads, 0, st>>>(sd, vs, ws, nvec, lg, fa, q, e);
       }
     }
-    if (!qt)
-      k_hv_spin<S, E><<<grid, kThreads, 0, st>>>(sd, reinterpret_cast<const S*>(v), reinterpret_cast<S*>(w), nvec, lg,
-                                                fa, nullptr, nullptr);
+    if (q == nullptr) {
+      if (narrow) k_hv_spin<S, E, false, uint32_t><<<grid, kThreads, 0, st>>>(sd, vs, ws, nvec, lg, fa, q, e);
+      else k_hv_spin<S, E, false, uint64_t><<<grid, kThreads, 0, st>>>(sd, vs, ws, nvec, lg, fa, q, e);
+    }
   }
   HPHI_CUDA_TRY(cudaGetLastError());
   return {};

@@ -1318,3 +1318,35 @@ def test_ritz_values_at_any_scale(scale):
     al, be = r["alpha"] / scale, r["beta"][:k - 1] / scale
     want = np.linalg.eigvalsh(np.diag(al) + np.diag(be, 1) + np.diag(be, -1))
     assert np.max(np.abs(r["eig"][:min(4, k)] / scale - want[:4])) <= 1e-13 * np.max(np.abs(want))
+
+
+# ----------------------------------------------------------------------------- merged entries of the generic kernel
+def _dm_ring(n, n_up, two=False):
+    """S^z-conserving ring with complex exchange: a bond's two patterns carry conjugate
+    coefficients (one merged entry); two: another coupling on every third bond."""
+    def J(a, b):
+        return np.array([[a, b, 0.0], [-b, a, 0.0], [0.0, 0.0, 0.7]])
+    cp = [(i, (i + 1) % n, J(0.5, -0.2) if two and i % 3 == 0 else J(1.0, 0.3)) for i in range(n)]
+    return wl.ModelSpec(kind=wl.SPIN, n_sites=n, couplings=cp, fields=[(i, (0.0, 0.0, 0.1 * (i % 2))) for i in range(n)],
+                        name=f"dm_ring_{n}").with_basis(wl.BASIS_SZ, n_up)
+
+
+@pytest.mark.parametrize("mk,nvec", [
+    (lambda: _dm_ring(14, 7), 1), (lambda: _dm_ring(15, 5, True), 3), (lambda: _dm_ring(34, 3), 1),
+    (lambda: _dm_ring(33, 2, True), 2), (lambda: wl.random_xxz_model(34, 40, seed=12).with_basis(wl.BASIS_SZ, 3), 1),
+    (lambda: wl.random_spin_model(10, 16, seed=13), 2), (lambda: _dm_ring(12, 0), 1), (lambda: _dm_ring(12, 1), 1),
+], ids=["dm14", "dm15-two", "dm34", "dm33-two", "xxz34", "full", "one-row", "twelve-rows"])
+def test_generic_merged_entries(mk, nvec):
+    """Products and Lanczos steps of the generic kernel: configurations of up to and above 32
+    bits, one and several class pairs, fewer rows than a chunk."""
+    spec = mk()
+    m = hp.Model.from_spec(spec)
+    v = wl.gaussian_vector(171, m.dim, nvec, complex_=m.is_complex)
+    ref = oracle.apply_H(spec, v)
+    ref = ref if m.is_complex else ref.real
+    for prec, tol in ((hp.FP64, 1e-12), (hp.FP32, 2e-5)):
+        assert _rel(m.apply_H(_to_dev(m, v, prec)).cpu().numpy(), ref) < tol
+        if m.dim > 12:
+            a, b = oracle.lanczos(spec, v[:, 0], 4)
+            r = m.lanczos(4, prec=prec, v0=torch.as_tensor(v[:, 0]))
+            assert _rel(r["alpha"], a) < tol and _rel(r["beta"], b) < tol
