@@ -1630,10 +1630,12 @@ hphi::Status lz_enqueue(LzPlan& L, cudaStream_t st) {
       if ((q = hphi::launch_lz_fin1(L.lz, k, L.partials, L.grid, st)).code) return q;
       hphi::QNext qn{};
       if (qnext) {
-        // the exact exponent of C_k: k_maxexp's slot (the copy's) at k = 0, else the one the
-        // previous pass 2 found; this pass 2 finds C_{k+1}'s into the other slot
+        // the exact exponent of C_k: at k = 0 k_maxexp's, moved out of the copy's slot because
+        // pass 2 overwrites that one while its CTAs read the exponent, else the one the previous
+        // pass 2 found; this pass 2 finds C_{k+1}'s into the other slot
         emax = qs.ec[(k + 1) & 1];
-        qn = hphi::QNext{qs.Q, qs.eq, qs.ep, k == 0 ? qs.eq : qs.ec[k & 1], qs.extra};
+        if (k == 0) HPHI_CUDA_TRY(cudaMemcpyAsync(qs.ec[0], qs.eq, sizeof(int), cudaMemcpyDeviceToDevice, st));
+        qn = hphi::QNext{qs.Q, qs.eq, qs.ep, qs.ec[k & 1], qs.extra};
         HPHI_CUDA_TRY(cudaMemsetAsync(emax, 0, sizeof(int), st));
       }
       if ((q = hphi::launch_lz_pass2(prec, cplx, L.lz, k, C, P, with_x ? ws.x.as<double>() : nullptr, L.n_real,
@@ -2048,7 +2050,8 @@ hphi::Status invit_impl(hphi_model* m, const hphi_invit_params* p, void* xv, hph
   for (DBuf* b : {&ws.vecA, &ws.vecB, &ws.cgp, &ws.cgq})
     if ((s = b->ensure(vb)).code) return s;
   void* scratch = nullptr;
-  const size_t need = hv_scratch_bytes(m, HPHI_FP64, 1, hphi::Epi::kStore);
+  const size_t need = std::max(hv_scratch_bytes(m, HPHI_FP64, 1, hphi::Epi::kStore),
+                               hv_scratch_bytes(m, HPHI_FP64, 1, hphi::Epi::kRefine));
   if (need && m->kind == HPHI_SPIN_HALF) {
     scratch = optional_scratch(m, need);
   } else if (need) {
@@ -2056,8 +2059,18 @@ hphi::Status invit_impl(hphi_model* m, const hphi_invit_params* p, void* xv, hph
     scratch = ws.work.p;
   }
   const int grid = hv_grid_for(m, 1, HPHI_FP64, hphi::Epi::kStore);
+  const int rgrid = hv_grid_for(m, 1, HPHI_FP64, hphi::Epi::kRefine);
   const int vgrid = launch_grid(n);
-  if ((s = ws.partials.ensure(sizeof(double) * (size_t)vgrid * hphi::kMaxRedQ)).code) return s;
+  if ((s = ws.partials.ensure(sizeof(double) * (size_t)std::max(rgrid, vgrid) * hphi::kMaxRedQ)).code) return s;
+  // fixed-point paths: the slots through which the direction kernel hands the product its copy
+  hphi::QSlots qs;
+  if (scratch != nullptr && !cplx) {
+    if (use_hub_fast(m, HPHI_FP64, 1, hphi::Epi::kRefine))
+      qs = hphi::hub_qslots(m->hdev, scratch);
+    else if (sec_runs(m, HPHI_FP64, 1, hphi::Epi::kRefine, ws.work.bytes))
+      qs = hphi::sec_qslots(*use_sec(m, HPHI_FP64, 1, hphi::Epi::kRefine), HPHI_FP64, hphi::Epi::kRefine, scratch);
+  }
+  const bool qnext = qs.Q != nullptr;
   if ((s = ws.scal.ensure(sizeof(double) * 18)).code) return s;
   hphi::CgDev cg;
   cg.s = ws.scal.as<double>();
@@ -2083,26 +2096,33 @@ hphi::Status invit_impl(hphi_model* m, const hphi_invit_params* p, void* xv, hph
   hphi::FusedArgs plain;  // H v without a flag
   hphi::FusedArgs flagged;
   flagged.done = cg.done;  // H p of a solve that has converged is skipped
+  flagged.partials = partials;
   const int hvk = hv_kernels(m, HPHI_FP64, 1, hphi::Epi::kStore);
+  const int hvr = hv_kernels(m, HPHI_FP64, 1, hphi::Epi::kRefine);
   int done_h = 0;
   for (int outer = 0; outer < p->outer; ++outer) {
     HPHI_CUDA_TRY(cudaMemsetAsync(cg.done, 0, sizeof(int), st));
     // start: y = b, r = b - A b, p = r
     plain.out = q;
     if ((s = hv_launch(m, HPHI_FP64, x, q, 1, hphi::Epi::kStore, plain, grid, scratch, st)).code) return s;
-    if ((s = hphi::launch_cg_shift(cg, x, q, n, partials, vgrid, st)).code) return s;
-    if ((s = hphi::launch_cg_update(cg, 0, x, y, rr, pp, q, n, partials, vgrid, st)).code) return s;
-    if ((s = hphi::launch_cg_fin(cg, 0, partials, vgrid, st)).code) return s;
-    launches += hvk + 3;
+    if ((s = hphi::launch_cg_update(cg, 0, x, y, rr, pp, q, n, partials, vgrid, nullptr, st)).code) return s;
+    if ((s = hphi::launch_cg_fin(cg, 0, partials, vgrid, nullptr, st)).code) return s;
+    launches += hvk + 2;
     for (int it = 0; it < p->max_cg; ++it) {
+      // H p with <p, H p> and <p, p>; from the second iteration on the quantised copy is ready
       flagged.out = q;
-      if ((s = hv_launch(m, HPHI_FP64, pp, q, 1, hphi::Epi::kStore, flagged, grid, scratch, st)).code) return s;
-      if ((s = hphi::launch_cg_shift(cg, pp, q, n, partials, vgrid, st)).code) return s;
-      if ((s = hphi::launch_cg_fin(cg, 1, partials, vgrid, st)).code) return s;
-      if ((s = hphi::launch_cg_update(cg, 1, nullptr, y, rr, pp, q, n, partials, vgrid, st)).code) return s;
-      if ((s = hphi::launch_cg_fin(cg, 2, partials, vgrid, st)).code) return s;
-      if ((s = hphi::launch_cg_dir(cg, rr, pp, n, vgrid, st)).code) return s;
-      launches += hvk + 5;
+      flagged.exp_ready = qnext && it > 0 ? 2 : 0;
+      if ((s = hv_launch(m, HPHI_FP64, pp, nullptr, 1, hphi::Epi::kRefine, flagged, rgrid, scratch, st)).code) return s;
+      if ((s = hphi::launch_cg_fin(cg, 1, partials, rgrid, qs.ep, st)).code) return s;
+      if ((s = hphi::launch_cg_update(cg, 1, nullptr, y, rr, pp, q, n, partials, vgrid, qs.ep, st)).code) return s;
+      int* ec_new = qnext ? qs.ec[(it + 1) & 1] : nullptr;
+      if ((s = hphi::launch_cg_fin(cg, 2, partials, vgrid, ec_new, st)).code) return s;
+      // E_p: the first product's scan left it in the copy's slot, which the direction kernel
+      // overwrites, so it is moved first; later what that kernel found
+      if (qnext && it == 0) HPHI_CUDA_TRY(cudaMemcpyAsync(qs.ec[0], qs.eq, sizeof(int), cudaMemcpyDeviceToDevice, st));
+      hphi::QNext qn{qs.Q, qs.eq, qs.ep, qs.ec[it & 1], qs.extra};
+      if ((s = hphi::launch_cg_dir(cg, rr, pp, n, vgrid, qnext ? &qn : nullptr, ec_new, st)).code) return s;
+      launches += hvr + 4 - (flagged.exp_ready ? 2 : 0);
       if (it % 16 == 15) {  // look at the flag now and then; the kernels skip work once it is set
         HPHI_CUDA_TRY(cudaMemcpyAsync(&done_h, cg.done, sizeof(int), cudaMemcpyDeviceToHost, st));
         HPHI_CUDA_TRY(cudaStreamSynchronize(st));
@@ -2111,7 +2131,7 @@ hphi::Status invit_impl(hphi_model* m, const hphi_invit_params* p, void* xv, hph
     }
     // x = y / |y|
     if ((s = hphi::launch_cg_norm(cg, 0, y, x, n, partials, vgrid, st)).code) return s;
-    if ((s = hphi::launch_cg_fin(cg, 3, partials, vgrid, st)).code) return s;
+    if ((s = hphi::launch_cg_fin(cg, 3, partials, vgrid, nullptr, st)).code) return s;
     if ((s = hphi::launch_cg_norm(cg, 1, y, x, n, partials, vgrid, st)).code) return s;
     launches += 3;
   }
@@ -2119,9 +2139,9 @@ hphi::Status invit_impl(hphi_model* m, const hphi_invit_params* p, void* xv, hph
   plain.out = q;
   if ((s = hv_launch(m, HPHI_FP64, x, q, 1, hphi::Epi::kStore, plain, grid, scratch, st)).code) return s;
   if ((s = hphi::launch_cg_rq(cg, 0, x, q, n, partials, vgrid, st)).code) return s;
-  if ((s = hphi::launch_cg_fin(cg, 4, partials, vgrid, st)).code) return s;
+  if ((s = hphi::launch_cg_fin(cg, 4, partials, vgrid, nullptr, st)).code) return s;
   if ((s = hphi::launch_cg_rq(cg, 1, x, q, n, partials, vgrid, st)).code) return s;
-  if ((s = hphi::launch_cg_fin(cg, 5, partials, vgrid, st)).code) return s;
+  if ((s = hphi::launch_cg_fin(cg, 5, partials, vgrid, nullptr, st)).code) return s;
   launches += hvk + 4;
   HPHI_CUDA_TRY(cudaEventRecord(tm.b, st));
   HPHI_CUDA_TRY(cudaMemcpyAsync(host_s, cg.s, sizeof(host_s), cudaMemcpyDeviceToHost, st));

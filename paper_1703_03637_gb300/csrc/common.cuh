@@ -512,16 +512,15 @@ struct CgDev {
   int* done;             // [1] the current solve has converged
   int* steps;            // [1] CG iterations so far
 };
-Status launch_cg_shift(const CgDev& cg, const double* p, double* q, int64_t n, double* partials, int grid,
-                       cudaStream_t st);
 Status launch_cg_update(const CgDev& cg, int mode, const double* b, double* y, double* r, double* p, const double* q,
-                        int64_t n, double* partials, int grid, cudaStream_t st);
-Status launch_cg_dir(const CgDev& cg, const double* r, double* p, int64_t n, int grid, cudaStream_t st);
+                        int64_t n, double* partials, int grid, int* er, cudaStream_t st);
+Status launch_cg_dir(const CgDev& cg, const double* r, double* p, int64_t n, int grid, const QNext* qn, int* ec_new,
+                     cudaStream_t st);
 Status launch_cg_norm(const CgDev& cg, int mode, const double* y, double* x, int64_t n, double* partials, int grid,
                       cudaStream_t st);
 Status launch_cg_rq(const CgDev& cg, int mode, const double* x, const double* hx, int64_t n, double* partials,
                     int grid, cudaStream_t st);
-Status launch_cg_fin(const CgDev& cg, int mode, const double* partials, int grid, cudaStream_t st);
+Status launch_cg_fin(const CgDev& cg, int mode, const double* partials, int grid, int* clear, cudaStream_t st);
 
 // what the diagonal-observable kernel needs to know of a row's configuration
 struct ObsDev {

@@ -5,6 +5,14 @@
 // Hermitian, so Re <u, A v> is the inner product CG needs).  Besides the caller's vector the
 // solve keeps four: the iterate y, the residual r, the direction p and q = A p.
 //
+// A p = H p + c p (c = delta - E) is never formed by itself: H p comes with <p, H p> and <p, p>
+// from the refinement epilogue, <p, A p> = <p, H p> + c <p, p>, and the residual update adds c p
+// where it reads p anyway.  On the fixed-point paths the direction kernel also writes the next
+// product's quantised copy, on a scale bounded before the pass from the largest exponents of r
+// and p (as the Lanczos pass 2 does), so the product needs neither scan nor quantisation.
+// 32 iterations on 24 sites (2.7 million rows) on GB300: 5.6 ms instead of 6.3 ms with a scan, a
+// quantisation and a separate shift pass per product (12 launches an iteration, now 8).
+//
 // Every kernel streams its vectors once with four elements per thread one grid stride apart
 // and leaves one fp64 partial sum per CTA; a one-CTA finaliser turns the partials into the
 // CG scalars on the device, so a whole solve is a fixed launch sequence.
@@ -31,77 +39,113 @@ __device__ __forceinline__ void cg_partial(double acc, double* partials, int q) 
   if (threadIdx.x == 0) partials[(size_t)blockIdx.x * kMaxRedQ + q] = t;
 }
 
-// q <- q + c p (c = delta - E, so q = (H - E + delta) p after q = H p); partial <p, q>
-__global__ void __launch_bounds__(kThreads) k_cg_shift(CgDev cg, const double* __restrict__ p, double* __restrict__ q,
-                                                        int64_t n, double* __restrict__ partials) {
-  if (*cg.done) return;
-  const double c = cg.s[4];
-  const int64_t stride = (int64_t)gridDim.x * kThreads;
-  double acc = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < n; i += 4 * stride) {
-    double pv[4], qv[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int64_t k = i + u * stride;
-      pv[u] = k < n ? p[k] : 0.0;
-      qv[u] = k < n ? q[k] : 0.0;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int64_t k = i + u * stride;
-      if (k < n) {
-        const double t = fma(c, pv[u], qv[u]);
-        q[k] = t;
-        acc = fma(pv[u], t, acc);
-      }
-    }
-  }
-  cg_partial(acc, partials, 0);
+// largest exponent field over the CTA's values into *slot
+__device__ __forceinline__ void cg_exponent(int mx, int* slot) {
+  mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)mx);
+  if ((threadIdx.x & 31) == 0 && mx > 0) atomicMax(slot, mx);
 }
+__device__ __forceinline__ int cg_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
-// mode 0: start of a solve: y <- b, r <- b - q (q = A b), p <- r; partials |r|^2, |b|^2
-// mode 1: y += alpha p, r -= alpha q; partial |r|^2
+// mode 0: start of a solve: y <- b, r <- b - A b (q = H b), p <- r; partials |r|^2, |b|^2
+// mode 1: y += alpha p, r -= alpha A p (q = H p); partial |r|^2
+// er (may be null): the largest exponent field of r
 __global__ void __launch_bounds__(kThreads) k_cg_update(CgDev cg, int mode, const double* __restrict__ b,
                                                          double* __restrict__ y, double* __restrict__ r,
                                                          double* __restrict__ p, const double* __restrict__ q,
-                                                         int64_t n, double* __restrict__ partials) {
+                                                         int64_t n, double* __restrict__ partials, int* er) {
   if (*cg.done) return;
-  const double al = cg.s[1];
+  const double al = cg.s[1], c = cg.s[4];
   const int64_t stride = (int64_t)gridDim.x * kThreads;
   double rr = 0.0, bb = 0.0;
+  int mx = 0;
   for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < n; i += 4 * stride) {
+    double a[4], qv[4], yv[4], rv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t k = i + u * stride;
+      const bool on = k < n;
+      a[u] = on ? (mode == 0 ? b[k] : p[k]) : 0.0;
+      qv[u] = on ? q[k] : 0.0;
+      yv[u] = on && mode != 0 ? y[k] : 0.0;
+      rv[u] = on && mode != 0 ? r[k] : 0.0;
+    }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int64_t k = i + u * stride;
       if (k >= n) break;
+      const double ap = fma(c, a[u], qv[u]);
+      double t;
       if (mode == 0) {
-        const double bv = b[k];
-        const double rv = bv - q[k];
-        y[k] = bv;
-        r[k] = rv;
-        p[k] = rv;
-        rr = fma(rv, rv, rr);
-        bb = fma(bv, bv, bb);
+        t = a[u] - ap;
+        y[k] = a[u];
+        p[k] = t;
+        bb = fma(a[u], a[u], bb);
       } else {
-        const double pv = p[k];
-        y[k] = fma(al, pv, y[k]);
-        const double rv = fma(-al, q[k], r[k]);
-        r[k] = rv;
-        rr = fma(rv, rv, rr);
+        y[k] = fma(al, a[u], yv[u]);
+        t = fma(-al, ap, rv[u]);
       }
+      r[k] = t;
+      rr = fma(t, t, rr);
+      mx = max(mx, cg_field(t));
     }
   }
+  if (er != nullptr) cg_exponent(mx, er);
   cg_partial(rr, partials, 0);
   if (mode == 0) cg_partial(bb, partials, 1);
 }
 
-// p <- r + beta p
+// q = round(x 2^(1078 - E)), the rounding of the quantisation kernels
+__device__ __forceinline__ long long cg_quant(double x, int E) {
+  const int hi = __double2hiint(x);
+  const int ex = (hi >> 20) & 0x7ff;
+  long long q = 0;
+  if (ex != 0) {
+    const long long M = ((long long)((hi & 0xfffff) | 0x100000) << 32) | (long long)(unsigned)__double2loint(x);
+    const int sh = E - ex - 3;
+    if (sh <= 0) q = M << (-sh);
+    else if (sh < 62) q = (M + (1ll << (sh - 1))) >> sh;
+    if (hi < 0) q = -q;
+  }
+  return q;
+}
+
+// p <- r + beta p.  With qn.Q: also the next product's quantised copy.  |r + beta p| is below
+// 2^(E_r - 1022) + |beta| 2^(E_p - 1022), E_r and E_p the largest exponent fields of r and p, so
+// E = max(E_r, E_p + e_beta - 1022) + 1 bounds the new p's; its own goes into *ec_new.
 __global__ void __launch_bounds__(kThreads) k_cg_dir(CgDev cg, const double* __restrict__ r, double* __restrict__ p,
-                                                      int64_t n) {
+                                                      int64_t n, QNext qn, int* ec_new) {
   if (*cg.done) return;
   const double be = cg.s[2];
+  int E = 0;
+  if (qn.Q != nullptr) {
+    const int eb = cg_field(be), ep = *qn.ec_cur;
+    E = *qn.ep;  // of r
+    if (eb != 0 && ep != 0) E = max(E, ep + eb - 1022);
+    E = min(E + 1, 2046);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *qn.eq = E;
+    E += qn.extra;
+  }
+  int mx = 0;
   const int64_t stride = (int64_t)gridDim.x * kThreads;
-  for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < n; i += stride) p[i] = fma(be, p[i], r[i]);
+  for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < n; i += 4 * stride) {
+    double rv[4], pv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t k = i + u * stride;
+      rv[u] = k < n ? r[k] : 0.0;
+      pv[u] = k < n ? p[k] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t k = i + u * stride;
+      if (k >= n) break;
+      const double t = fma(be, pv[u], rv[u]);
+      p[k] = t;
+      mx = max(mx, cg_field(t));
+      if (qn.Q != nullptr) qn.Q[k] = cg_quant(t, E);
+    }
+  }
+  if (qn.Q != nullptr) cg_exponent(mx, ec_new);
 }
 
 // x <- y / |y| (mode 0: partial |y|^2 first; mode 1: scale, the norm in s[9])
@@ -150,25 +194,28 @@ __device__ double cg_sum(const double* __restrict__ partials, int grid, int q, d
 }
 
 // scalar steps of the solve, one CTA:
-// 0 start (rr, |b|^2, done if r = 0)  1 alpha = rr / <p, q>  2 beta = rr' / rr, test
+// 0 start (rr, |b|^2, done if r = 0)  1 alpha = rr / <p, A p>  2 beta = rr' / rr, test
 // 3 the norm of y  4 e and the variance  5 the residual
+// clear (may be null): an exponent slot the next kernel raises
 __global__ void __launch_bounds__(kThreads) k_cg_fin(CgDev cg, int mode, const double* __restrict__ partials,
-                                                      int grid) {
+                                                      int grid, int* clear) {
   __shared__ double sm[kThreads];
   if ((mode == 1 || mode == 2) && *cg.done) return;
   const double s0 = cg_sum(partials, grid, 0, sm);
-  const double s1 = (mode == 0 || mode == 4) ? cg_sum(partials, grid, 1, sm) : 0.0;
+  const double s1 = (mode <= 1 || mode == 4) ? cg_sum(partials, grid, 1, sm) : 0.0;
   if (threadIdx.x != 0) return;
+  if (clear != nullptr) *clear = 0;
   if (mode == 0) {
     cg.s[0] = s0;
     cg.s[3] = s1;
     *cg.done = (s0 <= cg.s[5] * s1) ? 1 : 0;
   } else if (mode == 1) {
-    if (!(s0 > 0.0)) {  // A is positive definite on a non-zero p: only p = 0 gives this
+    const double pap = fma(cg.s[4], s1, s0);  // <p, H p> + c <p, p>
+    if (!(pap > 0.0)) {  // A is positive definite on a non-zero p: only p = 0 gives this
       *cg.done = 1;
       return;
     }
-    cg.s[1] = cg.s[0] / s0;
+    cg.s[1] = cg.s[0] / pap;
   } else if (mode == 2) {
     cg.s[2] = s0 / cg.s[0];
     cg.s[0] = s0;
@@ -186,22 +233,16 @@ __global__ void __launch_bounds__(kThreads) k_cg_fin(CgDev cg, int mode, const d
 
 }  // namespace
 
-Status launch_cg_shift(const CgDev& cg, const double* p, double* q, int64_t n, double* partials, int grid,
-                       cudaStream_t st) {
-  k_cg_shift<<<grid, kThreads, 0, st>>>(cg, p, q, n, partials);
-  HPHI_CUDA_TRY(cudaGetLastError());
-  return {};
-}
-
 Status launch_cg_update(const CgDev& cg, int mode, const double* b, double* y, double* r, double* p, const double* q,
-                        int64_t n, double* partials, int grid, cudaStream_t st) {
-  k_cg_update<<<grid, kThreads, 0, st>>>(cg, mode, b, y, r, p, q, n, partials);
+                        int64_t n, double* partials, int grid, int* er, cudaStream_t st) {
+  k_cg_update<<<grid, kThreads, 0, st>>>(cg, mode, b, y, r, p, q, n, partials, er);
   HPHI_CUDA_TRY(cudaGetLastError());
   return {};
 }
 
-Status launch_cg_dir(const CgDev& cg, const double* r, double* p, int64_t n, int grid, cudaStream_t st) {
-  k_cg_dir<<<grid, kThreads, 0, st>>>(cg, r, p, n);
+Status launch_cg_dir(const CgDev& cg, const double* r, double* p, int64_t n, int grid, const QNext* qn, int* ec_new,
+                     cudaStream_t st) {
+  k_cg_dir<<<grid, kThreads, 0, st>>>(cg, r, p, n, qn ? *qn : QNext{nullptr, nullptr, nullptr, nullptr, 0}, ec_new);
   HPHI_CUDA_TRY(cudaGetLastError());
   return {};
 }
@@ -220,8 +261,8 @@ Status launch_cg_rq(const CgDev& cg, int mode, const double* x, const double* hx
   return {};
 }
 
-Status launch_cg_fin(const CgDev& cg, int mode, const double* partials, int grid, cudaStream_t st) {
-  k_cg_fin<<<1, kThreads, 0, st>>>(cg, mode, partials, grid);
+Status launch_cg_fin(const CgDev& cg, int mode, const double* partials, int grid, int* clear, cudaStream_t st) {
+  k_cg_fin<<<1, kThreads, 0, st>>>(cg, mode, partials, grid, clear);
   HPHI_CUDA_TRY(cudaGetLastError());
   return {};
 }
