@@ -117,15 +117,18 @@ __global__ void __launch_bounds__(kThreads) k_hub_dn(const HubDev md, const R* _
   const int64_t dim_up = md.dim_up, dim_dn = md.dim_dn;
   const int64_t n_items = ((dim_up + SW - 1) / SW) * dim_dn;
   __shared__ int64_t s_item;
-  for (;;) {
-    __syncthreads();
-    if (tid == 0) s_item = (int64_t)atomicAdd(next_item, (unsigned long long)(kWarps * claim));
-    __syncthreads();
-    const int64_t base = s_item;
-    if (base >= n_items) break;
+  for (bool first = true;; first = false) {
+    int64_t base = (int64_t)blockIdx.x * kWarps;
+    if (claim > 0) {
+      __syncthreads();
+      if (tid == 0) s_item = (int64_t)atomicAdd(next_item, (unsigned long long)(kWarps * claim));
+      __syncthreads();
+      base = s_item;
+    }
+    if (base >= n_items || (claim == 0 && !first)) break;
     int64_t s = base / dim_dn, d = base - s * dim_dn + warp;  // the CTA's warps on neighbouring rows
-    for (int it = 0; it < claim; ++it, d += kWarps) {
-      while (d >= dim_dn) {
+    for (int it = 0; it < max(claim, 1); ++it, d += kWarps) {
+      while (d >= dim_dn) {  // (the warp's offset or the next round runs into the next stripe)
         d -= dim_dn;
         ++s;
       }
@@ -211,6 +214,50 @@ __global__ void __launch_bounds__(kThreads) k_maxexp(const double* __restrict__ 
   if ((threadIdx.x & 31) == 0 && mx > 0) atomicMax(E, mx);
 }
 
+// q = round(x 2^(1078 - E)), by integer operations on the bits of x
+__device__ __forceinline__ long long quant_one(double x, int E) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  const int ex = (hi >> 20) & 0x7ff;
+  long long q = 0;
+  if (ex != 0) {
+    const long long M = ((long long)((hi & 0xfffff) | 0x100000) << 32) | (long long)lo;  // x = M 2^(ex-1075)
+    const int sh = E - ex - 3;                                                           // q = M 2^-sh
+    if (sh <= 0) q = M << (-sh);
+    else if (sh < 62) q = (M + (1ll << (sh - 1))) >> sh;
+    if (hi < 0) q = -q;
+  }
+  return q;
+}
+
+// Exponent scan and quantisation of a short vector in one CTA: one launch instead of three (the
+// exponent slot's reset among them), which is what a few thousand elements wait for.  On the
+// 8-site cluster (4,900 rows), with pass D's counter gone too, a product takes 20.0 us instead of
+// 24.4 (three launches instead of six).  Sixteen elements a thread is what the one CTA holds in
+// registers; above that the grid's bandwidth is worth more than two launches.
+constexpr int kShortQuant = 16384;
+__global__ void __launch_bounds__(1024) k_quant_short(const double* __restrict__ X, long long* __restrict__ Q, int n,
+                                                      int* __restrict__ Ep, const int* __restrict__ done, int extra) {
+  if (done != nullptr && *done) return;
+  __shared__ int s_mx[32];
+  constexpr int kPer = kShortQuant / 1024;
+  const int tid = threadIdx.x;
+  double x[kPer];
+  int mx = 0;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) x[k] = tid + k * 1024 < n ? __ldg(X + tid + k * 1024) : 0.0;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) mx = max(mx, (__double2hiint(x[k]) >> 20) & 0x7ff);
+  mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)mx);
+  if ((tid & 31) == 0) s_mx[tid >> 5] = mx;
+  __syncthreads();
+  mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)s_mx[tid & 31]);
+  if (tid == 0) *Ep = mx;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k)
+    if (tid + k * 1024 < n) Q[tid + k * 1024] = quant_one(x[k], mx + extra);
+}
+
 // extra: headroom bits; q = round(x 2^(1078 - E - extra)), |q| < 2^(56 - extra)
 __global__ void __launch_bounds__(kThreads) k_quant(const double* __restrict__ X, long long* __restrict__ Q, int64_t n,
                                                      const int* __restrict__ Ep, const int* __restrict__ done,
@@ -218,19 +265,7 @@ __global__ void __launch_bounds__(kThreads) k_quant(const double* __restrict__ X
   if (done != nullptr && *done) return;
   const int E = *Ep + extra;
   for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kThreads) {
-    const double x = __ldg(X + i);
-    const int hi = __double2hiint(x);
-    const unsigned lo = (unsigned)__double2loint(x);
-    const int ex = (hi >> 20) & 0x7ff;
-    long long q = 0;
-    if (ex != 0) {
-      const long long M = ((long long)((hi & 0xfffff) | 0x100000) << 32) | (long long)lo;  // x = M 2^(ex-1075)
-      const int sh = E - ex - 3;                                                           // q = M 2^-sh
-      if (sh <= 0) q = M << (-sh);
-      else if (sh < 62) q = (M + (1ll << (sh - 1))) >> sh;
-      if (hi < 0) q = -q;
-    }
-    Q[i] = q;
+    Q[i] = quant_one(__ldg(X + i), E);
   }
 }
 
@@ -558,11 +593,12 @@ Status launch_dn(const HubDev& md, const R* X, R* W, const int* done, unsigned l
   int p = md.dn_ept;
   if (p != 1 && p != 2 && p != 4) p = items_of(kDnPieces) >= 2 * warps ? kDnPieces : 1;
   const int64_t items = items_of(p);
-  // items per warp and claim: four, fewer while that would leave warps without one
-  const int claim = (int)std::max<int64_t>(1, std::min<int64_t>(4, items / (2 * warps)));
   const int gd = (int)std::min<int64_t>((items + 7) / 8, (int64_t)num_sms() * 8);
+  // items per warp and claim: four, fewer while that would leave warps without one; 0: a warp for
+  // every item, no counter
+  const int claim = items <= (int64_t)gd * 8 ? 0 : (int)std::max<int64_t>(1, std::min<int64_t>(4, items / (2 * warps)));
   const bool vec = (md.dim_up * (int64_t)sizeof(R)) % 16 == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(W)) & 15u) == 0;
-  HPHI_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st));
+  if (claim > 0) HPHI_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st));
 #define HPHI_DN(PP)                                                                    \
   if (vec) k_hub_dn<R, PP, true><<<gd, kThreads, 0, st>>>(md, X, W, done, counter, claim);    \
   else k_hub_dn<R, PP, false><<<gd, kThreads, 0, st>>>(md, X, W, done, counter, claim)
@@ -632,15 +668,9 @@ Status launch_q(const HubDev& md, const void* v, void* w, void* scratch, const F
   long long* WQ = Q + md.dim;
   int* Ep = reinterpret_cast<int*>(WQ + md.dim);
   unsigned long long* counter = reinterpret_cast<unsigned long long*>(WQ + md.dim) + 1;
-  const int gv = (int)std::max<int64_t>(1, std::min<int64_t>((md.dim + kThreads - 1) / kThreads, (int64_t)num_sms() * 8));
-  if (!fa.exp_ready) {
-    HPHI_CUDA_TRY(cudaMemsetAsync(Ep, 0, sizeof(int), st));
-    k_maxexp<<<gv, kThreads, 0, st>>>(X, md.dim, Ep, fa.done);
-    HPHI_CUDA_TRY(cudaGetLastError());
-  }
   if (fa.exp_ready != 2) {  // 2: the previous Lanczos pass 2 wrote Q and its exponent
-    k_quant<<<gv, kThreads, 0, st>>>(X, Q, md.dim, Ep, fa.done, 0);
-    HPHI_CUDA_TRY(cudaGetLastError());
+    const Status s = launch_quant_vec(X, Q, md.dim, Ep, fa.done, fa.exp_ready != 0, 0, st);
+    if (s.code) return s;
   }
   if (fa.pexp != nullptr) HPHI_CUDA_TRY(cudaMemsetAsync(fa.pexp, 0, sizeof(int), st));
   Status sd = launch_dn<long long>(md, Q, WQ, fa.done, counter, st);
@@ -755,6 +785,11 @@ Status launch_hub_store_noalloc(const HubDev& md0, const void* v, void* w, cudaS
 
 Status launch_quant_vec(const double* X, long long* Q, int64_t n, int* Ep, const int* done, bool exp_ready, int extra,
                         cudaStream_t st) {
+  if (!exp_ready && n <= kShortQuant) {
+    k_quant_short<<<1, 1024, 0, st>>>(X, Q, (int)n, Ep, done, extra);
+    HPHI_CUDA_TRY(cudaGetLastError());
+    return {};
+  }
   const int gv = (int)std::max<int64_t>(1, std::min<int64_t>((n + kThreads - 1) / kThreads, (int64_t)num_sms() * 8));
   if (!exp_ready) {
     HPHI_CUDA_TRY(cudaMemsetAsync(Ep, 0, sizeof(int), st));

@@ -1274,6 +1274,27 @@ def test_hubbard_down_pass_pieces(n, nu, nd, offset):
             m.autotune(prec)
 
 
+# ----------------------------------------------------------------------------- short vectors
+@pytest.mark.parametrize("n,nu,nd", [(3, 1, 0), (4, 2, 2), (8, 4, 4), (9, 4, 4), (10, 3, 4)])
+@pytest.mark.parametrize("scale", [1.0, 2.0**900, 2.0**-900])
+def test_hubbard_short_vectors(n, nu, nd, scale):
+    """The one-CTA exponent scan and quantisation, from 3 rows to the last full round below its
+    limit (15,876 of 16,384) and the first size above it; zeros, values far below the largest and
+    the largest in the last row.  |q| < 2^56, so a product of at most 60 terms per row is within
+    60 x 2^-55 of the row sum of |H| times the largest entry: 1e-12 of the norm leaves the
+    reference's own rounding room."""
+    spec = wl.hubbard_ring(n, 1.0, 8.0).with_basis(wl.BASIS_NUMBER, nu, nd)
+    m = hp.Model.from_spec(spec)
+    v = wl.gaussian_vector(n + nd, m.dim)[:, 0]
+    v[::3] *= 1e-9
+    v[1::7] = 0.0
+    v[-1] = 3.0
+    ref = oracle.apply_H(spec, v).real
+    w = m.apply_H(torch.as_tensor(v * scale, device="cuda"))
+    assert _rel(w.cpu().numpy() / scale, ref) < 1e-12
+    assert torch.count_nonzero(m.apply_H(torch.zeros(m.dim, device="cuda", dtype=torch.float64))) == 0
+
+
 # ----------------------------------------------------------------------------- one-cluster Lanczos lists
 def _xyz_classes(n, values):
     """Full-basis ring whose bonds take `values` exchange couplings in turn, with a transverse field."""
