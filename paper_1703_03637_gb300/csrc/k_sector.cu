@@ -848,9 +848,10 @@ __device__ __forceinline__ void tile_load(const T* p, T* out) {
 // ahead across columns, W and the previous Lanczos vector are requested before the straddling
 // gathers, which run four bonds (4 K loads) at a time.
 //
-// 6x5 torus, S^z = 0 (155,117,520 rows), Lanczos step on GB300: fp64 2.77 ms (L = 14, two rows a
-// tile), bound by instruction issue (65 %) and shared-memory wavefronts (59 %); fp32 1.88 ms
-// (L = 15, four rows).  One row a tile at L = 17, every bond below L in state order and all
+// 6x5 torus, S^z = 0 (155,117,520 rows), Lanczos step on GB300: fp64 2.72 ms (L = 14, two rows a
+// tile), bound by instruction issue (65 %) and shared-memory wavefronts (59 %); fp32 1.62 ms
+// (L = 15, four rows).  Reading a bond's row pointers in 16-byte pieces and shifting the activity
+// bits instead of testing bond numbers gave 0.16 and 0.23 ms of that.  One row a tile at L = 17, every bond below L in state order and all
 // bonds across L gathered here, took 5.82 and 5.29 ms (pass H then 0.78 and 0.49 ms instead of
 // 1.09 and 0.76 ms).
 template <class T, int K, Epi E, int NT, bool ONE>
@@ -870,7 +871,7 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
   __shared__ uint32_t s_hdiag[K];
   __shared__ uint32_t s_hb[K];               // bit n: the high bit of straddling bond n
   __shared__ uint32_t s_spm[K][kSecMaxSl];
-  __shared__ const T* s_ptr[kSecMaxStr][K];  // partner row of row m through the bond
+  __shared__ __align__(16) const T* s_ptr[kSecMaxStr][K];  // partner row of row m through the bond
   __shared__ uint32_t s_hi0;
   __shared__ int s_nk;
   __shared__ unsigned long long s_t;
@@ -911,6 +912,7 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
   const double c1e = FIX ? (double)es.c1 * s_e2 : 0.0;
   const R coef0 = opaque((R)d.coef[0]);
   const int n_str = d.n_str, n_cls = d.n_cls;
+  const uint32_t str_mask = n_str < 32 ? (1u << n_str) - 1u : 0xffffffffu;
   const int64_t stride = d.lo_stride;
   constexpr int NQ = n_red<E>() > 0 ? n_red<E>() : 1;  // reduced quantities of the epilogue
   Red<FIX, NQ> red;
@@ -1051,22 +1053,34 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
       }
       uint32_t act[K];  // bond n acts on row m: its low bit differs from its high bit
 #pragma unroll
-      for (int m = 0; m < K; ++m) act[m] = (on && m < nk) ? info.y ^ s_hb[m] : 0u;
+      for (int m = 0; m < K; ++m) act[m] = (on && m < nk) ? (info.y ^ s_hb[m]) & str_mask : 0u;
       for (int n0 = 0; n0 < n_str; n0 += 4) {
         const uint2 r = rk;
         if (n0 + 4 < n_str) rk = __ldg(d.str_rank4 + (int64_t)(n0 / 4 + 1) * stride + lpad + u);
         T x[4][K];
 #pragma unroll
         for (int t4 = 0; t4 < 4; ++t4) {
-          const int n = n0 + t4;
           const uint32_t word = t4 < 2 ? r.x : r.y;
           const uint32_t col = (t4 & 1) ? word >> 16 : word & 0xffffu;
+          const T* pr[K];  // the rows' pointers in 16-byte reads
+          if constexpr (K >= 2) {
+#pragma unroll
+            for (int m = 0; m < K; m += 2) {
+              const ulonglong2 two = *reinterpret_cast<const ulonglong2*>(&s_ptr[n0 + t4][m]);
+              pr[m] = reinterpret_cast<const T*>(two.x);
+              pr[m + 1] = reinterpret_cast<const T*>(two.y);
+            }
+          } else {
+            pr[0] = s_ptr[n0 + t4][0];
+          }
 #pragma unroll
           for (int m = 0; m < K; ++m) {
             x[t4][m] = (T)0;
-            if (n < n_str && ((act[m] >> n) & 1u)) x[t4][m] = __ldg(s_ptr[n][m] + col);
+            if (act[m] & (1u << t4)) x[t4][m] = __ldg(pr[m] + col);
           }
         }
+#pragma unroll
+        for (int m = 0; m < K; ++m) act[m] >>= 4;
         if constexpr (ONE) {
 #pragma unroll
           for (int m = 0; m < K; ++m) acc[m] += (x[0][m] + x[1][m]) + (x[2][m] + x[3][m]);
