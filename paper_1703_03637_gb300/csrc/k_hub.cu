@@ -283,7 +283,9 @@ __global__ void __launch_bounds__(kThreads) k_quant(const double* __restrict__ X
 // electrons (165,636,900 rows), fp64 Lanczos step, two rows a tile: 2.13 ms instead of 4.16 ms,
 // bound by shared-memory wavefronts (71 %) and instruction issue (61 %); 7 + 6 electrons, fp32
 // product, four rows: 0.55 instead of 0.90 ms; 18 sites, 9 + 9 (2,363,904,400 rows), fp32 mTPQ
-// step, one 194 KB row: 28.0 instead of 64.3 ms, bound by instruction issue (83 %).
+// step, one 194 KB row: 26.6 instead of 64.3 ms, bound by instruction issue.  There whole chunks of
+// slots that add skip the tests of each group (*; 28.1 ms without; 1 % slower with two or four rows,
+// whose groups carry more work per test).
 template <class T, int K, Epi E, int NT>
 __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_hub_up(const HubDev md, const T* __restrict__ X, const T* W,
                                                const int* __restrict__ Ep, void* w, FusedArgs fa) {
@@ -415,27 +417,37 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_hub_up(const HubDe
         uint2 nxt[kGatherChunk];
 #pragma unroll
         for (int j = 0; j < kGatherChunk; ++j) nxt[j] = __ldg(q + j * stride);
+        if (K == 1 && 4 * (c0 + kGatherChunk) <= np) {  // a chunk that only adds: no tests per group (*)
+          T cs = (T)0;
 #pragma unroll
-        for (int j = 0; j < kGatherChunk; ++j) {
-          if (c0 + j < ng) {
+          for (int j = 0; j < kGatherChunk; ++j) {
             const uint2 r = cur[j];
-            T v[4][K];
-            load_k<T, K>(tile + (r.x & 0xffffu) * K, v[0]);
-            load_k<T, K>(tile + (r.x >> 16) * K, v[1]);
-            load_k<T, K>(tile + (r.y & 0xffffu) * K, v[2]);
-            load_k<T, K>(tile + (r.y >> 16) * K, v[3]);
-            const int left = np - 4 * (c0 + j);  // slots of this group that add
-            if (left >= 4) {
+            cs += (tile[r.x & 0xffffu] + tile[r.x >> 16]) + (tile[r.y & 0xffffu] + tile[r.y >> 16]);
+          }
+          acc[0] += cs;
+        } else {
 #pragma unroll
-              for (int m = 0; m < K; ++m) acc[m] += (v[0][m] + v[1][m]) + (v[2][m] + v[3][m]);
-            } else if (left <= 0) {
+          for (int j = 0; j < kGatherChunk; ++j) {
+            if (c0 + j < ng) {
+              const uint2 r = cur[j];
+              T v[4][K];
+              load_k<T, K>(tile + (r.x & 0xffffu) * K, v[0]);
+              load_k<T, K>(tile + (r.x >> 16) * K, v[1]);
+              load_k<T, K>(tile + (r.y & 0xffffu) * K, v[2]);
+              load_k<T, K>(tile + (r.y >> 16) * K, v[3]);
+              const int left = np - 4 * (c0 + j);  // slots of this group that add
+              if (left >= 4) {
 #pragma unroll
-              for (int m = 0; m < K; ++m) acc[m] -= (v[0][m] + v[1][m]) + (v[2][m] + v[3][m]);
-            } else {
+                for (int m = 0; m < K; ++m) acc[m] += (v[0][m] + v[1][m]) + (v[2][m] + v[3][m]);
+              } else if (left <= 0) {
 #pragma unroll
-              for (int s = 0; s < 4; ++s)
+                for (int m = 0; m < K; ++m) acc[m] -= (v[0][m] + v[1][m]) + (v[2][m] + v[3][m]);
+              } else {
 #pragma unroll
-                for (int m = 0; m < K; ++m) acc[m] += s < left ? v[s][m] : -v[s][m];
+                for (int s = 0; s < 4; ++s)
+#pragma unroll
+                  for (int m = 0; m < K; ++m) acc[m] += s < left ? v[s][m] : -v[s][m];
+              }
             }
           }
         }
