@@ -841,6 +841,16 @@ __device__ __forceinline__ void tile_load(const T* p, T* out) {
   }
 }
 
+// a tile's rows as pass R keeps them in shared memory
+template <int K>
+struct __align__(8) LoRows {
+  uint64_t roff[K];
+  uint32_t hrow[K], hdiag[K];
+  uint32_t hb[K];                // bit n: the high bit of straddling bond n
+  uint32_t spm[K][kSecMaxSl];
+  int nk;                        // 0: no tile left
+};
+
 // pass R: K rows of one class in shared memory; the bonds inside the row from the gather table,
 // straddling exchange gathered from the partner rows, diagonal from packed counts, plus the
 // pass-H sums Wh, then the fused epilogue.  X is the input (fp32) or its fixed-point copy.  A
@@ -848,12 +858,14 @@ __device__ __forceinline__ void tile_load(const T* p, T* out) {
 // ahead across columns, W and the previous Lanczos vector are requested before the straddling
 // gathers, which run four bonds (4 K loads) at a time.
 //
-// 6x5 torus, S^z = 0 (155,117,520 rows), Lanczos step on GB300: fp64 2.72 ms (L = 14, two rows a
-// tile), bound by instruction issue (65 %) and shared-memory wavefronts (59 %); fp32 1.62 ms
-// (L = 15, four rows).  Reading a bond's row pointers in 16-byte pieces and shifting the activity
-// bits instead of testing bond numbers gave 0.16 and 0.23 ms of that.  One row a tile at L = 17, every bond below L in state order and all
-// bonds across L gathered here, took 5.82 and 5.29 ms (pass H then 0.78 and 0.49 ms instead of
-// 1.09 and 0.76 ms).
+// 6x5 torus, S^z = 0 (155,117,520 rows), Lanczos step on GB300: fp64 2.58 ms (L = 14, two rows a
+// tile), fp32 1.62 ms (L = 15, four rows).  Instruction issue (65 %) and shared-memory wavefronts
+// (59 %) share it with the latencies of a tile's start and of the straddling gathers: with the
+// gathers in the tile left out it takes 0.2 ms less, with the straddling ones left out 0.75 ms.
+// Reading a bond's row pointers in 16-byte pieces and shifting the activity bits instead of testing
+// bond numbers gave 0.16 and 0.23 ms, knowing the next tile's rows ahead 0.14 ms in fp64.
+// One row a tile at L = 17, every bond below L in state order and all bonds across L gathered
+// here, took 5.82 and 5.29 ms (pass H then 0.78 and 0.49 ms instead of 1.09 and 0.76 ms).
 template <class T, int K, Epi E, int NT, bool ONE>
 __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDev d, const T* __restrict__ X,
                                                                     const T* Wh, void* w, FusedArgs fa,
@@ -866,15 +878,8 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
   T* tile = reinterpret_cast<T*>(smem_raw);
   R* s_dtab = reinterpret_cast<R*>(smem_raw + (((size_t)(d.nq_max + kZero) * K * sizeof(T) + 15) / 16) * 16);
   int* s_dti = reinterpret_cast<int*>(s_dtab + d.dtab_n);  // fp64 with d.dint: the table in units
-  __shared__ uint64_t s_roff[K];
-  __shared__ uint32_t s_hrow[K];
-  __shared__ uint32_t s_hdiag[K];
-  __shared__ uint32_t s_hb[K];               // bit n: the high bit of straddling bond n
-  __shared__ uint32_t s_spm[K][kSecMaxSl];
+  __shared__ LoRows<K> s_cur, s_nxt;         // the rows of this tile and of the next
   __shared__ __align__(16) const T* s_ptr[kSecMaxStr][K];  // partner row of row m through the bond
-  __shared__ uint32_t s_hi0;
-  __shared__ int s_nk;
-  __shared__ unsigned long long s_t;
   __shared__ T s_w[kSecMaxCls];
   __shared__ T s_sw[kSecMaxStr];             // weight of each straddling bond
   __shared__ double s_red[(NT / 32) * kMaxRedQ];
@@ -923,53 +928,64 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
   // the processing order (a fixed stride would let CTAs drift apart over thousands of tiles);
   // with a CTA for every tile each takes its own, so the partial sums keep their places
   const bool own = d.n_tiles <= (int64_t)gridDim.x;
-  for (bool first = true;; first = false) {
-    int64_t t = blockIdx.x;
-    __syncthreads();  // the previous tile's rows are no longer read
+  // The last warp claims the next tile and reads its rows' table entries, four dependent reads
+  // from memory, while the others gather: its share of a row is the shortest of a partial round.
+  auto fetch = [&](int l) {
+    __syncwarp();
+    int64_t t = s_nxt.nk < 0 ? (int64_t)blockIdx.x : d.n_tiles;  // own: the first time round only
+    __syncwarp();
     if (!own) {
-      if (tid == 0) s_t = atomicAdd(claim, 1ull);
-      __syncthreads();
-      t = (int64_t)s_t;
+      unsigned long long c = 0;
+      if (l == 0) c = atomicAdd(claim, 1ull);
+      t = (int64_t)__shfl_sync(0xffffffffu, c, 0);
     }
-    if (t >= d.n_tiles || (own && !first)) break;
-    if (tid < K) {
-      const uint32_t tw = __ldg(d.tiles + t);
-      const uint32_t start = tw & 0xffffffu;
-      const int nk = (int)(tw >> 24) + 1;
-      uint64_t roff = 0;
-      uint32_t hd = 0, hi = 0, hb = 0;
-      for (int l = 0; l < kSecMaxSl; ++l) s_spm[tid][l] = 0u;
-      if (tid < nk) {
-        hi = __ldg(d.hi_seq + start + tid);
-        if (tid == 0) s_hi0 = hi;
-        roff = __ldg(d.hi_off + hi);
-        hd = __ldg(d.hi_diag + hi);
-        for (int n = 0; n < d.n_sp; ++n)
-          if ((hi >> d.sp_a[n]) & 1u) s_spm[tid][d.sp_l[n]] |= 1u << d.sp_b[n];
-        for (int n = 0; n < n_str; ++n) hb |= ((hi >> d.str_a[n]) & 1u) << n;
-      }
-      if (tid == 0) s_nk = nk;
-      s_roff[tid] = roff;
-      s_hrow[tid] = hi;
-      s_hdiag[tid] = hd;
-      s_hb[tid] = hb;
+    if (t >= d.n_tiles) {
+      if (l == 0) s_nxt.nk = 0;
+      return;
     }
-    __syncthreads();
-    const int nk = s_nk;
-    if (tid < n_str) {  // partner rows, one bond per thread (read after the staging barrier)
-      const uint32_t a = d.str_a[tid];
-#pragma unroll
-      for (int m = 0; m < K; ++m) s_ptr[tid][m] = X + (m < nk ? __ldg(d.hi_off + (s_hrow[m] ^ (1u << a))) : 0ull);
+    if (l >= K) return;
+    const uint32_t tw = __ldg(d.tiles + t);
+    const uint32_t start = tw & 0xffffffu;
+    const int nk = (int)(tw >> 24) + 1;
+    uint64_t roff = 0;
+    uint32_t hd = 0, hi = 0, hb = 0;
+    for (int n = 0; n < kSecMaxSl; ++n) s_nxt.spm[l][n] = 0u;
+    if (l < nk) {
+      hi = __ldg(d.hi_seq + start + l);
+      roff = __ldg(d.hi_off + hi);
+      hd = __ldg(d.hi_diag + hi);
+      for (int n = 0; n < d.n_sp; ++n)
+        if ((hi >> d.sp_a[n]) & 1u) s_nxt.spm[l][d.sp_l[n]] |= 1u << d.sp_b[n];
+      for (int n = 0; n < n_str; ++n) hb |= ((hi >> d.str_a[n]) & 1u) << n;
     }
-    const int q = d.n_ones - __popc(s_hi0);
+    if (l == 0) s_nxt.nk = nk;
+    s_nxt.roff[l] = roff;
+    s_nxt.hrow[l] = hi;
+    s_nxt.hdiag[l] = hd;
+    s_nxt.hb[l] = hb;
+  };
+  if (tid == NT - 32) s_nxt.nk = -1;
+  for (;;) {
+    if (tid >= NT - 32) fetch(tid - (NT - 32));
+    __syncthreads();  // the previous tile's rows are no longer read, this tile's are known
+    const int nk = s_nxt.nk;
+    if (nk == 0) break;
+    for (int k = tid; k < (int)(sizeof(s_cur) / 8); k += NT)
+      reinterpret_cast<uint2*>(&s_cur)[k] = reinterpret_cast<const uint2*>(&s_nxt)[k];
+    const int q = d.n_ones - __popc(s_nxt.hrow[0]);
     const uint32_t lpad = d.lo_pad[q];
     const int nq = (int)(d.lo_off[q + 1] - d.lo_off[q]);
     const int nqp = (nq + 31) & ~31;
+    if (tid < n_str) {  // partner rows, one bond per thread (read after the staging barrier)
+      const uint32_t a = d.str_a[tid];
+#pragma unroll
+      for (int m = 0; m < K; ++m) s_ptr[tid][m] = X + (m < nk ? __ldg(d.hi_off + (s_nxt.hrow[m] ^ (1u << a))) : 0ull);
+    }
     // stage the rows, tile[u * K + m] = X[row m][u]
     for (int u = tid; u < nq; u += NT) {
 #pragma unroll
       for (int m = 0; m < K; ++m) {
-        if (m < nk) copy_async<(int)sizeof(T)>(tile + u * K + m, X + s_roff[m] + u);
+        if (m < nk) copy_async<(int)sizeof(T)>(tile + u * K + m, X + s_nxt.roff[m] + u);
         else tile[u * K + m] = (T)0;
       }
     }
@@ -1046,14 +1062,14 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
       R pin[K];
 #pragma unroll
       for (int m = 0; m < K; ++m) {
-        const int64_t idx = (int64_t)s_roff[m] + u;
+        const int64_t idx = (int64_t)s_cur.roff[m] + u;
         wv[m] = (on && m < nk) ? Wh[idx] : (T)0;
         if constexpr (E == Epi::kLanczos1)
           pin[m] = (on && m < nk) ? reinterpret_cast<const R*>(fa.in ? fa.in : fa.out)[idx] : (R)0;
       }
       uint32_t act[K];  // bond n acts on row m: its low bit differs from its high bit
 #pragma unroll
-      for (int m = 0; m < K; ++m) act[m] = (on && m < nk) ? (info.y ^ s_hb[m]) & str_mask : 0u;
+      for (int m = 0; m < K; ++m) act[m] = (on && m < nk) ? (info.y ^ s_cur.hb[m]) & str_mask : 0u;
       for (int n0 = 0; n0 < n_str; n0 += 4) {
         const uint2 r = rk;
         if (n0 + 4 < n_str) rk = __ldg(d.str_rank4 + (int64_t)(n0 / 4 + 1) * stride + lpad + u);
@@ -1100,10 +1116,10 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
 #pragma unroll
       for (int m = 0; m < K; ++m) {
         if (m >= nk) break;
-        uint32_t c = ldc + s_hdiag[m];
-        for (int l = 0; l < d.n_sl; ++l) c += (uint32_t)__popc(lo & s_spm[m][l]) << (8 * d.sp_lg[l]);
+        uint32_t c = ldc + s_cur.hdiag[m];
+        for (int l = 0; l < d.n_sl; ++l) c += (uint32_t)__popc(lo & s_cur.spm[m][l]) << (8 * d.sp_lg[l]);
         const int ci = (int)(c & 0xffu) + d.dstride * (int)(c >> 8);
-        const int64_t idx = (int64_t)s_roff[m] + u;
+        const int64_t idx = (int64_t)s_cur.roff[m] + u;
         const T xq = tile[u * K + m];
         const T S = acc[m] + wv[m];
         if constexpr (!FIX) {

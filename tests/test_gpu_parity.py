@@ -1274,6 +1274,23 @@ def test_hubbard_down_pass_pieces(n, nu, nd, offset):
             m.autotune(prec)
 
 
+# ----------------------------------------------------------------------------- tiles claimed ahead
+@pytest.mark.parametrize("mk", [wl.heisenberg_ring, wl.j1j2_ring], ids=["one-class", "two-classes"])
+@pytest.mark.parametrize("n,L,K", [(12, 11, 1), (16, 8, 1), (20, 11, 1), (20, 11, 4), (20, 8, 2)])
+def test_sector_tiles_claimed_ahead(mk, n, L, K):
+    """Pass R with one tile or two, a tile for every CTA, one or two tiles more than CTAs and many
+    of them: every row's alpha and beta contribution once, in both precisions."""
+    spec = mk(n).with_basis(wl.BASIS_SZ, n // 2)
+    m = hp.Model.from_spec(spec)
+    v0 = wl.gaussian_vector(n + L, m.dim)[:, 0]
+    a, b = oracle.lanczos(spec, v0, 6)
+    for prec, tol in ((hp.FP64, 1e-12), (hp.FP32, 1e-5)):
+        m.set_sector_split(prec, L, K)
+        for _ in range(2):
+            r = m.lanczos(6, prec=prec, v0=torch.as_tensor(v0))
+            assert _rel(r["alpha"], a) < tol and _rel(r["beta"], b) < tol
+
+
 # ----------------------------------------------------------------------------- short vectors
 @pytest.mark.parametrize("n,nu,nd", [(3, 1, 0), (4, 2, 2), (8, 4, 4), (9, 4, 4), (10, 3, 4)])
 @pytest.mark.parametrize("scale", [1.0, 2.0**900, 2.0**-900])
