@@ -40,9 +40,7 @@ METRIC = "H·v Gelem/s & %HBM peak; Lanczos/mTPQ steps/s, FP64 vs mixed+batched 
 FALLBACK_HBM_GBS = 6800.0
 # DRAM bytes (read + write) per fused H v launch group from an ncu capture of the current
 # kernels, with where they come from; absent where no capture of the current kernels exists
-MEASURED_TRAFFIC = {("heisenberg_6x6_sz0", "fp64"): (1_001_300_000_000, "ncu capture at full size (1-pass DRAM "
-                                                       "counters): k_sec_hi + k_sec_lo of one step after the "
-                                                       "first, split (15, 2), 1 KB pass-H stripes")}
+MEASURED_TRAFFIC = {}
 # fp64 FMA throughput of this machine's GB300 from a throughput probe (thread-level T op/s); the
 # chip issues fp64 at 1/64 of its fp32 rate
 FP64_PEAK_TOPS = 0.50
@@ -147,9 +145,12 @@ def hv_group_name(spec, m, prec, nvec, what):
     import paper_1703_03637_gb300 as hp
     kind = "spin" if spec.kind == wl.SPIN else "hubbard"
     if kind == "hubbard" and not m.is_complex:
-        ks = "k_maxexp + k_quant + k_hub_dn + k_hub_up_q" if prec == hp.FP64 else "k_hub_dn + k_hub_up"
+        ks = "k_maxexp + k_quant + k_hub_dn + k_hub_up" if prec == hp.FP64 else "k_hub_dn + k_hub_up"
     elif kind == "spin" and spec.basis == wl.BASIS_FULL and nvec in (32, 64, 128, 256):
-        ks = "k_maxexp_cols + k_quant_cols + k_hv_batch" if prec == hp.FP64 else "k_hv_batch"
+        if spec.n_sites >= 16:  # enough tiles for the tile passes
+            ks = "k_maxexp_cols + k_hv_tile" if prec == hp.FP64 else "k_hv_tile"
+        else:
+            ks = "k_maxexp_cols + k_quant_cols + k_hv_batch" if prec == hp.FP64 else "k_hv_batch"
     else:
         ks = "k_hv_hub" if kind == "hubbard" else "k_hv_spin"
     return f"{ks} ({what})"
@@ -390,7 +391,7 @@ def hv_group_kernels(spec, m, prec):
                     "previous pass 2 wrote; k_maxexp + k_quant in the first step only)")
         return "k_sec_hi + k_sec_lo (split-row H v fused with Lanczos pass 1)"
     if spec.kind == wl.HUBBARD and not m.is_complex and prec == hp.FP64:
-        return ("k_hub_dn + k_hub_up_q (two-pass H v fused with Lanczos pass 1, on the int64 copy that the "
+        return ("k_hub_dn + k_hub_up (two-pass H v fused with Lanczos pass 1, on the int64 copy that the "
                 "previous pass 2 wrote; k_maxexp + k_quant in the first step only)")
     return hv_group_name(spec, m, prec, 1, "Lanczos pass 1")
 
@@ -473,7 +474,7 @@ def run_hubbard_sub(args, world, local, rank):
             "lanczos_steps_per_s": round(W["steps"] / (ms_step / 1e3), 2), "e0": t["res"]["eig"][0],
             "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
                          "frac": round(achieved / hbm, 4), "traffic": traffic[0] if traffic else None,
-                         "kernel": "k_hub_dn + k_hub_up_q (Lanczos pass 1; k_maxexp + k_quant in the first step only)",
+                         "kernel": "k_hub_dn + k_hub_up (Lanczos pass 1; k_maxexp + k_quant in the first step only)",
                          "kernel_avg_ms": round(t["hv_avg_ms"], 4), "algorithmic_bytes_per_launch": D * 24},
             "autotune": tune, "gpu_launches": t["launches"], "clocks": t["clocks"]}
 
