@@ -899,8 +899,9 @@ hphi::Status hv_launch(hphi_model* m, int prec, const void* v, void* w, int nvec
 }
 
 // Times one plain H v of the split-row path for every candidate split (L, K) -- the default
-// low part and one or two bits fewer, each with every tile height that fits -- and keeps the
-// fastest for precision prec.  Tables of the losing candidates are freed.
+// low part at its tile height, half and twice that, and one bit more or fewer -- and keeps the
+// fastest for precision prec.  Tables of the losing candidates are freed.  Every height that fits
+// at four low parts (12 to 14 shapes) took 0.30 s instead of 0.12 s on the 6x5 torus.
 hphi::Status sec_autotune(hphi_model* m, int prec, hphi_tune_result* res, cudaStream_t st) {
   const int pi = prec == HPHI_FP64 ? 0 : 1;
   const int esz = prec == HPHI_FP64 ? 8 : 4;
@@ -909,11 +910,13 @@ hphi::Status sec_autotune(hphi_model* m, int prec, hphi_tune_result* res, cudaSt
   if (L0 <= 0) return {};
   const std::array<int, 3> dflt = sec_shape(m, prec);
   std::vector<std::array<int, 3>> cand = {dflt};
-  for (int L = L0 + 1; L >= std::max(1, L0 - 2); --L) {
-    if (m->n_sites - L > hphi::kSecMaxH) break;
-    const int kmax = hphi::sec_tallest_K(m->sec_terms, L, esz);
-    for (int K = 1; K <= kmax; K *= 2)
+  for (int L : {L0, L0 + 1, L0 - 1}) {
+    if (L < 1 || L >= m->n_sites || m->n_sites - L > hphi::kSecMaxH) continue;
+    const int K0 = hphi::sec_default_K(m->sec_terms, L, esz);
+    for (int K : {K0, K0 / 2, 2 * K0}) {
+      if (K < 1 || (L != L0 && K != K0)) continue;
       if (hphi::sec_fits(m->sec_terms, L, K, esz) && std::array<int, 3>{L, K, esz} != dflt) cand.push_back({L, K, esz});
+    }
   }
   hphi::Status s;
   if ((s = m->ws.vecA.ensure((size_t)esz * (size_t)m->dim)).code) return s;

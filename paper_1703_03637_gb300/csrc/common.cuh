@@ -421,10 +421,8 @@ struct SecTablesDeleter {
 bool sec_applicable(const SecTerms& t, int prec, std::string* why);
 // the split used when nothing else is asked for element size esz (0: no row fits a tile)
 int sec_default_L(const SecTerms& t, int esz);
-// tile rows K for low-part length L at element size esz: 16-byte tile entries if they fit, and
-// the tallest tile the autotuner tries
+// tile rows K for low-part length L at element size esz: 16-byte tile entries if they fit
 int sec_default_K(const SecTerms& t, int L, int esz);
-int sec_tallest_K(const SecTerms& t, int L, int esz);
 // K rows of the longest row of split L fit one tile at element size esz
 bool sec_fits(const SecTerms& t, int L, int K, int esz);
 Status sec_build(const SecTerms& t, int L, int K, int esz, SecTables** out, cudaStream_t st);

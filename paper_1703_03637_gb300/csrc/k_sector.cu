@@ -357,7 +357,6 @@ static int tallest(const SecTerms& t, int L, int esz, int kmax) {
 // a neighbour; taller tiles are left to the autotuner (8-byte elements stop at 4 rows: 8 int64
 // rows run out of registers)
 int sec_default_K(const SecTerms& t, int L, int esz) { return tallest(t, L, esz, 16 / esz); }
-int sec_tallest_K(const SecTerms& t, int L, int esz) { return tallest(t, L, esz, esz >= 8 ? 4 : 8); }
 
 // ====================================================================== device tables
 struct SecTables {
