@@ -720,21 +720,6 @@ __device__ __forceinline__ double cl_take(const double* slots, int ncta) {
   return __shfl_sync(0xffffffffu, v, 0);
 }
 
-// sqrt(x) and 1 / sqrt(x) to the last place or so in ten fp64 operations (x > 0): the fp32
-// reciprocal root, one third-order step, one residual step for the root
-__device__ __forceinline__ void cl_sqrt(double x, double& root, double& inv) {
-  const int hi = __double2hiint(x);
-  const int k = ((hi >> 20) - 1023) >> 1;  // x = m 4^k, m in [1, 4)
-  const double m = __hiloint2double(hi - (k << 21), __double2loint(x));
-  double y = (double)rsqrtf((float)m);
-  const double e = fma(-(m * y), y, 1.0);
-  y = fma(y * e, fma(0.375, e, 0.5), y);
-  double r = m * y;
-  r = fma(fma(-r, r, m), 0.5 * y, r);
-  root = r * __hiloint2double((k + 1023) << 20, 0);
-  inv = y * __hiloint2double((1023 - k) << 20, 0);
-}
-
 __device__ __forceinline__ unsigned cl_rank() {
   unsigned r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -920,13 +905,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_lz_cl(const SpinDev md, LzDev
     cl_sync();  // the new vector complete everywhere, sums of beta in their slots
     if (tid < 32) {
       const double ps = cl_take(s_slot[1], ncta);
-      double b, sn;
-      if (ps >= 2.2250738585072014e-308 && ps <= 1.7976931348623157e308) {
-        cl_sqrt(ps, b, sn);
-      } else {  // zero, subnormal, infinite or NaN
-        b = sqrt(ps);
-        sn = 1.0 / b;
-      }
+      const double b = sqrt(ps), sn = 1.0 / b;
       if (tid == 0) {
         const bool stop = !(b > brk * fmax(1.0, fabs(a)));
         s_done = stop ? 1 : 0;
