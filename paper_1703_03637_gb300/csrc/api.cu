@@ -761,7 +761,7 @@ const hphi::TilePlan* use_tile(hphi_model* m, int prec, int nvec, hphi::Epi epi)
 // S^z-sector spin model), else null.  The path also needs its scratch (sec_scratch_bytes).
 const hphi::SecDev* use_sec(hphi_model* m, int prec, int nvec, hphi::Epi epi) {
   if (m->kind != HPHI_SPIN_HALF || nvec != 1 || m->cplx_model) return nullptr;
-  if (epi == hphi::Epi::kRefine && prec != HPHI_FP64) return nullptr;
+  if ((epi == hphi::Epi::kRefine || epi == hphi::Epi::kShift) && prec != HPHI_FP64) return nullptr;
   return sec_find(m, prec);
 }
 
@@ -2054,7 +2054,7 @@ hphi::Status invit_impl(hphi_model* m, const hphi_invit_params* p, void* xv, hph
     if ((s = b->ensure(vb)).code) return s;
   void* scratch = nullptr;
   const size_t need = std::max(hv_scratch_bytes(m, HPHI_FP64, 1, hphi::Epi::kStore),
-                               hv_scratch_bytes(m, HPHI_FP64, 1, hphi::Epi::kRefine));
+                               hv_scratch_bytes(m, HPHI_FP64, 1, hphi::Epi::kShift));
   if (need && m->kind == HPHI_SPIN_HALF) {
     scratch = optional_scratch(m, need);
   } else if (need) {
@@ -2062,16 +2062,16 @@ hphi::Status invit_impl(hphi_model* m, const hphi_invit_params* p, void* xv, hph
     scratch = ws.work.p;
   }
   const int grid = hv_grid_for(m, 1, HPHI_FP64, hphi::Epi::kStore);
-  const int rgrid = hv_grid_for(m, 1, HPHI_FP64, hphi::Epi::kRefine);
+  const int rgrid = hv_grid_for(m, 1, HPHI_FP64, hphi::Epi::kShift);
   const int vgrid = launch_grid(n);
   if ((s = ws.partials.ensure(sizeof(double) * (size_t)std::max(rgrid, vgrid) * hphi::kMaxRedQ)).code) return s;
   // fixed-point paths: the slots through which the direction kernel hands the product its copy
   hphi::QSlots qs;
   if (scratch != nullptr && !cplx) {
-    if (use_hub_fast(m, HPHI_FP64, 1, hphi::Epi::kRefine))
+    if (use_hub_fast(m, HPHI_FP64, 1, hphi::Epi::kShift))
       qs = hphi::hub_qslots(m->hdev, scratch);
-    else if (sec_runs(m, HPHI_FP64, 1, hphi::Epi::kRefine, ws.work.bytes))
-      qs = hphi::sec_qslots(*use_sec(m, HPHI_FP64, 1, hphi::Epi::kRefine), HPHI_FP64, hphi::Epi::kRefine, scratch);
+    else if (sec_runs(m, HPHI_FP64, 1, hphi::Epi::kShift, ws.work.bytes))
+      qs = hphi::sec_qslots(*use_sec(m, HPHI_FP64, 1, hphi::Epi::kShift), HPHI_FP64, hphi::Epi::kShift, scratch);
   }
   const bool qnext = qs.Q != nullptr;
   if ((s = ws.scal.ensure(sizeof(double) * 18)).code) return s;
@@ -2100,8 +2100,9 @@ hphi::Status invit_impl(hphi_model* m, const hphi_invit_params* p, void* xv, hph
   hphi::FusedArgs flagged;
   flagged.done = cg.done;  // H p of a solve that has converged is skipped
   flagged.partials = partials;
+  flagged.scal = cg.s + 4;  // delta - E
   const int hvk = hv_kernels(m, HPHI_FP64, 1, hphi::Epi::kStore);
-  const int hvr = hv_kernels(m, HPHI_FP64, 1, hphi::Epi::kRefine);
+  const int hvr = hv_kernels(m, HPHI_FP64, 1, hphi::Epi::kShift);
   int done_h = 0;
   for (int outer = 0; outer < p->outer; ++outer) {
     HPHI_CUDA_TRY(cudaMemsetAsync(cg.done, 0, sizeof(int), st));
@@ -2112,10 +2113,10 @@ hphi::Status invit_impl(hphi_model* m, const hphi_invit_params* p, void* xv, hph
     if ((s = hphi::launch_cg_fin(cg, 0, partials, vgrid, nullptr, st)).code) return s;
     launches += hvk + 2;
     for (int it = 0; it < p->max_cg; ++it) {
-      // H p with <p, H p> and <p, p>; from the second iteration on the quantised copy is ready
+      // H p with <p, A p>; from the second iteration on the quantised copy is ready
       flagged.out = q;
       flagged.exp_ready = qnext && it > 0 ? 2 : 0;
-      if ((s = hv_launch(m, HPHI_FP64, pp, nullptr, 1, hphi::Epi::kRefine, flagged, rgrid, scratch, st)).code) return s;
+      if ((s = hv_launch(m, HPHI_FP64, pp, nullptr, 1, hphi::Epi::kShift, flagged, rgrid, scratch, st)).code) return s;
       if ((s = hphi::launch_cg_fin(cg, 1, partials, rgrid, qs.ep, st)).code) return s;
       if ((s = hphi::launch_cg_update(cg, 1, nullptr, y, rr, pp, q, n, partials, vgrid, qs.ep, st)).code) return s;
       int* ec_new = qnext ? qs.ec[(it + 1) & 1] : nullptr;

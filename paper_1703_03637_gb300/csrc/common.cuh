@@ -255,12 +255,13 @@ Status launch_philox_raw(const uint32_t* ctr, const uint32_t* key, uint32_t* out
 Status launch_random(void* v, int64_t n_elem, bool cplx, bool f64, uint64_t seed, cudaStream_t st);
 
 // H v and fused solver kernels (k_hv.cu) -----------------------------------------------
-enum class Epi { kStore = 0, kLanczos1 = 1, kTpq = 2, kRefine = 3 };
+enum class Epi { kStore = 0, kLanczos1 = 1, kTpq = 2, kRefine = 3, kShift = 4 };
 
 struct FusedArgs {
   // Lanczos pass 1: P <- c1 * Y - c2 * P; partial sum of self * Y.
   // TPQ: Xn <- inv[c] * (l * X - Y / Ns); partial sums <X, Y>, |Y|^2 per column.
-  // Refine: stores Y and reduces <x, Y>, <x, x>.
+  // Refine: stores Y and reduces <x, Y>, <x, x>, <Y, Y>.
+  // Shift (fp64): stores Y and reduces <x, Y + c x>, c = scal[0].
   void* out = nullptr;             // P (Lanczos) / X_{k+1} (TPQ) / Hx (refine)
   const void* in = nullptr;        // Lanczos: previous vector read by pass 1 (null: same as out)
   const double* scal = nullptr;    // device scalars read at kernel start

@@ -163,7 +163,7 @@ __device__ __forceinline__ R opaque(R x) {
 
 template <class R>
 struct EpiScalars {
-  R c1, c2;  // Lanczos pass 1
+  R c1, c2;  // Lanczos pass 1; c1: the shift c
   R l, ins;  // mTPQ: l and 1 / N_s
 };
 
@@ -173,6 +173,8 @@ __device__ __forceinline__ EpiScalars<R> epi_scalars(const FusedArgs& fa) {
   if constexpr (E == Epi::kLanczos1) {
     es.c1 = opaque((R)fa.scal[0]);
     es.c2 = opaque((R)fa.scal[1]);
+  } else if constexpr (E == Epi::kShift) {
+    es.c1 = opaque((R)fa.scal[0]);
   } else if constexpr (E == Epi::kTpq) {
     es.l = opaque((R)fa.l);
     es.ins = opaque((R)fa.inv_ns);
@@ -214,6 +216,13 @@ __device__ __forceinline__ void epilogue(int64_t idx, typename Traits<S>::R sr, 
       red.add(1, hi, hi);
     }
     red.tick();
+  } else if constexpr (E == Epi::kShift) {
+    // H x stored; partial <x, (H + c) x>, element by element: with x near an eigenvector the sums of
+    // <x, H x> and c <x, x> would cancel, and their roundings with them be all that is left
+    st<S>(reinterpret_cast<S*>(fa.out), idx, hr, hi);
+    red.add(0, sr, fma(es.c1, sr, hr));
+    if constexpr (C) red.add(0, si, fma(es.c1, si, hi));
+    red.tick();
   } else {  // kRefine: Hx stored; partials <x, Hx>, <x, x>, <Hx, Hx>
     st<S>(reinterpret_cast<S*>(fa.out), idx, hr, hi);
     red.add(0, sr, hr);
@@ -239,6 +248,14 @@ __device__ __forceinline__ void refine_folded(double hvu, double xr, double s_e2
   red.add(2, hvu, hvu);
 }
 
+// The shifted product's element in folded units; cs = c 2^-k, hv = hvu 2^(eoff + k), x = xr 2^eoff.
+template <int NQ>
+__device__ __forceinline__ void shift_folded(double hvu, double xr, double cs, double s_e2, int64_t idx,
+                                             const FusedArgs& fa, Red<true, NQ>& red) {
+  reinterpret_cast<double*>(fa.out)[idx] = hvu * s_e2;
+  red.add(0, xr, fma(cs, xr, hvu));
+}
+
 // A sum of folded products back in plain units: quantity 0 is x hv, 1 x x and 2 hv hv.
 __device__ __forceinline__ double folded_sum(double x, int q, double s_eoff, double s_e2) {
   const double a = q == 2 ? s_e2 : s_eoff, b = q == 1 ? s_eoff : s_e2;
@@ -246,7 +263,7 @@ __device__ __forceinline__ double folded_sum(double x, int q, double s_eoff, dou
 }
 
 template <Epi E> __host__ __device__ constexpr int n_red() {
-  return E == Epi::kStore ? 0 : (E == Epi::kLanczos1 ? 1 : (E == Epi::kTpq ? 2 : 3));
+  return E == Epi::kStore ? 0 : (E == Epi::kLanczos1 || E == Epi::kShift ? 1 : (E == Epi::kTpq ? 2 : 3));
 }
 
 }  // namespace hphi

@@ -644,6 +644,7 @@ int batch_grid(int prec, bool cplx, int nvec, Epi epi, int64_t dim) {
     case Epi::kLanczos1: b = occupancy_e<Epi::kLanczos1>(prec, cplx, nvec); break;
     case Epi::kTpq: b = occupancy_e<Epi::kTpq>(prec, cplx, nvec); break;
     case Epi::kRefine: b = occupancy_e<Epi::kRefine>(HPHI_FP64, cplx, nvec); break;
+    case Epi::kShift: break;
   }
   const int64_t need = (dim + kThreads / 32 - 1) / (kThreads / 32);
   return (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)num_sms() * b));
@@ -665,6 +666,7 @@ Status launch_batch(const SpinDev& md, const BatchPlan* plan, int prec, bool cpl
     case Epi::kRefine:
       if (prec != HPHI_FP64) break;
       return launch_e<Epi::kRefine>(md, plan, prec, cplx, v, w, scratch, nvec, fa, grid, st);
+    case Epi::kShift: break;  // one vector only
   }
   return {HPHI_ERR_INVALID_ARG, "batched rows: unsupported precision / epilogue"};
 }

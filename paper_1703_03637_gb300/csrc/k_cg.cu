@@ -5,9 +5,9 @@
 // Hermitian, so Re <u, A v> is the inner product CG needs).  Besides the caller's vector the
 // solve keeps four: the iterate y, the residual r, the direction p and q = A p.
 //
-// A p = H p + c p (c = delta - E) is never formed by itself: H p comes with <p, H p> and <p, p>
-// from the refinement epilogue, <p, A p> = <p, H p> + c <p, p>, and the residual update adds c p
-// where it reads p anyway.  On the fixed-point paths the direction kernel also writes the next
+// A p = H p + c p (c = delta - E) is never stored: H p comes with <p, (H + c) p>, summed element
+// by element, from the product's shift epilogue, and the residual update adds c p where it reads p
+// anyway.  On the fixed-point paths the direction kernel also writes the next
 // product's quantised copy, on a scale bounded before the pass from the largest exponents of r
 // and p (as the Lanczos pass 2 does), so the product needs neither scan nor quantisation.
 // 32 iterations on 24 sites (2.7 million rows) on GB300: 5.6 ms instead of 6.3 ms with a scan, a
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kThreads) k_cg_fin(CgDev cg, int mode, const d
   __shared__ double sm[kThreads];
   if ((mode == 1 || mode == 2) && *cg.done) return;
   const double s0 = cg_sum(partials, grid, 0, sm);
-  const double s1 = (mode <= 1 || mode == 4) ? cg_sum(partials, grid, 1, sm) : 0.0;
+  const double s1 = (mode == 0 || mode == 4) ? cg_sum(partials, grid, 1, sm) : 0.0;
   if (threadIdx.x != 0) return;
   if (clear != nullptr) *clear = 0;
   if (mode == 0) {
@@ -210,12 +210,11 @@ __global__ void __launch_bounds__(kThreads) k_cg_fin(CgDev cg, int mode, const d
     cg.s[3] = s1;
     *cg.done = (s0 <= cg.s[5] * s1) ? 1 : 0;
   } else if (mode == 1) {
-    const double pap = fma(cg.s[4], s1, s0);  // <p, H p> + c <p, p>
-    if (!(pap > 0.0)) {  // A is positive definite on a non-zero p: only p = 0 gives this
+    if (!(s0 > 0.0)) {  // A is positive definite on a non-zero p: only p = 0 gives this
       *cg.done = 1;
       return;
     }
-    cg.s[1] = cg.s[0] / pap;
+    cg.s[1] = cg.s[0] / s0;
   } else if (mode == 2) {
     cg.s[2] = s0 / cg.s[0];
     cg.s[0] = s0;

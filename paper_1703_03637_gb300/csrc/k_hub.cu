@@ -480,6 +480,8 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_hub_up(const HubDe
               }
             } else if constexpr (E == Epi::kRefine) {
               refine_folded(hvu, __ll2double_rn(xq), s_e2, idx, fa, red);
+            } else if constexpr (E == Epi::kShift) {
+              shift_folded(hvu, __ll2double_rn(xq), es.c1 * r_k, s_e2, idx, fa, red);
             }
             continue;
           }
@@ -530,6 +532,8 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_hub_up(const HubDe
             red.tick();
           } else if constexpr (E == Epi::kRefine) {
             refine_folded(hvu, xr, s_e2, idx, fa, red);
+          } else if constexpr (E == Epi::kShift) {
+            shift_folded(hvu, xr, es.c1 * r_k, s_e2, idx, fa, red);
           }
         } else {
           const double x = fix_to_double(xq, eoff);
@@ -704,6 +708,7 @@ int upq_grid(const HubDev& md, Epi epi) {
     case Epi::kLanczos1: occ = up_occupancy<long long, KK, Epi::kLanczos1>(md); break;   \
     case Epi::kTpq: occ = up_occupancy<long long, KK, Epi::kTpq>(md); break;             \
     case Epi::kRefine: occ = up_occupancy<long long, KK, Epi::kRefine>(md); break;       \
+    case Epi::kShift: occ = up_occupancy<long long, KK, Epi::kShift>(md); break;         \
   }
   if (K == 2) { HPHI_OCCQ(2) } else { HPHI_OCCQ(1) }
 #undef HPHI_OCCQ
@@ -741,6 +746,7 @@ int up_grid_r(const HubDev& md, Epi epi) {
     case Epi::kLanczos1: occ = up_occupancy<R, KK, Epi::kLanczos1>(md); break; \
     case Epi::kTpq: occ = up_occupancy<R, KK, Epi::kTpq>(md); break;           \
     case Epi::kRefine: occ = up_occupancy<R, KK, Epi::kRefine>(md); break;     \
+    case Epi::kShift: break;                                                   \
   }
   if (k == 4) { HPHI_OCC(4) } else if (k == 2) { HPHI_OCC(2) } else { HPHI_OCC(1) }
 #undef HPHI_OCC
@@ -830,7 +836,7 @@ bool hub_fast_ok(const HubDev& md, int prec, bool cplx, int nvec, Epi epi) {
   if (!md.fast || cplx || nvec != 1) return false;
   // fixed-point sums of at most 127 terms (|q| < 2^56) stay exact in 64 bits
   if (prec == HPHI_FP64 && md.maxdeg_up + md.maxdeg_dn > 126) return false;
-  if (epi == Epi::kRefine && prec != HPHI_FP64) return false;
+  if ((epi == Epi::kRefine || epi == Epi::kShift) && prec != HPHI_FP64) return false;
   return hub_up_row_fits(md, prec);
 }
 
@@ -885,13 +891,15 @@ Status launch_hub_fast(const HubDev& md0, int prec, const void* v, void* w, void
       case Epi::kLanczos1: return launch_q<Epi::kLanczos1>(md, v, w, scratch, fa, grid_up, st);
       case Epi::kTpq: return launch_q<Epi::kTpq>(md, v, w, scratch, fa, grid_up, st);
       case Epi::kRefine: return launch_q<Epi::kRefine>(md, v, w, scratch, fa, grid_up, st);
+      case Epi::kShift: return launch_q<Epi::kShift>(md, v, w, scratch, fa, grid_up, st);
     }
   } else {
     switch (epi) {
       case Epi::kStore: return launch_r<float, Epi::kStore>(md, v, w, scratch, fa, grid_up, st);
       case Epi::kLanczos1: return launch_r<float, Epi::kLanczos1>(md, v, w, scratch, fa, grid_up, st);
       case Epi::kTpq: return launch_r<float, Epi::kTpq>(md, v, w, scratch, fa, grid_up, st);
-      case Epi::kRefine: break;
+      case Epi::kRefine:
+      case Epi::kShift: break;
     }
   }
   return {HPHI_ERR_INVALID_ARG, "two-pass Hubbard path: unsupported precision / epilogue"};

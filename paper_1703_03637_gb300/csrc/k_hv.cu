@@ -624,6 +624,7 @@ int hv_resident_grid(bool hubbard, int prec, bool cplx, Epi epi) {
     case Epi::kLanczos1: b = occupancy_e<Epi::kLanczos1>(hubbard, prec, cplx); break;
     case Epi::kTpq: b = occupancy_e<Epi::kTpq>(hubbard, prec, cplx); break;
     case Epi::kRefine: b = occupancy_e<Epi::kRefine>(hubbard, HPHI_FP64, cplx); break;
+    case Epi::kShift: b = cplx ? occupancy_t<double2, Epi::kShift>(hubbard) : occupancy_t<double, Epi::kShift>(hubbard); break;
   }
   return num_sms() * b;
 }
@@ -647,6 +648,10 @@ Status launch_hv(bool hubbard, const void* md, int prec, bool cplx, const void* 
     case Epi::kRefine:
       if (prec != HPHI_FP64) return {HPHI_ERR_INVALID_ARG, "refinement runs in fp64"};
       return launch_e<Epi::kRefine>(hubbard, md, prec, cplx, v, w, nvec, fa, grid, scratch, st);
+    case Epi::kShift:
+      if (prec != HPHI_FP64) return {HPHI_ERR_INVALID_ARG, "refinement runs in fp64"};
+      return cplx ? launch_t<double2, Epi::kShift>(hubbard, md, v, w, nvec, fa, grid, scratch, st)
+                  : launch_t<double, Epi::kShift>(hubbard, md, v, w, nvec, fa, grid, scratch, st);
   }
   return {HPHI_ERR_INVALID_ARG, "unknown epilogue"};
 }

@@ -913,7 +913,7 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
   for (int k = tid; k < kZero * K; k += NT) tile[(size_t)d.nq_max * K + k] = (T)0;  // entries unused slots read
   const EpiScalars<R> es = epi_scalars<R, E>(fa);
   const R inv = E == Epi::kTpq ? opaque((R)fa.scal[0]) : (R)0;
-  const double c1e = FIX ? (double)es.c1 * s_e2 : 0.0;
+  const double c1e = FIX ? (double)es.c1 * (E == Epi::kShift ? r_k : s_e2) : 0.0;  // c1 in folded units
   const R coef0 = opaque((R)d.coef[0]);
   const int n_str = d.n_str, n_cls = d.n_cls;
   const uint32_t str_mask = n_str < 32 ? (1u << n_str) - 1u : 0xffffffffu;
@@ -1149,6 +1149,8 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
               }
             } else if constexpr (E == Epi::kRefine) {
               refine_folded(hvu, __ll2double_rn(xq), s_e2, idx, fa, red);
+            } else if constexpr (E == Epi::kShift) {
+              shift_folded(hvu, __ll2double_rn(xq), c1e, s_e2, idx, fa, red);
             }
             continue;
           }
@@ -1166,6 +1168,8 @@ __global__ void __launch_bounds__(NT, (NT >= 1024) ? 1 : 2) k_sec_lo(const SecDe
               red.tick();
             } else if constexpr (E == Epi::kRefine) {
               refine_folded(hvu, xr, s_e2, idx, fa, red);
+            } else if constexpr (E == Epi::kShift) {
+              shift_folded(hvu, xr, c1e, s_e2, idx, fa, red);
             }
           } else {
             const double x = fix_to_double(xq, eoff);
@@ -1350,6 +1354,7 @@ int sec_grid(const SecDev& d, int prec, Epi epi) {
     case Epi::kLanczos1: occ = lo_occupancy_k<TT, Epi::kLanczos1>(d); break; \
     case Epi::kTpq: occ = lo_occupancy_k<TT, Epi::kTpq>(d); break;           \
     case Epi::kRefine: occ = lo_occupancy_k<TT, Epi::kRefine>(d); break;     \
+    case Epi::kShift: occ = lo_occupancy_k<long long, Epi::kShift>(d); break; \
   }
   if (prec == HPHI_FP64) { HPHI_SECOCC(long long) } else { HPHI_SECOCC(float) }
 #undef HPHI_SECOCC
@@ -1358,7 +1363,8 @@ int sec_grid(const SecDev& d, int prec, Epi epi) {
 
 Status launch_sec(const SecDev& d, int prec, const void* v, void* w, void* scratch, Epi epi, const FusedArgs& fa,
                   int grid, cudaStream_t st) {
-  if (epi == Epi::kRefine && prec != HPHI_FP64) return {HPHI_ERR_INVALID_ARG, "refinement runs in fp64"};
+  if ((epi == Epi::kRefine || epi == Epi::kShift) && prec != HPHI_FP64)
+    return {HPHI_ERR_INVALID_ARG, "refinement runs in fp64"};
   char* sc = static_cast<char*>(scratch);
   char* tail = sc + sec_scratch_bytes(d, prec, epi) - 256;
   int* Ep = reinterpret_cast<int*>(tail);
@@ -1383,6 +1389,7 @@ Status launch_sec(const SecDev& d, int prec, const void* v, void* w, void* scrat
       case Epi::kLanczos1: return launch_lo_k<long long, Epi::kLanczos1>(d, Q, W, w, fa, Ep, grid, claim, st);
       case Epi::kTpq: return launch_lo_k<long long, Epi::kTpq>(d, Q, W, w, fa, Ep, grid, claim, st);
       case Epi::kRefine: return launch_lo_k<long long, Epi::kRefine>(d, Q, W, w, fa, Ep, grid, claim, st);
+      case Epi::kShift: return launch_lo_k<long long, Epi::kShift>(d, Q, W, w, fa, Ep, grid, claim, st);
     }
   } else {
     const float* X = reinterpret_cast<const float*>(v);
@@ -1393,7 +1400,8 @@ Status launch_sec(const SecDev& d, int prec, const void* v, void* w, void* scrat
       case Epi::kStore: return launch_lo_k<float, Epi::kStore>(d, X, W, w, fa, Ep, grid, claim, st);
       case Epi::kLanczos1: return launch_lo_k<float, Epi::kLanczos1>(d, X, W, w, fa, Ep, grid, claim, st);
       case Epi::kTpq: return launch_lo_k<float, Epi::kTpq>(d, X, W, w, fa, Ep, grid, claim, st);
-      case Epi::kRefine: break;
+      case Epi::kRefine:
+      case Epi::kShift: break;
     }
   }
   return {HPHI_ERR_INVALID_ARG, "split-row path: unsupported precision / epilogue"};

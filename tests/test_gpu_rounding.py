@@ -30,3 +30,60 @@ def test_one_cluster_square_root_and_reciprocal():
             s = 1.0 / b
             assert r["alpha"][0] == 1.5 and r["beta"][0] == b, (h1, h2)
             assert r["alpha"][1] == xs * s * s, (h1, h2)
+
+
+# ----------------------------------------------------------------------------- inverse iteration
+def _product_state(h, excited):
+    """Amplitudes of the product eigenstate of -sum h_i . S_i with spin `excited` (or none) flipped
+    against its field, in long double; bit i of the index is spin i up."""
+    L = np.longdouble
+    v = np.ones(1, L)
+    for i, (hx, _, hz) in enumerate(h):
+        g = np.array([L(hx), np.sqrt(L(hx) ** 2 + L(hz) ** 2) + L(hz)], L)  # down, up
+        g /= np.sqrt((g * g).sum())
+        if i == excited:
+            g = np.array([-g[1], g[0]], L)
+        v = np.outer(g, v).ravel()
+    return v
+
+
+def _fields_times(h, x):
+    L = np.longdouble
+    out = np.zeros_like(x)
+    for i, (hx, _, hz) in enumerate(h):
+        a, o = x.reshape(-1, 2, 1 << i), out.reshape(-1, 2, 1 << i)
+        o[:, 0] += L(hz) / 2 * a[:, 0] - L(hx) / 2 * a[:, 1]
+        o[:, 1] -= L(hx) / 2 * a[:, 0] + L(hz) / 2 * a[:, 1]
+    return out
+
+
+@pytest.mark.parametrize("k", range(4))
+def test_inverse_iteration_step_next_to_an_eigenvalue(k):
+    """One CG step from b = e + zeta g, A e = e and A g = lambda g with lambda = 2^-30 of the size of
+    H: the direction is zeta g, so the step length is 1 / <g, A g> and the iterate shows it.
+    Each of the products p_i (A p)_i carries a rounding of |E| p_i, independent of the others:
+    an error of 2^-53 |E| (sum g^4)^(1/2) / lambda of the step; 16 times that is allowed.  The
+    difference of the sums <p, H p> and c <p, p> would err by 2^-53 |E| / lambda instead, 400 times
+    the root here."""
+    n, lam, zeta = 16, 2.0 ** -30 * (1 + k / 16), 2.0 ** -13
+    rng = np.random.default_rng(4)
+    ang = rng.uniform(-10, 10, n) * np.pi / 180
+    mag = np.concatenate([[1 - lam], rng.uniform(1.0, 1.5, n - 1)])
+    h = [(float(m * np.cos(a)), 0.0, float(m * np.sin(a))) for m, a in zip(mag, ang)]
+    L = np.longdouble
+    size = [np.sqrt(L(x) ** 2 + L(z) ** 2) for x, _, z in h]
+    e0 = -sum(size) / 2
+    g, e = _product_state(h, None), _product_state(h, 0)
+    b = (e + L(zeta) * g).astype(np.float64)
+    energy = float(e0 + size[0])  # c = 1 - energy puts e at one
+    c = L(1.0 - energy)
+    r = b - (_fields_times(h, b.astype(L)) + c * b)
+    step = (r @ r) / (r @ (_fields_times(h, r) + c * r))
+    m = hp.Model.from_spec(wl.ModelSpec(kind=wl.SPIN, n_sites=n, couplings=[], fields=list(enumerate(h)), name="fields"))
+    x = torch.as_tensor(b).cuda()
+    m.inverse_iteration(x, energy, shift=1.0, outer=1, max_cg=1)
+    x = x.cpu().numpy().astype(L)
+    t = (g @ x) / (e @ x)  # x ~ b + step r
+    got = (t * (e @ b) - g @ b) / (g @ r - t * (e @ r))
+    s4 = float(np.sqrt((g ** 4).sum()))
+    assert abs(got / step - 1) <= 16 * 2.0 ** -53 * abs(float(e0)) * s4 / lam
