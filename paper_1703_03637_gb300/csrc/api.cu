@@ -2065,15 +2065,14 @@ hphi::Status invit_impl(hphi_model* m, const hphi_invit_params* p, void* xv, hph
   const int rgrid = hv_grid_for(m, 1, HPHI_FP64, hphi::Epi::kShift);
   const int vgrid = launch_grid(n);
   if ((s = ws.partials.ensure(sizeof(double) * (size_t)std::max(rgrid, vgrid) * hphi::kMaxRedQ)).code) return s;
-  // fixed-point paths: the slots through which the direction kernel hands the product its copy
-  hphi::QSlots qs;
+  // fixed-point paths: the slot through which the direction kernel hands the product its exponent
+  int* emax = nullptr;
   if (scratch != nullptr && !cplx) {
     if (use_hub_fast(m, HPHI_FP64, 1, hphi::Epi::kShift))
-      qs = hphi::hub_qslots(m->hdev, scratch);
+      emax = hphi::hub_exponent_slot(m->hdev, scratch);
     else if (sec_runs(m, HPHI_FP64, 1, hphi::Epi::kShift, ws.work.bytes))
-      qs = hphi::sec_qslots(*use_sec(m, HPHI_FP64, 1, hphi::Epi::kShift), HPHI_FP64, hphi::Epi::kShift, scratch);
+      emax = hphi::sec_exponent_slot(*use_sec(m, HPHI_FP64, 1, hphi::Epi::kShift), HPHI_FP64, hphi::Epi::kShift, scratch);
   }
-  const bool qnext = qs.Q != nullptr;
   if ((s = ws.scal.ensure(sizeof(double) * 18)).code) return s;
   hphi::CgDev cg;
   cg.s = ws.scal.as<double>();
@@ -2109,24 +2108,19 @@ hphi::Status invit_impl(hphi_model* m, const hphi_invit_params* p, void* xv, hph
     // start: y = b, r = b - A b, p = r
     plain.out = q;
     if ((s = hv_launch(m, HPHI_FP64, x, q, 1, hphi::Epi::kStore, plain, grid, scratch, st)).code) return s;
-    if ((s = hphi::launch_cg_update(cg, 0, x, y, rr, pp, q, n, partials, vgrid, nullptr, st)).code) return s;
+    if ((s = hphi::launch_cg_update(cg, 0, x, y, rr, pp, q, n, partials, vgrid, st)).code) return s;
     if ((s = hphi::launch_cg_fin(cg, 0, partials, vgrid, nullptr, st)).code) return s;
     launches += hvk + 2;
     for (int it = 0; it < p->max_cg; ++it) {
-      // H p with <p, A p>; from the second iteration on the quantised copy is ready
+      // H p with <p, A p>; from the second iteration on the exponent is in the slot
       flagged.out = q;
-      flagged.exp_ready = qnext && it > 0 ? 2 : 0;
+      flagged.exp_ready = emax != nullptr && it > 0 ? 1 : 0;
       if ((s = hv_launch(m, HPHI_FP64, pp, nullptr, 1, hphi::Epi::kShift, flagged, rgrid, scratch, st)).code) return s;
-      if ((s = hphi::launch_cg_fin(cg, 1, partials, rgrid, qs.ep, st)).code) return s;
-      if ((s = hphi::launch_cg_update(cg, 1, nullptr, y, rr, pp, q, n, partials, vgrid, qs.ep, st)).code) return s;
-      int* ec_new = qnext ? qs.ec[(it + 1) & 1] : nullptr;
-      if ((s = hphi::launch_cg_fin(cg, 2, partials, vgrid, ec_new, st)).code) return s;
-      // E_p: the first product's scan left it in the copy's slot, which the direction kernel
-      // overwrites, so it is moved first; later what that kernel found
-      if (qnext && it == 0) HPHI_CUDA_TRY(cudaMemcpyAsync(qs.ec[0], qs.eq, sizeof(int), cudaMemcpyDeviceToDevice, st));
-      hphi::QNext qn{qs.Q, qs.eq, qs.ep, qs.ec[it & 1], qs.extra};
-      if ((s = hphi::launch_cg_dir(cg, rr, pp, n, vgrid, qnext ? &qn : nullptr, ec_new, st)).code) return s;
-      launches += hvr + 4 - (flagged.exp_ready ? 2 : 0);
+      if ((s = hphi::launch_cg_fin(cg, 1, partials, rgrid, nullptr, st)).code) return s;
+      if ((s = hphi::launch_cg_update(cg, 1, nullptr, y, rr, pp, q, n, partials, vgrid, st)).code) return s;
+      if ((s = hphi::launch_cg_fin(cg, 2, partials, vgrid, emax, st)).code) return s;
+      if ((s = hphi::launch_cg_dir(cg, rr, pp, n, vgrid, emax, st)).code) return s;
+      launches += hvr + 4 - (flagged.exp_ready ? 1 : 0);
       if (it % 16 == 15) {  // look at the flag now and then; the kernels skip work once it is set
         HPHI_CUDA_TRY(cudaMemcpyAsync(&done_h, cg.done, sizeof(int), cudaMemcpyDeviceToHost, st));
         HPHI_CUDA_TRY(cudaStreamSynchronize(st));

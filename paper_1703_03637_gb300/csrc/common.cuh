@@ -512,9 +512,8 @@ struct CgDev {
   int* steps;            // [1] CG iterations so far
 };
 Status launch_cg_update(const CgDev& cg, int mode, const double* b, double* y, double* r, double* p, const double* q,
-                        int64_t n, double* partials, int grid, int* er, cudaStream_t st);
-Status launch_cg_dir(const CgDev& cg, const double* r, double* p, int64_t n, int grid, const QNext* qn, int* ec_new,
-                     cudaStream_t st);
+                        int64_t n, double* partials, int grid, cudaStream_t st);
+Status launch_cg_dir(const CgDev& cg, const double* r, double* p, int64_t n, int grid, int* emax, cudaStream_t st);
 Status launch_cg_norm(const CgDev& cg, int mode, const double* y, double* x, int64_t n, double* partials, int grid,
                       cudaStream_t st);
 Status launch_cg_rq(const CgDev& cg, int mode, const double* x, const double* hx, int64_t n, double* partials,

@@ -7,11 +7,8 @@
 //
 // A p = H p + c p (c = delta - E) is never stored: H p comes with <p, (H + c) p>, summed element
 // by element, from the product's shift epilogue, and the residual update adds c p where it reads p
-// anyway.  On the fixed-point paths the direction kernel also writes the next
-// product's quantised copy, on a scale bounded before the pass from the largest exponents of r
-// and p (as the Lanczos pass 2 does), so the product needs neither scan nor quantisation.
-// 32 iterations on 24 sites (2.7 million rows) on GB300: 5.6 ms instead of 6.3 ms with a scan, a
-// quantisation and a separate shift pass per product (12 launches an iteration, now 8).
+// anyway.  On the fixed-point paths the direction kernel also finds the new direction's largest
+// exponent, so the next product quantises it on its own scale without a scan.
 //
 // Every kernel streams its vectors once with four elements per thread one grid stride apart
 // and leaves one fp64 partial sum per CTA; a one-CTA finaliser turns the partials into the
@@ -39,25 +36,16 @@ __device__ __forceinline__ void cg_partial(double acc, double* partials, int q) 
   if (threadIdx.x == 0) partials[(size_t)blockIdx.x * kMaxRedQ + q] = t;
 }
 
-// largest exponent field over the CTA's values into *slot
-__device__ __forceinline__ void cg_exponent(int mx, int* slot) {
-  mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)mx);
-  if ((threadIdx.x & 31) == 0 && mx > 0) atomicMax(slot, mx);
-}
-__device__ __forceinline__ int cg_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-
 // mode 0: start of a solve: y <- b, r <- b - A b (q = H b), p <- r; partials |r|^2, |b|^2
 // mode 1: y += alpha p, r -= alpha A p (q = H p); partial |r|^2
-// er (may be null): the largest exponent field of r
 __global__ void __launch_bounds__(kThreads) k_cg_update(CgDev cg, int mode, const double* __restrict__ b,
                                                          double* __restrict__ y, double* __restrict__ r,
                                                          double* __restrict__ p, const double* __restrict__ q,
-                                                         int64_t n, double* __restrict__ partials, int* er) {
+                                                         int64_t n, double* __restrict__ partials) {
   if (*cg.done) return;
   const double al = cg.s[1], c = cg.s[4];
   const int64_t stride = (int64_t)gridDim.x * kThreads;
   double rr = 0.0, bb = 0.0;
-  int mx = 0;
   for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < n; i += 4 * stride) {
     double a[4], qv[4], yv[4], rv[4];
 #pragma unroll
@@ -86,45 +74,17 @@ __global__ void __launch_bounds__(kThreads) k_cg_update(CgDev cg, int mode, cons
       }
       r[k] = t;
       rr = fma(t, t, rr);
-      mx = max(mx, cg_field(t));
     }
   }
-  if (er != nullptr) cg_exponent(mx, er);
   cg_partial(rr, partials, 0);
   if (mode == 0) cg_partial(bb, partials, 1);
 }
 
-// q = round(x 2^(1078 - E)), the rounding of the quantisation kernels
-__device__ __forceinline__ long long cg_quant(double x, int E) {
-  const int hi = __double2hiint(x);
-  const int ex = (hi >> 20) & 0x7ff;
-  long long q = 0;
-  if (ex != 0) {
-    const long long M = ((long long)((hi & 0xfffff) | 0x100000) << 32) | (long long)(unsigned)__double2loint(x);
-    const int sh = E - ex - 3;
-    if (sh <= 0) q = M << (-sh);
-    else if (sh < 62) q = (M + (1ll << (sh - 1))) >> sh;
-    if (hi < 0) q = -q;
-  }
-  return q;
-}
-
-// p <- r + beta p.  With qn.Q: also the next product's quantised copy.  |r + beta p| is below
-// 2^(E_r - 1022) + |beta| 2^(E_p - 1022), E_r and E_p the largest exponent fields of r and p, so
-// E = max(E_r, E_p + e_beta - 1022) + 1 bounds the new p's; its own goes into *ec_new.
+// p <- r + beta p; emax (may be null): the largest exponent field of the new p
 __global__ void __launch_bounds__(kThreads) k_cg_dir(CgDev cg, const double* __restrict__ r, double* __restrict__ p,
-                                                      int64_t n, QNext qn, int* ec_new) {
+                                                      int64_t n, int* emax) {
   if (*cg.done) return;
   const double be = cg.s[2];
-  int E = 0;
-  if (qn.Q != nullptr) {
-    const int eb = cg_field(be), ep = *qn.ec_cur;
-    E = *qn.ep;  // of r
-    if (eb != 0 && ep != 0) E = max(E, ep + eb - 1022);
-    E = min(E + 1, 2046);
-    if (blockIdx.x == 0 && threadIdx.x == 0) *qn.eq = E;
-    E += qn.extra;
-  }
   int mx = 0;
   const int64_t stride = (int64_t)gridDim.x * kThreads;
   for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < n; i += 4 * stride) {
@@ -141,11 +101,13 @@ __global__ void __launch_bounds__(kThreads) k_cg_dir(CgDev cg, const double* __r
       if (k >= n) break;
       const double t = fma(be, pv[u], rv[u]);
       p[k] = t;
-      mx = max(mx, cg_field(t));
-      if (qn.Q != nullptr) qn.Q[k] = cg_quant(t, E);
+      mx = max(mx, (__double2hiint(t) >> 20) & 0x7ff);
     }
   }
-  if (qn.Q != nullptr) cg_exponent(mx, ec_new);
+  if (emax != nullptr) {
+    mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)mx);
+    if ((threadIdx.x & 31) == 0 && mx > 0) atomicMax(emax, mx);
+  }
 }
 
 // x <- y / |y| (mode 0: partial |y|^2 first; mode 1: scale, the norm in s[9])
@@ -233,15 +195,14 @@ __global__ void __launch_bounds__(kThreads) k_cg_fin(CgDev cg, int mode, const d
 }  // namespace
 
 Status launch_cg_update(const CgDev& cg, int mode, const double* b, double* y, double* r, double* p, const double* q,
-                        int64_t n, double* partials, int grid, int* er, cudaStream_t st) {
-  k_cg_update<<<grid, kThreads, 0, st>>>(cg, mode, b, y, r, p, q, n, partials, er);
+                        int64_t n, double* partials, int grid, cudaStream_t st) {
+  k_cg_update<<<grid, kThreads, 0, st>>>(cg, mode, b, y, r, p, q, n, partials);
   HPHI_CUDA_TRY(cudaGetLastError());
   return {};
 }
 
-Status launch_cg_dir(const CgDev& cg, const double* r, double* p, int64_t n, int grid, const QNext* qn, int* ec_new,
-                     cudaStream_t st) {
-  k_cg_dir<<<grid, kThreads, 0, st>>>(cg, r, p, n, qn ? *qn : QNext{nullptr, nullptr, nullptr, nullptr, 0}, ec_new);
+Status launch_cg_dir(const CgDev& cg, const double* r, double* p, int64_t n, int grid, int* emax, cudaStream_t st) {
+  k_cg_dir<<<grid, kThreads, 0, st>>>(cg, r, p, n, emax);
   HPHI_CUDA_TRY(cudaGetLastError());
   return {};
 }

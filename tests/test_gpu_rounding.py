@@ -87,3 +87,47 @@ def test_inverse_iteration_step_next_to_an_eigenvalue(k):
     got = (t * (e @ b) - g @ b) / (g @ r - t * (e @ r))
     s4 = float(np.sqrt((g ** 4).sum()))
     assert abs(got / step - 1) <= 16 * 2.0 ** -53 * abs(float(e0)) * s4 / lam
+
+
+def test_inverse_iteration_iterate_in_extended_precision():
+    """Six CG steps on a split-row sector (12,870 rows) against the same recurrence in long double.
+    The products' input is quantised at 2^-57 of its largest element, at most 2^-53 of the typical
+    one here, so every operation errs by about one fp64 rounding; 16 of them per element, in the
+    root mean square over the vector, cover the six steps' four operations each (24^(1/2) = 5) with
+    the conditioning of the recurrence."""
+    n, steps, c = 16, 6, 0.1 + 0.4461935 * 16
+    spec = wl.heisenberg_ring(n).with_basis(wl.BASIS_SZ, n // 2)
+    m = hp.Model.from_spec(spec)
+    states = m.basis_states().cpu().numpy()
+    rank = np.zeros(1 << n, dtype=np.int64)
+    rank[states] = np.arange(len(states))
+    L = np.longdouble
+    diag, pairs = np.zeros(len(states), L), []
+    for i in range(n):
+        j = (i + 1) % n
+        anti = ((states >> i) ^ (states >> j)) & 1
+        diag += np.where(anti, L(-0.25), L(0.25))
+        rows = np.nonzero(anti)[0]
+        pairs.append((rows, rank[states[rows] ^ (1 << i) ^ (1 << j)]))
+
+    def product(x):
+        out = (diag + L(1.0 - (1.0 - c))) * x
+        for rows, partner in pairs:
+            out[rows] += x[partner] / 2
+        return out
+
+    b = np.random.default_rng(11).standard_normal(len(states))
+    y = b.astype(L)
+    r = y - product(y)
+    p = r.copy()
+    for _ in range(steps):
+        q = product(p)
+        rr = r @ r
+        al = rr / (p @ q)
+        y = y + al * p
+        r = r - al * q
+        p = r + (r @ r) / rr * p
+    x = torch.as_tensor(b).cuda()
+    m.inverse_iteration(x, 1.0 - c, shift=1.0, outer=1, max_cg=steps)
+    err = x.cpu().numpy().astype(L) - y / np.sqrt(y @ y)
+    assert float(np.sqrt(err @ err)) <= 16 * 2.0 ** -53
