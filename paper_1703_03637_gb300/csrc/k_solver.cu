@@ -10,6 +10,7 @@
 
 #include "common.cuh"
 #include "reduce.cuh"
+#include "squares.cuh"
 
 namespace hphi {
 

@@ -87,29 +87,4 @@ __device__ __forceinline__ double widen(float f) {
 }
 __device__ __forceinline__ double widen(double x) { return x; }
 
-// Sum of the squares of N fp32 values as fp64.  In fp64 each value would cost a conversion and a
-// multiply-add, at 1/64 of the fp32 rate; instead the squares are summed in one fp32 pair (exact
-// products, TwoSum) that is converted once.  The pair's rounding, about 2^-48 of the group with
-// random sign, averages out over the groups: over 2^30 values the total is as close to the exact
-// sum as the plain fp64 one.  Groups whose squares leave the fp32 range take the fp64 sum.
-template <int N>
-__device__ __forceinline__ double sum_squares(const float* x) {
-  float hi = 0.f, lo = 0.f;
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    const float p = __fmul_rn(x[k], x[k]);
-    const float e = fmaf(x[k], x[k], -p);
-    const float t = __fadd_rn(hi, p);
-    const float z = __fsub_rn(t, hi);
-    const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(p, z));
-    hi = t;
-    lo = __fadd_rn(lo, __fadd_rn(err, e));
-  }
-  if (hi > 1e-24f && hi < 1e37f) return (double)hi + (double)lo;
-  double s = 0.0;
-#pragma unroll 1
-  for (int k = 0; k < N; ++k) s = fma((double)x[k], (double)x[k], s);
-  return s;
-}
-
 }  // namespace hphi
