@@ -142,9 +142,13 @@ HPHI_HD uint64_t gauss_numerator(uint64_t k) {
 
 // sqrt(-2 ln(A / 2^54)) = rad 2^-62 2^ex, rad in [2^62, 2^63) (0 for A = 2^54)
 HPHI_HD uint64_t gauss_radius(uint64_t A, const GaussTables& t, int& ex) {
+  if (A >> 54) {  // u = 1: no logarithm to normalise
+    ex = 0;
+    return 0;
+  }
   const int nz = clz64(A);
   const int n = nz - 9;                                    // u = m 2^-n, m = M / 2^53 in [1, 2)
-  const uint64_t M = A << (nz - 10 < 0 ? 0 : nz - 10) >> (nz - 10 < 0 ? 1 : 0);
+  const uint64_t M = A << (nz - 10);
   const uint32_t j = ((uint32_t)(M >> 44) + 1) / 2 - 256;  // nearest centre 1 + j / 256
   const int64_t r0 = (int64_t)(M * t.rc[j] - (1ull << 63));  // r, Q63, exact
   const int64_t r = r0 * 128;                              // Q70
@@ -158,11 +162,7 @@ HPHI_HD uint64_t gauss_radius(uint64_t A, const GaussTables& t, int& ex) {
   const int64_t g = mulhi_s(r, h2);                                      // r h2, Q69
   uint64_t X;  // -ln u = X 2^-q
   int q;
-  if (n == 1 && j == 256) {  // n ln 2 - ln c_j = 0 and r <= 0
-    if (r0 == 0) {
-      ex = 0;
-      return 0;
-    }
+  if (n == 1 && j == 256) {  // n ln 2 - ln c_j = 0 and r < 0
     const int s = clz64((uint64_t)(-r0)) - 1;
     const int64_t rn = -r0 * (int64_t)(1ull << s);  // |r|, Q(63 + s), below 2^63
     X = (uint64_t)rn + (uint64_t)(mulhi_s(rn, -g) >> 5);

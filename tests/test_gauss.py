@@ -70,3 +70,21 @@ def test_pairs_against_extended_precision(pairs, what):
         # (2^-52.4 of the radius), below it the series is relative; cos and sin 2^-60
         bound = 0.5 * np.spacing(np.abs(ref).astype(np.float64)) + L(2) ** -52 * np.abs(rad)
         assert np.all(np.abs(got.astype(L) - ref) <= bound)
+
+
+def test_pairs_stay_inside_the_language(tmp_path):
+    """Every 53-bit word is defined behaviour, the one that rounds to u = 1 (radius zero) included;
+    the largest word below it is not."""
+    top = (1 << 53) - 1
+    words = [0, 1, top, top - 1, top - 2, 1 << 52, (1 << 52) - 1, 12345678901]
+    main = SRC + "#include <cstdio>\nint main() { const uint64_t w[] = {" + ", ".join(f"{w}ull" for w in words) + "};\n" \
+        "  for (uint64_t a : w) for (uint64_t b : w) { double g[2]; pairs(&a, &b, g, g + 1, 1);" \
+        " std::printf(\"%d\", (g[0] != 0) + 2 * (g[1] != 0)); } }\n"
+    (tmp_path / "m.cpp").write_text(main)
+    exe = str(tmp_path / "m")
+    subprocess.run(["g++", "-O1", "-std=c++17", "-fsanitize=undefined", "-fno-sanitize-recover=undefined", "-I", CSRC, "-o", exe, str(tmp_path / "m.cpp")], check=True)
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0 and not r.stderr, r.stderr
+    n = len(words)
+    zero = [set(r.stdout[n * k:n * k + n]) == {"0"} for k in range(n)]
+    assert zero == [w == top for w in words]
