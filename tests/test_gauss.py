@@ -72,6 +72,26 @@ def test_pairs_against_extended_precision(pairs, what):
         assert np.all(np.abs(got.astype(L) - ref) <= bound)
 
 
+@pytest.mark.parametrize("what", ["uniform", "ends", "centres", "angles"])
+def test_pairs_relative_to_each_number(pairs, what):
+    """Each number within 3 2^-53 of itself: the final rounding, half of the 2^-52 by which the
+    logarithm may be off, and 2^-60 of the radius on components of at least pi / 256 (0.64 2^-53);
+    components next to an axis keep their relative accuracy."""
+    if np.finfo(np.longdouble).nmant < 63:
+        pytest.skip("long double is no wider than double here")
+    a = _edges(what)
+    for b in (a[::-1].copy(), np.roll(a, 7)):
+        L = np.longdouble
+        ua, ub = ((x.astype(np.float64) + 0.5).astype(L) / L(2) ** 53 for x in (a, b))
+        rad = np.sqrt(-2 * np.log1p(ua - 1))
+        quad = np.rint(4 * ub)
+        x = (ub - quad / 4) * (2 * L("3.14159265358979323846264338327950288"))
+        c, s = np.cos(x), np.sin(x)
+        q = quad.astype(int) % 4
+        for got, ref in zip(pairs(a, b), (rad * np.choose(q, [c, -s, -c, s]), rad * np.choose(q, [s, c, -s, -c]))):
+            assert np.all(np.abs(got.astype(L) - ref) <= 3 * L(2) ** -53 * np.abs(ref))
+
+
 def test_pairs_stay_inside_the_language(tmp_path):
     """Every 53-bit word is defined behaviour, the one that rounds to u = 1 (radius zero) included;
     the largest word below it is not."""
