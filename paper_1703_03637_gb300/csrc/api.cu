@@ -394,6 +394,7 @@ hphi::Status compile_spin(hphi_model* m, cudaStream_t st) {
       tp.pass[p].n_ent = th.e0[p + 1] - th.e0[p];
       tp.pass[p].dep = m->d_tile_dep[k].as<uint32_t>() + (size_t)p * 1024;
       tp.pass[p].t = 8 + k;
+      tp.pass[p].holes = th.holes[p];
       memcpy(tp.pass[p].pos, th.pos[p], sizeof(th.pos[p]));
     }
   }

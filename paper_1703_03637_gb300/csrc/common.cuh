@@ -361,6 +361,7 @@ constexpr int kTileMaxEntries = 128;  // terms of one pass
 constexpr int kTilePerRow4 = 1;       // TileEntry::flags: the phase depends on which of 4 rows,
 constexpr int kTilePerRow8 = 2;       // or of 8 rows, of a thread,
 constexpr int kTileReal = 4;          // the class coefficient and the phase are real
+constexpr int kTileLive = 4;          // bit kTileLive + b_i + 2 b_j: the element is not zero there
 struct TileEntry {
   uint32_t lmask;    // flipped sites as local row bits
   uint16_t phases;   // as in SpinEntry
@@ -374,6 +375,7 @@ struct TilePass {
   const TileEntry* ents = nullptr;
   const uint32_t* dep = nullptr;  // [4][256] visit-index byte -> row bits (the set's sites first)
   int n_ent = 0, t = 0, first = 0;
+  int holes = 0;                  // some entry's element is zero for some settings of its bits
   uint8_t pos[12] = {};           // local row bit -> site
 };
 struct TilePlan {
@@ -383,6 +385,7 @@ struct TilePlan {
 struct TileHost {                 // a plan's tables before their upload
   int n_pass = 0, max_run = 0;
   int e0[kMaxPasses + 1] = {};
+  int holes[kMaxPasses] = {};
   uint8_t pos[kMaxPasses][12] = {};
   std::vector<TileEntry> ents;
   std::vector<uint32_t> dep;

@@ -16,7 +16,8 @@
 // four high ones number its rows, which share their columns, and for most terms their phase.
 // A warp's partner reads are XOR images of its own consecutive units, so they never conflict.
 //
-// fp32 multiplies each value by its phase times the class coefficient.  fp64 quantises the rows
+// fp32 multiplies each value by its phase times the class coefficient; where the element is zero it
+// reads a zero unit behind the tile, so an infinity stays in the rows coupled to it.  fp64 quantises the rows
 // while staging them (one scale per column, q = round(x 2^(1078 - E_c))), sums each class's run
 // exactly in 64-bit integers and converts once per class and pass.
 //
@@ -36,6 +37,7 @@ namespace hphi {
 namespace {
 
 constexpr int kTileUnits = 4096;     // units of 16 bytes per tile
+constexpr int kTileBytes = kTileUnits * 16;  // a zero unit follows
 constexpr int kTileSteps = kTileUnits / kThreads;  // rows per thread
 static_assert(kTileSteps == 16, "a thread's rows are numbered by four local bits");
 constexpr int kTileRows = 1024;      // most rows per tile (U >= 4)
@@ -124,7 +126,8 @@ __device__ __forceinline__ R tile_diag(const SpinDev& md, uint32_t s) {
   return d;
 }
 
-template <class S, Epi E, bool LAST>
+// HOLES (fp32): some entry of the pass is zero for some settings of its bits
+template <class S, Epi E, bool LAST, bool HOLES>
 __global__ void __launch_bounds__(kThreads, 3)
     k_hv_tile(const SpinDev md, const TilePass tp, const S* __restrict__ v, S* out, int nvec, FusedArgs fa,
               const int* __restrict__ Ec) {
@@ -141,6 +144,7 @@ __global__ void __launch_bounds__(kThreads, 3)
   if (fa.done != nullptr && *fa.done) return;
   const int tid = threadIdx.x;
   const int ne = tp.n_ent;
+  if (tid < 4) reinterpret_cast<uint32_t*>(smem_raw + kTileBytes)[tid] = 0u;
   for (int k = tid; k < ne; k += kThreads) s_ent[k] = tp.ents[k];
   if constexpr (!F64) {
     for (int k = tid; k < ne * 4; k += kThreads) {
@@ -286,13 +290,14 @@ __global__ void __launch_bounds__(kThreads, 3)
           cur = en.cls;
         }
         T x[NR][NW];
+        const uint32_t sel = ((sg >> en.i) & 1u) | (((sg >> en.j) & 1u) << 1);
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
-          const uint32_t o = (g0 + (uint32_t)r * kstride) ^ (en.lmask << (4 + lgU));
+          uint32_t o = (g0 + (uint32_t)r * kstride) ^ (en.lmask << (4 + lgU));
+          if (HOLES && !((en.flags >> (kTileLive + (sel ^ tile_flip(en, r)))) & 1)) o = (uint32_t)kTileBytes;
           const uint4 p = *reinterpret_cast<const uint4*>(tb + o);
           memcpy(&x[r][0], &p, 16);
         }
-        const uint32_t sel = ((sg >> en.i) & 1u) | (((sg >> en.j) & 1u) << 1);
         const bool per_row = (en.flags & (NR == 8 ? kTilePerRow8 : kTilePerRow4)) != 0;
         if constexpr (!F64) {
           const float2* tab = s_ph[n];
@@ -375,16 +380,24 @@ __global__ void __launch_bounds__(kThreads, 3)
   }
 }
 
-constexpr size_t kTileSmem = (size_t)kTileUnits * 16;
+constexpr size_t kTileSmem = kTileBytes + 16;
+
+template <class S, Epi E, bool LAST, bool HOLES>
+Status launch_holes(const SpinDev& md, const TilePass& tp, const void* v, void* out, int nvec, const FusedArgs& fa,
+                   int grid, const int* Ec, cudaStream_t st) {
+  HPHI_CUDA_TRY(cudaFuncSetAttribute(k_hv_tile<S, E, LAST, HOLES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmem));
+  k_hv_tile<S, E, LAST, HOLES><<<grid, kThreads, kTileSmem, st>>>(md, tp, reinterpret_cast<const S*>(v),
+                                                           reinterpret_cast<S*>(out), nvec, fa, Ec);
+  HPHI_CUDA_TRY(cudaGetLastError());
+  return {};
+}
 
 template <class S, Epi E, bool LAST>
 Status launch_pass(const SpinDev& md, const TilePass& tp, const void* v, void* out, int nvec, const FusedArgs& fa,
                    int grid, const int* Ec, cudaStream_t st) {
-  HPHI_CUDA_TRY(cudaFuncSetAttribute(k_hv_tile<S, E, LAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmem));
-  k_hv_tile<S, E, LAST><<<grid, kThreads, kTileSmem, st>>>(md, tp, reinterpret_cast<const S*>(v),
-                                                           reinterpret_cast<S*>(out), nvec, fa, Ec);
-  HPHI_CUDA_TRY(cudaGetLastError());
-  return {};
+  if constexpr (!Traits<S>::kF64)
+    if (tp.holes) return launch_holes<S, E, LAST, true>(md, tp, v, out, nvec, fa, grid, Ec, st);
+  return launch_holes<S, E, LAST, false>(md, tp, v, out, nvec, fa, grid, Ec, st);
 }
 
 template <class S>
@@ -486,10 +499,14 @@ bool batch_tile_plan(int n_sites, int t, const std::vector<SpinEntry>& ents, con
       e.phases = ents[k].phases;
       e.cls = ents[k].cls;
       bool real = true;
+      int live = e.i == e.j ? 6 : 0;  // (settings that a one-site term never reads)
       for (int s = 0; s < 4; ++s) {
         const int code = (ents[k].phases >> (3 * s)) & 7;
         real = real && (code == 0 || code == 1 || code == 3);
+        if (code) live |= 1 << s;
       }
+      e.flags |= (uint16_t)(live << kTileLive);
+      if (live != 15) out->holes[p] = 1;
       if (real && cls[ents[k].cls].y == 0.0) e.flags |= kTileReal;
       for (int b = 0; b < 3; ++b) {
         const int site = use[t - 4 + b].second;

@@ -131,3 +131,27 @@ def test_inverse_iteration_iterate_in_extended_precision():
     m.inverse_iteration(x, 1.0 - c, shift=1.0, outer=1, max_cg=steps)
     err = x.cpu().numpy().astype(L) - y / np.sqrt(y @ y)
     assert float(np.sqrt(err @ err)) <= 16 * 2.0 ** -53
+
+
+# ----------------------------------------------------------------------------- infinities in blocks of vectors
+@pytest.mark.parametrize("n,nvec,complex_", [(19, 16, False), (16, 64, False), (17, 16, True), (16, 64, True)])
+def test_infinity_stays_in_coupled_rows(n, nvec, complex_):
+    """An infinite amplitude in a single-precision block reaches the rows with a matrix element to
+    its own and no others: all others are bit for bit those of the block with a zero there."""
+    D = 0.3 if complex_ else 0.0
+    J = np.array([[1.0, D, 0.0], [-D, 1.0, 0.0], [0.0, 0.0, 0.7]])  # an exchange: zero on parallel spins
+    m = hp.Model.from_spec(wl.ModelSpec(kind=wl.SPIN, n_sites=n, couplings=[(i, (i + 1) % n, J) for i in range(n)],
+                                        name="exchange_ring"))
+    assert m.is_complex == complex_
+    g = torch.Generator().manual_seed(3)
+    v = torch.randn((m.dim, nvec), dtype=m.dtype(hp.FP32), generator=g).cuda()
+    row = int("0110100111010010110"[:n], 2)
+    coupled = [row] + [row ^ (1 << i) ^ (1 << ((i + 1) % n)) for i in range(n) if (row >> i ^ row >> ((i + 1) % n)) & 1]
+    v[row, 1] = 0
+    clean = m.apply_H(v)
+    v[row, 1] = float("inf")
+    w = m.apply_H(v)
+    rest = torch.ones(m.dim, dtype=torch.bool, device="cuda")
+    rest[coupled] = False
+    assert torch.equal(torch.view_as_real(w[rest]) if complex_ else w[rest], torch.view_as_real(clean[rest]) if complex_ else clean[rest])
+    assert not torch.isfinite(w[coupled, 1]).any()
