@@ -135,7 +135,7 @@ struct hphi_model {
   std::map<int, std::unique_ptr<WinCache>> win;
   // tile plans of the full basis for t = 8 .. 10 sites (built with the sector tables)
   hphi::TilePlan tile[3];
-  DBuf d_tile_ents[3], d_tile_dep[3];
+  DBuf d_tile_ents[3], d_tile_dep[3], d_tile_fix[3];
   // split-row path of real S^z-sector spin models: the compiled terms, whether each precision
   // may take the path, the split asked for per precision (-1 off, 0 default, else L) and
   // rows per tile (0 default), and the device tables built so far by (L, K, element size)
@@ -385,16 +385,21 @@ hphi::Status compile_spin(hphi_model* m, cudaStream_t st) {
     if (sector || !hphi::batch_tile_plan(N, 8 + k, ents, cls, &th)) continue;
     if ((s = upload(m->d_tile_ents[k], th.ents, st)).code) return s;
     if ((s = upload(m->d_tile_dep[k], th.dep, st)).code) return s;
+    if ((s = upload(m->d_tile_fix[k], th.fix, st)).code) return s;
     HPHI_CUDA_TRY(cudaStreamSynchronize(st));  // th dies here
     hphi::TilePlan& tp = m->tile[k];
     tp.n_pass = th.n_pass;
-    tp.max_run = th.max_run;
+    tp.f64 = th.f64;
     for (int p = 0; p < th.n_pass; ++p) {
       tp.pass[p].ents = m->d_tile_ents[k].as<hphi::TileEntry>() + th.e0[p];
       tp.pass[p].n_ent = th.e0[p + 1] - th.e0[p];
       tp.pass[p].dep = m->d_tile_dep[k].as<uint32_t>() + (size_t)p * 1024;
       tp.pass[p].t = 8 + k;
       tp.pass[p].holes = th.holes[p];
+      tp.pass[p].fix = m->d_tile_fix[k].as<longlong2>();
+      tp.pass[p].fix_shift = th.fix_shift;
+      tp.pass[p].fix_exp = th.fix_exp;
+      tp.pass[p].fix_half = th.fix_half;
       memcpy(tp.pass[p].pos, th.pos[p], sizeof(th.pos[p]));
     }
   }

@@ -17,16 +17,24 @@
 // A warp's partner reads are XOR images of its own consecutive units, so they never conflict.
 //
 // fp32 multiplies each value by its phase times the class coefficient; where the element is zero it
-// reads a zero unit behind the tile, so an infinity stays in the rows coupled to it.  fp64 quantises the rows
-// while staging them (one scale per column, q = round(x 2^(1078 - E_c))), sums each class's run
-// exactly in 64-bit integers and converts once per class and pass.
+// reads a zero unit behind the tile, so an infinity stays in the rows coupled to it.
+//
+// fp64 quantises the rows while staging them (one scale per column, q = round(x 2^(1078 - E_c))),
+// sums each class's run exactly in 64-bit integers and multiplies the sums by the class
+// coefficients in fixed point (high halves of 64 x 64-bit products, tile_fix).  The partial sums
+// stay integers from pass to pass; the last one converts once, so an element is rounded twice, in
+// the conversion and with the diagonal, whatever the number of classes and passes.
 //
 // Measured on GB300, one mTPQ step of 64 starts against the gather kernel: 2^24 rows c64 26.3 ms
 // instead of 49.4 ms (three passes; bound by shared-memory wavefronts, 73 %, with DRAM at 48 %),
 // 2^18 rows c128 1.81 ms instead of 1.99 ms (two passes; bound by the fp64 pipe, 64 to 76 %);
 // 16 starts, 2^24 rows c64 28.2 instead of 156 ms for four steps.
+#include <math.h>
+
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
+#include <vector>
 
 #include "common.cuh"
 #include "epilogue.cuh"
@@ -179,6 +187,7 @@ __global__ void __launch_bounds__(kThreads, 3)
   int eq[NC];
 #pragma unroll
   for (int q = 0; q < NC; ++q) eq[q] = F64 ? Ec[col + q] : 0;
+  using H = std::conditional_t<F64, long long, float>;  // a row's sums, fp64 in units of 2^(fix_exp + eq - 1078)
   const EpiScalars<R> es = epi_scalars<R, E>(fa);
   R inv[NC];
 #pragma unroll
@@ -225,12 +234,12 @@ __global__ void __launch_bounds__(kThreads, 3)
     if constexpr (!F64) asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     for (int k0 = 0; k0 < kTileSteps; k0 += NR) {
-      R hs[NR][F64 ? NW : 4];  // the row's sums: NW scalars (re, im pairs or columns)
+      H hs[NR][NW];  // the row's sums: NW scalars (re, im pairs or columns)
 #pragma unroll
       for (int r = 0; r < NR; ++r) {
         if (tp.first) {
 #pragma unroll
-          for (int e = 0; e < NW; ++e) hs[r][e] = (R)0;
+          for (int e = 0; e < NW; ++e) hs[r][e] = (H)0;
         } else {
           const uint4 p = __ldcs(reinterpret_cast<const uint4*>(out + (int64_t)(s0 | kbits(k0 + r)) * nvec + col));
           memcpy(&hs[r][0], &p, 16);
@@ -239,33 +248,15 @@ __global__ void __launch_bounds__(kThreads, 3)
       T ac[F64 ? NR : 1][2];
       auto flush = [&](int cls) {
         if constexpr (F64) {
-          // c 2^eoff is exact unless it leaves the normal range, so the sums need one conversion
-          // and one multiply-add each
-          const double2 cc = md.cls_coef[cls];
+          const longlong2 cf = __ldg(tp.fix + cls);
 #pragma unroll
-          for (int q = 0; q < NC; ++q) {
-            const int eo = eq[q] - 1078;
-            const double sc = eo >= -1022 ? __longlong_as_double((long long)(eo + 1023) << 52) : 0.0;
-            double cx = cc.x * sc, cy = cc.y * sc;
-            const bool slow = !(fabs(cx) >= 1e-290) || (cc.y != 0.0 && !(fabs(cy) >= 1e-290));
-            if (slow) {
-              cx = cc.x;
-              cy = cc.y;
-            }
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-              const double vr = slow ? fix_to_double(ac[r][C ? 0 : q], eo) : __ll2double_rn(ac[r][C ? 0 : q]);
-              if constexpr (C) {
-                const double vi2 = slow ? fix_to_double(ac[r][1], eo) : __ll2double_rn(ac[r][1]);
-                hs[r][0] = fma(cx, vr, hs[r][0]);
-                hs[r][1] = fma(cx, vi2, hs[r][1]);
-                if (cc.y != 0.0) {
-                  hs[r][0] = fma(-cy, vi2, hs[r][0]);
-                  hs[r][1] = fma(cy, vr, hs[r][1]);
-                }
-              } else {
-                hs[r][q] = fma(cx, vr, hs[r][q]);
-              }
+          for (int r = 0; r < NR; ++r) {
+            const long long v0 = ac[r][0] << tp.fix_shift, v1 = ac[r][1] << tp.fix_shift;
+            hs[r][0] += __mul64hi(v0, cf.x);
+            hs[r][1] += __mul64hi(v1, cf.x);
+            if (C && cf.y != 0) {
+              hs[r][0] += __mul64hi(v1, -cf.y);
+              hs[r][1] += __mul64hi(v0, cf.y);
             }
           }
 #pragma unroll
@@ -337,25 +328,32 @@ __global__ void __launch_bounds__(kThreads, 3)
             memcpy(x0, &p, 16);
           }
           const R d = s_d[lrow + ((k0 + r) << lb)];
+          R hv[NW];
 #pragma unroll
-          for (int e = 0; e < NW; ++e) hs[r][e] = fma(d, x0[e], hs[r][e]);
+          for (int e = 0; e < NW; ++e) {
+            if constexpr (F64) hv[e] = fma(d, x0[e], fix_to_double(hs[r][e] + tp.fix_half, eq[C ? 0 : e] + tp.fix_exp - 1078));
+            else hv[e] = fma(d, x0[e], hs[r][e]);
+          }
           if constexpr (E == Epi::kTpq) {
 #pragma unroll
             for (int e = 0; e < NW; ++e) {
               const int q = C ? e / 2 : e;
-              red[q].add(0, x0[e], hs[r][e]);
-              red[q].add(1, hs[r][e], hs[r][e]);
-              if constexpr (F64) hs[r][e] = fma(-in_[q], hs[r][e], il[q] * x0[e]);
-              else hs[r][e] = inv[q] * (es.l * x0[e] - hs[r][e] * es.ins);
+              red[q].add(0, x0[e], hv[e]);
+              red[q].add(1, hv[e], hv[e]);
+              if constexpr (F64) hv[e] = fma(-in_[q], hv[e], il[q] * x0[e]);
+              else hv[e] = inv[q] * (es.l * x0[e] - hv[e] * es.ins);
             }
 #pragma unroll
             for (int q = 0; q < NC; ++q) red[q].tick();
           }
+          uint4 p;
+          memcpy(&p, &hv[0], 16);
+          *reinterpret_cast<uint4*>(out + idx) = p;
+        } else {
+          uint4 p;
+          memcpy(&p, &hs[r][0], 16);
+          __stcs(reinterpret_cast<uint4*>(out + idx), p);
         }
-        uint4 p;
-        memcpy(&p, &hs[r][0], 16);
-        if constexpr (LAST) *reinterpret_cast<uint4*>(out + idx) = p;
-        else __stcs(reinterpret_cast<uint4*>(out + idx), p);
       }
     }
   }
@@ -423,6 +421,58 @@ Status launch_s(const SpinDev& md, const TilePlan& plan, const void* v, void* w,
 }
 
 }  // namespace
+
+// The integers of fp64.  A class sum S of a pass is below 2^56 times its longest run, so
+// S 2^shift fits 63 bits with shift = 7 - log2(run); the coefficients times 2^s fit 63 bits with
+// s = 62 - log2(c_max); and the sum of all products over 2^64 must stay below 2^62, which lowers
+// first the shift, then s.  A product is exact when the coefficient's trailing zeros and the shift
+// make up 64 bits (c = +-2^k), else its floor is half a unit low on average: fix_half makes up for
+// these.  Against the whole vector the
+// products' floors are below the rounding of the elements (rms over the norm, 18-site Heisenberg ring
+// in a field of 1e-3: 0.60 2^-53, the gather kernel 0.77); rows that only a coefficient c reaches lose a further c_max / (12 c) of
+// their own rounding, so models whose coefficients span more than 1,024 keep to the gather kernels.
+static void tile_fix(const std::vector<SpinEntry>& ents, const std::vector<double2>& cls, TileHost* out) {
+  double cmax = 0.0, cmin = 1e308, sum = 0.0;
+  for (const SpinEntry& e : ents) {
+    for (double c : {fabs(cls[e.cls].x), fabs(cls[e.cls].y)}) {
+      if (c == 0.0) continue;
+      cmax = std::max(cmax, c);
+      cmin = std::min(cmin, c);
+      sum += c;
+    }
+  }
+  int run = 1;
+  for (int p = 0; p < out->n_pass; ++p)
+    for (int k = out->e0[p], r = 0; k < out->e0[p + 1]; ++k) {
+      r = (k > out->e0[p] && out->ents[k].cls == out->ents[k - 1].cls) ? r + 1 : 1;
+      run = std::max(run, r);
+    }
+  out->fix.assign(cls.size(), longlong2{0, 0});
+  out->f64 = run <= 127 && cmax > 0.0 && cmin >= cmax / 1024 && cmax < 1e300 && cmin > 1e-290;
+  if (!out->f64) return;
+  const int lg = std::ilogb(cmax);
+  int s = 62 - lg, run2 = 0, sum2 = 0;
+  while ((1 << run2) < run) ++run2;
+  while (std::ldexp(cmax, sum2) < sum * 1.001) ++sum2;  // sum <= 2^(lg + 1 + sum2)
+  out->fix_shift = std::min(7 - run2, 7 - sum2);
+  if (out->fix_shift < 0) {
+    s += out->fix_shift;
+    out->fix_shift = 0;
+  }
+  out->fix_exp = 64 - s - out->fix_shift;
+  auto fixed = [&](double c, int* inexact) -> long long {
+    const long long v = std::llrint(std::ldexp(c, s));
+    if (v != 0 && __builtin_ctzll((unsigned long long)v) + out->fix_shift < 64) *inexact += 1;
+    return v;
+  };
+  std::vector<int> floors(cls.size(), 0);  // per component
+  for (size_t k = 0; k < cls.size(); ++k) out->fix[k] = longlong2{fixed(cls[k].x, &floors[k]), fixed(cls[k].y, &floors[k])};
+  int n = 0;
+  for (int p = 0; p < out->n_pass; ++p)
+    for (int k = out->e0[p]; k < out->e0[p + 1]; ++k)
+      if (k == out->e0[p] || out->ents[k].cls != out->ents[k - 1].cls) n += floors[out->ents[k].cls];
+  out->fix_half = n / 2;
+}
 
 // Covers the flip masks by site sets of at most t sites: the set grows by the mask that covers
 // most new masks per added site (ties: the one whose new sites fewest masks touch, which walks
@@ -534,12 +584,7 @@ bool batch_tile_plan(int n_sites, int t, const std::vector<SpinEntry>& ents, con
       }
   }
   out->e0[out->n_pass] = (int)out->ents.size();
-  out->max_run = 0;
-  for (int p = 0; p < out->n_pass; ++p)
-    for (int k = out->e0[p], run = 0; k < out->e0[p + 1]; ++k) {
-      run = (k > out->e0[p] && out->ents[k].cls == out->ents[k - 1].cls) ? run + 1 : 1;
-      out->max_run = std::max(out->max_run, run);
-    }
+  tile_fix(ents, cls, out);
   return true;
 }
 
@@ -568,7 +613,7 @@ const TilePlan* tile_choose(const TilePlan* plans, const SpinDev& md, int prec, 
   for (int t = 8; t <= 10; ++t) {
     const TilePlan& pl = plans[t - 8];
     if (pl.n_pass == 0 || (16 << (12 - t)) > nvec * esz) continue;
-    if (prec == HPHI_FP64 && pl.max_run > 127) continue;  // the exact-integer limit
+    if (prec == HPHI_FP64 && !pl.f64) continue;
     if (tile_count(md, t, nvec, esz) < 2 * num_sms()) continue;
     const double c = (3.0 * pl.n_pass - 1.0) * (t == 10 ? 1.1 : 1.0);
     if (c < bc) {
