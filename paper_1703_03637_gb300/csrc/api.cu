@@ -802,12 +802,13 @@ const hphi::BatchPlan* batch_plan(hphi_model* m, int prec, int nvec) {
   return it->second ? &it->second->plan : nullptr;
 }
 
-// kernels one hv_launch runs (for the launch counts the results report)
-int hv_kernels(hphi_model* m, int prec, int nvec, hphi::Epi epi) {
-  if (use_hub_fast(m, prec, nvec, epi)) return prec == HPHI_FP64 ? 4 : 2;  // (max-exponent, quantise,) D, U
+// kernels one hv_launch runs (for the launch counts the results report); exp_ready as in FusedArgs
+int hv_kernels(hphi_model* m, int prec, int nvec, hphi::Epi epi, int exp_ready = 0) {
+  const int quant = prec == HPHI_FP64 ? hphi::quant_kernels(m->dim, exp_ready) : 0;
+  if (use_hub_fast(m, prec, nvec, epi)) return quant + 2;  // D, U
   if (use_sec(m, prec, nvec, epi) && m->ws.work.p != nullptr &&
       m->ws.work.bytes >= hphi::sec_scratch_bytes(*use_sec(m, prec, nvec, epi), prec, epi))
-    return prec == HPHI_FP64 ? 4 : 2;  // (max-exponent, quantise,) pass H, pass R
+    return quant + 2;  // pass H, pass R
   if (const hphi::TilePlan* tp = use_tile(m, prec, nvec, epi)) return tp->n_pass + (prec == HPHI_FP64 ? 1 : 0);
   if (use_batch(m, nvec)) {
     const hphi::BatchPlan* plan = epi == hphi::Epi::kLanczos1 ? nullptr : batch_plan(m, prec, nvec);
@@ -1611,7 +1612,8 @@ hphi::Status lz_enqueue(LzPlan& L, cudaStream_t st) {
   const bool qnext = qs.Q != nullptr;
   auto run_pass = [&](bool with_x) -> hphi::Status {
     hphi::Status q;
-    L.launches += 2 + (3 + hv_kernels(m, prec, 1, hphi::Epi::kLanczos1)) * steps - (qnext ? 2 * (steps - 1) : 0);
+    L.launches += 2 + 3 * steps + hv_kernels(m, prec, 1, hphi::Epi::kLanczos1) +
+                  (steps - 1) * hv_kernels(m, prec, 1, hphi::Epi::kLanczos1, qnext ? 2 : 0);
     if ((q = hphi::launch_lz_init(prec, cplx, v0_dev, c0, p0, L.n_real, L.partials, L.vgrid, st)).code) return q;
     if ((q = hphi::launch_lz_init_fin(L.lz, L.partials, L.vgrid, st)).code) return q;
     if (with_x) HPHI_CUDA_TRY(cudaMemsetAsync(ws.x.p, 0, 8 * (size_t)L.n_real, st));
@@ -2107,7 +2109,6 @@ hphi::Status invit_impl(hphi_model* m, const hphi_invit_params* p, void* xv, hph
   flagged.partials = partials;
   flagged.scal = cg.s + 4;  // delta - E
   const int hvk = hv_kernels(m, HPHI_FP64, 1, hphi::Epi::kStore);
-  const int hvr = hv_kernels(m, HPHI_FP64, 1, hphi::Epi::kShift);
   int done_h = 0;
   for (int outer = 0; outer < p->outer; ++outer) {
     HPHI_CUDA_TRY(cudaMemsetAsync(cg.done, 0, sizeof(int), st));
@@ -2126,7 +2127,7 @@ hphi::Status invit_impl(hphi_model* m, const hphi_invit_params* p, void* xv, hph
       if ((s = hphi::launch_cg_update(cg, 1, nullptr, y, rr, pp, q, n, partials, vgrid, st)).code) return s;
       if ((s = hphi::launch_cg_fin(cg, 2, partials, vgrid, emax, st)).code) return s;
       if ((s = hphi::launch_cg_dir(cg, rr, pp, n, vgrid, emax, st)).code) return s;
-      launches += hvr + 4 - (flagged.exp_ready ? 1 : 0);
+      launches += hv_kernels(m, HPHI_FP64, 1, hphi::Epi::kShift, flagged.exp_ready) + 4;
       if (it % 16 == 15) {  // look at the flag now and then; the kernels skip work once it is set
         HPHI_CUDA_TRY(cudaMemcpyAsync(&done_h, cg.done, sizeof(int), cudaMemcpyDeviceToHost, st));
         HPHI_CUDA_TRY(cudaStreamSynchronize(st));

@@ -412,6 +412,8 @@ Status launch_maxexp_cols(const double* v, int64_t rows, int nvec, int ncomp, in
 // E the largest exponent field of x (computed into *Ep unless exp_ready), |q| < 2^(56 - extra)
 Status launch_quant_vec(const double* X, long long* Q, int64_t n, int* Ep, const int* done, bool exp_ready, int extra,
                         cudaStream_t st);
+// kernels that the copy takes for FusedArgs::exp_ready (2: none)
+int quant_kernels(int64_t n, int exp_ready);
 
 // Split-row spin-sector H v (k_sector.cu) ---------------------------------------------
 // The compiled terms of a real S^z-sector spin model, as the term compiler produced them.

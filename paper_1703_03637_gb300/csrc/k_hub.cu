@@ -801,6 +801,10 @@ Status launch_hub_store_noalloc(const HubDev& md0, const void* v, void* w, cudaS
   return launch_q<Epi::kStore>(md, v, w, scratch, fa, upq_grid(md, Epi::kStore), st);
 }
 
+int quant_kernels(int64_t n, int exp_ready) {
+  return exp_ready == 2 ? 0 : (exp_ready != 0 || n <= kShortQuant ? 1 : 2);
+}
+
 Status launch_quant_vec(const double* X, long long* Q, int64_t n, int* Ep, const int* done, bool exp_ready, int extra,
                         cudaStream_t st) {
   if (!exp_ready && n <= kShortQuant) {
