@@ -62,6 +62,19 @@ hphi::Status upload(DBuf& b, const std::vector<T>& v, cudaStream_t st) {
   return {};
 }
 
+// Several host tables in one device buffer: put() returns a table's offset, upload() copies them
+// all (one allocation and one copy instead of one of each per table).
+struct Pack {
+  std::vector<unsigned char> bytes;
+  template <class T>
+  size_t put(const std::vector<T>& v) {
+    const size_t at = bytes.size();
+    bytes.resize(at + (sizeof(T) * v.size() + 15) / 16 * 16);
+    if (!v.empty()) memcpy(bytes.data() + at, v.data(), sizeof(T) * v.size());
+    return at;
+  }
+};
+
 uint64_t binom_host(int n, int k) {
   if (k < 0 || k > n || n < 0) return 0;
   if (k > n - k) k = n - k;
@@ -115,7 +128,7 @@ struct hphi_model {
   std::string err;
   int device = 0;
   // device data
-  DBuf d_entries, d_merged, d_cls, d_lin, d_pairs, d_pcoef, d_hi_off, d_lo_rank, d_lo_list, d_lo_off;
+  DBuf d_terms, d_hi_off, d_lo_rank, d_lo_list, d_lo_off;
   DBuf d_nbr_up, d_deg_up, d_nbr_dn, d_deg_dn, d_npos_up, d_npos_dn, d_counter;
   DBuf d_up_rec[3], d_up_hdr[3];  // pass U gather tables by entry width
   hphi::SpinDev sdev{};
@@ -127,6 +140,10 @@ struct hphi_model {
   // window passes of the batched-row kernel: the compiled entries, the size setting
   // (-1 off, 0 sized from L2, else the window's sites) and the plans built so far by size
   std::vector<hphi::SpinEntry> host_entries;
+  // compiled Hubbard terms: hops (up first), classes and U groups
+  std::vector<hphi::HopEntry> host_hops;
+  std::vector<double2> host_cls;
+  std::vector<hphi::LinGroup> host_ulin;
   int win_bits_opt = -1;
   struct WinCache {
     DBuf ents, dep;
@@ -135,7 +152,6 @@ struct hphi_model {
   std::map<int, std::unique_ptr<WinCache>> win;
   // tile plans of the full basis for t = 8 .. 10 sites (built with the sector tables)
   hphi::TilePlan tile[3];
-  DBuf d_tile_ents[3], d_tile_dep[3], d_tile_fix[3];
   // split-row path of real S^z-sector spin models: the compiled terms, whether each precision
   // may take the path, the split asked for per precision (-1 off, 0 default, else L) and
   // rows per tile (0 default), and the device tables built so far by (L, K, element size)
@@ -362,45 +378,52 @@ hphi::Status compile_spin(hphi_model* m, cudaStream_t st) {
     return {HPHI_ERR_UNSUPPORTED, "too many distinct S^z S^z couplings"};
   std::stable_sort(pe.begin(), pe.end(), [](const hphi::PairEntry& x, const hphi::PairEntry& y) { return x.grp < y.grp; });
 
+  // one buffer: the generic tables, then entries, coefficients and visit orders of the tile plans
+  Pack pk;
+  const size_t o_ents = pk.put(ents), o_merged = pk.put(merged), o_cls = pk.put(cls), o_lin = pk.put(lg), o_pairs = pk.put(pe),
+               o_pc = pk.put(pc);
+  hphi::TileHost th[3];
+  size_t o_tile[3][3] = {};
+  for (int k = 0; k < 3; ++k) {
+    if (sector || !hphi::batch_tile_plan(N, 8 + k, ents, cls, &th[k])) {
+      th[k].n_pass = 0;
+      continue;
+    }
+    o_tile[k][0] = pk.put(th[k].ents);
+    o_tile[k][1] = pk.put(th[k].fix);
+    o_tile[k][2] = pk.put(th[k].dep);
+  }
   hphi::Status s;
-  if ((s = upload(m->d_entries, ents, st)).code) return s;
-  if ((s = upload(m->d_merged, merged, st)).code) return s;
-  if ((s = upload(m->d_cls, cls, st)).code) return s;
-  if ((s = upload(m->d_lin, lg, st)).code) return s;
-  if ((s = upload(m->d_pairs, pe, st)).code) return s;
-  if ((s = upload(m->d_pcoef, pc, st)).code) return s;
+  if ((s = upload(m->d_terms, pk.bytes, st)).code) return s;
+  HPHI_CUDA_TRY(cudaStreamSynchronize(st));  // pk dies here
+  const unsigned char* base = m->d_terms.as<unsigned char>();
   hphi::SpinDev& d = m->sdev;
   d = hphi::SpinDev{};
   d.n_sites = N;
   d.sector = sector ? 1 : 0;
   d.n_entries = (int)ents.size();
   d.n_merged = (int)merged.size();
-  d.merged = m->d_merged.as<hphi::SpinMerged>();
+  d.merged = reinterpret_cast<const hphi::SpinMerged*>(base + o_merged);
   d.max_run = max_run;
   m->host_entries = ents;
   m->win.clear();
   for (int k = 0; k < 3; ++k) {
     m->tile[k] = hphi::TilePlan{};
-    hphi::TileHost th;
-    if (sector || !hphi::batch_tile_plan(N, 8 + k, ents, cls, &th)) continue;
-    if ((s = upload(m->d_tile_ents[k], th.ents, st)).code) return s;
-    if ((s = upload(m->d_tile_dep[k], th.dep, st)).code) return s;
-    if ((s = upload(m->d_tile_fix[k], th.fix, st)).code) return s;
-    HPHI_CUDA_TRY(cudaStreamSynchronize(st));  // th dies here
     hphi::TilePlan& tp = m->tile[k];
-    tp.n_pass = th.n_pass;
-    tp.f64 = th.f64;
-    for (int p = 0; p < th.n_pass; ++p) {
-      tp.pass[p].ents = m->d_tile_ents[k].as<hphi::TileEntry>() + th.e0[p];
-      tp.pass[p].n_ent = th.e0[p + 1] - th.e0[p];
-      tp.pass[p].dep = m->d_tile_dep[k].as<uint32_t>() + (size_t)p * 1024;
-      tp.pass[p].t = 8 + k;
-      tp.pass[p].holes = th.holes[p];
-      tp.pass[p].fix = m->d_tile_fix[k].as<longlong2>();
-      tp.pass[p].fix_shift = th.fix_shift;
-      tp.pass[p].fix_exp = th.fix_exp;
-      tp.pass[p].fix_half = th.fix_half;
-      memcpy(tp.pass[p].pos, th.pos[p], sizeof(th.pos[p]));
+    tp.n_pass = th[k].n_pass;
+    tp.f64 = th[k].f64;
+    for (int p = 0; p < tp.n_pass; ++p) {
+      hphi::TilePass& q = tp.pass[p];
+      q.ents = reinterpret_cast<const hphi::TileEntry*>(base + o_tile[k][0]) + th[k].e0[p];
+      q.n_ent = th[k].e0[p + 1] - th[k].e0[p];
+      q.fix = reinterpret_cast<const longlong2*>(base + o_tile[k][1]);
+      q.dep = reinterpret_cast<const uint32_t*>(base + o_tile[k][2]) + (size_t)p * 1024;
+      q.t = 8 + k;
+      q.holes = th[k].holes[p];
+      q.fix_shift = th[k].fix_shift;
+      q.fix_exp = th[k].fix_exp;
+      q.fix_half = th[k].fix_half;
+      memcpy(q.pos, th[k].pos[p], sizeof(q.pos));
     }
   }
   d.n_classes = (int)cls.size();
@@ -408,11 +431,11 @@ hphi::Status compile_spin(hphi_model* m, cudaStream_t st) {
   d.n_pairs = (int)pe.size();
   d.n_pair_groups = (int)pc.size();
   d.c0 = c0;
-  d.entries = m->d_entries.as<hphi::SpinEntry>();
-  d.cls_coef = m->d_cls.as<double2>();
-  d.lin = m->d_lin.as<hphi::LinGroup>();
-  d.pairs = m->d_pairs.as<hphi::PairEntry>();
-  d.pair_coef = m->d_pcoef.as<double>();
+  d.entries = reinterpret_cast<const hphi::SpinEntry*>(base + o_ents);
+  d.cls_coef = reinterpret_cast<const double2*>(base + o_cls);
+  d.lin = reinterpret_cast<const hphi::LinGroup*>(base + o_lin);
+  d.pairs = reinterpret_cast<const hphi::PairEntry*>(base + o_pairs);
+  d.pair_coef = reinterpret_cast<const double*>(base + o_pc);
   m->cplx_model = cplx_model;
   m->sec_terms = hphi::SecTerms{};
   m->sec_tab.clear();
@@ -491,12 +514,12 @@ hphi::Status compile_hub(hphi_model* m, cudaStream_t st) {
   for (const cplx& c : ct.coefs) cls.push_back(make_double2(c.real(), c.imag()));
   std::vector<hphi::LinGroup> lin_all = ul;
   lin_all.insert(lin_all.end(), ml.begin(), ml.end());
+  Pack pk;
+  const size_t o_hops = pk.put(all), o_cls = pk.put(cls), o_lin = pk.put(lin_all), o_pairs = pk.put(pe), o_pc = pk.put(pc);
   hphi::Status s;
-  if ((s = upload(m->d_entries, all, st)).code) return s;
-  if ((s = upload(m->d_cls, cls, st)).code) return s;
-  if ((s = upload(m->d_lin, lin_all, st)).code) return s;
-  if ((s = upload(m->d_pairs, pe, st)).code) return s;
-  if ((s = upload(m->d_pcoef, pc, st)).code) return s;
+  if ((s = upload(m->d_terms, pk.bytes, st)).code) return s;
+  HPHI_CUDA_TRY(cudaStreamSynchronize(st));  // pk dies here
+  const unsigned char* base = m->d_terms.as<unsigned char>();
   hphi::HubDev& d = m->hdev;
   d = hphi::HubDev{};
   d.n_sites = N;
@@ -508,12 +531,15 @@ hphi::Status compile_hub(hphi_model* m, cudaStream_t st) {
   d.n_pairs = (int)pe.size();
   d.n_pair_groups = (int)pc.size();
   d.c0 = 0.0;
-  d.hops = m->d_entries.as<hphi::HopEntry>();
-  d.cls_coef = m->d_cls.as<double2>();
-  d.ulin = m->d_lin.as<hphi::LinGroup>();
-  d.mulin = m->d_lin.as<hphi::LinGroup>() + ul.size();
-  d.pairs = m->d_pairs.as<hphi::PairEntry>();
-  d.pair_coef = m->d_pcoef.as<double>();
+  d.hops = reinterpret_cast<const hphi::HopEntry*>(base + o_hops);
+  d.cls_coef = reinterpret_cast<const double2*>(base + o_cls);
+  d.ulin = reinterpret_cast<const hphi::LinGroup*>(base + o_lin);
+  d.mulin = d.ulin + ul.size();
+  d.pairs = reinterpret_cast<const hphi::PairEntry*>(base + o_pairs);
+  d.pair_coef = reinterpret_cast<const double*>(base + o_pc);
+  m->host_hops = all;
+  m->host_cls = cls;
+  m->host_ulin = ul;
   m->cplx_model = cplx_model;
   return {};
 }
@@ -543,7 +569,7 @@ hphi::Status hub_ensure_table(hphi_model* m, int prec, cudaStream_t st) {
   hphi::Status s;
   if ((s = m->d_up_rec[wi].ensure(sizeof(uint2) * (size_t)stride * (size_t)(slots / 4))).code) return s;
   if ((s = m->d_up_hdr[wi].ensure(sizeof(uint4) * (size_t)(stride / 32))).code) return s;
-  if ((s = hphi::build_gather_table(d.nbr_up, d.dim_up, d.deg_up, (int)d.dim_up, 31, 2, (int)d.dim_up, 4 << wi,
+  if ((s = hphi::build_gather_table(d.nbr_up, d.dim_up, d.deg_up, d.maxdeg_up, (int)d.dim_up, 31, 2, (int)d.dim_up, 4 << wi,
                                     m->d_up_rec[wi].as<uint2>(), stride, 0, slots, m->d_up_hdr[wi].as<uint4>(), st))
           .code)
     return s;
@@ -578,12 +604,8 @@ hphi::Status build_hub_fast(hphi_model* m, cudaStream_t st) {
     }
   }
   if (cnt[0] > 255 || cnt[1] > 255) return {};
-  std::vector<hphi::HopEntry> host(cnt[0] + cnt[1]);
-  if (!host.empty())
-    HPHI_CUDA_TRY(cudaMemcpyAsync(host.data(), d.hops, sizeof(hphi::HopEntry) * host.size(), cudaMemcpyDeviceToHost, st));
-  std::vector<double2> cc(std::max(1, d.n_classes));
-  HPHI_CUDA_TRY(cudaMemcpyAsync(cc.data(), d.cls_coef, sizeof(double2) * cc.size(), cudaMemcpyDeviceToHost, st));
-  HPHI_CUDA_TRY(cudaStreamSynchronize(st));
+  const std::vector<hphi::HopEntry>& host = m->host_hops;
+  const std::vector<double2>& cc = m->host_cls;
   for (int k = 0; k < (int)host.size(); ++k) {
     const int sp = k < cnt[0] ? 0 : 1;
     if (cls[sp] < 0) cls[sp] = host[k].cls;
@@ -617,11 +639,7 @@ hphi::Status build_hub_fast(hphi_model* m, cudaStream_t st) {
   d.up_stride = (d.dim_up + 31) / 32 * 32;
   for (int prec : {HPHI_FP64, HPHI_FP32})
     if ((s = hub_ensure_table(m, prec, st)).code) return s;
-  std::vector<hphi::LinGroup> ulin(d.n_ulin);
-  if (d.n_ulin)
-    HPHI_CUDA_TRY(cudaMemcpyAsync(ulin.data(), d.ulin, sizeof(hphi::LinGroup) * ulin.size(), cudaMemcpyDeviceToHost, st));
-  HPHI_CUDA_TRY(cudaStreamSynchronize(st));
-  d.dint = hub_diag_integer(d, ulin) ? 1 : 0;
+  d.dint = hub_diag_integer(d, m->host_ulin) ? 1 : 0;
   d.fast = 1;
   return {};
 }

@@ -298,12 +298,12 @@ size_t spin_scratch_bytes(const SpinDev& md, int prec, bool cplx, int nvec);
 int hv_grid(int nvec);  // upper bound of any H v grid (partials sizing)
 
 // Gather table of n states (k_gather.cu; layout in gather.cuh).  nbr[q * nbr_stride + k] is
-// term q < deg[k] of state k, target | phase << shift with phase < n_phase; zero0 is the index
+// term q < deg[k] <= max_deg of state k, target | phase << shift, phase < n_phase; zero0 is the index
 // of the first zero entry; entry_bytes (4, 8 or 16) the width of a staged entry.  State k's
 // records go to rec[group * stride + out0 + k], 32 states' header to hdr[(out0 + k) / 32];
 // out0 is a multiple of 32 and the table has room for max_slots slots and whole warps.
-Status build_gather_table(const uint32_t* nbr, int64_t nbr_stride, const uint8_t* deg, int n, int shift, int n_phase,
-                          int zero0, int entry_bytes, uint2* rec, int64_t stride, int64_t out0, int max_slots,
+Status build_gather_table(const uint32_t* nbr, int64_t nbr_stride, const uint8_t* deg, int max_deg, int n, int shift,
+                          int n_phase, int zero0, int entry_bytes, uint2* rec, int64_t stride, int64_t out0, int max_slots,
                           uint4* hdr, cudaStream_t st);
 
 // Two-pass Hubbard path (k_hub.cu): neighbour tables, and H v = diag + up hops (row tiles

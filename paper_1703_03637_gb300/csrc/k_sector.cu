@@ -677,7 +677,7 @@ Status sec_build(const SecTerms& t, int L, int K, int esz, SecTables** out, cuda
     const int n = (int)(d.lo_off[q + 1] - d.lo_off[q]);
     k_sec_nbr<<<(n + kThreads - 1) / kThreads, kThreads, 0, st>>>(g_list + d.lo_off[q], n, g_rank, g_ll, n_ll, g_nbr, g_deg);
     HPHI_CUDA_TRY(cudaGetLastError());
-    if ((s = build_gather_table(g_nbr, n, g_deg, n, 24, std::max(1, d.n_cls), d.nq_max, entry, rec, d.lo_stride,
+    if ((s = build_gather_table(g_nbr, n, g_deg, n_ll, n, 24, std::max(1, d.n_cls), d.nq_max, entry, rec, d.lo_stride,
                                 d.lo_pad[q], slots, hdr, st)).code)
       return s;
   }

@@ -484,54 +484,69 @@ bool batch_tile_plan(int n_sites, int t, const std::vector<SpinEntry>& ents, con
   out->dep.clear();
   out->n_pass = 0;
   if (t < 8 || t > 10 || n_sites < 13 || n_sites > 32 || ents.empty() || (int)ents.size() > 512) return false;
-  auto pc = [](uint64_t x) { return __builtin_popcountll(x); };
+  auto pc = [](uint32_t x) { return __builtin_popcount(x); };
+  // distinct masks of the entries not placed yet, in the entries' order, with their counts
+  uint32_t masks[512];
+  int counts[512], n_masks = 0;
+  for (const SpinEntry& e : ents) {
+    int k = 0;
+    while (k < n_masks && masks[k] != (uint32_t)e.mask) ++k;
+    if (k == n_masks) {
+      masks[n_masks] = (uint32_t)e.mask;
+      counts[n_masks++] = 0;
+    }
+    ++counts[k];
+  }
   std::vector<int> pass_of(ents.size(), -1);
-  size_t left = ents.size();
-  while (left) {
+  while (n_masks > 0) {
     if (out->n_pass >= kMaxPasses) return false;
-    uint64_t S = 0;
-    for (;;) {
+    uint32_t S = 0;
+    for (int cov0 = 0;;) {
       double bg = -1.0;
-      int bd = 0;
-      uint64_t bU = 0;
-      int cov0 = 0;
-      for (size_t k = 0; k < ents.size(); ++k) cov0 += pass_of[k] < 0 && (ents[k].mask & ~S) == 0;
+      int bd = 0, bc = 0;
+      uint32_t bU = 0;
       for (int near = S ? 1 : 0; near >= 0 && bg < 0.0; --near) {
-        for (size_t k = 0; k < ents.size(); ++k) {
-          const uint64_t U = S | ents[k].mask;
-          if (pass_of[k] >= 0 || U == S || pc(U) > t || (near && !(ents[k].mask & S))) continue;
+        for (int k = 0; k < n_masks; ++k) {
+          const uint32_t U = S | masks[k];
+          if (U == S || (near && !(masks[k] & S)) || pc(U) > t) continue;
+          const uint32_t out_of_U = ~U, added = U & ~S;
           int cov = 0, deg = 0;
-          for (size_t j = 0; j < ents.size(); ++j)
-            if (pass_of[j] < 0) {
-              cov += (ents[j].mask & ~U) == 0;
-              deg += (ents[j].mask & U & ~S) != 0;
-            }
+          for (int o = 0; o < n_masks; ++o) {
+            cov += (masks[o] & out_of_U) == 0u ? counts[o] : 0;
+            deg += (masks[o] & added) != 0u ? counts[o] : 0;
+          }
           const double gain = (double)(cov - cov0) / (pc(U) - pc(S));
           if (gain > bg || (gain == bg && deg < bd)) {
             bg = gain;
             bd = deg;
+            bc = cov;
             bU = U;
           }
         }
       }
       if (bg < 0.0) break;
       S = bU;
+      cov0 = bc;
     }
     if (S == 0) return false;  // a mask wider than t sites
     const int p = out->n_pass++;
     out->e0[p] = (int)out->ents.size();
     for (size_t k = 0; k < ents.size(); ++k)
-      if (pass_of[k] < 0 && (ents[k].mask & ~S) == 0) {
-        pass_of[k] = p;
-        --left;
+      if (pass_of[k] < 0 && ((uint32_t)ents[k].mask & ~S) == 0) pass_of[k] = p;
+    int kept = 0;
+    for (int k = 0; k < n_masks; ++k)
+      if (masks[k] & ~S) {
+        masks[kept] = masks[k];
+        counts[kept++] = counts[k];
       }
-    for (int b = 0; b < n_sites && pc(S) < t; ++b) S |= 1ull << b;  // whole tiles
+    n_masks = kept;
+    for (int b = 0; b < n_sites && pc(S) < t; ++b) S |= 1u << b;  // whole tiles
     // local positions: the four highest bits number a thread's rows, the first of them innermost,
     // so the sites that fewest of the pass's entries read go there (the phase is then the same
     // for a thread's rows), the least read first
     std::vector<std::pair<int, int>> use;
     for (int b = 0; b < n_sites; ++b)
-      if ((S >> b) & 1ull) {
+      if ((S >> b) & 1u) {
         int n = 0;
         for (size_t k = 0; k < ents.size(); ++k) n += pass_of[k] == p && (ents[k].i == b || ents[k].j == b);
         use.emplace_back(-n, b);
@@ -572,15 +587,13 @@ bool batch_tile_plan(int n_sites, int t, const std::vector<SpinEntry>& ents, con
     int pos[32], n = 0;
     for (int l = 0; l < t; ++l) pos[n++] = out->pos[p][l];
     for (int b = 0; b < n_sites; ++b)
-      if (!((S >> b) & 1ull)) pos[n++] = b;
+      if (!((S >> b) & 1u)) pos[n++] = b;
     const size_t d0 = out->dep.size();
     out->dep.resize(d0 + 1024, 0u);
     for (int byte = 0; byte < 4; ++byte)
-      for (int val = 0; val < 256; ++val) {
-        uint32_t r = 0;
-        for (int b = 0; b < 8; ++b)
-          if (((val >> b) & 1) && byte * 8 + b < n_sites) r |= 1u << pos[byte * 8 + b];
-        out->dep[d0 + byte * 256 + val] = r;
+      for (int val = 1; val < 256; ++val) {  // the value without its lowest bit, and that bit
+        const int bit = byte * 8 + __builtin_ctz((unsigned)val);
+        out->dep[d0 + byte * 256 + val] = out->dep[d0 + byte * 256 + (val & (val - 1))] | (bit < n_sites ? 1u << pos[bit] : 0u);
       }
   }
   out->e0[out->n_pass] = (int)out->ents.size();
