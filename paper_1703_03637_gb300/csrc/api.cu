@@ -162,6 +162,7 @@ struct hphi_model {
   int sec_hi_cols[2] = {0, 0};  // pass H columns per lane per precision (0: built-in)
   int sec_L0[2] = {0, 0};  // the default split of each precision
   std::map<std::array<int, 3>, std::unique_ptr<hphi::SecTables, hphi::SecTablesDeleter>> sec_tab;
+  hphi::SecHighCache sec_high;  // what sec_tab's entries share
 };
 
 namespace {
@@ -439,6 +440,7 @@ hphi::Status compile_spin(hphi_model* m, cudaStream_t st) {
   m->cplx_model = cplx_model;
   m->sec_terms = hphi::SecTerms{};
   m->sec_tab.clear();
+  m->sec_high.clear();
   m->sec_ok[0] = m->sec_ok[1] = false;
   if (sector && !cplx_model) {
     hphi::SecTerms& t = m->sec_terms;
@@ -662,7 +664,7 @@ hphi::Status sec_ensure(hphi_model* m, int prec, cudaStream_t st) {
   const std::array<int, 3> sh = sec_shape(m, prec);
   if (sh[0] == 0 || m->sec_tab.count(sh)) return {};
   hphi::SecTables* t = nullptr;
-  hphi::Status s = hphi::sec_build(m->sec_terms, sh[0], sh[1], sh[2], &t, st);
+  hphi::Status s = hphi::sec_build(m->sec_terms, sh[0], sh[1], sh[2], m->sec_high, &t, st);
   if (s.code) return s;
   m->sec_tab[sh].reset(t);
   return {};

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <map>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -439,7 +441,10 @@ int sec_default_L(const SecTerms& t, int esz);
 int sec_default_K(const SecTerms& t, int L, int esz);
 // K rows of the longest row of split L fit one tile at element size esz
 bool sec_fits(const SecTerms& t, int L, int K, int esz);
-Status sec_build(const SecTerms& t, int L, int K, int esz, SecTables** out, cudaStream_t st);
+// pass H's tables by its split hL, shared by the shapes of one model (12 bytes per high part)
+struct SecHigh;
+using SecHighCache = std::map<int, std::weak_ptr<SecHigh>>;
+Status sec_build(const SecTerms& t, int L, int K, int esz, SecHighCache& high, SecTables** out, cudaStream_t st);
 const SecDev& sec_dev(const SecTables* t);
 size_t sec_scratch_bytes(const SecDev& d, int prec, Epi epi);
 int sec_grid(const SecDev& d, int prec, Epi epi);

@@ -359,9 +359,19 @@ static int tallest(const SecTerms& t, int L, int esz, int kmax) {
 int sec_default_K(const SecTerms& t, int L, int esz) { return tallest(t, L, esz, 16 / esz); }
 
 // ====================================================================== device tables
+struct SecHigh {
+  uint32_t* cls = nullptr;  // SecDev::h_cls
+  uint64_t* off = nullptr;  // SecDev::h_off
+  ~SecHigh() {
+    if (cls) cudaFree(cls);
+    if (off) cudaFree(off);
+  }
+};
+
 struct SecTables {
   SecDev dev{};
   std::vector<void*> bufs;
+  std::shared_ptr<SecHigh> high;
 };
 
 void sec_free(SecTables* t) {
@@ -424,7 +434,7 @@ __global__ void k_sec_nbr(const uint32_t* __restrict__ list, int n, const uint32
 
 }  // namespace
 
-Status sec_build(const SecTerms& t, int L, int K, int esz, SecTables** out, cudaStream_t st) {
+Status sec_build(const SecTerms& t, int L, int K, int esz, SecHighCache& high, SecTables** out, cudaStream_t st) {
   *out = nullptr;
   Analysis a = analyse(t);
   if (!a.ok) return {HPHI_ERR_UNSUPPORTED, a.why};
@@ -662,16 +672,10 @@ Status sec_build(const SecTerms& t, int L, int K, int esz, SecTables** out, cuda
   uint8_t* g_deg = nullptr;
   uint2* rec = nullptr;
   uint4* hdr = nullptr;
-  uint32_t *h_cls = nullptr, *h_rank = nullptr;
-  uint64_t* h_off = nullptr;
-  const size_t n_h = (size_t)1 << d.hH;
   if ((s = room(&tmp, (size_t)std::max(1, n_ll) * nqmax, &g_nbr)).code) return s;
   if ((s = room(&tmp, nqmax, &g_deg)).code) return s;
-  if ((s = room(&tmp, n_h, &h_rank)).code) return s;
   if ((s = room(T.get(), (size_t)(slots / 4) * (size_t)d.lo_stride, &rec)).code) return s;
   if ((s = room(T.get(), (size_t)d.lo_stride / 32, &hdr)).code) return s;
-  if ((s = room(T.get(), n_h, &h_cls)).code) return s;
-  if ((s = room(T.get(), n_h, &h_off)).code) return s;
   const int entry = (int)(K * esz);
   for (int q = qmin; q <= qmax; ++q) {
     const int n = (int)(d.lo_off[q + 1] - d.lo_off[q]);
@@ -681,18 +685,27 @@ Status sec_build(const SecTerms& t, int L, int K, int esz, SecTables** out, cuda
                                 d.lo_pad[q], slots, hdr, st)).code)
       return s;
   }
-  {
+  T->high = high[d.hL].lock();
+  if (!T->high) {
+    T->high = std::make_shared<SecHigh>();
+    const size_t n_h = (size_t)1 << d.hH;
+    SecTables own;  // (its buffers pass to T->high)
+    uint32_t* h_rank = nullptr;
+    if ((s = room(&tmp, n_h, &h_rank)).code) return s;
+    if ((s = room(&own, n_h, &T->high->cls)).code) return s;
+    if ((s = room(&own, n_h, &T->high->off)).code) return s;
     std::vector<uint32_t> off(d.hH + 2, 0);
     for (int p = 0; p <= d.hH; ++p) off[p + 1] = off[p] + (uint32_t)binom_u(d.hH, p);
     if ((s = up(&tmp, off, &g_off, st)).code) return s;
     HPHI_CUDA_TRY(cudaStreamSynchronize(st));  // `off` dies here
-    if ((s = build_popcount_tables(d.hH, h_rank, h_cls, g_off, st)).code) return s;
-    if ((s = build_hi_offsets(d.hL, d.hH, n1, h_off, st)).code) return s;
+    if ((s = build_popcount_tables(d.hH, h_rank, T->high->cls, g_off, st)).code) return s;
+    if ((s = build_hi_offsets(d.hL, d.hH, n1, T->high->off, st)).code) return s;
+    high[d.hL] = T->high;
   }
   d.lo_rec = rec;
   d.lo_hdr = hdr;
-  d.h_cls = h_cls;
-  d.h_off = h_off;
+  d.h_cls = T->high->cls;
+  d.h_off = T->high->off;
   HPHI_CUDA_TRY(cudaStreamSynchronize(st));  // host vectors die here
   *out = T.release();
   return {};

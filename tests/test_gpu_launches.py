@@ -41,3 +41,22 @@ def test_launch_counts(mk, rows, quant):
     if m.kind == hp.HUBBARD:
         r = m.tpq(1, 3, l=8.0)
         assert r["launches"] == 1 + 2 + 3 * (quant + 2 + 1)
+
+
+def test_high_part_tables_are_shared():
+    """Pass H's tables (12 bytes for each of 2^22 high parts here) belong to the sector: neither the
+    second precision nor another split of the row pass adds a copy."""
+    def used():
+        torch.cuda.synchronize()
+        free, total = torch.cuda.mem_get_info()
+        return total - free
+
+    hp.Model.from_spec(wl.heisenberg_ring(18).with_basis(wl.BASIS_SZ, 2))  # the context's own memory
+    high = 12 << 22
+    before = used()
+    m = hp.Model.from_spec(wl.heisenberg_ring(34).with_basis(wl.BASIS_SZ, 4))
+    built = used()
+    assert high <= built - before < 2 * high
+    m.set_sector_split(hp.FP64, 15, 2)
+    m.set_sector_split(hp.FP32, 16, 1)
+    assert used() - built < high
