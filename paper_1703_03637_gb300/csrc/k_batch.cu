@@ -21,6 +21,7 @@
 
 #include "common.cuh"
 #include "epilogue.cuh"
+#include "quant.cuh"
 #include "reduce.cuh"
 
 namespace hphi {
@@ -131,20 +132,7 @@ __global__ void __launch_bounds__(kThreads) k_quant_cols(const double* __restric
                                                           const int* __restrict__ Ec) {
   for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kThreads) {
     const int c = (int)((i & ((1ll << lg_rowlen) - 1)) >> lg_ncomp);
-    const int E = Ec[c];
-    const double x = __ldg(X + i);
-    const int hi = __double2hiint(x);
-    const unsigned lo = (unsigned)__double2loint(x);
-    const int ex = (hi >> 20) & 0x7ff;
-    long long q = 0;
-    if (ex != 0) {
-      const long long M = ((long long)((hi & 0xfffff) | 0x100000) << 32) | (long long)lo;  // x = M 2^(ex-1075)
-      const int sh = E - ex - 3;                                                           // q = M 2^-sh
-      if (sh <= 0) q = M << (-sh);
-      else if (sh < 62) q = (M + (1ll << (sh - 1))) >> sh;
-      if (hi < 0) q = -q;
-    }
-    Q[i] = q;
+    Q[i] = quant_one(__ldg(X + i), Ec[c]);
   }
 }
 

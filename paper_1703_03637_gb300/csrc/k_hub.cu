@@ -20,6 +20,7 @@
 #include "common.cuh"
 #include "epilogue.cuh"
 #include "gather.cuh"
+#include "quant.cuh"
 #include "reduce.cuh"
 
 namespace hphi {
@@ -212,22 +213,6 @@ __global__ void __launch_bounds__(kThreads) k_maxexp(const double* __restrict__ 
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) mx = max(mx, __shfl_down_sync(0xffffffffu, mx, off));
   if ((threadIdx.x & 31) == 0 && mx > 0) atomicMax(E, mx);
-}
-
-// q = round(x 2^(1078 - E)), by integer operations on the bits of x
-__device__ __forceinline__ long long quant_one(double x, int E) {
-  const int hi = __double2hiint(x);
-  const unsigned lo = (unsigned)__double2loint(x);
-  const int ex = (hi >> 20) & 0x7ff;
-  long long q = 0;
-  if (ex != 0) {
-    const long long M = ((long long)((hi & 0xfffff) | 0x100000) << 32) | (long long)lo;  // x = M 2^(ex-1075)
-    const int sh = E - ex - 3;                                                           // q = M 2^-sh
-    if (sh <= 0) q = M << (-sh);
-    else if (sh < 62) q = (M + (1ll << (sh - 1))) >> sh;
-    if (hi < 0) q = -q;
-  }
-  return q;
 }
 
 // Exponent scan and quantisation of a short vector in one CTA: one launch instead of three (the

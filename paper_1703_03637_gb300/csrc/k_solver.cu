@@ -9,6 +9,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "quant.cuh"
 #include "reduce.cuh"
 #include "squares.cuh"
 
@@ -109,23 +110,6 @@ __global__ void __launch_bounds__(kThreads) k_lz_fin(LzDev lz, int mode, int k, 
 
 // P <- P - gamma C ; partial |P|^2 ; optionally x += xc * C (fp64 accumulator); optionally
 // (emax) the largest exponent field of the new P, which the next step's quantisation needs
-// q = round(p 2^(1078 - E)) by integer operations on the bits of p (|q| < 2^56 when the
-// exponent field of p is at most E); the same rounding as the quantisation kernels
-__device__ __forceinline__ long long quant_bits(double p, int E) {
-  const int hi = __double2hiint(p);
-  const unsigned lo = (unsigned)__double2loint(p);
-  const int ex = (hi >> 20) & 0x7ff;
-  long long q = 0;
-  if (ex != 0) {
-    const long long M = ((long long)((hi & 0xfffff) | 0x100000) << 32) | (long long)lo;  // p = M 2^(ex-1075)
-    const int sh = E - ex - 3;                                                           // q = M 2^-sh
-    if (sh <= 0) q = M << (-sh);
-    else if (sh < 62) q = (M + (1ll << (sh - 1))) >> sh;
-    if (hi < 0) q = -q;
-  }
-  return q;
-}
-
 // With Q: the next step's quantised copy is written here instead of by a separate pass.  Its
 // exponent must be fixed before any element is seen, so it is a bound: |P - gamma C| <
 // 2^(EP - 1022) + |gamma| 2^(EC - 1022), EP the largest exponent field pass 1 wrote, EC the
@@ -177,7 +161,7 @@ __global__ void __launch_bounds__(kThreads) k_lz_pass2(LzDev lz, const R* __rest
         if (X) x[k] = fma(xc, (double)c[u], x[k]);
         if constexpr (F64) {
           mx = max(mx, (int)((__double_as_longlong((double)p) >> 52) & 0x7ff));
-          if (qn.Q != nullptr) qn.Q[k] = quant_bits((double)p, Eq);
+          if (qn.Q != nullptr) qn.Q[k] = quant_one((double)p, Eq);
         }
       }
     }

@@ -38,6 +38,7 @@
 
 #include "common.cuh"
 #include "epilogue.cuh"
+#include "quant.cuh"
 #include "reduce.cuh"
 
 namespace hphi {
@@ -59,21 +60,6 @@ template <class S> struct TileUnit {
 // change of an entry's phase index on the thread's row r (its two bits per row bit, host-made)
 __device__ __forceinline__ uint32_t tile_flip(const TileEntry& en, int r) {
   return (((r & 1) ? en.flip : 0u) ^ ((r & 2) ? en.flip >> 2 : 0u) ^ ((r & 4) ? en.flip >> 4 : 0u)) & 3u;
-}
-
-// x to the 64-bit fixed point of exponent field E (the rounding of k_quant)
-__device__ __forceinline__ long long tile_quant(double x, int E) {
-  const int hi = __double2hiint(x);
-  const int ex = (hi >> 20) & 0x7ff;
-  long long q = 0;
-  if (ex != 0) {
-    const long long M = ((long long)((hi & 0xfffff) | 0x100000) << 32) | (long long)(unsigned)__double2loint(x);
-    const int sh = E - ex - 3;
-    if (sh <= 0) q = M << (-sh);
-    else if (sh < 62) q = (M + (1ll << (sh - 1))) >> sh;
-    if (hi < 0) q = -q;
-  }
-  return q;
 }
 
 // (ar, ai) += phase(code) * (xr, xi) of NR rows; one branch for all of them
@@ -219,8 +205,8 @@ __global__ void __launch_bounds__(kThreads, 3)
       for (int k = 0; k < kTileSteps; ++k) {
         const double2 x = __ldg(reinterpret_cast<const double2*>(v + (int64_t)(s0 | kbits(k)) * nvec + col));
         longlong2 q;
-        q.x = tile_quant(x.x, eq[0]);
-        q.y = tile_quant(x.y, eq[NC - 1]);
+        q.x = quant_one(x.x, eq[0]);
+        q.y = quant_one(x.y, eq[NC - 1]);
         *reinterpret_cast<longlong2*>(tb + off0 + k * kstride) = q;
       }
     }
