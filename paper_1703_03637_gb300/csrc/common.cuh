@@ -130,10 +130,9 @@ struct HubDev {
   const uint4* up_hdr[3];
   const uint32_t* nbr_up;
   const uint8_t* deg_up;
-  const uint8_t* npos_up;    // entries [0, npos) carry sign +1, [npos, deg) sign -1
   const uint32_t* nbr_dn;
   const uint8_t* deg_dn;
-  const uint8_t* npos_dn;
+  const uint8_t* npos_dn;    // entries [0, npos) carry sign +1, [npos, deg) sign -1
 };
 
 // Split-row view of a fixed-S^z sector (section 3.1's split of a configuration into a high
@@ -310,6 +309,7 @@ Status build_gather_table(const uint32_t* nbr, int64_t nbr_stride, const uint8_t
 
 // Two-pass Hubbard path (k_hub.cu): neighbour tables, and H v = diag + up hops (row tiles
 // in shared memory) + down hops (stripe-major row combinations into the scratch vector W).
+// npos (may be null): the number of a state's positive targets, which come first.
 Status build_hub_neighbours(const HubDev& md, int species, uint32_t* nbr, uint8_t* deg, uint8_t* npos,
                             cudaStream_t st);
 bool hub_fast_ok(const HubDev& md, int prec, bool cplx, int nvec, Epi epi);
@@ -322,7 +322,6 @@ size_t hub_scratch_bytes(const HubDev& md, int prec, Epi epi);  // scratch the l
 int* hub_exponent_slot(const HubDev& md, void* scratch);
 // fp64 H v of the two-pass path with its scratch in a fixed device array (no allocation)
 Status launch_hub_store_noalloc(const HubDev& md, const void* v, void* w, cudaStream_t st);
-size_t noalloc_capacity_bytes();
 Status launch_hub_fast(const HubDev& md, int prec, const void* v, void* w, void* scratch, Epi epi,
                        const FusedArgs& fa, int grid_up, cudaStream_t st);
 // resident CTAs of the chosen kernel instance over the whole GPU (occupancy API)

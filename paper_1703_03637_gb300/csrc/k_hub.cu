@@ -92,7 +92,7 @@ __global__ void k_hub_nbr(const HubDev md, int species, uint32_t* __restrict__ n
       if (pass == 0) np = cnt;
     }
     deg[k] = (uint8_t)cnt;
-    npos[k] = (uint8_t)np;
+    if (npos != nullptr) npos[k] = (uint8_t)np;
   }
 }
 
@@ -769,8 +769,6 @@ Status noalloc_scratch(void** out, cudaStream_t st) {
 }  // namespace
 
 HubDev with_shape(const HubDev& md, int prec);
-
-size_t noalloc_capacity_bytes() { return kNoAllocScratchBytes; }
 
 Status launch_hub_store_noalloc(const HubDev& md0, const void* v, void* w, cudaStream_t st) {
   const HubDev md = with_shape(md0, HPHI_FP64);

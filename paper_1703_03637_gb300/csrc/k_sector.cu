@@ -717,10 +717,6 @@ namespace {
 constexpr int kHiWarps = kThreads / 32;
 constexpr int kHiClaim = 4;  // items per warp per counter claim
 
-template <class T> struct SecAcc;
-template <> struct SecAcc<float> { using A = float; };
-template <> struct SecAcc<long long> { using A = long long; };
-
 // weight of exchange class c: fp32 the coefficient, fixed point the integer multiple
 template <class T>
 __device__ __forceinline__ T sec_w(const SecDev& d, int c);
