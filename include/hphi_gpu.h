@@ -174,14 +174,23 @@ typedef struct {
  * hphi_lanczos_run / hphi_tpq_run on this model.  The two-pass Hubbard path is tuned over
  * 16-byte pieces per lane of the down-spin pass x rows per tile of the up-spin pass.  Real spin
  * models in an S^z sector that take the split-row path (see hphi_set_sector_split) are tuned
- * over the split: the default low part, one bit more and up to two fewer, each with every tile height
- * that fits, and then over the high pass's columns per lane on the chosen split.  A real spin model in its full basis has every S^z sector of at least 2^20 rows
- * tuned that way: hphi_lanczos_run_sectors keeps those sectors' shapes; the result then
- * counts the candidates of all of them and reports the timings of the largest.  Other models
+ * over the split: the default low part at its default tile height, half and twice that, and one
+ * bit more or fewer at its default height, as far as they fit; then over the high pass's columns
+ * per lane on the chosen split.  A real spin model in its full basis has every S^z sector of at
+ * least 2^20 rows tuned that way: hphi_lanczos_run_sectors keeps those sectors' shapes; the result
+ * then counts the candidates of all of them and reports the timings of the largest.  Other models
  * report n_candidates = 0.  Uses the model's workspace (and the sectors' own); synchronises
  * the stream.  *out may be NULL.  No counterpart in the paper (its CPU code has no launch
  * shapes). */
 int hphi_autotune(hphi_model* m, int prec, hphi_tune_result* out, void* stream);
+
+/* Launch shape of the two-pass Hubbard path for precision prec: pieces = 1, 2 or 4 16-byte pieces
+ * per lane of the down-spin pass, rows = 1, 2 or 4 rows per shared-memory tile of the up-spin pass
+ * (at most as many as fit; two in fp64); 0 restores either default.  What hphi_autotune chooses,
+ * set by hand; the up-spin pass's table for that many rows is built here if it is not there yet
+ * (on `stream`, which is synchronised).  Returns HPHI_ERR_UNSUPPORTED for a model that does not
+ * take the path.  No counterpart in the paper. */
+int hphi_set_hubbard_shape(hphi_model* m, int prec, int pieces, int rows, void* stream);
 
 /* Split-row H v of real spin models in an S^z sector, section 3.1's split of a configuration
  * into a high and a low part (the split-half search) turned into the data layout: the rows
@@ -196,9 +205,10 @@ int hphi_autotune(hphi_model* m, int prec, hphi_tune_result* out, void* stream);
  * L = -1 turns the path off (generic kernel), L = 0 restores the default (14 bits in fp64, 15
  * in fp32, fewer on small clusters), 1..20 forces the low part's length; K = 0 picks 16-byte
  * tile entries (two fp64 or four fp32 rows) if they fit, 1/2/4/8 forces the rows per tile.  The
- * high-part combinations use a shorter split of their own (12 bits where the tables allow).  The device tables of
- * the split are built here (a host loop over 2^L low and 2^(N-L) high parts, then an upload
- * on `stream`, which is synchronised).  Results agree with the generic kernel to rounding
+ * high-part combinations use a shorter split of their own (12 bits where the tables allow).  The
+ * device tables of the split are built here on `stream`, which is synchronised: the lists of low
+ * and high parts by a host loop and an upload, the gather table and the high-part combinations'
+ * tables by kernels (the latter once per model).  Results agree with the generic kernel to rounding
  * (fp32) or exactly up to the final conversion (fp64 fixed-point sums).  Returns
  * HPHI_ERR_UNSUPPORTED (with the reason) for a model the path does not cover and
  * HPHI_ERR_INVALID_ARG when the forced split does not fit.  No counterpart in the paper. */

@@ -30,7 +30,7 @@ EXPORTS = [
     "hphi_build_sector", "hphi_dim", "hphi_is_complex", "hphi_basis_states", "hphi_basis_ranks", "hphi_apply_H",
     "hphi_random_vector", "hphi_philox4x32_10", "hphi_lanczos_run", "hphi_tpq_run", "hphi_apply_H_noalloc",
     "hphi_lanczos_run_sectors", "hphi_autotune", "hphi_set_window_bits", "hphi_set_sector_split",
-    "hphi_release_workspace", "hphi_inverse_iteration",
+    "hphi_release_workspace", "hphi_inverse_iteration", "hphi_set_hubbard_shape",
 ]
 
 
@@ -129,6 +129,7 @@ def load(build_if_missing: bool = True):
         L.hphi_autotune.argtypes = [P, I, ctypes.POINTER(TuneResult), P]
         L.hphi_set_window_bits.argtypes = [P, I]
         L.hphi_set_sector_split.argtypes = [P, I, I, I, P]
+        L.hphi_set_hubbard_shape.argtypes = [P, I, I, I, P]
         L.hphi_release_workspace.argtypes = [P]
         L.hphi_inverse_iteration.argtypes = [P, ctypes.POINTER(InvitParams), P, ctypes.POINTER(InvitResult), P]
         L.hphi_lanczos_run_sectors.argtypes = [P, P, I, ctypes.POINTER(LanczosParams), ctypes.POINTER(LanczosResult), P]
@@ -279,6 +280,12 @@ class Model:
         return dict(n_candidates=r.n_candidates, dn_ept=r.best_dn_ept, up_k=r.best_up_k, best_ms=r.best_ms,
                     default_ms=r.default_ms, worst_ms=r.worst_ms, split_L=r.best_split_L, split_K=r.best_split_K,
                     split_hi_cols=r.best_split_hi_cols)
+
+    def set_hubbard_shape(self, prec=FP64, pieces: int = 0, rows: int = 0):
+        """Two-pass Hubbard path (see hphi_set_hubbard_shape): 16-byte pieces per lane of the down-spin
+        pass and rows per tile of the up-spin pass; 0 restores a default."""
+        _torch()
+        self._check(self._L.hphi_set_hubbard_shape(self._h, prec, int(pieces), int(rows), _stream()))
 
     def set_sector_split(self, prec=FP64, L: int = 0, K: int = 0):
         """Split-row spin path (see hphi_set_sector_split): L = -1 off, 0 default, else the low

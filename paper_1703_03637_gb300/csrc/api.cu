@@ -1411,6 +1411,30 @@ int hphi_autotune(hphi_model* m, int prec, hphi_tune_result* out, void* stream) 
   return HPHI_OK;
 }
 
+int hphi_set_hubbard_shape(hphi_model* m, int prec, int pieces, int rows, void* stream) {
+  int rc = check_built(m);
+  if (rc) return rc;
+  if (prec != HPHI_FP64 && prec != HPHI_FP32) return fail(m, HPHI_ERR_INVALID_ARG, "set_hubbard_shape: prec FP64 or FP32");
+  auto known = [](int x) { return x == 0 || x == 1 || x == 2 || x == 4; };
+  if (!known(pieces) || !known(rows))
+    return fail(m, HPHI_ERR_INVALID_ARG, "set_hubbard_shape: pieces and rows in {0, 1, 2, 4}");
+  if (!use_hub_fast(m, prec, 1, hphi::Epi::kStore))
+    return fail(m, HPHI_ERR_UNSUPPORTED, "set_hubbard_shape: the model does not take the two-pass Hubbard path");
+  const int pi = prec == HPHI_FP64 ? 0 : 1;
+  const int old_pieces = m->hdev.tuned_ept[pi], old_rows = m->hdev.tuned_k[pi];
+  m->hdev.tuned_ept[pi] = pieces;
+  m->hdev.tuned_k[pi] = rows;
+  hphi::Status s = hub_ensure_table(m, prec, (cudaStream_t)stream);
+  if (s.code == 0 && cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess)
+    s = {HPHI_ERR_CUDA, std::string("set_hubbard_shape: ") + cudaGetErrorString(cudaGetLastError())};
+  if (s.code) {
+    m->hdev.tuned_ept[pi] = old_pieces;
+    m->hdev.tuned_k[pi] = old_rows;
+    return fail(m, s);
+  }
+  return HPHI_OK;
+}
+
 int hphi_apply_H_noalloc(hphi_model* m, const void* v, void* w, void* stream) {
   int rc = check_built(m);
   if (rc) return rc;
