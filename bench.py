@@ -140,17 +140,28 @@ def l2_note(vector_bytes: int) -> str:
     return f"vectors ({vector_bytes / 1e6:.2f} MB) fit in L2: on-chip workload, no flush"
 
 
-def hv_group_name(spec, m, prec, nvec, what):
+def tile_passes_run(spec, m, prec, nvec, sms):
+    """Whether the library's tile passes take a full-basis block: a power of two of vectors in rows of
+    at least 64 bytes, and two 64 KB tiles for every SM."""
+    import paper_1703_03637_gb300 as hp
+    row = nvec * (8 if prec == hp.FP64 else 4) * (2 if m.is_complex else 1)
+    return (13 <= spec.n_sites <= 32 and 2 <= nvec <= 256 and nvec & (nvec - 1) == 0 and row >= 64
+            and (row << spec.n_sites) >> 16 >= 2 * sms)
+
+
+def hv_group_name(spec, m, prec, nvec, what, sms=None):
     """The kernels of one fused H v launch group, as the library picks them."""
     import paper_1703_03637_gb300 as hp
+    if sms is None:
+        import torch
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
     kind = "spin" if spec.kind == wl.SPIN else "hubbard"
     if kind == "hubbard" and not m.is_complex:
         ks = "k_maxexp + k_quant + k_hub_dn + k_hub_up" if prec == hp.FP64 else "k_hub_dn + k_hub_up"
+    elif kind == "spin" and spec.basis == wl.BASIS_FULL and tile_passes_run(spec, m, prec, nvec, sms):
+        ks = "k_maxexp_cols + k_hv_tile" if prec == hp.FP64 else "k_hv_tile"
     elif kind == "spin" and spec.basis == wl.BASIS_FULL and nvec in (32, 64, 128, 256):
-        if spec.n_sites >= 16:  # enough tiles for the tile passes
-            ks = "k_maxexp_cols + k_hv_tile" if prec == hp.FP64 else "k_hv_tile"
-        else:
-            ks = "k_maxexp_cols + k_quant_cols + k_hv_batch" if prec == hp.FP64 else "k_hv_batch"
+        ks = "k_maxexp_cols + k_quant_cols + k_hv_batch" if prec == hp.FP64 else "k_hv_batch"
     else:
         ks = "k_hv_hub" if kind == "hubbard" else "k_hv_spin"
     return f"{ks} ({what})"
