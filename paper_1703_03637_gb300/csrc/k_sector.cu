@@ -315,9 +315,12 @@ std::string straddle_limits(const Analysis& a, int L) {
 }
 
 // Pass H's split.  Rows of C(12, 6) = 924 entries fill 128-column stripes to nine tenths; fp64
-// Lanczos group (pass H + pass R) at hL = 9 / 10 / 11 / 12 / 13 on GB300: 6x5 torus, S^z = 0
-// 4.69 / 4.18 / 3.98 / 3.98 / 3.95 ms; 28-site J1-J2 ring, 9 up 0.50 / 0.40 / 0.36 / 0.33 ms
-// (at 9 bits a row's part-filled stripes cost more than the bonds it takes over).
+// Lanczos group (pass H + pass R) on GB300 at hL = 9 / 10 / 11 / 12 / 13, 6x5 torus, S^z = 0:
+// 4.69 / 4.18 / 3.98 / 3.98 / 3.95 ms, and at 9 / 10 / 11 / 12, 28-site J1-J2 ring, 9 up:
+// 0.50 / 0.40 / 0.36 / 0.33 ms (at 9 bits a row's part-filled stripes cost more than the bonds it
+// takes over; 13 is within 1 % of 12).  Both sizes' stripes fit L2 (50 MB on 6x5).  On 36 sites the
+// largest class's stripe is C(24, 12) KB = 2.8 GB and partner reads go to DRAM; a longer split for
+// that size is not measured.
 int high_L(int N, int L) { return std::min(L, std::max(kSecHighL, N - kSecMaxHH)); }
 
 }  // namespace
@@ -1302,13 +1305,9 @@ Status launch_hi(const SecDev& d, const T* X, T* W, const int* done, unsigned lo
   HPHI_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st));
   const int grid = num_sms() * 8;
   const bool one = d.one_cls != 0;
-  // 1 KB row stripes per warp item (4 int64 / 8 fp32 columns per lane).  The kernel is bound by
-  // instruction issue (64-bit adds, addresses, neighbour lists), so wider stripes spread each
-  // neighbour's overhead over more columns: on the 6x6 sector 256-byte stripes measured 185 ms,
-  // 512-byte 124 ms, and 1 KB about 2.5 % less again, although one stripe of the largest class
-  // (360 MB) then far exceeds L2.
-  // The autotuner may halve them (d.hi_cols): on the 6x6 sector a 1 KB stripe of the largest
-  // class is 360 MB, so the partner reads partly come from DRAM.
+  // 1 KB row stripes per warp item (4 int64 / 8 fp32 columns per lane): wide stripes spread each
+  // partner's address arithmetic and offset read over more columns.  The autotuner may halve them
+  // (d.hi_cols), which halves the stripe of a class that should stay in L2.
   constexpr int EPT = sizeof(T) == 8 ? 4 : 8;
   if (d.hi_cols == EPT / 2) {
     if (one) k_sec_hi<T, EPT / 2, true><<<grid, kThreads, 0, st>>>(d, X, W, done, counter);
