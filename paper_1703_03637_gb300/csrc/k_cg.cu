@@ -10,7 +10,7 @@
 // anyway.  On the fixed-point paths the direction kernel also finds the new direction's largest
 // exponent, so the next product quantises it on its own scale without a scan.
 // 32 iterations on 24 sites (2.7 million rows) on GB300: 5.5 ms; 6.3 ms with a scan and a separate
-// shift pass per product (11 launches an iteration instead of 7).
+// shift pass per product (9 kernels an iteration instead of 7).
 //
 // Every kernel streams its vectors once with four elements per thread one grid stride apart
 // and leaves one fp64 partial sum per CTA; a one-CTA finaliser turns the partials into the

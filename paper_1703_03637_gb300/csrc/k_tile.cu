@@ -27,7 +27,8 @@
 //
 // Measured on GB300, one mTPQ step of 64 starts against the gather kernel: 2^24 rows c64 26.3 ms
 // instead of 49.4 ms (three passes; bound by shared-memory wavefronts, 73 %, with DRAM at 48 %),
-// 2^18 rows c128 1.81 ms instead of 1.99 ms (two passes; bound by the fp64 pipe, 64 to 76 %);
+// 2^18 rows c128 1.60 ms instead of 1.99 ms (two passes: 0.47 ms, issue 59 % and integer pipe 56 %, and
+// 1.07 ms with the diagonal and the epilogue, fp64 pipe 69 %; 1.81 ms with a conversion per class and pass);
 // 16 starts, 2^24 rows c64 28.2 instead of 156 ms for four steps.
 #include <math.h>
 

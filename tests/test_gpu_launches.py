@@ -1,5 +1,7 @@
 """The launch counts that results report, kernel by kernel, below and above the size up to which one
 kernel scans and quantises an fp64 vector."""
+import gc
+
 import pytest
 
 import workloads as wl
@@ -47,6 +49,7 @@ def test_high_part_tables_are_shared():
     """Pass H's tables (12 bytes for each of 2^22 high parts here) belong to the sector: neither the
     second precision nor another split of the row pass adds a copy."""
     def used():
+        gc.collect()  # models of earlier tests
         torch.cuda.synchronize()
         free, total = torch.cuda.mem_get_info()
         return total - free
