@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(kGtWarps * 32) k_gather_table(const uint32_t* 
       s_load[wid][lane] = 0;
       __syncwarp();
       for (int i = 0; i < cnt; ++i) atomicAdd(&load[list[i * 32 + lane] % W], 1);
+      __syncwarp();  // all lanes' terms are counted
       const int m = __reduce_max_sync(0xffffffffu, cnt);
       int useb, loadb = s_load[wid][lane];  // bank `me` of this bank pass: uses in the slot, terms left
       for (int q = 0; q < m; ++q) {
