@@ -423,7 +423,6 @@ hphi::Status compile_spin(hphi_model* m, cudaStream_t st) {
       q.holes = th[k].holes[p];
       q.fix_shift = th[k].fix_shift;
       q.fix_exp = th[k].fix_exp;
-      q.fix_half = th[k].fix_half;
       memcpy(q.pos, th[k].pos[p], sizeof(q.pos));
     }
   }

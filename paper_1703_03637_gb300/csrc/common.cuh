@@ -377,9 +377,9 @@ struct TilePass {
   const uint32_t* dep = nullptr;  // [4][256] visit-index byte -> row bits (the set's sites first)
   int n_ent = 0, t = 0, first = 0;
   // fp64: the class coefficients as integers, c 2^(64 - exp - shift), the sums' left shift before
-  // the product with them, the exponent of the products' unit and half a unit per inexact product
+  // the product with them and the exponent of the products' unit
   const longlong2* fix = nullptr;
-  int fix_shift = 0, fix_exp = 0, fix_half = 0;
+  int fix_shift = 0, fix_exp = 0;
   int holes = 0;                  // some entry's element is zero for some settings of its bits
   uint8_t pos[12] = {};           // local row bit -> site
 };
@@ -391,7 +391,7 @@ struct TilePlan {
 struct TileHost {                 // a plan's tables before their upload
   int n_pass = 0;
   bool f64 = false;
-  int fix_shift = 0, fix_exp = 0, fix_half = 0;
+  int fix_shift = 0, fix_exp = 0;
   std::vector<longlong2> fix;
   int e0[kMaxPasses + 1] = {};
   int holes[kMaxPasses] = {};

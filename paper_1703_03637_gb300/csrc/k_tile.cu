@@ -21,14 +21,14 @@
 //
 // fp64 quantises the rows while staging them (one scale per column, q = round(x 2^(1078 - E_c))),
 // sums each class's run exactly in 64-bit integers and multiplies the sums by the class
-// coefficients in fixed point (high halves of 64 x 64-bit products, tile_fix).  The partial sums
+// coefficients in fixed point (rounded high halves of 64 x 64-bit products, tile_fix).  The partial sums
 // stay integers from pass to pass; the last one converts once, so an element is rounded twice, in
 // the conversion and with the diagonal, whatever the number of classes and passes.
 //
 // Measured on GB300, one mTPQ step of 64 starts against the gather kernel: 2^24 rows c64 26.3 ms
 // instead of 49.4 ms (three passes; bound by shared-memory wavefronts, 73 %, with DRAM at 48 %),
-// 2^18 rows c128 1.60 ms instead of 1.99 ms (two passes: 0.47 ms, issue 59 % and integer pipe 56 %, and
-// 1.07 ms with the diagonal and the epilogue, fp64 pipe 69 %; 1.81 ms with a conversion per class and pass);
+// 2^18 rows c128 1.62 ms instead of 1.99 ms (two passes: 0.48 ms, issue 59 % and integer pipe 56 %, and
+// 1.08 ms with the diagonal and the epilogue, fp64 pipe 69 %; 1.81 ms with a conversion per class and pass);
 // 16 starts, 2^24 rows c64 28.2 instead of 156 ms for four steps.
 #include <math.h>
 
@@ -61,6 +61,11 @@ template <class S> struct TileUnit {
 // change of an entry's phase index on the thread's row r (its two bits per row bit, host-made)
 __device__ __forceinline__ uint32_t tile_flip(const TileEntry& en, int r) {
   return (((r & 1) ? en.flip : 0u) ^ ((r & 2) ? en.flip >> 2 : 0u) ^ ((r & 4) ? en.flip >> 4 : 0u)) & 3u;
+}
+
+// a b / 2^64, rounded to nearest (so a zero sum stays zero)
+__device__ __forceinline__ long long tile_mul(long long a, long long b) {
+  return (long long)(((__int128)a * b + ((__int128)1 << 63)) >> 64);
 }
 
 // (ar, ai) += phase(code) * (xr, xi) of NR rows; one branch for all of them
@@ -239,11 +244,11 @@ __global__ void __launch_bounds__(kThreads, 3)
 #pragma unroll
           for (int r = 0; r < NR; ++r) {
             const long long v0 = ac[r][0] << tp.fix_shift, v1 = ac[r][1] << tp.fix_shift;
-            hs[r][0] += __mul64hi(v0, cf.x);
-            hs[r][1] += __mul64hi(v1, cf.x);
+            hs[r][0] += tile_mul(v0, cf.x);
+            hs[r][1] += tile_mul(v1, cf.x);
             if (C && cf.y != 0) {
-              hs[r][0] += __mul64hi(v1, -cf.y);
-              hs[r][1] += __mul64hi(v0, cf.y);
+              hs[r][0] -= tile_mul(v1, cf.y);
+              hs[r][1] += tile_mul(v0, cf.y);
             }
           }
 #pragma unroll
@@ -318,7 +323,7 @@ __global__ void __launch_bounds__(kThreads, 3)
           R hv[NW];
 #pragma unroll
           for (int e = 0; e < NW; ++e) {
-            if constexpr (F64) hv[e] = fma(d, x0[e], fix_to_double(hs[r][e] + tp.fix_half, eq[C ? 0 : e] + tp.fix_exp - 1078));
+            if constexpr (F64) hv[e] = fma(d, x0[e], fix_to_double(hs[r][e], eq[C ? 0 : e] + tp.fix_exp - 1078));
             else hv[e] = fma(d, x0[e], hs[r][e]);
           }
           if constexpr (E == Epi::kTpq) {
@@ -412,12 +417,11 @@ Status launch_s(const SpinDev& md, const TilePlan& plan, const void* v, void* w,
 // The integers of fp64.  A class sum S of a pass is below 2^56 times its longest run, so
 // S 2^shift fits 63 bits with shift = 7 - log2(run); the coefficients times 2^s fit 63 bits with
 // s = 62 - log2(c_max); and the sum of all products over 2^64 must stay below 2^62, which lowers
-// first the shift, then s.  A product is exact when the coefficient's trailing zeros and the shift
-// make up 64 bits (c = +-2^k), else its floor is half a unit low on average: fix_half makes up for
-// these.  Against the whole vector the
-// products' floors are below the rounding of the elements (rms over the norm, 18-site Heisenberg ring
-// in a field of 1e-3: 0.60 2^-53, the gather kernel 0.77); rows that only a coefficient c reaches lose a further c_max / (12 c) of
-// their own rounding, so models whose coefficients span more than 1,024 keep to the gather kernels.
+// first the shift, then s.  Products are rounded to nearest (with a shift of two or more those with
+// c_max = 2^k are exact); against the whole vector that is below the rounding of the elements (rms over
+// the norm, 18-site Heisenberg ring in a field of 1e-3: 0.60 2^-53, the gather kernel 0.77).  Rows that
+// only a coefficient c reaches lose a further c_max / (12 c) of their own rounding, so models whose
+// coefficients span more than 1,024 keep to the gather kernels.
 static void tile_fix(const std::vector<SpinEntry>& ents, const std::vector<double2>& cls, TileHost* out) {
   double cmax = 0.0, cmin = 1e308, sum = 0.0;
   for (const SpinEntry& e : ents) {
@@ -447,18 +451,8 @@ static void tile_fix(const std::vector<SpinEntry>& ents, const std::vector<doubl
     out->fix_shift = 0;
   }
   out->fix_exp = 64 - s - out->fix_shift;
-  auto fixed = [&](double c, int* inexact) -> long long {
-    const long long v = std::llrint(std::ldexp(c, s));
-    if (v != 0 && __builtin_ctzll((unsigned long long)v) + out->fix_shift < 64) *inexact += 1;
-    return v;
-  };
-  std::vector<int> floors(cls.size(), 0);  // per component
-  for (size_t k = 0; k < cls.size(); ++k) out->fix[k] = longlong2{fixed(cls[k].x, &floors[k]), fixed(cls[k].y, &floors[k])};
-  int n = 0;
-  for (int p = 0; p < out->n_pass; ++p)
-    for (int k = out->e0[p]; k < out->e0[p + 1]; ++k)
-      if (k == out->e0[p] || out->ents[k].cls != out->ents[k - 1].cls) n += floors[out->ents[k].cls];
-  out->fix_half = n / 2;
+  for (size_t k = 0; k < cls.size(); ++k)
+    out->fix[k] = longlong2{std::llrint(std::ldexp(cls[k].x, s)), std::llrint(std::ldexp(cls[k].y, s))};
 }
 
 // Covers the flip masks by site sets of at most t sites: the set grows by the mask that covers

@@ -189,3 +189,23 @@ def test_block_products_round_twice(mk, n, hx, nvec):
         assert float((off @ off) / (ref @ ref)) < 1.1 ** 2
         err = w[:, c].astype(L) - ref
         assert float(np.sqrt((err @ err) / (ref @ ref))) <= 0.63 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("mk,nvec", [(lambda: wl.kitaev_honeycomb(4, 2), 64), (lambda: wl.kitaev_honeycomb(4, 2, h=0.3), 32),
+                                     (lambda: wl.random_spin_model(16, 12, seed=21), 64)],
+                         ids=["kitaev", "kitaev-strong-field", "random"])
+def test_block_products_keep_zeros(mk, nvec):
+    """fp64 blocks of basis vectors: an element without a matrix element to its column's basis vector is
+    zero, and so is a zero column, also where the coefficients' products are rounded."""
+    spec = mk()
+    m = hp.Model.from_spec(spec)
+    rng = np.random.default_rng(12)
+    rows = rng.integers(0, m.dim, nvec - 1)
+    v = np.zeros((m.dim, nvec), dtype=np.complex128 if m.is_complex else np.float64)
+    v[rows, np.arange(nvec - 1)] = rng.uniform(0.5, 2, nvec - 1)
+    w = m.apply_H(torch.as_tensor(v).cuda()).cpu().numpy()
+    assert not w[:, -1].any()
+    for c in range(0, nvec - 1, 7):
+        allowed = {rows[c]} | {rows[c] ^ (1 << i) ^ (1 << j) for i, j, _ in spec.couplings}
+        allowed |= {rows[c] ^ (1 << i) for i in range(spec.n_sites)}  # fields, and S^z times S^x or S^y
+        assert set(np.nonzero(w[:, c])[0].tolist()) <= allowed
